@@ -28,6 +28,8 @@ constexpr int64_t kMaxChannelElems = 65535; // one-CTA paths: keeps the clamp-ed
                                             // kernel, which checks every candidate against the clip range
 constexpr int64_t kMaxKernels = (1 << sq::kIdxBits) - 1;   // kernels per channel: the select keys hold 18 index bits
 constexpr size_t kMaxPlans = 64;
+constexpr int kWideSmemGoal = 112 << 10;     // the same of a cluster's thread block: two of them
+constexpr int kGroupedSmemGoal = 55 << 10;   // shared memory of a grouped CTA with which four of them share a multiprocessor
 
 std::mutex g_mutex;
 std::atomic<int64_t> g_launches{0};
@@ -46,6 +48,7 @@ int cuda_fail(cudaError_t e, const char *what)
     } while (0)
 
 inline int align16(int v) { return (v + 15) & ~15; }
+inline int64_t align16_64(int64_t v) { return (v + 15) & ~static_cast<int64_t>(15); }
 
 struct HostPlan {
     std::vector<LayerDesc> layers;
@@ -102,6 +105,28 @@ int validate(const squant_layer *layers, int32_t n_layers, const squant_options 
     return SQUANT_OK;
 }
 
+// Layout of a channel with staged weights and per-kernel arrays: the pipelined kernel's layers, E|C on
+// larger kernels, 1x1 rows beyond the registers of one thread block.
+void layout_staged(const squant_layer &l, LayerDesc &d, unsigned mode)
+{
+    d.g = group_size(d.NK);
+    d.g_shift = 0;
+    while ((1 << d.g_shift) < d.g) ++d.g_shift;
+    int off = align16(4 * d.NK);              // staged weights
+    d.off_codes = off; off += align16(d.NK);  // staged codes
+    const bool ec_only = (mode & SQUANT_MODE_C) && !(mode & SQUANT_MODE_K);   // elements are the candidates
+    if ((d.K == 1 || ec_only) && !l.scales_in) {   // perturbations overwrite the weights
+        d.off_ev = 0; d.off_vv = 0; d.off_vi = 0;
+    } else {
+        d.off_ev = off; off += align16(4 * d.N);
+        d.off_vv = off; off += align16(4 * d.N);
+        d.off_vi = off; off += align16(2 * d.N);
+    }
+    d.off_hist = off; off += 4 * sq::kHistBins;
+    d.off_red = off; off += 256;
+    d.slice_bytes = off;
+}
+
 // Device-side descriptor of one layer: group size and the layout of a group's shared-memory
 // slice.  Returns the dynamic shared memory one CTA needs for this layer.
 int64_t layout_layer(const squant_layer &l, LayerDesc &d, unsigned mode, unsigned flags)
@@ -122,20 +147,32 @@ int64_t layout_layer(const squant_layer &l, LayerDesc &d, unsigned mode, unsigne
         d.slice_bytes = align16(5 * d.K);
         return static_cast<int64_t>(sq::kCtaThreads) * d.slice_bytes;
     }
-    int off = align16(4 * d.NK);              // staged weights
-    d.off_codes = off; off += align16(d.NK);  // staged codes
-    const bool ec_only = (mode & SQUANT_MODE_C) && !(mode & SQUANT_MODE_K);   // elements are the candidates
-    if ((d.K == 1 || ec_only) && !l.scales_in) {   // perturbations overwrite the weights
-        d.off_ev = 0; d.off_vv = 0; d.off_vi = 0;
-    } else {
-        d.off_ev = off; off += align16(4 * d.N);
-        d.off_vv = off; off += align16(4 * d.N);
-        d.off_vi = off; off += align16(2 * d.N);
+    if (d.K == 1) {   // a channel that fits the registers of at most one thread block: no staging
+        const int first = static_cast<int>((reinterpret_cast<uintptr_t>(l.w) >> 2) & 3);
+        const int vecs = (d.N & 3) ? (d.N + 6) >> 2 : (d.N + first + 3) >> 2;   // of the most misaligned row
+        const int g = sq::row_group(vecs);
+        if (g) {
+            d.g = g;
+            d.g_shift = 0;
+            while ((1 << d.g_shift) < d.g) ++d.g_shift;
+            d.off_codes = 0; d.off_ev = 0; d.off_vv = 0; d.off_vi = vecs; d.off_hist = 0; d.off_red = 0;
+            d.slice_bytes = align16(sq::row_bytes(g, vecs));
+            return static_cast<int64_t>(sq::kCtaThreads / d.g) * d.slice_bytes;
+        }
     }
-    d.off_hist = off; off += 4 * sq::kHistBins;
-    d.off_red = off; off += 256;
-    d.slice_bytes = off;
-    return static_cast<int64_t>(sq::kCtaThreads / d.g) * off;
+    if (d.K > 1 && !((mode & SQUANT_MODE_C) && !(mode & SQUANT_MODE_K))) {   // kernels: a thread settles up to four of them (larger than 3x3: two)
+        const int per = d.K <= 9 ? 4 : 2;
+        int g = 32;
+        while (g < sq::kCtaThreads && (per * g < d.N || sq::kCtaThreads / g * sq::conv_bytes(g, d.NK, d.K) > kGroupedSmemGoal)) g *= 2;
+        d.g = g;
+        d.g_shift = 0;
+        while ((1 << d.g_shift) < d.g) ++d.g_shift;
+        d.off_codes = 0; d.off_ev = 0; d.off_vv = 0; d.off_vi = 0; d.off_hist = 0; d.off_red = 0;
+        d.slice_bytes = align16(sq::conv_bytes(g, d.NK, d.K));
+        return static_cast<int64_t>(sq::kCtaThreads / d.g) * d.slice_bytes;
+    }
+    layout_staged(l, d, mode);
+    return static_cast<int64_t>(sq::kCtaThreads / d.g) * d.slice_bytes;
 }
 
 // Work list in a table (global-memory variant): CTA-sized items, heaviest first.
@@ -153,7 +190,9 @@ int build_plan(const squant_layer *layers, int32_t n_layers, const squant_option
         LayerDesc &d = p.layers[i];
         const int64_t cta_smem = layout_layer(layers[i], d, o.mode, o.flags);
         const int groups = sq::kCtaThreads / d.g;
-        if (cta_smem > max_smem) return SQUANT_ERR_TOO_WIDE;
+        LayerDesc staged = d;
+        layout_staged(layers[i], staged, o.mode);   // (the limit: a channel staged with its per-kernel arrays)
+        if (cta_smem > max_smem || static_cast<int64_t>(sq::kCtaThreads / staged.g) * staged.slice_bytes > max_smem) return SQUANT_ERR_TOO_WIDE;
         if (cta_smem > p.smem_bytes) p.smem_bytes = static_cast<int>(cta_smem);
         for (int c = 0; c < d.M; c += groups) {
             const int nch = (d.M - c < groups) ? d.M - c : groups;
@@ -179,6 +218,9 @@ struct ParamPlan {
     // cluster kernel (channels wider than one CTA): one launch per layer
     struct Wide { LayerDesc d; int cluster, kpc, smem; };
     std::vector<Wide> wide;
+    // row kernel (1x1 rows too long for a group): one item per output channel
+    std::vector<sq::LaunchTable> row_tables;
+    std::vector<int> row_grids, row_smem;
     // pipelined kernel (layers of long 3x3 channels): one item per output channel
     std::vector<sq::LaunchTable> pipe_tables;
     std::vector<int> pipe_items, pipe_set_stride, pipe_slot;
@@ -229,28 +271,67 @@ int build_param_plan(const squant_layer *layers, int32_t n_layers, const squant_
              ((o.flags & SQUANT_FLAG_NARROW_RANGE) ? 0u : sq::kModeWideRange);
     p.smem_bytes = 0;
     std::vector<LayerDesc> descs(n_layers);
-    std::vector<int> order, piped, streamed;
+    std::vector<int> order, piped, streamed, rows;
     for (int i = 0; i < n_layers; ++i) {
         const int64_t cta_smem = layout_layer(layers[i], descs[i], o.mode, o.flags);
         if (cta_smem > max_smem || descs[i].NK > kMaxChannelElems) {
             // a cluster of 2, 4 or 8 CTAs per output channel, each with an even number of kernels
             if ((o.mode & SQUANT_MODE_C) && !(o.mode & SQUANT_MODE_K) && descs[i].K > 1) return SQUANT_ERR_TOO_WIDE;   // E|C selects among elements: one CTA only
+            // (the limit: what eight of them hold at 5 B a weight and 10 B a larger kernel)
             ParamPlan::Wide w{descs[i], 0, 0, 0};
-            for (int c = 2; c <= sq::kWideMaxCluster && !w.cluster; c *= 2) {
-                const int kpc = (((descs[i].N + c - 1) / c) + 1) & ~1;
-                const sq::WideLayout wl = sq::wide_layout(kpc, descs[i].K);
-                if (wl.total <= max_smem) { w.cluster = c; w.kpc = kpc; w.smem = wl.total; }
+            const int64_t k8 = (((descs[i].N + 7) / 8) + 1) & ~1;
+            if (align16_64(4 * k8 * descs[i].K) + align16_64(k8 * descs[i].K) + (descs[i].K > 1 ? 2 * align16_64(4 * k8) + align16_64(2 * k8) : 0) + 2304 > max_smem)
+                return SQUANT_ERR_TOO_WIDE;
+            // two thread blocks per multiprocessor if the channel can be cut that small: while one waits for its
+            // weights or for its cluster the other works
+            for (int goal = kWideSmemGoal;; goal = max_smem) {
+                for (int c = 2; c <= sq::kWideMaxCluster && !w.cluster; c *= 2) {
+                    const int kpc = (((descs[i].N + c - 1) / c) + 3) & ~3;
+                    const int64_t bytes = sq::wide_bytes(kpc, descs[i].K);
+                    if (bytes <= goal) { w.cluster = c; w.kpc = kpc; w.smem = static_cast<int>(bytes); }
+                }
+                if (w.cluster || goal == max_smem) break;
             }
             if (!w.cluster) return SQUANT_ERR_TOO_WIDE;
+            w.d.off_vi = (w.kpc + 6) >> 2;
             p.wide.push_back(w);
             continue;
         }
-        if (pipe_eligible(layers[i], descs[i], o, max_smem)) {
+        LayerDesc staged = descs[i];
+        layout_staged(layers[i], staged, o.mode);
+        if (pipe_eligible(layers[i], staged, o, max_smem)) {
+            descs[i] = staged;
             (stream_eligible(layers[i], descs[i], o, max_smem) ? streamed : piped).push_back(i);
+            continue;
+        }
+        if (descs[i].K == 1 && descs[i].off_hist != 0 && descs[i].N <= sq::kRowBlockElems) {   // too long for a group, 164 KB at most
+            rows.push_back(i);
             continue;
         }
         if (cta_smem > p.smem_bytes) p.smem_bytes = static_cast<int>(cta_smem);
         order.push_back(i);
+    }
+    // long rows, longest first: a thread block per output channel
+    std::stable_sort(rows.begin(), rows.end(), [&](int a, int b) { return descs[a].N > descs[b].N; });
+    for (size_t base = 0; base < rows.size(); base += sq::kMaxParamLayers) {
+        const int n = static_cast<int>(std::min<size_t>(rows.size() - base, sq::kMaxParamLayers));
+        p.row_tables.emplace_back();
+        sq::LaunchTable &t = p.row_tables.back();
+        std::memset(&t, 0, sizeof(t));
+        t.n_layers = n;
+        for (int st = 1; st < n; st <<= 1) t.top_step = st;
+        int items = 0, smem = 0;
+        for (int j = 0; j < n; ++j) {
+            LayerDesc d = descs[rows[base + j]];
+            d.off_vi = (d.N + 6) >> 2;
+            smem = std::max(smem, sq::row_bytes(sq::kBlockThreads, d.off_vi, sq::kBlock));
+            t.layers[j] = d;
+            t.first_item[j] = items;
+            items += d.M;
+        }
+        for (int j = n; j <= sq::kMaxParamLayers; ++j) t.first_item[j] = items;
+        p.row_grids.push_back(items);
+        p.row_smem.push_back(smem);
     }
     for (int kind = 0; kind < 2; ++kind) {
     const std::vector<int> &piped_k = kind ? streamed : piped;
@@ -362,6 +443,8 @@ int device_smem_limit(int device, int &limit)
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, v));
         SQ_CUDA(cudaFuncSetAttribute(sq::squant_pipe_kernel,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, v));
+        SQ_CUDA(cudaFuncSetAttribute(sq::squant_row_kernel,
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, v));
         SQ_CUDA(cudaFuncSetAttribute(sq::squant_wide_kernel,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, v));
         SQ_CUDA(cudaFuncSetAttribute(sq::squant_stream_kernel,
@@ -454,6 +537,11 @@ int launch_plan(const ParamPlan &p, cudaStream_t stream)
         SQ_CUDA(cudaGetLastError());
         g_launches.fetch_add(1, std::memory_order_relaxed);
     }
+    for (size_t c = 0; c < p.row_tables.size(); ++c) {
+        sq::squant_row_kernel<<<p.row_grids[c], sq::kBlockThreads, p.row_smem[c], stream>>>(p.row_tables[c], p.qmax, p.mode);
+        SQ_CUDA(cudaGetLastError());
+        g_launches.fetch_add(1, std::memory_order_relaxed);
+    }
     for (size_t c = 0; c < p.tables.size(); ++c) {
         if (p.grids[c] == 0) continue;
         sq::squant_model_kernel<<<p.grids[c], sq::kCtaThreads, p.smem_bytes, stream>>>(p.tables[c], p.qmax, p.mode);
@@ -463,7 +551,7 @@ int launch_plan(const ParamPlan &p, cudaStream_t stream)
     for (const ParamPlan::Wide &w : p.wide) {   // one cluster per output channel
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(static_cast<unsigned>(w.d.M) * w.cluster);
-        cfg.blockDim = dim3(sq::kWideThreads);
+        cfg.blockDim = dim3(sq::kBlockThreads);
         cfg.dynamicSmemBytes = static_cast<size_t>(w.smem);
         cfg.stream = stream;
         cudaLaunchAttribute attr;

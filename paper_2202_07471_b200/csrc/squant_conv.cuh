@@ -1,0 +1,455 @@
+// Layers with kernels of more than one element: a group of 32 to 256 threads takes an output channel,
+// one thread a whole kernel at a time.
+//
+// The channel is staged in shared memory by asynchronous copies; a thread reads its kernel's K weights
+// from there (for odd K the lanes of a warp fall on different banks), settles SQuant-E, SQuant-K and the
+// candidate of Algorithm 3 in registers (3x3) or in place, and leaves candidate, error sum and position
+// in the place of the kernel's first three weights.  SQuant-C is select_top over the kernels' candidates.
+// What bounds it is the number of instructions: 9 loads, 30 for SQuant-E and about 90 for the selection
+// per 3x3 kernel.  A thread with four kernels at once (128-bit loads) needs fewer of them, but leaves half
+// of a short channel's threads idle, needs N to be a multiple of four and an aligned row, and its 1500
+// instructions of straight code are fetched anew by every warp; this body is a loop of about 170.
+#pragma once
+
+#include "squant_rows.cuh"
+
+namespace sq {
+
+// Shared memory of a group: selection, the staged row (with the misalignment of the row in global
+// memory), the codes (likewise).
+__host__ __device__ inline int conv_bytes(int g, int nk, int K, Owner own = kGroup)
+{
+    return sel_bytes(g, own, K) + ((4 * nk + 12 + 15) & ~15) + ((nk + 15 + 15) & ~15);
+}
+
+// Exact SQuant-K + Algorithm 3 on a kernel of K elements whose integer perturbations (2^-30 units, sum e)
+// are at P and whose SQuant-E code bytes are at cb; both are updated in place.  Out of line.
+struct KernelOut64 {
+    long long e;
+    int v, idx;
+};
+
+__device__ __noinline__ KernelOut64 kernel_flip(int *P, unsigned char *cb, int K, bool do_k, long long e)
+{
+    KernelOut64 o;
+    o.v = 0;
+    o.idx = 0;
+    if (e != 0) {
+        const int sgn = e > 0 ? 1 : -1;
+        const long long abs_e = e > 0 ? e : -e;
+        const int k = do_k ? flip_count(abs_e) : 0;
+        int flips = 0, last = -1, cand = -1;
+#pragma unroll 1
+        for (int r = 0; r <= k; ++r) {
+            int best = 0, bi = -1;
+#pragma unroll 4
+            for (int i = 0; i < K; ++i) {
+                const int key = sgn * P[i];
+                if (key > best) { best = key; bi = i; }
+            }
+            if (bi < 0) break;
+            if (r < k) {   // a flipped element changes sign and leaves the candidates by itself
+                P[bi] -= sgn * kOne;
+                cb[bi] = static_cast<unsigned char>(cb[bi] - sgn);
+                last = bi;
+                ++flips;
+            } else {
+                cand = bi;
+            }
+        }
+        e -= static_cast<long long>(sgn) * flips * kOne;
+        const int pick = (static_cast<long long>(flips) * kOne > abs_e) ? last : cand;   // Over SQuant: flip back
+        if (pick >= 0) {
+            o.idx = pick;
+            o.v = P[pick];
+        }
+    }
+    o.e = e;
+    return o;
+}
+
+// Straight-line SQuant-K + Algorithm 3 on a kernel of K = 2 .. 7 elements (1x3, 7x1, ..), as kernel9_select:
+// P are its integer perturbations, cb its staged code bytes.  With |e| <= K / 2 the flips and the candidate
+// are among the (K + 1) / 2 largest keys, which an insertion network finds.  True: not settled (keys below
+// 2^27 need not be ordered like the perturbations; the staged codes are then untouched).
+template <int K>
+__device__ __forceinline__ bool kernel_small_select(const int (&P)[K], unsigned char *cb, int &e_out, int &v_out, int &idx_out)
+{
+    constexpr int R = (K + 1) / 2;
+    long long e = P[0];
+#pragma unroll
+    for (int i = 1; i < K; ++i) e += P[i];
+    const int sgn = e < 0 ? -1 : 1;
+    const unsigned eabs = static_cast<unsigned>(e < 0 ? -e : e);   // <= 3.5 * 2^30
+    int top[R];
+#pragma unroll
+    for (int j = 0; j < R; ++j) top[j] = -0x7fffffff;
+#pragma unroll
+    for (int i = 0; i < K; ++i) {
+        int x = ((P[i] * sgn) & ~15) | (15 - i);
+#pragma unroll
+        for (int j = 0; j < R; ++j) {
+            const int y = min(top[j], x);
+            top[j] = max(top[j], x);
+            x = y;
+        }
+    }
+    const unsigned t = (eabs & static_cast<unsigned>(kOne - 1)) != 0u ? 1u : 0u;
+    const unsigned jx = (eabs - t) >> 29;   // floor(2 |e|), exact halves falling to the lower value
+    const bool zero = eabs == 0u;
+    const int c = min(static_cast<int>(jx >> 1), R - 1);   // rank of the candidate, from 0
+    int mc = top[0];
+#pragma unroll
+    for (int j = 1; j < R; ++j) mc = c == j ? top[j] : mc;
+    if (!zero && mc < (1 << 27)) return true;
+    const int k = zero ? 0 : static_cast<int>((jx + 1u) >> 1);
+#pragma unroll
+    for (int j = 0; j < R; ++j)
+        if (j < k) {
+            unsigned char *p = cb + min(~top[j] & 15, K - 1);
+            *p = static_cast<unsigned char>(*p - sgn);
+        }
+    e_out = zero ? 0 : sgn * static_cast<int>(eabs - (static_cast<unsigned>(k) << 30));
+    v_out = zero ? 0 : sgn * ((mc & ~15) - static_cast<int>((jx & 1u) << 30));   // Over: value after the flip
+    idx_out = min(~mc & 15, K - 1);
+    return false;
+}
+
+// The same under the clip of Sec. 2.2 and from the weights (kernel_clip), out of line.
+__device__ __noinline__ KernelOut64 kernel_clip_out(float *wk, int K, float s, bool do_k, int qmin, int qmax, int8_t *ck)
+{
+    KernelOut64 o;
+    kernel_clip(wk, K, s, do_k, qmin, qmax, ck, o.e, o.v, o.idx);
+    return o;
+}
+
+// ---------------------------------------------------------------- codes and their products to global memory
+// The n codes at cel (shared memory, visible to the whole group), which are those from element `first` of
+// the layer on: int8 or packed int4 (from byte first4 on), and code * s as fp32 and bfloat16.  cel has the
+// misalignment of the int8 codes modulo 16.
+__device__ __forceinline__ void emit_codes(const LayerDesc &L, size_t first, size_t first4, const Group &G, const unsigned char *cel, int n,
+                                           float s, unsigned mode)
+{
+    if (!(mode & kModePackInt4)) {
+        unsigned char *row = reinterpret_cast<unsigned char *>(L.codes) + first;
+        const int head = min(static_cast<int>((16 - (reinterpret_cast<uintptr_t>(row) & 15)) & 15), n);
+        const int nv = (n - head) >> 4, tail = head + 16 * nv;
+        for (int i = G.t; i < nv; i += G.g)
+            __stcs(reinterpret_cast<int4 *>(row + head) + i, reinterpret_cast<const int4 *>(cel + head)[i]);
+        for (int i = G.t; i < head + (n - tail); i += G.g) {
+            const int e = i < head ? i : tail + i - head;
+            row[e] = cel[e];
+        }
+    } else {   // two codes per byte, low nibble = even flat index
+        unsigned char *row = reinterpret_cast<unsigned char *>(L.codes) + first4;
+        // eight codes at a time where the packed row is aligned, the rest byte by byte
+        const int head = min(static_cast<int>((4 - (reinterpret_cast<uintptr_t>(row) & 3)) & 3), n >> 1);   // packed bytes
+        const int nv = ((n >> 1) - head) >> 2, tail = head + 4 * nv;
+        for (int i = G.t; i < nv; i += G.g) {
+            const unsigned char *c = cel + 2 * (head + 4 * i);
+            unsigned o = 0u;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) o |= static_cast<unsigned>(c[k] & 15) << (4 * k);
+            __stcs(reinterpret_cast<unsigned *>(row + head) + i, o);
+        }
+        for (int i = G.t; i < head + ((n + 1) >> 1) - tail; i += G.g) {
+            const int b = i < head ? i : tail + i - head;
+            row[b] = static_cast<unsigned char>((cel[2 * b] & 15) | (2 * b + 1 < n ? cel[2 * b + 1] << 4 : 0));
+        }
+    }
+    if (L.deq) {   // Algorithm 1's own return value: code * s
+        float *row = L.deq + first;
+        const Span sp(row, n, G.t);
+        const bool words = ((reinterpret_cast<uintptr_t>(cel) - sp.r) & 3) == 0;
+        for (int q = sp.q_lo + G.t; q < sp.q_hi; q += G.g) {
+            const unsigned char *c = cel + (4 * q - sp.r);
+            const unsigned c4 = words ? *reinterpret_cast<const unsigned *>(c) : c[0] | (c[1] << 8) | (c[2] << 16) | (static_cast<unsigned>(c[3]) << 24);
+            __stcs(reinterpret_cast<float4 *>(row + (4 * q - sp.r)), make_float4(row_deq(c4, s), row_deq(c4 >> 8, s), row_deq(c4 >> 16, s), row_deq(c4 >> 24, s)));
+        }
+        if (sp.rag >= 0) row[sp.rag] = row_deq(cel[sp.rag], s);
+    }
+    if (L.deq16) {   // the same product as bfloat16
+        uint16_t *row = L.deq16 + first;
+        const int head = min(static_cast<int>(((8 - (reinterpret_cast<uintptr_t>(row) & 7)) & 7) >> 1), n);
+        const int nv = (n - head) >> 2, tail = head + 4 * nv;
+        const bool words = (reinterpret_cast<uintptr_t>(cel + head) & 3) == 0;
+        for (int i = G.t; i < nv; i += G.g) {
+            const unsigned char *c = cel + head + 4 * i;
+            const unsigned c4 = words ? *reinterpret_cast<const unsigned *>(c) : c[0] | (c[1] << 8) | (c[2] << 16) | (static_cast<unsigned>(c[3]) << 24);
+            const unsigned b0 = bf16_bits(row_deq(c4, s)), b1 = bf16_bits(row_deq(c4 >> 8, s));
+            const unsigned b2 = bf16_bits(row_deq(c4 >> 16, s)), b3 = bf16_bits(row_deq(c4 >> 24, s));
+            __stcs(reinterpret_cast<uint2 *>(row + head) + i, make_uint2(b0 | (b1 << 16), b2 | (b3 << 16)));
+        }
+        for (int i = G.t; i < head + (n - tail); i += G.g) {
+            const int e = i < head ? i : tail + i - head;
+            row[e] = static_cast<uint16_t>(bf16_bits(row_deq(cel[e], s)));
+        }
+    }
+}
+
+// ---------------------------------------------------------------- one channel
+// KT = 3, 7, 9: kernels of that many elements with SQuant-K in the mode mask; KT = 0: any kernel size and
+// mode but E|C.
+// kClip: caller-supplied scales, the clip of Sec. 2.2 can fire.
+// kCluster: this thread block has the kernels n0 .. n0 + nloc - 1 (n0 even).
+template <int KT, bool kClip, Owner kOwn = kGroup>
+__device__ __forceinline__ void conv_body(const LayerDesc &L, int m, const Group &G, unsigned char *slice, int qmax, unsigned mode,
+                                          int n0 = 0, int nloc = 0)
+{
+    const int g = G.g, N = kOwn == kCluster ? nloc : L.N, K = KT ? KT : L.K, NK = kOwn == kCluster ? nloc * K : L.NK;   // here
+    const size_t first = static_cast<size_t>(m) * L.NK + static_cast<size_t>(n0) * K;   // of these elements in the layer
+    SelScratch *sc = reinterpret_cast<SelScratch *>(slice);
+    if (G.t == 0) {
+        sc->amax = 0u; sc->count = 0; sc->top = 0;
+        sc->total[0] = 0;
+        sc->sum64 = 0ull;
+    }
+    // ---- stage the row, take its absmax (each thread over what it has copied itself)
+    const float *wrow = L.w + first;
+    float *wel;
+    float amax = 0.0f;
+    {
+        const Span sp(wrow, NK, G.t);
+        float4 *buf = reinterpret_cast<float4 *>(slice + sel_bytes(g, kOwn, K));
+        wel = reinterpret_cast<float *>(buf) + sp.r;
+        const float4 *src = reinterpret_cast<const float4 *>(wrow - sp.r);
+#pragma unroll 2
+        for (int q = sp.q_lo + G.t; q < sp.q_hi; q += g) copy_async16(buf + q, src + q);
+        if (sp.rag >= 0) copy_async4(wel + sp.rag, wrow + sp.rag);
+        copy_async_wait();
+#pragma unroll 2
+        for (int q = sp.q_lo + G.t; q < sp.q_hi; q += g) {
+            const float4 v = buf[q];
+            amax = absmax3(absmax3(amax, v.x, v.y), v.z, v.w);
+        }
+        if (sp.rag >= 0) amax = fmaxf(amax, fabsf(wel[sp.rag]));
+    }
+    unsigned char *cel;   // codes, with the misalignment of their row in global memory
+    {
+        unsigned char *c0 = slice + sel_bytes(g, kOwn, K) + ((4 * NK + 12 + 15) & ~15);
+        cel = c0 + ((reinterpret_cast<uintptr_t>(L.codes) + first) & 15);
+    }
+
+    // ---- scale
+    float s;
+    {
+        unsigned u = __reduce_max_sync(kFull, __float_as_uint(amax));   // >= 0: uint order = float order
+        G.sync();   // the scratch words are cleared, the staged weights are visible
+        if (g > 32) {
+            if ((G.t & 31) == 0) atomicMax(&sc->amax, u);
+            G.sync();
+            u = sc->amax;
+        }
+        if (kOwn == kCluster) {
+            cg::cluster_group cl = cg::this_cluster();
+            cl.sync();
+            const int lane = threadIdx.x & 31;
+            u = __reduce_max_sync(kFull, lane < static_cast<int>(cl.num_blocks()) ? remote(&sc->amax, lane) : 0u);
+        }
+        amax = __uint_as_float(u);
+        s = (amax < 0x1p-100f) ? 1.0f : __fdiv_rn(amax, static_cast<float>(qmax));
+        if (kClip && (kOwn != kCluster || L.sin)) {
+            s = L.sin[m];
+            if (!(s > 0.0f && s < __int_as_float(0x7f800000))) s = 1.0f;
+        }
+    }
+
+    // ---- SQuant-E, SQuant-K, candidates: one thread per kernel
+    const bool do_k = KT != 0 || (mode & 2u) != 0;
+    const bool fast = s >= 0x1p-60f && s <= 0x1p60f;
+    const int qmin = (mode & kModeWideRange) ? -qmax - 1 : -qmax;
+    float *kerr = L.kerr ? L.kerr + static_cast<size_t>(m) * L.N + n0 : nullptr;
+    const float s2 = fast ? __fmul_rn(s, 0x1p-30f) : 0.0f;
+    const E2 c2 = make_e2(fast ? __frcp_rn(s2) : 0.0f, s2);
+    long long esum = 0;
+    int hi0 = 0, lo0 = 0;   // extremes of the candidates
+    // few kernels of many elements (a 7x7 stem has three per channel): a warp per kernel, lanes over its elements
+    const bool by_warp = KT == 0 && !kClip && K >= 16 && 4 * N <= g;
+#pragma unroll 1
+    for (int n = by_warp ? G.t >> 5 : G.t; n < N; n += by_warp ? g >> 5 : g) {
+        float *wk = wel + n * K;
+        unsigned char *ck = cel + n * K;
+        long long e = 0;
+        int v = 0, idx = 0;
+        if (by_warp) {
+            kernel_warp(wk, K, s, do_k, reinterpret_cast<int8_t *>(ck), G.t & 31, e, v, idx);
+            if ((G.t & 31) != 0) continue;
+        } else if (KT == 9 && fast) {
+            float2 P2[5];
+            unsigned edge = 0u;
+            {
+                float w[9];
+#pragma unroll
+                for (int i = 0; i < 9; ++i) w[i] = wk[i];
+#pragma unroll
+                for (int p = 0; p < 5; ++p) {
+                    const float2 w2 = make_float2(w[2 * p], p < 4 ? w[2 * p + 1] : 0.0f);
+                    float2 t;
+                    if (!kClip) {
+                        squant_e_fast2(w2, c2, t, P2[p]);
+                    } else {
+                        // the codes on the edge of the range and the clipped ones: a flip can be barred there
+                        const float2 x0 = __fmul2_rn(w2, c2.y);
+                        const float2 X = __ffma2_rn(__ffma2_rn(x0, c2.ns2, w2), c2.y, x0);
+                        t = __fadd2_rn(X, c2.magic);
+                        P2[p] = __ffma2_rn(X, c2.neg1, __fadd2_rn(t, c2.nmagic));
+                        const float lim_hi = (static_cast<float>(qmax) - 0.5f) * 1073741824.0f, lim_lo = (static_cast<float>(qmin) + 0.5f) * 1073741824.0f;
+                        edge |= (X.x < lim_hi && X.x > lim_lo && X.y < lim_hi && X.y > lim_lo) ? 0u : 1u;
+                    }
+                    ck[2 * p] = static_cast<unsigned char>(__float_as_uint(t.x));
+                    if (p < 4) ck[2 * p + 1] = static_cast<unsigned char>(__float_as_uint(t.y));
+                }
+            }
+            const float2 s01 = __fadd2_rn(__fadd2_rn(P2[0], P2[1]), __fadd2_rn(P2[2], P2[3]));
+            const float ef = __fadd_rn(__fadd_rn(s01.x, s01.y), P2[4].x);
+            const float gs = copysignf(1.0f, ef);
+            const float2 G2 = make_float2(gs, gs);
+            float Pk[9];
+#pragma unroll
+            for (int p = 0; p < 5; ++p) {
+                const float2 q = __fmul2_rn(P2[p], G2);
+                Pk[2 * p] = q.x;
+                if (p < 4) Pk[2 * p + 1] = q.y;
+            }
+            int e32;
+            unsigned ix;
+            if (kClip && edge != 0u) {
+                const KernelOut64 o = kernel_clip_out(wk, 9, s, true, qmin, qmax, reinterpret_cast<int8_t *>(ck));
+                e = o.e; v = o.v; idx = o.idx;
+            } else {
+                if (kernel9_select(Pk, ef, ck, e32, v, ix)) {   // about one in 10^5: settled exactly
+                    int *P = reinterpret_cast<int *>(wk);
+                    const int gi = (__float_as_int(ef) >> 31) | 1;
+#pragma unroll
+                    for (int i = 0; i < 9; ++i) P[i] = gi * __float2int_rn(Pk[i]);
+                    long long e64 = 0;
+#pragma unroll
+                    for (int i = 0; i < 9; ++i) e64 += P[i];
+                    const KernelOut64 o = kernel_flip(P, ck, 9, true, e64);
+                    e32 = static_cast<int>(o.e); v = o.v; ix = static_cast<unsigned>(o.idx);
+                }
+                e = e32;
+                idx = static_cast<int>(ix);
+            }
+        } else if (kClip) {
+            const KernelOut64 o = kernel_clip_out(wk, K, s, do_k, qmin, qmax, reinterpret_cast<int8_t *>(ck));
+            e = o.e; v = o.v; idx = o.idx;
+        } else if (KT > 1 && KT < 9 && fast) {
+            int P[KT > 1 ? KT : 2];
+#pragma unroll
+            for (int i = 0; i < KT; ++i) {
+                unsigned tb;
+                squant_e_fast(wk[i], c2.y.x, s2, tb, P[i]);
+                ck[i] = static_cast<unsigned char>(tb);
+            }
+            int e32;
+            if (kernel_small_select<(KT > 1 && KT < 9 ? KT : 2)>(reinterpret_cast<const int (&)[KT > 1 && KT < 9 ? KT : 2]>(P), ck, e32, v, idx)) {
+                int *Ps = reinterpret_cast<int *>(wk);
+                e = 0;
+#pragma unroll
+                for (int i = 0; i < KT; ++i) { Ps[i] = P[i]; e += P[i]; }
+                const KernelOut64 o = kernel_flip(Ps, ck, KT, true, e);
+                e32 = static_cast<int>(o.e); v = o.v; idx = o.idx;
+            }
+            e = e32;
+        } else {
+            int *P = reinterpret_cast<int *>(wk);
+#pragma unroll 4
+            for (int i = 0; i < K; ++i) {
+                int p;
+                if (fast) {
+                    unsigned tb;
+                    squant_e_fast(wk[i], c2.y.x, s2, tb, p);
+                    ck[i] = static_cast<unsigned char>(tb);
+                } else {
+                    int q;
+                    squant_e(wk[i], s, q, p);
+                    ck[i] = static_cast<unsigned char>(q);
+                }
+                P[i] = p;
+                e += p;
+            }
+            const KernelOut64 o = kernel_flip(P, ck, K, do_k, e);
+            e = o.e; v = o.v; idx = o.idx;
+        }
+        esum += e;
+        if (kerr) kerr[n] = __fmul_rn(KT != 0 && !kClip ? __int2float_rn(static_cast<int>(e)) : __ll2float_rn(e), 0x1p-30f);
+        // for SQuant-C, in the place of the kernel's weights (of two elements: the position is the low bit of the sum)
+        int *rec = reinterpret_cast<int *>(wk);
+        // a kernel that can be flipped has |e| <= 1/2
+        const int es = KT != 0 && !kClip ? static_cast<int>(e) : static_cast<int>(max(min(e, 0x3fffffffll), -0x3fffffffll));
+        rec[0] = v;
+        rec[1] = K > 2 ? es : 2 * es + idx;
+        if (K > 2) rec[2] = idx;
+        hi0 = max(hi0, v);
+        lo0 = min(lo0, v);
+    }
+
+    // ---- channel sum
+    long long ec = 0;
+    if ((mode & 4u) || L.cerr) {
+        for (int o = 16; o > 0; o >>= 1) esum += __shfl_xor_sync(kFull, esum, o);
+        if (g > 32) {
+            if ((G.t & 31) == 0) atomicAdd(&sc->sum64, static_cast<unsigned long long>(esum));
+            G.sync();
+            esum = static_cast<long long>(sc->sum64);
+            if (kOwn == kCluster) {
+                cg::cluster_group cl = cg::this_cluster();
+                cl.sync();
+                esum = 0;
+                for (int c = 0; c < static_cast<int>(cl.num_blocks()); ++c) esum += static_cast<long long>(remote(&sc->sum64, c));
+            }
+        }
+        ec = esum;
+    }
+
+    // ---- SQuant-C: Algorithm 2 on the channel, keys = the kernels' candidates
+    if (mode & 4u) {
+        const int sgn = ec > 0 ? 1 : -1;
+        const long long abs_e = ec > 0 ? ec : -ec;
+        const int kc = static_cast<int>(min((abs_e + (kHalf - 1)) >> 30, 1ll << 30));   // a clipped channel's sum can be huge
+        if (kc > 0) {   // uniform in the group
+            auto each = [&](int t, auto fn) {
+#pragma unroll 2
+                for (int n = by_warp ? ((G.t & 31) ? N : G.t >> 5) : G.t; n < N; n += by_warp ? g >> 5 : g) {
+                    const int a = reinterpret_cast<const int *>(wel)[n * K] * sgn;
+                    if (a >= t) fn(a, n0 + n);
+                }
+            };
+            auto flip = [&](int, int n_abs) {
+                const int n = n_abs - n0;
+                const int *rec = reinterpret_cast<const int *>(wel + n * K);
+                const int idx = K > 2 ? rec[2] : rec[1] & 1;
+                SQ_DBG(n >= 0 && n < N && idx >= 0 && idx < K, 2);
+                unsigned char *cb = cel + n * K + idx;
+                *cb = static_cast<unsigned char>(*cb - sgn);
+                if (kerr) kerr[n] = __fmul_rn(__int2float_rn((K > 2 ? rec[1] : rec[1] >> 1) - sgn * kOne), 0x1p-30f);
+            };
+            const int m0 = sgn > 0 ? hi0 : -lo0;
+            // Over-SQuant candidates reach one, but few come near it: the search starts at the largest
+            int top = static_cast<int>(__reduce_max_sync(kFull, static_cast<unsigned>(m0)));
+            if (g > 32) {
+                if ((G.t & 31) == 0) atomicMax(&sc->top, top);
+                G.sync();
+                top = sc->top;
+                if (kOwn == kCluster) {
+                    cg::cluster_group cl = cg::this_cluster();
+                    cl.sync();
+                    const int lane = threadIdx.x & 31;
+                    top = __reduce_max_sync(kFull, lane < static_cast<int>(cl.num_blocks()) ? remote(&sc->top, lane) : 0);
+                }
+            }
+            const int k_eff = select_top<kOwn>(G, each, flip, m0, 0, top + 1, 3.0f, kc, L.N, true, sc, K);
+            ec -= static_cast<long long>(sgn) * k_eff * kOne;
+        }
+    }
+    G.sync();   // all codes are final
+
+    emit_codes(L, first, static_cast<size_t>(m) * ((L.NK + 1) >> 1) + ((static_cast<size_t>(n0) * K) >> 1), G, cel, NK, s, mode);
+    if (G.t == 0 && n0 == 0) {
+        L.scales[m] = s;
+        if (L.cerr) L.cerr[m] = __fmul_rn(__ll2float_rn(ec), 0x1p-30f);
+    }
+}
+
+}  // namespace sq

@@ -36,7 +36,7 @@ struct LayerDesc {
     int32_t g;            // threads per channel group: 32, 64, 128 or 256
     int32_t g_shift;      // log2(g)
     int32_t slice_bytes;  // shared memory per group
-    int32_t off_codes, off_ev, off_vv, off_vi, off_hist, off_red;
+    int32_t off_codes, off_ev, off_vv, off_vi, off_hist, off_red;   // 1x1 layers (off_hist = 0): off_vi = vectors of a row
 };
 
 // One CTA: channels ch0 .. ch0 + 256/g - 1 of one layer, one per group.
@@ -63,7 +63,7 @@ struct Group {
     int bar;  // named barrier of the group (groups wider than a warp)
     __device__ __forceinline__ void sync() const
     {
-        if (g == 32) __syncwarp();
+        if (g <= 32) __syncwarp();   // groups of 8 and 16 threads share a warp and keep step with each other
         else asm volatile("bar.sync %0, %1;" ::"r"(bar), "r"(g) : "memory");
     }
 };
@@ -1590,6 +1590,12 @@ __global__ void debug_wait_kernel(int max_polls)
     }
 }
 
+}  // namespace sq
+
+#include "squant_conv.cuh"
+
+namespace sq {
+
 // ---------------------------------------------------------------- grouped launch
 // One CTA per work item.  The descriptor of the CTA's layer comes either from the launch table
 // in the kernel's parameter space (kParams) or from a table in global memory.
@@ -1610,31 +1616,48 @@ __device__ __forceinline__ void run_item(const LayerDesc &L, int ch0, unsigned c
     const int gi = threadIdx.x >> L.g_shift;
     G.bar = 1 + gi;
     const int m = ch0 + gi;
-    if (m >= L.M) return;   // the whole group leaves together; it shares no barrier with others
     unsigned char *slice = smem + static_cast<size_t>(gi) * L.slice_bytes;
+    if (L.K == 1 && L.off_hist == 0) {   // 1x1, in registers; groups without a channel stay with their warp
+        SQ_DBG(ch0 >= 0 && L.g >= 8 && (1 << L.g_shift) == L.g && row_bytes(L.g, L.off_vi) <= L.slice_bytes &&
+               static_cast<size_t>(gi + 1) * L.slice_bytes <= dynamic_smem_bytes(), 5);
+        if (L.g >= 32 && m >= L.M) return;
+        if (L.sin) row_body<true>(L, m, G, slice, qmax, mode, m < L.M);
+        else row_body<false>(L, m, G, slice, qmax, mode, m < L.M);
+        return;
+    }
+    if (m >= L.M) return;   // the whole group leaves together; it shares no barrier with others
+    if (L.off_hist == 0) {   // larger kernels
+        SQ_DBG(ch0 >= 0 && L.g >= 32 && (1 << L.g_shift) == L.g && conv_bytes(L.g, L.NK, L.K) <= L.slice_bytes &&
+               static_cast<size_t>(gi + 1) * L.slice_bytes <= dynamic_smem_bytes(), 6);
+        if (L.K == 9 && (mode & 2u)) {
+            if (L.sin) conv_body<9, true>(L, m, G, slice, qmax, mode);
+            else conv_body<9, false>(L, m, G, slice, qmax, mode);
+        } else if (L.sin) {
+            conv_body<0, true>(L, m, G, slice, qmax, mode);
+        } else if (L.K == 7 && (mode & 2u)) {
+            conv_body<7, false>(L, m, G, slice, qmax, mode);
+        } else if (L.K == 3 && (mode & 2u)) {
+            conv_body<3, false>(L, m, G, slice, qmax, mode);
+        } else {
+            conv_body<0, false>(L, m, G, slice, qmax, mode);
+        }
+        return;
+    }
     SQ_DBG(ch0 >= 0 && L.g >= 32 && (L.g & (L.g - 1)) == 0 && (1 << L.g_shift) == L.g, 5);
     SQ_DBG(static_cast<size_t>(gi + 1) * L.slice_bytes <= dynamic_smem_bytes(), 6);
     SQ_DBG(L.off_red + 256 <= L.slice_bytes && L.off_hist + 4 * kHistBins <= L.off_red && L.off_codes + L.NK <= L.slice_bytes, 7);
     const float s = stage_channel(L, m, G, slice, qmax);
     if (s == 0.0f) return;   // staging wait ran out (status word set); nothing is written
-    if (L.sin) {   // Algorithm 1 with its scale as an input
+    if (L.K > 1) {   // E + C without K
+        channel_body_ec(L, m, G, slice, s, mode);
+    } else if (L.sin) {   // 1x1 rows too long for the registers of one thread block
         float sc = L.sin[m];
         if (!(sc > 0.0f && sc < __int_as_float(0x7f800000))) sc = 1.0f;
         channel_body_clip(L, m, G, slice, sc, mode, qmax);
-    } else if (L.K > 1 && (mode & 6u) == 4u) {   // E + C without K
-        channel_body_ec(L, m, G, slice, s, mode);
-    } else if (L.K == 1) {
-        if ((L.N & 3) == 0 && s >= 0x1p-60f && s <= 0x1p60f)
-            channel_body_k1_fast(L, m, G, slice, s, mode);
-        else
-            channel_body<1>(L, m, G, slice, s, mode);
-    } else if (L.K == 9) {
-        if ((L.N & 3) == 0 && (mode & 2u) && s >= 0x1p-60f && s <= 0x1p60f)
-            channel_body_k9_fast(L, m, G, slice, s, mode);
-        else
-            channel_body<9>(L, m, G, slice, s, mode);
+    } else if ((L.N & 3) == 0 && s >= 0x1p-60f && s <= 0x1p60f) {
+        channel_body_k1_fast(L, m, G, slice, s, mode);
     } else {
-        channel_body<0>(L, m, G, slice, s, mode);
+        channel_body<1>(L, m, G, slice, s, mode);
     }
 }
 

@@ -1,0 +1,662 @@
+// 1x1 layers (fully connected and pointwise): a group of 8 to 256 threads takes a whole output
+// channel, up to 32 weights a thread.
+//
+// Every element is its own kernel, so SQuant-K is a no-op (Sec. 3.4) and the work is absmax,
+// SQuant-E, the channel sum and SQuant-C's choice of the k_c largest perturbations of one sign.
+// What bounds such a channel is not bandwidth but instructions and the chain of its steps: by way
+// of staged weights, a histogram in shared atomics and a 256-bin scan per channel, a ResNet-50
+// spent 70 thread-instructions per weight, most of them fixed costs of short channels.  Here
+//   - the weights are requested all at once and put into shared memory, each thread's for itself (no
+//     barrier); the perturbations take their place, where a thread looks again only if its largest one
+//     comes into question;
+//   - short channels share a warp (8 or 16 threads each), so the fixed costs are shared too;
+//   - SQuant-C needs no histogram.  Each thread knows its largest candidates; a value T0 that at
+//     least k_c of those maxima reach is a lower bound of the k_c-th largest candidate whatever the
+//     distribution, and few other elements reach it (with k_c of m maxima about m ln(m / (m - k_c))
+//     elements).  T0 is searched among the maxima, the elements from T0 on are listed, and those of
+//     the first k_c ranks are flipped.  What that cannot settle (k_c beyond the number of maxima, a
+//     full list) goes to an exact search over the 48-bit keys.
+#pragma once
+
+#include <cooperative_groups.h>
+
+#include "squant_device.cuh"
+
+namespace sq {
+
+namespace cg = cooperative_groups;
+
+constexpr int kRowVecs = 8;                       // float4 a thread holds
+
+// Threads per channel for rows of `vecs` vectors (8, 16, .. 256), 0: too long for one thread block.
+__host__ __device__ inline int row_group(int vecs)
+{
+    int g = 8;
+    while (g * kRowVecs < vecs) g *= 2;
+    return g <= kCtaThreads ? g : 0;
+}
+
+// Control words of one group, followed by its list and, for groups wider than a warp, the threads'
+// maxima.
+struct SelScratch {
+    unsigned amax;             // absmax accumulator (bit pattern of a non-negative float)
+    unsigned sum;              // channel sum modulo 2^32
+    int approx;                // channel sum in units of 2^20
+    int count;                 // listed elements
+    int total[3];              // rotating counters of the exact search
+    int top;                   // largest candidate (larger kernels)
+    unsigned long long sum64;  // channel sum (supplied scales)
+    int found[2];              // rotating counters of the search over a cluster
+};
+
+// Who owns a channel: a group inside a thread block, a whole thread block, a cluster of thread blocks
+// (each a run of the channel's kernels; they read each other's control words and lists through
+// distributed shared memory).
+enum Owner { kGroup, kBlock, kCluster };
+constexpr int kBlockThreads = 512;   // kBlock, kCluster
+// kCluster: room for the lists of all thread blocks together.  Kernels of more than 16 elements are few
+// and leave little shared memory: short lists there.
+__host__ __device__ constexpr int merged_cap(int K) { return K > 16 ? 128 : 1024; }
+
+__host__ __device__ constexpr int sel_cap(int g, int K = 1) { return g <= 64 || (g > 256 && K > 16) ? 64 : g; }
+__host__ __device__ constexpr int sel_maxima(int g) { return g <= 64 ? 2 * g : g; }   // two per thread up to 64 threads
+__host__ __device__ constexpr int sel_bytes(int g, Owner own = kGroup, int K = 1)
+{
+    return static_cast<int>(sizeof(SelScratch)) + 8 * sel_cap(g, K) +
+           (own == kGroup ? (g > 32 ? 4 * sel_maxima(g) : 0) : (own == kCluster ? 8 * merged_cap(K) : 0));
+}
+// The same of a 1x1 channel of `vecs` vectors: selection, perturbations, codes.
+__host__ __device__ constexpr int row_bytes(int g, int vecs, Owner own = kGroup) { return sel_bytes(g, own) + 20 * vecs; }
+
+// How a run of n 4-byte elements that starts anywhere is cut into 16-byte vectors: vector q holds the
+// elements 4q - r .. 4q - r + 3; those with q_lo <= q < q_hi are whole, the up to six elements outside
+// them go to one thread each (rag, -1: none).
+struct Span {
+    int r, q_lo, q_hi, rag;
+    bool ragged;   // there are such elements (uniform)
+    __device__ __forceinline__ Span(const void *p, int n, int t) : Span(static_cast<int>((reinterpret_cast<uintptr_t>(p) >> 2) & 3), n, t) {}
+    __device__ __forceinline__ Span(int r_, int n, int t)
+    {
+        r = r_;
+        q_lo = min((r + 3) >> 2, (n + r + 3) >> 2);
+        q_hi = max((n + r) >> 2, q_lo);
+        const int head = min((4 - r) & 3, n), tail = max(4 * q_hi - r, 0);
+        ragged = head > 0 || tail < n;
+        rag = t < head ? t : (tail >= head && t - head < n - tail ? tail + t - head : -1);
+    }
+};
+
+__device__ __forceinline__ void copy_async16(void *dst, const void *src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copy_async4(void *dst, const void *src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_addr(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copy_async_wait()
+{
+    asm volatile("cp.async.wait_all;" ::: "memory");
+}
+
+// max(a, |x|, |y|) in one instruction
+__device__ __forceinline__ float absmax3(float a, float x, float y)
+{
+    float d;
+    asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(fabsf(x)), "f"(fabsf(y)));
+    return d;
+}
+
+// ---------------------------------------------------------------- reductions inside a warp's group
+__device__ __forceinline__ unsigned lanes_max(int g, unsigned v)
+{
+    if (g >= 32) return __reduce_max_sync(kFull, v);
+    for (int o = g >> 1; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(kFull, v, o));
+    return v;
+}
+
+__device__ __forceinline__ int lanes_add(int g, int v)
+{
+    if (g >= 32) return __reduce_add_sync(kFull, v);
+    for (int o = g >> 1; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
+    return v;
+}
+
+// ---------------------------------------------------------------- reductions over the owner of a channel
+// (of kBlock and kCluster; every thread calls them)
+// Word w of another thread block's control words.
+template <class T>
+__device__ __forceinline__ T remote(const T *w, int rank)
+{
+    return *cg::this_cluster().map_shared_rank(w, rank);
+}
+
+// Sum over the cluster of *w, which every thread block has completed before its last barrier.
+__device__ __forceinline__ int cluster_sum(const int *w)
+{
+    cg::cluster_group cl = cg::this_cluster();
+    cl.sync();
+    const int lane = threadIdx.x & 31;
+    return __reduce_add_sync(kFull, lane < static_cast<int>(cl.num_blocks()) ? remote(w, lane) : 0);
+}
+
+// ---------------------------------------------------------------- SQuant-C: the k_c largest candidates
+// each(t, f) visits those of the calling thread's elements that reach t >= 1, f(a, n) with a = the
+// candidate's value in the direction of the flips and n its kernel index in the channel; m0, m1: the
+// thread's maxima of a over two disjoint parts of its elements, top a value above every candidate, spread the expected
+// distance between the largest candidates in units of top / n_all.  flip(a, n) is called once for each
+// of the min(kc, candidates) largest (equal values: lower index first), by some thread of the
+// group.  want: this group selects at all (kc >= 1).  Returns the number of flips.  Every thread of
+// the group calls it, groups that share a warp together; it starts with no barrier and ends
+// with none.
+template <Owner kOwn, class Each, class Flip>
+__device__ __forceinline__ int select_top(const Group &G, Each each, Flip flip, int m0, int m1, int top, float spread, int kc, int n_all, bool want,
+                                          SelScratch *sc, int K = 1)
+{
+    const int g = G.g, lane = threadIdx.x & 31;
+    const unsigned gmask = g >= 32 ? kFull : (((1u << g) - 1u) << (lane & ~(g - 1)));
+    unsigned long long *list = reinterpret_cast<unsigned long long *>(sc + 1);
+    const int cap = sel_cap(g, kOwn == kCluster ? K : 1);
+    const int nmax = kOwn == kGroup ? sel_maxima(g) : 2 * g * (kOwn == kCluster ? static_cast<int>(cg::this_cluster().num_blocks()) : 1);
+    int *mx = reinterpret_cast<int *>(list + cap);
+    if (kOwn == kGroup && g > 32) {
+        if (g <= 64) { mx[G.t] = m0; mx[G.t + g] = m1; }
+        else mx[G.t] = max(m0, m1);
+        G.sync();
+    }
+
+    // ---- T0: at least kc of the maxima reach it, and not many more.  The first guess supposes an even
+    // spread; the distance to the top is doubled until it is enough, then the interval is halved (1x1:
+    // 1.1 rounds on normal and heavy-tailed weights of 4 and 8 bit, 3x3: 1.3 to 2.6; the list holds about
+    // kc + 3 elements for small, 1.6 kc for large kc).
+    int lo = 1, hi = top;
+    bool sure = false;   // lo has been counted
+    bool done = !want || kc > nmax;
+    const int slack = kc + (kc >> 1) + 6;
+    int mid = max(top - 1 - __float2int_rz(__fmul_rn(__fmul_rn(static_cast<float>(kc) + 1.0f, spread), __fdividef(static_cast<float>(top), static_cast<float>(n_all)))), 1);
+#pragma unroll 1
+    for (int it = 0; __any_sync(kFull, !done); ++it) {
+        int c;
+        if (kOwn != kGroup) {
+            c = __syncthreads_count(m0 >= mid) + __syncthreads_count(m1 >= mid);
+            if (kOwn == kCluster) {
+                if (G.t == 0) sc->found[it & 1] = c;
+                __syncthreads();
+                c = cluster_sum(&sc->found[it & 1]);
+            }
+        } else if (g <= 32) {
+            c = __popc(__ballot_sync(kFull, m0 >= mid) & gmask) + __popc(__ballot_sync(kFull, m1 >= mid) & gmask);
+        } else {
+            c = 0;
+#pragma unroll 1
+            for (int i = lane; i < (nmax >> 2); i += 32) {
+                const int4 q = reinterpret_cast<const int4 *>(mx)[i];
+                c += (q.x >= mid) + (q.y >= mid) + (q.z >= mid) + (q.w >= mid);
+            }
+            c = __reduce_add_sync(kFull, c);
+        }
+        if (!done) {
+            if (c >= kc) { lo = mid; sure = true; done = c <= slack; }
+            else hi = mid;
+            done = done || hi - lo <= 1;
+            mid = sure ? lo + ((hi - lo) >> 1) : max(hi - (top - hi), 1);
+        }
+    }
+    const int T0 = lo;
+    bool slow = want && !sure;   // fewer than kc maxima are candidates at all
+
+    // ---- list the elements from T0 on
+    if (want && !slow && max(m0, m1) >= T0)
+        each(T0, [&](int a, int n) {
+            const int pos = atomicAdd(&sc->count, 1);
+            if (pos < cap)
+                list[pos] = (static_cast<unsigned long long>(static_cast<unsigned>(a)) << kIdxBits) |
+                            static_cast<unsigned long long>(((1 << kIdxBits) - 1) - n);
+        });
+    G.sync();
+    int cnt = sc->count, all = cnt;   // this list, all lists
+    int k_eff = want ? kc : 0;
+    const unsigned long long *merged = list;
+    if (kOwn == kCluster) {   // every thread block collects all lists
+        cg::cluster_group cl = cg::this_cluster();
+        cl.sync();
+        unsigned long long *dst = list + cap;
+        merged = dst;
+        all = 0;
+        bool full = false;
+        for (int c = 0; c < static_cast<int>(cl.num_blocks()); ++c) {
+            const int n = remote(&sc->count, c);
+            full = full || n > cap || all + n > merged_cap(K);
+            if (!full)
+                for (int y = G.t; y < n; y += g) dst[all + y] = remote(list + y, c);
+            all += n;
+        }
+        if (full) slow = true;
+        G.sync();
+    } else if (want && !slow && cnt > cap) {
+        slow = true;
+    }
+    if (kOwn != kGroup && want && !slow) {   // exact ranks, a warp per entry: keys are distinct
+#pragma unroll 1
+        for (int x = G.t >> 5; x < cnt; x += g >> 5) {
+            const unsigned long long me = list[x];
+            int rank = 0;
+            for (int y = lane; y < all; y += 32) rank += merged[y] > me ? 1 : 0;
+            rank = __reduce_add_sync(kFull, rank);
+            if (rank < kc && lane == 0) flip(static_cast<int>(me >> kIdxBits), ((1 << kIdxBits) - 1) - static_cast<int>(me & ((1ull << kIdxBits) - 1)));
+        }
+    }
+    if (kOwn == kGroup && want && !slow) {   // exact ranks inside the list: keys are distinct
+#pragma unroll 1
+        for (int x = G.t; x < cnt; x += g) {
+            const unsigned long long me = list[x];
+            int rank = 0;
+            if (cnt > kc) {
+#pragma unroll 4
+                for (int y = 0; y < cnt; ++y) rank += list[y] > me ? 1 : 0;
+            }
+            if (rank < kc) flip(static_cast<int>(me >> kIdxBits), ((1 << kIdxBits) - 1) - static_cast<int>(me & ((1ull << kIdxBits) - 1)));
+        }
+    }
+
+    // ---- exact search: the value v with at most kc - 1 candidates above it and at least kc from it on, by
+    // counting (eight rounds interpolate, then the interval is halved); all candidates above v are
+    // flipped, and of those that tie at v the ones with the lowest indices
+    if (__any_sync(kFull, slow)) {   // group-uniform for groups of whole warps
+        int vlo = 1, vhi = top, vm = 1, c_lo = 0, c_hi = 0, tie = 0;   // count(vlo) >= kc > count(vhi)
+        int ilo = 0, ihi = n_all, im = 0;                      // ties with index < ihi suffice, with index < ilo do not
+        int phase = slow ? 0 : 2;
+#pragma unroll 1
+        for (int it = 0; __any_sync(kFull, phase < 2); ++it) {
+            int c = 0;
+            if (phase == 0) each(vm, [&](int, int) { ++c; });
+            if (phase == 1) each(vlo, [&](int a, int n) { c += (a == vlo && n < im) ? 1 : 0; });
+            c = lanes_add(g, c);
+            if (g > 32) {
+                if (lane == 0) atomicAdd(&sc->total[it % 3], c);
+                if (G.t == 0) sc->total[(it + 1) % 3] = 0;
+                G.sync();
+                c = kOwn == kCluster ? cluster_sum(&sc->total[it % 3]) : sc->total[it % 3];
+            }
+            if (phase == 0) {
+                if (it == 0 && c <= kc) { k_eff = c; vlo = 1; ihi = n_all; phase = 2; }        // every candidate is flipped
+                else if (c >= kc) { vlo = vm; c_lo = c; if (c == kc) phase = 2; }
+                else { vhi = vm; c_hi = c; }
+                if (phase == 0) {
+                    if (vhi - vlo <= 1) {   // more candidates of value vlo than there is room for
+                        tie = kc - c_hi;
+                        phase = 1;
+                        im = n_all >> 1;
+                    } else if (it < 9) {
+                        const float f = __fdividef(static_cast<float>(c_lo - kc) + 0.5f, static_cast<float>(c_lo - c_hi) + 0.5f);
+                        vm = max(vlo + 1, min(vlo + static_cast<int>(f * static_cast<float>(vhi - vlo)), vhi - 1));
+                    } else {
+                        vm = vlo + ((vhi - vlo) >> 1);
+                    }
+                }
+            } else if (phase == 1) {
+                if (c >= tie) ihi = im;
+                else ilo = im;
+                if (c == tie || ihi - ilo <= 1) phase = 2;
+                im = ilo + ((ihi - ilo) >> 1);
+            }
+        }
+        if (slow) each(vlo, [&](int a, int n) { if (a > vlo || n < ihi) flip(a, n); });
+    }
+    return k_eff;
+}
+
+// SQuant-E on four weights by plain IEEE division, codes clamped to [lo, hi]: for scales outside the
+// range of the reciprocal sequence.  Out of line: rare, and its code would be in the way.
+__device__ __noinline__ unsigned row_e_div(float4 w, float s, int lo, int hi, float2 &Pa, float2 &Pb)
+{
+    float P[4];
+    unsigned c4 = 0u;
+    const float ws[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        const float x = __fdiv_rn(ws[c], s);
+        const float qf = fminf(fmaxf(rintf(x), static_cast<float>(lo)), static_cast<float>(hi));
+        P[c] = __fmul_rn(__fsub_rn(qf, x), 1073741824.0f);
+        c4 |= (static_cast<unsigned>(__float2int_rn(qf)) & 255u) << (8 * c);
+    }
+    Pa = make_float2(P[0], P[1]);
+    Pb = make_float2(P[2], P[3]);
+    return c4;
+}
+
+// One element under the clip: its exact perturbation Pf goes into the 64-bit sum and, as a float,
+// into o; P (Pf as an integer, saturated) becomes 0 if the element is no candidate in either direction
+// because the flipped code (low byte of c) would leave the range - every clipped element among them.
+__device__ __forceinline__ void row_clip_one(float Pf, int &P, unsigned c, int qmin, int qmax, long long &sum64, float &o)
+{
+    const bool large = !(fabsf(Pf) < 0x1p30f);
+    sum64 += large ? __float2ll_rn(Pf) : static_cast<long long>(P);
+    o = large ? Pf : __int2float_rn(P);
+    const int q8 = static_cast<int>(static_cast<signed char>(c & 255u));
+    if ((P > 0 && q8 == qmin) || (P < 0 && q8 == qmax)) P = 0;
+}
+
+// code (low byte of c) * s
+__device__ __forceinline__ float row_deq(unsigned c, float s)
+{
+    return __fmul_rn(__int2float_rn(static_cast<int>(static_cast<signed char>(c & 255u))), s);
+}
+
+// ---------------------------------------------------------------- one 1x1 channel
+// kClip: the clip of Sec. 2.2 can fire (caller-supplied scales) or the element at the edge of the
+// range can reach the selection (channels of 2^16 and more kernels): codes are clamped, sums are 64
+// bit and an element whose flipped code would leave the range is no candidate.  valid = false: the
+// group has no channel (its lanes take part in the warp's steps and write nothing).
+// kCluster: this thread block has the elements n0 .. n0 + nloc - 1 (n0 a multiple of four).
+template <bool kClip, Owner kOwn = kGroup>
+__device__ __forceinline__ void row_body(const LayerDesc &L, int m, const Group &G, unsigned char *slice, int qmax, unsigned mode,
+                                         bool valid, int n0 = 0, int nloc = 0)
+{
+    const int g = G.g, N = kOwn == kCluster ? nloc : (valid ? L.N : 0);   // elements here
+    SelScratch *sc = reinterpret_cast<SelScratch *>(slice);
+    if (G.t == 0) {
+        sc->amax = 0u; sc->sum = 0u; sc->approx = 0; sc->count = 0;
+        sc->total[0] = 0;
+        sc->sum64 = 0ull;
+    }
+    const size_t first = static_cast<size_t>(m) * L.N + n0;   // of these elements in the layer
+    const float *wrow = L.w + first;
+    // The row is cut into vectors at 16-byte boundaries of the weights (packed codes pair elements from
+    // the row's start, so there the vectors start with the row).
+    const bool pack = (mode & kModePackInt4) != 0;
+    const Span sp(pack ? 0 : static_cast<int>((reinterpret_cast<uintptr_t>(wrow) >> 2) & 3), N, G.t);
+    const int r = sp.r, q_hi = sp.q_hi, rag = sp.rag, q0 = sp.q_lo + G.t;
+    int4 *Pbuf = reinterpret_cast<int4 *>(slice + sel_bytes(g, kOwn));              // what SQuant-C may choose from
+    unsigned *cbuf = reinterpret_cast<unsigned *>(slice + sel_bytes(g, kOwn) + 16 * L.off_vi);   // codes, by vectors
+    int *Pel = reinterpret_cast<int *>(Pbuf) + r;                                   // the same by elements
+    unsigned char *cel = reinterpret_cast<unsigned char *>(cbuf) + r;
+    float *kerr = L.kerr ? L.kerr + first : nullptr;
+
+    // ---- weights: every thread copies its vectors to shared memory, all requests at once, and takes their
+    // absmax.  (Short loops, here and below: unrolled over eight vectors in registers, this body was no
+    // faster than the old one, because code that every warp runs through once waits for its instructions.)
+    float amax = 0.0f;
+    {
+        const float4 *src = reinterpret_cast<const float4 *>(wrow - r);
+        if ((reinterpret_cast<uintptr_t>(src) & 15) == 0) {
+#pragma unroll 2
+            for (int q = q0; q < q_hi; q += g) copy_async16(Pbuf + q, src + q);
+        } else {   // packed codes of a misaligned row
+#pragma unroll 1
+            for (int q = q0; q < q_hi; q += g)
+                for (int c = 0; c < 4; ++c) copy_async4(Pel + 4 * q + c, wrow + 4 * q + c);
+        }
+        if (rag >= 0) copy_async4(Pel + rag, wrow + rag);
+        copy_async_wait();
+#pragma unroll 2
+        for (int q = q0; q < q_hi; q += g) {
+            const float4 v = reinterpret_cast<const float4 *>(Pbuf)[q];
+            amax = absmax3(absmax3(amax, v.x, v.y), v.z, v.w);
+        }
+    }
+    float w_rag = 0.0f;
+    if (rag >= 0) w_rag = reinterpret_cast<const float *>(Pel)[rag];
+    amax = fmaxf(amax, fabsf(w_rag));
+
+    // ---- scale
+    float s;
+    {
+        unsigned u = lanes_max(g, __float_as_uint(amax));   // >= 0: uint order = float order
+        G.sync();   // the scratch words are cleared
+        if (g > 32) {
+            if ((G.t & 31) == 0) atomicMax(&sc->amax, u);
+            G.sync();
+            u = sc->amax;
+        }
+        if (kOwn == kCluster) {
+            cg::cluster_group cl = cg::this_cluster();
+            cl.sync();
+            const int lane = threadIdx.x & 31;
+            u = __reduce_max_sync(kFull, lane < static_cast<int>(cl.num_blocks()) ? remote(&sc->amax, lane) : 0u);
+        }
+        amax = __uint_as_float(u);
+        s = (amax < 0x1p-100f) ? 1.0f : __fdiv_rn(amax, static_cast<float>(qmax));
+        if (kClip && L.sin && valid) {
+            s = L.sin[m];
+            if (!(s > 0.0f && s < __int_as_float(0x7f800000))) s = 1.0f;
+        }
+    }
+
+    // ---- SQuant-E: codes and perturbations; the kernels' error sums leave at once (SQuant-C corrects
+    // the few it flips)
+    const bool fast = s >= 0x1p-60f && s <= 0x1p60f;
+    const int qmin = (mode & kModeWideRange) ? -qmax - 1 : -qmax;
+    unsigned sum = 0u;
+    float2 fs = make_float2(0.0f, 0.0f);
+    long long sum64 = 0;
+    int hi0 = 0, hi1 = 0, lo0 = 0, lo1 = 0;   // extremes over every other vector
+    {
+        const float s2 = fast ? __fmul_rn(s, 0x1p-30f) : 0.0f;
+        const E2 c2 = make_e2(fast ? __frcp_rn(s2) : 0.0f, s2);
+        const float tmin = kMagic + static_cast<float>(qmin) * 1073741824.0f, tmax = kMagic + static_cast<float>(qmax) * 1073741824.0f;
+        const bool kvec = ((reinterpret_cast<uintptr_t>(kerr) - 4 * r) & 15) == 0;
+        auto quantize = [&](const float4 w, int4 &p, float2 &oa, float2 &ob) -> unsigned {
+            float2 Pa, Pb;
+            unsigned c4;
+            if (fast) {
+                const float2 wa = make_float2(w.x, w.y), wb = make_float2(w.z, w.w);
+                float2 ta, tb;
+                if (!kClip) {
+                    squant_e_fast2(wa, c2, ta, Pa);
+                    squant_e_fast2(wb, c2, tb, Pb);
+                } else {
+                    const float2 xa = __fmul2_rn(wa, c2.y), xb = __fmul2_rn(wb, c2.y);
+                    const float2 Xa = __ffma2_rn(__ffma2_rn(xa, c2.ns2, wa), c2.y, xa), Xb = __ffma2_rn(__ffma2_rn(xb, c2.ns2, wb), c2.y, xb);
+                    ta = __fadd2_rn(Xa, c2.magic);
+                    tb = __fadd2_rn(Xb, c2.magic);
+                    ta.x = fminf(fmaxf(ta.x, tmin), tmax);   // the clip of Sec. 2.2
+                    ta.y = fminf(fmaxf(ta.y, tmin), tmax);
+                    tb.x = fminf(fmaxf(tb.x, tmin), tmax);
+                    tb.y = fminf(fmaxf(tb.y, tmin), tmax);
+                    Pa = __ffma2_rn(Xa, c2.neg1, __fadd2_rn(ta, c2.nmagic));
+                    Pb = __ffma2_rn(Xb, c2.neg1, __fadd2_rn(tb, c2.nmagic));
+                }
+                c4 = __byte_perm(__byte_perm(__float_as_uint(ta.x), __float_as_uint(ta.y), 0x0040),
+                                 __byte_perm(__float_as_uint(tb.x), __float_as_uint(tb.y), 0x0040), 0x5410);
+            } else {
+                c4 = row_e_div(w, s, kClip ? qmin : -255, kClip ? qmax : 255, Pa, Pb);
+            }
+            p = make_int4(__float2int_rn(Pa.x), __float2int_rn(Pa.y), __float2int_rn(Pb.x), __float2int_rn(Pb.y));
+            if (!kClip) {
+                fs = __fadd2_rn(fs, Pa);
+                fs = __fadd2_rn(fs, Pb);
+                sum += static_cast<unsigned>(p.x) + static_cast<unsigned>(p.y);
+                sum += static_cast<unsigned>(p.z) + static_cast<unsigned>(p.w);
+                oa = make_float2(__int2float_rn(p.x), __int2float_rn(p.y));
+                ob = make_float2(__int2float_rn(p.z), __int2float_rn(p.w));
+            } else {
+                row_clip_one(Pa.x, p.x, c4, qmin, qmax, sum64, oa.x);
+                row_clip_one(Pa.y, p.y, c4 >> 8, qmin, qmax, sum64, oa.y);
+                row_clip_one(Pb.x, p.z, c4 >> 16, qmin, qmax, sum64, ob.x);
+                row_clip_one(Pb.y, p.w, c4 >> 24, qmin, qmax, sum64, ob.y);
+            }
+            if (mode & 4u) {   // the extremes change places with those of the thread's other vectors
+                const int h1 = __vimax3_s32(hi0, p.x, p.y), l1 = __vimin3_s32(lo0, p.x, p.y);
+                hi0 = hi1; lo0 = lo1;
+                hi1 = __vimax3_s32(h1, p.z, p.w); lo1 = __vimin3_s32(l1, p.z, p.w);
+            }
+            const float2 k30 = make_float2(0x1p-30f, 0x1p-30f);
+            oa = __fmul2_rn(oa, k30);
+            ob = __fmul2_rn(ob, k30);
+            return c4;
+        };
+#pragma unroll 2
+        for (int q = q0; q < q_hi; q += g) {
+            int4 p;
+            float2 oa, ob;
+            cbuf[q] = quantize(reinterpret_cast<const float4 *>(Pbuf)[q], p, oa, ob);
+            Pbuf[q] = p;
+            if (kerr) {
+                float *ke = kerr + (4 * q - r);
+                if (kvec) __stcs(reinterpret_cast<float4 *>(ke), make_float4(oa.x, oa.y, ob.x, ob.y));
+                else { ke[0] = oa.x; ke[1] = oa.y; ke[2] = ob.x; ke[3] = ob.y; }
+            }
+        }
+        if (sp.ragged) {
+            int4 p;
+            float2 oa, ob;
+            const unsigned c4 = quantize(make_float4(w_rag, 0.0f, 0.0f, 0.0f), p, oa, ob);
+            if (rag >= 0) {
+                cel[rag] = static_cast<unsigned char>(c4);
+                Pel[rag] = p.x;
+                if (kerr) kerr[rag] = oa.x;
+            }
+        }
+    }
+
+    // ---- channel sum.  !kClip: its value modulo 2^32 is exact, its size is known from the float sums
+    // (2^16 elements of at most one half: the float sums are off by far less than 2^31)
+    long long ec = 0;
+    if ((mode & 4u) || L.cerr) {
+        unsigned tot = 0u;
+        int apx = 0;
+        if (!kClip) {
+            tot = static_cast<unsigned>(lanes_add(g, static_cast<int>(sum)));
+            apx = lanes_add(g, __float2int_rn(__fmul_rn(__fadd_rn(fs.x, fs.y), 0x1p-20f)));
+        } else {
+            for (int o = min(g, 32) >> 1; o > 0; o >>= 1) sum64 += __shfl_xor_sync(kFull, sum64, o);
+        }
+        if (g > 32) {
+            if ((G.t & 31) == 0) {
+                if (!kClip) {
+                    atomicAdd(&sc->sum, tot);
+                    atomicAdd(&sc->approx, apx);
+                } else {
+                    atomicAdd(&sc->sum64, static_cast<unsigned long long>(sum64));
+                }
+            }
+            G.sync();
+            tot = sc->sum;
+            apx = sc->approx;
+            sum64 = static_cast<long long>(sc->sum64);
+            if (kOwn == kCluster) {
+                cg::cluster_group cl = cg::this_cluster();
+                cl.sync();
+                tot = 0u;
+                apx = 0;
+                sum64 = 0;
+                for (int c = 0; c < static_cast<int>(cl.num_blocks()); ++c) {
+                    tot += remote(&sc->sum, c);
+                    apx += remote(&sc->approx, c);
+                    sum64 += static_cast<long long>(remote(&sc->sum64, c));
+                }
+            }
+        }
+        if (!kClip) {
+            const unsigned base = static_cast<unsigned>(apx) << 20;
+            ec = static_cast<long long>(apx) * (1ll << 20) + static_cast<int>(tot - base);
+        } else {
+            ec = sum64;
+        }
+    }
+
+    // ---- SQuant-C: Algorithm 2 on the channel, the perturbations are the keys
+    if (mode & 4u) {
+        const int sgn = ec > 0 ? 1 : -1;
+        const long long abs_e = ec > 0 ? ec : -ec;
+        const int kc = static_cast<int>(min((abs_e + (kHalf - 1)) >> 30, 1ll << 30));
+        const bool want = kc > 0;
+        if (g <= 32 ? __any_sync(kFull, want) : want) {
+            const int m0 = sgn > 0 ? hi0 : -lo0, m1 = sgn > 0 ? hi1 : -lo1;
+            const int sx = sgn > 0 ? 0 : -1;   // p ^ sx = the value in the direction of the flips, less one if that is downward
+            auto each = [&](int t, auto fn) {
+                const int tx = t + sx;
+                for (int qb = q0; qb < q_hi; qb += kRowVecs * g) {   // (kGroup: once)
+                unsigned hit = 0u, bit = 1u;   // a bit for each of these 32 elements that count
+#pragma unroll 2
+                for (int q = qb; q < min(q_hi, qb + kRowVecs * g); q += g, bit <<= 4) {
+                    const int4 p = Pbuf[q];
+                    if ((p.x ^ sx) >= tx) hit |= bit;
+                    if ((p.y ^ sx) >= tx) hit |= 2u * bit;
+                    if ((p.z ^ sx) >= tx) hit |= 4u * bit;
+                    if ((p.w ^ sx) >= tx) hit |= 8u * bit;
+                }
+#pragma unroll 1
+                for (; hit != 0u; hit &= hit - 1u) {
+                    const int b = __ffs(hit) - 1, n = 4 * (qb + (b >> 2) * g) - r + (b & 3);
+                    fn((Pel[n] ^ sx) - sx, n0 + n);
+                }
+                if (kOwn == kGroup) break;
+                }
+                if (rag >= 0) {
+                    const int v = Pel[rag] ^ sx;
+                    if (v >= tx) fn(v - sx, n0 + rag);
+                }
+            };
+            auto flip = [&](int a, int n_abs) {
+                const int n = n_abs - n0;
+                SQ_DBG(n >= 0 && n < N, 3);
+                unsigned char *cb = cel + n;
+                *cb = static_cast<unsigned char>(*cb - sgn);
+                if (kerr) kerr[n] = __fmul_rn(__int2float_rn(sgn > 0 ? a - kOne : kOne - a), 0x1p-30f);
+            };
+            const int k_eff = select_top<kOwn>(G, each, flip, m0, m1, kHalf + (1 << 14) + 1, 2.0f, kc, L.N, want, sc);
+            ec -= static_cast<long long>(sgn) * k_eff * kOne;
+        }
+    }
+    G.sync();   // all codes are final
+    if (!valid) return;
+
+    // ---- codes, scale, channel error
+    if (!pack) {
+        unsigned char *crow = reinterpret_cast<unsigned char *>(L.codes) + first;
+        if (((reinterpret_cast<uintptr_t>(crow) - r) & 3) == 0) {
+            unsigned *dst = reinterpret_cast<unsigned *>(crow - r);
+#pragma unroll 4
+            for (int q = q0; q < q_hi; q += g) __stcs(dst + q, cbuf[q]);
+            if (rag >= 0) crow[rag] = cel[rag];
+        } else {
+            for (int n = G.t; n < N; n += g) crow[n] = cel[n];
+        }
+    } else {   // two codes per byte, low nibble = even flat index; r = 0
+        unsigned char *crow = reinterpret_cast<unsigned char *>(L.codes) + static_cast<size_t>(m) * ((L.N + 1) >> 1) + (n0 >> 1);
+        const bool two = (reinterpret_cast<uintptr_t>(crow) & 1) == 0;
+        for (int q = q0; q < q_hi; q += g) {
+            const unsigned b = cbuf[q] & 0x0f0f0f0fu, h = b | (b >> 4);
+            if (two) {
+                *reinterpret_cast<unsigned short *>(crow + 2 * q) = static_cast<unsigned short>((h & 255u) | ((h >> 8) & 0xff00u));
+            } else {
+                crow[2 * q] = static_cast<unsigned char>(h);
+                crow[2 * q + 1] = static_cast<unsigned char>(h >> 16);
+            }
+        }
+        if (rag >= 0 && (rag & 1) == 0) crow[rag >> 1] = static_cast<unsigned char>((cel[rag] & 15) | (rag + 1 < N ? cel[rag + 1] << 4 : 0));
+    }
+    if (L.deq) {   // Algorithm 1's own return value: code * s
+        float *dg = L.deq + first;
+        const bool vec = ((reinterpret_cast<uintptr_t>(dg) - 4 * r) & 15) == 0;
+        for (int q = q0; q < q_hi; q += g) {
+            const unsigned c4 = cbuf[q];
+            const float4 d = make_float4(row_deq(c4, s), row_deq(c4 >> 8, s), row_deq(c4 >> 16, s), row_deq(c4 >> 24, s));
+            float *o = dg + (4 * q - r);
+            if (vec) __stcs(reinterpret_cast<float4 *>(o), d);
+            else { o[0] = d.x; o[1] = d.y; o[2] = d.z; o[3] = d.w; }
+        }
+        if (rag >= 0) dg[rag] = row_deq(cel[rag], s);
+    }
+    if (L.deq16) {   // the same product as bfloat16
+        uint16_t *dg = L.deq16 + first;
+        const bool vec = ((reinterpret_cast<uintptr_t>(dg) - 2 * r) & 7) == 0;
+        for (int q = q0; q < q_hi; q += g) {
+            const unsigned c4 = cbuf[q];
+            const unsigned b0 = bf16_bits(row_deq(c4, s)), b1 = bf16_bits(row_deq(c4 >> 8, s));
+            const unsigned b2 = bf16_bits(row_deq(c4 >> 16, s)), b3 = bf16_bits(row_deq(c4 >> 24, s));
+            uint16_t *o = dg + (4 * q - r);
+            if (vec) __stcs(reinterpret_cast<uint2 *>(o), make_uint2(b0 | (b1 << 16), b2 | (b3 << 16)));
+            else { o[0] = static_cast<uint16_t>(b0); o[1] = static_cast<uint16_t>(b1); o[2] = static_cast<uint16_t>(b2); o[3] = static_cast<uint16_t>(b3); }
+        }
+        if (rag >= 0) dg[rag] = static_cast<uint16_t>(bf16_bits(row_deq(cel[rag], s)));
+    }
+    if (G.t == 0 && n0 == 0) {
+        L.scales[m] = s;
+        if (L.cerr) L.cerr[m] = __fmul_rn(__ll2float_rn(ec), 0x1p-30f);
+    }
+}
+
+}  // namespace sq

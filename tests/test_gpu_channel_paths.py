@@ -1,0 +1,72 @@
+"""The grouped kernel's channel paths at the sizes where their bookkeeping can go wrong (needs a B200):
+1x1 rows around every group size and vector remainder, kernels of every specialised size around the
+group sizes, rows that start anywhere, all output forms, many flips and massive ties (the selection's
+exact search).  Whole numbers and raw float words must equal the checker's."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import paper_2202_07471_b200 as sq
+from paper_2202_07471_b200 import workloads as W
+
+from cases import adversarial_layer, coarse
+
+pytestmark = pytest.mark.gpu
+
+ROWS = (1, 2, 3, 5, 31, 32, 33, 252, 253, 256, 257, 509, 512, 1021, 1024, 1025, 2045, 2048, 4093, 4096, 8181, 8188, 8192)
+KERNELS = (1, 2, 3, 31, 33, 127, 128, 129, 256, 257, 511, 512, 513, 1025)
+
+
+def layers(shape, seed):
+    """Special channels; one-signed values (hundreds of flips per channel); a coarse grid (ties)."""
+    out = [adversarial_layer(shape, seed)]
+    if shape[1] >= 100:
+        out += [np.abs(W.random_layer((3,) + shape[1:], seed)), coarse(W.random_layer((3,) + shape[1:], seed), steps=24, div=4)]
+    return out
+
+
+def check(ws, bits, mode=sq.MODE_EKC, flags=sq.FLAG_NARROW_RANGE, start=0, outputs=False, clip=None):
+    pack = bool(flags & sq.FLAG_PACK_INT4)
+    bufs, scales = [], []
+    for i, w in enumerate(ws):
+        t = torch.zeros(w.size + 4, device="cuda")[start:start + w.size].view(w.shape)
+        t.copy_(torch.from_numpy(w))
+        b = sq.alloc_outputs(t, pack_int4=pack, dequant=outputs, dequant_bf16=outputs)
+        b.codes.fill_(-128)
+        b.kernel_err.fill_(float("nan"))
+        sc = None
+        if clip:
+            a = np.abs(w).reshape(w.shape[0], -1).max(1)
+            sc = (np.where(a > 0, a, 1) * clip / (2 ** (bits - 1) - 1)).astype(np.float32)
+            b.scales_in = torch.from_numpy(sc).cuda()
+        scales.append(sc)
+        bufs.append(b)
+    sq.squant_quantize_model(bufs, bits=bits, mode=mode, flags=flags)
+    sq.squant_device_status()
+    for b, w, sc in zip(bufs, ws, scales):
+        r = oracle.quantize_layer(w, bits=bits, mode=mode, flags=flags, details=True, scales_in=sc)
+        pairs = [(b.codes, r.codes), (b.scales, r.scales), (b.kernel_err, r.kernel_err), (b.channel_err, r.channel_err)]
+        if outputs:
+            pairs += [(b.dequant, r.dequant), (b.dequant_bf16.view(torch.int16), r.dequant_bf16.view(np.int16))]
+        for k, (got, want) in enumerate(pairs):
+            got = got.cpu().numpy()
+            assert np.array_equal(got.view(np.uint8), np.ascontiguousarray(want).view(np.uint8)), (w.shape, bits, mode, flags, start, clip, k)
+
+
+def shapes(kind):
+    if kind == "rows":
+        return [(5 if n > 1000 else 37, n, 1, 1) for n in ROWS]
+    return [(5 if n > 200 else 19, n) + k for k in ((3, 3), (1, 7), (3, 1), (2, 2), (5, 5)) for n in KERNELS if n * k[0] * k[1] <= 14000]
+
+
+@pytest.mark.parametrize("kind", ["rows", "kernels"])
+@pytest.mark.parametrize("bits,mode,flags", [(4, 7, 1), (8, 7, 0), (2, 7, 1), (4, 3, 1), (4, 1, 0)])
+def test_channel_paths(kind, bits, mode, flags):
+    ws = [w for i, s in enumerate(shapes(kind)) for w in layers(s, 40 * bits + i)]
+    check(ws, bits, mode, flags)
+    check(ws, bits, mode, flags, start=1, outputs=True)
+    if bits <= 4:
+        check(ws, bits, mode, flags | sq.FLAG_PACK_INT4, start=3)
+    check(ws, bits, mode, flags, start=2, clip=0.6)
+    check(ws, bits, mode, flags, outputs=True, clip=0.9)
