@@ -13,7 +13,6 @@
 #include <vector>
 
 #include "squant_device.cuh"
-#include "squant_pipe.cuh"
 #include "squant_stream.cuh"
 #include "squant_wide.cuh"
 
@@ -28,6 +27,7 @@ constexpr int64_t kMaxChannelElems = 65535; // one-CTA paths: keeps the clamp-ed
                                             // kernel, which checks every candidate against the clip range
 constexpr int64_t kMaxKernels = (1 << sq::kIdxBits) - 1;   // kernels per channel: the select keys hold 18 index bits
 constexpr size_t kMaxPlans = 64;
+constexpr int kLongChannel = 8192;           // weights: longer channels are launched apart from the others
 constexpr int kWideSmemGoal = 112 << 10;     // the same of a cluster's thread block: two of them
 constexpr int kGroupedSmemGoal = 55 << 10;   // shared memory of a grouped CTA with which four of them share a multiprocessor
 
@@ -105,7 +105,7 @@ int validate(const squant_layer *layers, int32_t n_layers, const squant_options 
     return SQUANT_OK;
 }
 
-// Layout of a channel with staged weights and per-kernel arrays: the pipelined kernel's layers, E|C on
+// Layout of a channel with staged weights and per-kernel arrays: E|C on
 // larger kernels, 1x1 rows beyond the registers of one thread block.
 void layout_staged(const squant_layer &l, LayerDesc &d, unsigned mode)
 {
@@ -211,9 +211,9 @@ int build_plan(const squant_layer *layers, int32_t n_layers, const squant_option
 // CTAs (heaviest first, so the tail of the launch is made of light CTAs), at most
 // kMaxParamLayers per launch.
 struct ParamPlan {
-    std::vector<sq::LaunchTable> tables;   // grouped kernel: one CTA per item
-    std::vector<int> grids;
-    int smem_bytes = 0, qmax = 0;
+    struct Grouped { sq::LaunchTable table; int grid, smem; };
+    std::vector<Grouped> grouped;   // grouped kernel: one CTA per item
+    int qmax = 0;
     unsigned mode = 0;
     // cluster kernel (channels wider than one CTA): one launch per layer
     struct Wide { LayerDesc d; int cluster, kpc, smem; };
@@ -221,14 +221,20 @@ struct ParamPlan {
     // row kernel (1x1 rows too long for a group): one item per output channel
     std::vector<sq::LaunchTable> row_tables;
     std::vector<int> row_grids, row_smem;
-    // pipelined kernel (layers of long 3x3 channels): one item per output channel
-    std::vector<sq::LaunchTable> pipe_tables;
-    std::vector<int> pipe_items, pipe_set_stride, pipe_slot;
-    std::vector<int> pipe_stream;   // 1: the launch goes to the streaming kernel (plain int8 output); pipe_set_stride then
-    std::vector<int> pipe_nmax;     // holds the longest channel in weights and pipe_nmax the same in kernels
-    // Scratch of the streaming kernel's launches (what SQuant-C needs of every kernel one step later: four
-    // sets of 18 KB per thread block), allocated at the plan's first launch, freed with the plan.
-    mutable std::vector<void *> pipe_scratch;
+    // streaming kernel (layers of long 3x3 channels): one item per output channel
+    struct Stream {
+        sq::LaunchTable table;
+        int items, nk_max, n_max, slot;
+        bool out;                     // packed or dequantized outputs wanted
+        // Scratch (what SQuant-C needs of every kernel one step later: four sets of 18 KB per thread block),
+        // allocated at the plan's first launch, freed with the plan.
+        void *scratch;
+        // Layers with packed or dequantized outputs can also go to the grouped kernel, which needs no scratch:
+        // where it cannot be allocated (a full device, the plan's first launch inside a stream capture).
+        sq::LaunchTable grouped;
+        int grouped_grid, grouped_smem;
+    };
+    mutable std::vector<Stream> streams;
     ParamPlan() = default;
     ParamPlan(ParamPlan &&) = default;
     ParamPlan &operator=(ParamPlan &&) = default;
@@ -236,31 +242,45 @@ struct ParamPlan {
     ParamPlan &operator=(const ParamPlan &) = delete;
     ~ParamPlan()
     {
-        for (void *q : pipe_scratch)
-            if (q) cudaFree(q);
+        for (Stream &st : streams)
+            if (st.scratch) cudaFree(st.scratch);
     }
-    mutable bool slots_clean = false;   // the work counters of pipe_slot have been zeroed on the stream of the plan's first launch
+    mutable bool slots_clean = false;   // the streams' work counters have been zeroed on the stream of the plan's first launch
 };
 
-int g_next_slot = 0;   // next work-counter slot of the pipelined kernel; guarded by g_mutex
+int g_next_slot = 0;   // next work-counter slot of the streaming kernel; guarded by g_mutex
 
-// Layers the pipelined kernel takes: 3x3, more than 8192 weights per output channel (the grouped
-// kernel gives such a channel a whole CTA), input channels a multiple of four, SQuant-K on, absmax
-// scales, and two buffer sets fit the shared memory of one SM.
-bool pipe_eligible(const squant_layer &l, const LayerDesc &d, const squant_options &o, int max_smem)
-{
-    if (d.K != 9 || (d.N & 3) != 0 || d.NK <= 8192) return false;
-    if (!(o.mode & SQUANT_MODE_K) || l.scales_in) return false;
-    if ((reinterpret_cast<uintptr_t>(l.w) & 15) || (reinterpret_cast<uintptr_t>(l.codes) & 15)) return false;
-    return 2 * d.slice_bytes + sq::kPipeCtrlBytes <= max_smem;
-}
-
-// Of those, the streaming kernel takes the layers with plain int8 codes and nothing else to emit.
+// Layers the streaming kernel takes: 3x3 channels so long that no four CTAs of the grouped kernel fit a
+// multiprocessor (from 1184 input channels on: 2048 channels take 42.4 us in the grouped kernel and 59.8 us
+// in this one at N = 1028, 46.5 and 52.7 us at 1152, 55.0 and 53.1 us at 1280, 89.0 and 57.5 us at 2048; with
+// packed codes 44 and 59, 58 and 60, 94 and 68 us at 1028, 1280, 2048), input channels a multiple of four and one quad of kernels per
+// quantizer thread, SQuant-K on, absmax scales, and its buffers fit the shared memory of one SM.
 bool stream_eligible(const squant_layer &l, const LayerDesc &d, const squant_options &o, int max_smem)
 {
-    if (l.dequant || l.dequant_bf16 || (o.flags & SQUANT_FLAG_PACK_INT4)) return false;
-    if (d.N > 4 * sq::kStreamQuantThreads) return false;   // one quad of kernels per quantizer thread
+    if (d.K != 9 || (d.N & 3) != 0 || sq::conv_bytes(sq::kCtaThreads, d.NK, d.K) <= kGroupedSmemGoal) return false;
+    if (!(o.mode & SQUANT_MODE_K) || l.scales_in) return false;
+    if ((reinterpret_cast<uintptr_t>(l.w) & 15) || (reinterpret_cast<uintptr_t>(l.codes) & 15)) return false;
+    if (d.N > 4 * sq::kStreamQuantThreads) return false;
     return sq::stream_layout(d.NK, d.N).total <= max_smem;
+}
+
+// Launch table of n layers; work items are CTAs of the grouped kernel or single output channels.  Returns
+// the number of items.
+int fill_table(sq::LaunchTable &t, const std::vector<LayerDesc> &descs, const int *layers, int n, bool ctas)
+{
+    std::memset(&t, 0, sizeof(t));
+    t.n_layers = n;
+    for (int step = 1; step < n; step <<= 1) t.top_step = step;
+    int items = 0;
+    for (int j = 0; j < n; ++j) {
+        const LayerDesc &d = descs[layers[j]];
+        const int groups = ctas ? sq::kCtaThreads / d.g : 1;
+        t.layers[j] = d;
+        t.first_item[j] = items;
+        items += (d.M + groups - 1) / groups;
+    }
+    for (int j = n; j <= sq::kMaxParamLayers; ++j) t.first_item[j] = items;
+    return items;
 }
 
 int build_param_plan(const squant_layer *layers, int32_t n_layers, const squant_options &o,
@@ -269,9 +289,8 @@ int build_param_plan(const squant_layer *layers, int32_t n_layers, const squant_
     p.qmax = (1 << (o.bits - 1)) - 1;
     p.mode = o.mode | ((o.flags & SQUANT_FLAG_PACK_INT4) ? sq::kModePackInt4 : 0u) |
              ((o.flags & SQUANT_FLAG_NARROW_RANGE) ? 0u : sq::kModeWideRange);
-    p.smem_bytes = 0;
     std::vector<LayerDesc> descs(n_layers);
-    std::vector<int> order, piped, streamed, rows;
+    std::vector<int> order, streamed[2], rows;
     for (int i = 0; i < n_layers; ++i) {
         const int64_t cta_smem = layout_layer(layers[i], descs[i], o.mode, o.flags);
         if (cta_smem > max_smem || descs[i].NK > kMaxChannelElems) {
@@ -297,116 +316,77 @@ int build_param_plan(const squant_layer *layers, int32_t n_layers, const squant_
             p.wide.push_back(w);
             continue;
         }
-        LayerDesc staged = descs[i];
-        layout_staged(layers[i], staged, o.mode);
-        if (pipe_eligible(layers[i], staged, o, max_smem)) {
-            descs[i] = staged;
-            (stream_eligible(layers[i], descs[i], o, max_smem) ? streamed : piped).push_back(i);
+        if (stream_eligible(layers[i], descs[i], o, max_smem)) {
+            const squant_layer &l = layers[i];
+            streamed[l.dequant || l.dequant_bf16 || (o.flags & SQUANT_FLAG_PACK_INT4) ? 1 : 0].push_back(i);
             continue;
         }
         if (descs[i].K == 1 && descs[i].off_hist != 0 && descs[i].N <= sq::kRowBlockElems) {   // too long for a group, 164 KB at most
             rows.push_back(i);
             continue;
         }
-        if (cta_smem > p.smem_bytes) p.smem_bytes = static_cast<int>(cta_smem);
         order.push_back(i);
     }
     // long rows, longest first: a thread block per output channel
     std::stable_sort(rows.begin(), rows.end(), [&](int a, int b) { return descs[a].N > descs[b].N; });
     for (size_t base = 0; base < rows.size(); base += sq::kMaxParamLayers) {
         const int n = static_cast<int>(std::min<size_t>(rows.size() - base, sq::kMaxParamLayers));
-        p.row_tables.emplace_back();
-        sq::LaunchTable &t = p.row_tables.back();
-        std::memset(&t, 0, sizeof(t));
-        t.n_layers = n;
-        for (int st = 1; st < n; st <<= 1) t.top_step = st;
-        int items = 0, smem = 0;
+        int smem = 0;
         for (int j = 0; j < n; ++j) {
-            LayerDesc d = descs[rows[base + j]];
+            LayerDesc &d = descs[rows[base + j]];
             d.off_vi = (d.N + 6) >> 2;
             smem = std::max(smem, sq::row_bytes(sq::kBlockThreads, d.off_vi, sq::kBlock));
-            t.layers[j] = d;
-            t.first_item[j] = items;
-            items += d.M;
         }
-        for (int j = n; j <= sq::kMaxParamLayers; ++j) t.first_item[j] = items;
-        p.row_grids.push_back(items);
+        p.row_tables.emplace_back();
+        p.row_grids.push_back(fill_table(p.row_tables.back(), descs, rows.data() + base, n, false));
         p.row_smem.push_back(smem);
     }
-    for (int kind = 0; kind < 2; ++kind) {
-    const std::vector<int> &piped_k = kind ? streamed : piped;
-    for (size_t base = 0; base < piped_k.size(); base += sq::kMaxParamLayers) {
-        const int n = static_cast<int>(std::min<size_t>(piped_k.size() - base, sq::kMaxParamLayers));
-        p.pipe_tables.emplace_back();
-        sq::LaunchTable &t = p.pipe_tables.back();
-        std::memset(&t, 0, sizeof(t));
-        t.n_layers = n;
-        for (int st = 1; st < n; st <<= 1) t.top_step = st;
-        int items = 0, stride = 0;
-        for (int j = 0; j < n; ++j) {
-            const LayerDesc &d = descs[piped_k[base + j]];
-            t.layers[j] = d;
-            t.first_item[j] = items;
-            items += d.M;
-            stride = std::max(stride, d.slice_bytes);
+    for (int kind = 1; kind >= 0; --kind) {
+        const std::vector<int> &list = streamed[kind];
+        for (size_t base = 0; base < list.size(); base += sq::kMaxParamLayers) {
+            const int n = static_cast<int>(std::min<size_t>(list.size() - base, sq::kMaxParamLayers));
+            p.streams.emplace_back();
+            ParamPlan::Stream &st = p.streams.back();
+            std::memset(&st, 0, sizeof(st));
+            st.items = fill_table(st.table, descs, list.data() + base, n, false);
+            st.grouped_grid = fill_table(st.grouped, descs, list.data() + base, n, true);
+            for (int j = 0; j < n; ++j) {
+                const LayerDesc &d = descs[list[base + j]];
+                st.nk_max = std::max(st.nk_max, d.NK);
+                st.n_max = std::max(st.n_max, d.N);
+                st.grouped_smem = std::max(st.grouped_smem, sq::kCtaThreads / d.g * d.slice_bytes);
+            }
+            st.out = kind != 0;
+            st.slot = g_next_slot;
+            g_next_slot = (g_next_slot + 1) % sq::kTicketSlots;
         }
-        for (int j = n; j <= sq::kMaxParamLayers; ++j) t.first_item[j] = items;
-        // One layout for every layer of the launch, that of the widest one: the staging area of a
-        // long channel must not reach into the buffers the finishers still use for a shorter one
-        // that had the set before, and the channel-step scratch is found (and cleared) without
-        // knowing the layer.  It sits at the end of a set.
-        int widest = 0;
-        for (int j = 1; j < n; ++j)
-            if (t.layers[j].slice_bytes > t.layers[widest].slice_bytes) widest = j;
-        for (int j = 0; j < n; ++j) {
-            LayerDesc &d = t.layers[j];
-            const LayerDesc &wd = t.layers[widest];
-            d.off_codes = wd.off_codes; d.off_ev = wd.off_ev; d.off_vv = wd.off_vv; d.off_vi = wd.off_vi;
-            d.off_hist = wd.off_hist; d.off_red = wd.off_red; d.slice_bytes = wd.slice_bytes;
-        }
-        int nk_max = 0, n_max = 0;
-        for (int j = 0; j < n; ++j) {
-            nk_max = std::max(nk_max, t.layers[j].NK);
-            n_max = std::max(n_max, t.layers[j].N);
-        }
-        p.pipe_items.push_back(items);
-        p.pipe_set_stride.push_back(kind ? nk_max : stride);
-        p.pipe_stream.push_back(kind);
-        p.pipe_scratch.push_back(nullptr);
-        p.pipe_nmax.push_back(n_max);
-        p.pipe_slot.push_back(g_next_slot);
-        g_next_slot = (g_next_slot + 1) % sq::kTicketSlots;
     }
-    }
-    n_layers = static_cast<int32_t>(order.size());   // the grouped kernel takes the rest
-    // Estimated duration of one CTA of the layer.  Kernel sizes other than 1x1 and 3x3 take the
-    // general per-thread path, which is latency-bound and far slower per weight (a 7x7 stem CTA
-    // is the longest of a whole ResNet), so those start first.
+    // The grouped kernel takes the rest, layers of long channels in launches of their own: their CTAs need
+    // shared memory that would cost the others their fourth CTA per multiprocessor.
+    // Estimated duration of one CTA of the layer.  Kernel sizes without a body of their own take the
+    // general per-thread path, which is latency-bound and far slower per weight, so those start first.
     auto cta_work = [&](int i) {
         const LayerDesc &d = descs[i];
         const int64_t groups = sq::kCtaThreads / d.g;
-        const int64_t per_channel = (d.K == 1 || d.K == 9) ? d.NK : static_cast<int64_t>(d.NK) * 64 * d.K;
-        return (groups < d.M ? groups : d.M) * per_channel;
+        const bool own = d.K == 1 || d.K == 3 || d.K == 7 || d.K == 9;
+        return (groups < d.M ? groups : d.M) * (own ? d.NK : static_cast<int64_t>(d.NK) * 64 * d.K);
     };
-    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return cta_work(a) > cta_work(b); });
-    for (int base = 0; base < n_layers; base += sq::kMaxParamLayers) {
-        const int n = (n_layers - base < sq::kMaxParamLayers) ? n_layers - base : sq::kMaxParamLayers;
-        p.tables.emplace_back();
-        sq::LaunchTable &t = p.tables.back();
-        std::memset(&t, 0, sizeof(t));
-        t.n_layers = n;
-        t.top_step = 0;
-        for (int st = 1; st < n; st <<= 1) t.top_step = st;
-        int items = 0;
-        for (int j = 0; j < n; ++j) {
+    auto is_long = [&](int i) { return descs[i].NK > kLongChannel; };
+    std::stable_sort(order.begin(), order.end(), [&](int a, int b) {
+        return is_long(a) != is_long(b) ? is_long(a) : cta_work(a) > cta_work(b);
+    });
+    for (size_t base = 0; base < order.size();) {
+        size_t n = 1;
+        while (base + n < order.size() && n < sq::kMaxParamLayers && is_long(order[base + n]) == is_long(order[base])) ++n;
+        p.grouped.emplace_back();
+        ParamPlan::Grouped &gl = p.grouped.back();
+        gl.smem = 0;
+        for (size_t j = 0; j < n; ++j) {
             const LayerDesc &d = descs[order[base + j]];
-            const int groups = sq::kCtaThreads / d.g;
-            t.layers[j] = d;
-            t.first_item[j] = items;
-            items += (d.M + groups - 1) / groups;
+            gl.smem = std::max(gl.smem, sq::kCtaThreads / d.g * d.slice_bytes);
         }
-        for (int j = n; j <= sq::kMaxParamLayers; ++j) t.first_item[j] = items;
-        p.grids.push_back(items);
+        gl.grid = fill_table(gl.table, descs, order.data() + base, static_cast<int>(n), true);
+        base += n;
     }
     return SQUANT_OK;
 }
@@ -441,13 +421,13 @@ int device_smem_limit(int device, int &limit)
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, v));
         SQ_CUDA(cudaFuncSetAttribute(sq::squant_table_kernel,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, v));
-        SQ_CUDA(cudaFuncSetAttribute(sq::squant_pipe_kernel,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, v));
         SQ_CUDA(cudaFuncSetAttribute(sq::squant_row_kernel,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, v));
         SQ_CUDA(cudaFuncSetAttribute(sq::squant_wide_kernel,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, v));
-        SQ_CUDA(cudaFuncSetAttribute(sq::squant_stream_kernel,
+        SQ_CUDA(cudaFuncSetAttribute(sq::squant_stream_kernel<false>,
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, v));
+        SQ_CUDA(cudaFuncSetAttribute(sq::squant_stream_kernel<true>,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, v));
         int sms = 0;
         SQ_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device));
@@ -504,35 +484,38 @@ int launch_plan(const ParamPlan &p, cudaStream_t stream)
     // A work-counter slot comes to a plan in an unknown state (a plan that was evicted, or a launch
     // that failed, may have left it dirty): zero it in stream order before the plan's first launch.
     if (!p.slots_clean) {
-        for (size_t c = 0; c < p.pipe_tables.size(); ++c) {
-            SQ_CUDA(cudaMemsetAsync(ticket_address(p.pipe_slot[c], false), 0, sizeof(unsigned), stream));
-            SQ_CUDA(cudaMemsetAsync(ticket_address(p.pipe_slot[c], true), 0, sizeof(unsigned), stream));
+        for (const ParamPlan::Stream &st : p.streams) {
+            SQ_CUDA(cudaMemsetAsync(ticket_address(st.slot, false), 0, sizeof(unsigned), stream));
+            SQ_CUDA(cudaMemsetAsync(ticket_address(st.slot, true), 0, sizeof(unsigned), stream));
         }
         p.slots_clean = true;
     }
     // long 3x3 channels first: one persistent CTA per multiprocessor
-    for (size_t c = 0; c < p.pipe_tables.size(); ++c) {
-        if (p.pipe_items[c] == 0) continue;
+    for (ParamPlan::Stream &st : p.streams) {
         int device = 0;
         SQ_CUDA(cudaGetDevice(&device));
-        const int grid = std::min(p.pipe_items[c], std::max(g_sm_count_by_device[device], 1));
-        if (p.pipe_stream[c]) {
-            const int smem = sq::stream_layout(p.pipe_set_stride[c], p.pipe_nmax[c]).total;
-            if (!p.pipe_scratch[c]) {
-                const size_t bytes = static_cast<size_t>(std::max(g_sm_count_by_device[device], 1)) * sq::kStreamHeldSets * sq::kStreamHeldBytes;
-                if (cudaMalloc(&p.pipe_scratch[c], bytes) != cudaSuccess) {
-                    cudaGetLastError();   // the failed allocation is reported by the return code, not left pending
-                    p.pipe_scratch[c] = nullptr;
-                    return SQUANT_ERR_NOMEM;
-                }
+        const int sms = std::max(g_sm_count_by_device[device], 1);
+        if (!st.scratch) {
+            bool try_alloc = true;
+            if (st.out) {
+                cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+                SQ_CUDA(cudaStreamIsCapturing(stream, &cap));
+                try_alloc = cap == cudaStreamCaptureStatusNone;
             }
-            sq::squant_stream_kernel<<<grid, sq::kStreamThreads, smem, stream>>>(p.pipe_tables[c], p.qmax, p.mode, p.pipe_items[c],
-                                                                             p.pipe_slot[c], p.pipe_set_stride[c], p.pipe_nmax[c],
-                                                                             static_cast<unsigned char *>(p.pipe_scratch[c]));
+            const size_t bytes = static_cast<size_t>(sms) * sq::kStreamHeldSets * sq::kStreamHeldBytes;
+            if (try_alloc && cudaMalloc(&st.scratch, bytes) != cudaSuccess) {
+                cudaGetLastError();   // the failed allocation is reported by the return code, not left pending
+                st.scratch = nullptr;
+                if (!st.out) return SQUANT_ERR_NOMEM;
+            }
+        }
+        if (st.scratch) {
+            const int grid = std::min(st.items, sms), smem = sq::stream_layout(st.nk_max, st.n_max).total;
+            auto kernel = st.out ? sq::squant_stream_kernel<true> : sq::squant_stream_kernel<false>;
+            kernel<<<grid, sq::kStreamThreads, smem, stream>>>(st.table, p.qmax, p.mode, st.items, st.slot, st.nk_max, st.n_max,
+                                                               static_cast<unsigned char *>(st.scratch));
         } else {
-            const int smem = 2 * p.pipe_set_stride[c] + sq::kPipeCtrlBytes;
-            sq::squant_pipe_kernel<<<grid, sq::kPipeThreads, smem, stream>>>(p.pipe_tables[c], p.qmax, p.mode, p.pipe_items[c],
-                                                                         p.pipe_slot[c], p.pipe_set_stride[c]);
+            sq::squant_model_kernel<<<st.grouped_grid, sq::kCtaThreads, st.grouped_smem, stream>>>(st.grouped, p.qmax, p.mode);
         }
         SQ_CUDA(cudaGetLastError());
         g_launches.fetch_add(1, std::memory_order_relaxed);
@@ -542,9 +525,8 @@ int launch_plan(const ParamPlan &p, cudaStream_t stream)
         SQ_CUDA(cudaGetLastError());
         g_launches.fetch_add(1, std::memory_order_relaxed);
     }
-    for (size_t c = 0; c < p.tables.size(); ++c) {
-        if (p.grids[c] == 0) continue;
-        sq::squant_model_kernel<<<p.grids[c], sq::kCtaThreads, p.smem_bytes, stream>>>(p.tables[c], p.qmax, p.mode);
+    for (const ParamPlan::Grouped &gl : p.grouped) {
+        sq::squant_model_kernel<<<gl.grid, sq::kCtaThreads, gl.smem, stream>>>(gl.table, p.qmax, p.mode);
         SQ_CUDA(cudaGetLastError());
         g_launches.fetch_add(1, std::memory_order_relaxed);
     }

@@ -265,58 +265,6 @@ __device__ __forceinline__ void kernel_generic(float *wk, int K, float s, bool d
     idx_out = idx;
 }
 
-// ---------------------------------------------------------------- one kernel, K in registers
-template <int K>
-__device__ __forceinline__ void kernel_regs(const float *wk, float s, bool do_k, int8_t *ck,
-                                            long long &e_out, int &v_out, int &idx_out)
-{
-    int P[K], q[K];
-    long long e = 0;
-#pragma unroll
-    for (int i = 0; i < K; ++i) {
-        squant_e(wk[i], s, q[i], P[i]);
-        e += P[i];
-    }
-    int v = 0, idx = 0;
-    if (e != 0) {
-        const int sgn = e > 0 ? 1 : -1;
-        const long long abs_e = e > 0 ? e : -e;
-        const int k = do_k ? flip_count(abs_e) : 0;
-        int flips = 0, last = -1, cand = -1;
-        for (int r = 0; r <= k; ++r) {
-            int best = 0, bi = -1;
-#pragma unroll
-            for (int i = 0; i < K; ++i) {
-                const int key = sgn * P[i];
-                if (key > best) { best = key; bi = i; }
-            }
-            if (bi < 0) break;
-            if (r < k) {
-#pragma unroll
-                for (int i = 0; i < K; ++i)
-                    if (i == bi) { P[i] -= sgn * kOne; q[i] -= sgn; }
-                last = bi;
-                ++flips;
-            } else {
-                cand = bi;
-            }
-        }
-        e -= static_cast<long long>(sgn) * flips * kOne;
-        const int pick = (static_cast<long long>(flips) * kOne > abs_e) ? last : cand;
-        if (pick >= 0) {
-            idx = pick;
-#pragma unroll
-            for (int i = 0; i < K; ++i)
-                if (i == pick) v = P[i];
-        }
-    }
-#pragma unroll
-    for (int i = 0; i < K; ++i) ck[i] = static_cast<int8_t>(q[i]);
-    e_out = e;
-    v_out = v;
-    idx_out = idx;
-}
-
 // ---------------------------------------------------------------- SQuant-C selection
 // Key of a kernel's candidate in Algorithm 2's order on the channel: larger |v| first, equal |v|
 // by lower kernel index.  0 = not a candidate for this sign.
@@ -535,11 +483,6 @@ __device__ __noinline__ KernelOut kernel9_exact_t(const float *wk, float y, floa
     return o;
 }
 
-__device__ __forceinline__ KernelOut kernel9_exact(const float *wk, float y, float s2, unsigned char *cb)
-{
-    return kernel9_exact_t<false>(wk, y, s2, cb);
-}
-
 // Fast SQuant-K + Algorithm 3 on one 3x3 kernel whose exact perturbations Pf[0..8] (floats, in
 // 2^-30 units, before the conversion to integers) are in registers and whose code bytes are
 // already staged at cb.  Straight-line on purpose: every lane runs the same instructions; a
@@ -648,7 +591,6 @@ __device__ __forceinline__ float stage_channel(const LayerDesc &L, int m, const 
         for (int i = G.t; i < kHistBins; i += G.g) hist[i] = 0;
         if (G.t == 0) {
             reinterpret_cast<int *>(red + 128)[5] = 0;                    // boundary-list count
-            reinterpret_cast<int *>(red + 128)[6] = 0;                    // redo-list count (3x3 fast path)
             *reinterpret_cast<unsigned long long *>(red + 208) = 0ull;   // channel-sum accumulator
             *reinterpret_cast<unsigned *>(red + 216) = 0u;               // absmax slot
         }
@@ -904,104 +846,41 @@ __device__ __forceinline__ void channel_single(const LayerDesc &L, int m, unsign
     if (L.cerr) L.cerr[m] = ef;
 }
 
-// ---------------------------------------------------------------- channel body, any kernel size
-template <int KT>
-__device__ __forceinline__ void channel_body(const LayerDesc &L, int m, const Group &G,
-                                             unsigned char *slice, float s, unsigned mode)
+// ---------------------------------------------------------------- 1x1 rows beyond the row kernel's shared memory
+// (and, in the entry point without device allocation, beyond a group's registers): staged in the shared
+// memory of one CTA, any length and scale.  The perturbations overwrite the weights.
+__device__ __forceinline__ void channel_body_row(const LayerDesc &L, int m, const Group &G, unsigned char *slice, float s, unsigned mode)
 {
-    const int K = KT ? KT : L.K;
     const int N = L.N;
     float *wbuf = reinterpret_cast<float *>(slice);
     int8_t *cbuf = reinterpret_cast<int8_t *>(slice + L.off_codes);
-    int *ev = reinterpret_cast<int *>(slice + L.off_ev);
-    int *vv = reinterpret_cast<int *>(slice + L.off_vv);
-    unsigned short *vi = reinterpret_cast<unsigned short *>(slice + L.off_vi);
-
-    // ---- SQuant-E, SQuant-K, candidate: one thread per kernel
-    // Without SQuant-K a kernel sum can reach K/2 and no longer fits 32 bits; it is then
-    // emitted right here (no channel step follows: E|C on larger kernels has its own body).
-    const bool do_k = (mode & 2u) != 0;
-    const bool keep = do_k || KT == 1 || K == 1;
+    int *ev = reinterpret_cast<int *>(slice);
     float *kerr = L.kerr ? L.kerr + static_cast<size_t>(m) * N : nullptr;
     long long esum = 0;
-    if (KT == 0 && K >= 16 && 4 * N <= G.g) {
-        // few kernels of many elements: a warp per kernel, lanes over its elements
-        const int lane = G.t & 31;
-        for (int n = G.t >> 5; n < N; n += G.g >> 5) {
-            long long e1;
-            int v, idx;
-            kernel_warp(wbuf + static_cast<size_t>(n) * K, K, s, do_k, cbuf + static_cast<size_t>(n) * K, lane, e1, v, idx);
-            if (lane == 0) {
-                if (keep) {
-                    ev[n] = static_cast<int>(e1);
-                    vv[n] = v;
-                    vi[n] = static_cast<unsigned short>(idx);
-                } else if (kerr) {
-                    kerr[n] = __fmul_rn(__ll2float_rn(e1), 0x1p-30f);
-                }
-                esum += e1;
-            }
-        }
-    } else
     for (int n = G.t; n < N; n += G.g) {
-        long long e1;
-        if (KT == 1) {
-            int q, P;
-            squant_e(wbuf[n], s, q, P);
-            cbuf[n] = static_cast<int8_t>(q);
-            e1 = P;                  // a 1x1 kernel is its own candidate; ev and vv alias wbuf
-            ev[n] = P;
-        } else {
-            int v, idx;
-            if (KT == 0) kernel_generic(wbuf + static_cast<size_t>(n) * K, K, s, do_k, cbuf + static_cast<size_t>(n) * K, e1, v, idx);
-            else kernel_regs<(KT > 1 ? KT : 2)>(wbuf + n * K, s, do_k, cbuf + n * K, e1, v, idx);
-            if (keep) {
-                ev[n] = static_cast<int>(e1);
-                vv[n] = v;
-                vi[n] = static_cast<unsigned short>(idx);
-            } else if (kerr) {
-                kerr[n] = __fmul_rn(__ll2float_rn(e1), 0x1p-30f);
-            }
-        }
-        esum += e1;
+        int q, P;
+        squant_e(wbuf[n], s, q, P);
+        cbuf[n] = static_cast<int8_t>(q);
+        ev[n] = P;   // a 1x1 kernel is its own candidate
+        esum += P;
     }
-
-    // ---- SQuant-C: Algorithm 2 on the channel, keys = the kernels' candidates
     const ChannelStep cs = channel_step(L, G, slice, esum, mode);
-    const long long ec = cs.ec;
-    const int sgn_c = cs.sgn_c, k_eff = cs.k_eff;
-    const unsigned long long T = cs.T;
-
-    // ---- apply the channel flips, emit the kernels' error sums
-    if (keep && (k_eff > 0 || kerr)) {
+    if (cs.k_eff > 0 || kerr) {
         for (int n = G.t; n < N; n += G.g) {
             int e1 = ev[n];
-            if (k_eff > 0) {
-                const unsigned long long ck = cand_key(vv[n], sgn_c, n);
-                if (ck != 0 && ck >= T) {
-                    e1 -= sgn_c * kOne;
-                    const size_t j = (KT == 1) ? n : static_cast<size_t>(n) * K + vi[n];
-                    if (SQ_DBG_OK(j < static_cast<size_t>(L.NK) && (KT == 1 || vi[n] < K), 2)) cbuf[j] = static_cast<int8_t>(cbuf[j] - sgn_c);
+            if (cs.k_eff > 0) {
+                const unsigned long long ck = cand_key(e1, cs.sgn_c, n);
+                if (ck != 0 && ck >= cs.T) {
+                    e1 -= cs.sgn_c * kOne;
+                    cbuf[n] = static_cast<int8_t>(cbuf[n] - cs.sgn_c);
                 }
             }
             if (kerr) kerr[n] = __fmul_rn(__int2float_rn(e1), 0x1p-30f);
         }
     }
     G.sync();
-#ifdef SQUANT_DEBUG_BOUNDS
-    // Checked build, kernels kept in shared memory: the perturbations staged after SQuant-K, summed
-    // again, minus one unit per channel flip must equal the channel sum.
-    if (KT == 0 && ((mode & 4u) || L.cerr)) {
-        const int *Pall = reinterpret_cast<const int *>(slice);
-        long long chk = 0;
-        for (int j = G.t; j < N * K; j += G.g) chk += Pall[j];
-        chk = group_sum(G, chk, slice + L.off_red);
-        if (G.t == 0) SQ_DBG(chk - static_cast<long long>(sgn_c) * k_eff * kOne == ec, 9);
-    }
-#endif
-
-    // ---- codes, scale, channel error (the staged weights / perturbations are dead: scratch)
-    emit_channel(L, m, G, reinterpret_cast<const unsigned char *>(cbuf), slice, s, ec, mode);
+    // codes, scale, channel error (the perturbations are dead: scratch)
+    emit_channel(L, m, G, reinterpret_cast<const unsigned char *>(cbuf), slice, s, cs.ec, mode);
 }
 
 // ---------------------------------------------------------------- channel body, caller-supplied scale
@@ -1169,21 +1048,15 @@ __device__ __forceinline__ void hist_add(int *hist, int v)
     atomicAdd(&hist[min(a >> 22, static_cast<unsigned>(kHistBins - 1))], (v > 0 ? 1 : 0) | (v < 0 ? 0x10000 : 0));
 }
 
-// Second half of a fast-path channel: channel sum, SQuant-C by the candidate histogram, flips,
-// patched error sums, stores.  KT = 9: kernel n's candidate byte is cbuf[9 n + vi[n]];
-// KT = 1: every element is its own kernel and candidate (vv = ev = the perturbations, byte n).
-// Needs N % 4 = 0.
-template <int KT>
-__device__ __forceinline__ void finish_channel_hist(const LayerDesc &L, int m, const Group &G,
-                                                    unsigned char *slice, float s, unsigned mode,
-                                                    long long esum, float *kerr, float y, float s2,
-                                                    void *w_release = nullptr, unsigned char *pack_scratch = nullptr)
+// Second half of a long 1x1 row: channel sum, SQuant-C by the candidate histogram, flips, patched error
+// sums, stores.  Every element is its own kernel and candidate (the perturbations are at the slice's
+// start).  Needs N % 4 = 0.
+__device__ __forceinline__ void finish_row_hist(const LayerDesc &L, int m, const Group &G, unsigned char *slice, float s, unsigned mode,
+                                                long long esum, float *kerr)
 {
     const int N = L.N;
     unsigned char *cbuf = slice + L.off_codes;
-    int *ev = reinterpret_cast<int *>(slice + L.off_ev);
-    int *vv = reinterpret_cast<int *>(slice + L.off_vv);
-    unsigned char *vi = slice + L.off_vi;
+    int *vv = reinterpret_cast<int *>(slice);
     int *hist = reinterpret_cast<int *>(slice + L.off_hist);
     unsigned char *red = slice + L.off_red;
     int *bc = reinterpret_cast<int *>(red + 128);               // [0..3] scan result, [5] list count
@@ -1198,34 +1071,7 @@ __device__ __forceinline__ void finish_channel_hist(const LayerDesc &L, int m, c
         if ((G.t & 31) == 0)
             atomicAdd(acc, static_cast<unsigned long long>((static_cast<long long>(hi) << 16) + lo));
     }
-    G.sync();   // per-kernel data, histogram, channel sum and redo list visible
-    if (KT == 9) {
-        // Kernels the fast selection reported: redone exactly from the staged weights, one
-        // thread per kernel.  The list holds N / 2 entries; beyond that (inputs made of ties or
-        // of weights tiny against the channel's scale) every thread redoes its own marked kernels.
-        const int cnt = bc[6];
-        if (cnt > 0) {   // group-uniform
-            const float *wbuf = reinterpret_cast<const float *>(slice);
-            const unsigned short *redo = reinterpret_cast<const unsigned short *>(vi + N);
-            const bool listed = cnt <= (N >> 1);
-            const int end = listed ? cnt : N;
-            for (int i = G.t; i < end; i += G.g) {
-                int n = i;
-                if (listed) n = redo[i];
-                else if (vi[i] != kRedoMark) continue;
-                const KernelOut o = kernel9_exact(wbuf + n * 9, y, s2, cbuf + n * 9);
-                ev[n] = o.e;
-                vv[n] = o.v;
-                vi[n] = static_cast<unsigned char>(o.idx);
-                if (kerr) kerr[n] = __fmul_rn(__int2float_rn(o.e), 0x1p-30f);
-                if (o.v != 0) hist_add(hist, o.v);
-                atomicAdd(acc, static_cast<unsigned long long>(static_cast<long long>(o.e)));
-            }
-            G.sync();
-        }
-        // the staged weights are dead from here on: a pipelined caller lets the next copy start
-        if (w_release != nullptr && G.t == 0) mbar_arrive(w_release);
-    }
+    G.sync();   // perturbations, histogram and channel sum visible
     long long ec = static_cast<long long>(*acc);
 
     // ---- SQuant-C: boundary bin of the candidate histogram
@@ -1315,10 +1161,10 @@ __device__ __forceinline__ void finish_channel_hist(const LayerDesc &L, int m, c
                         }
                     }
                     if (take) {
-                        SQ_DBG(n < N && (KT == 1 || vi[n] < 9), 3);
-                        unsigned char *bp = cbuf + (KT == 1 ? n : n * 9 + vi[n]);
+                        SQ_DBG(n < N, 3);
+                        unsigned char *bp = cbuf + n;
                         *bp = static_cast<unsigned char>(*bp - sgn_c);
-                        if (kerr) kerr[n] = __fmul_rn(__int2float_rn(ev[n] - sgn_c * kOne), 0x1p-30f);
+                        if (kerr) kerr[n] = __fmul_rn(__int2float_rn(vv[n] - sgn_c * kOne), 0x1p-30f);
                     }
                 }
             }
@@ -1335,157 +1181,16 @@ __device__ __forceinline__ void finish_channel_hist(const LayerDesc &L, int m, c
             }
             if (rank < rem) {
                 SQ_DBG(me.y >= 0 && me.y < N && cb <= kListCap, 4);
-                unsigned char *bp = cbuf + (KT == 1 ? me.y : me.y * 9 + vi[me.y]);
+                unsigned char *bp = cbuf + me.y;
                 *bp = static_cast<unsigned char>(*bp - sgn_c);
-                if (kerr) kerr[me.y] = __fmul_rn(__int2float_rn(ev[me.y] - sgn_c * kOne), 0x1p-30f);
+                if (kerr) kerr[me.y] = __fmul_rn(__int2float_rn(vv[me.y] - sgn_c * kOne), 0x1p-30f);
             }
         }
         G.sync();
     }
 
-#ifdef SQUANT_DEBUG_BOUNDS
-    // Checked build, grouped kernel, 3x3: the staged weights are still there, so the channel's error
-    // sum can be taken again from scratch - plain IEEE division of every weight, perturbation of
-    // its FINAL code - and must equal what the selection machinery arrived at.
-    if (KT == 9 && w_release == nullptr && pack_scratch == nullptr) {
-        G.sync();
-        const float *wchk = reinterpret_cast<const float *>(slice);
-        long long chk = 0;
-        for (int j = G.t; j < 9 * N; j += G.g) {
-            // rounded code and its perturbation (that difference is exact), then whole steps for the flips
-            const float x = __fdiv_rn(wchk[j], s), q0 = rintf(x);
-            const long long P0 = __float2ll_rn(__fmul_rn(__fsub_rn(q0, x), 1073741824.0f));
-            chk += P0 + (static_cast<long long>(static_cast<signed char>(cbuf[j])) - __float2int_rn(q0)) * kOne;
-        }
-        chk = group_sum(G, chk, red);
-        if (G.t == 0) SQ_DBG(chk == ec, 8);
-    }
-#endif
-    // ---- codes, scale, channel error (the staged weights / perturbations are dead: scratch)
-    emit_channel(L, m, G, cbuf, pack_scratch ? pack_scratch : slice, s, ec, mode);
-}
-
-// ---------------------------------------------------------------- channel body, 3x3 fast path
-// Needs K = 9, N a multiple of 4, SQuant-K in the mode mask and 2^-60 <= s <= 2^60.
-// A thread owns four consecutive kernels = 36 consecutive weights: nine conflict-free 128-bit
-// shared loads in, nine conflict-free 32-bit stores of packed code bytes out; flips are byte
-// read-modify-writes on the staged codes.  Kernel error sums are written as soon as SQuant-K is
-// done; SQuant-C later patches the few kernels it flips.
-//
-// SQuant-C needs ONE histogram, filled while the kernels are processed: bin = |v| >> 22 of each
-// kernel's candidate, positive and negative candidates counted in the two halves of one 32-bit
-// word.  Once the channel sum (hence the sign and k_c) is known, one warp scans the histogram
-// of that sign for the boundary bin;
-// kernels above it are flipped, the few inside it are collected in a list and ranked exactly
-// (|v| descending, kernel index ascending).  A boundary bin too crowded for the list (massive
-// ties) falls back to the general radix select.
-__device__ __forceinline__ long long k9_quantize(const LayerDesc &L, int m, const Group &G,
-                                                 unsigned char *slice, float s, float s2, float y)
-{
-    const int N = L.N;
-    const float *wbuf = reinterpret_cast<const float *>(slice);
-    unsigned char *cbuf = slice + L.off_codes;
-    int *ev = reinterpret_cast<int *>(slice + L.off_ev);
-    int *vv = reinterpret_cast<int *>(slice + L.off_vv);
-    unsigned char *vi = slice + L.off_vi;
-    int *hist = reinterpret_cast<int *>(slice + L.off_hist);
-    float *kerr = L.kerr ? L.kerr + static_cast<size_t>(m) * N : nullptr;
-    const bool kvec = (reinterpret_cast<uintptr_t>(kerr) & 15) == 0;
-
-    (void)s;
-    const int quads = N >> 2;
-    int *redo_cnt = reinterpret_cast<int *>(slice + L.off_red + 128) + 6;
-    unsigned short *redo = reinterpret_cast<unsigned short *>(vi + N);   // upper half of the index area
-    const int redo_cap = N >> 1;
-    long long esum = 0;
-    const E2 c2 = make_e2(y, s2);
-    for (int Q = G.t; Q < quads; Q += G.g) {
-        const float4 *src = reinterpret_cast<const float4 *>(wbuf) + Q * 9;
-        unsigned *dst = reinterpret_cast<unsigned *>(cbuf) + Q * 9;
-        float2 P2[18];   // the quad's 36 perturbations, pair p = elements 2p, 2p + 1
-#pragma unroll
-        for (int j = 0; j < 9; ++j) {
-            const float4 w = src[j];
-            float2 ta, tb;
-            squant_e_fast2(make_float2(w.x, w.y), c2, ta, P2[2 * j]);
-            squant_e_fast2(make_float2(w.z, w.w), c2, tb, P2[2 * j + 1]);
-            dst[j] = __byte_perm(__byte_perm(__float_as_uint(ta.x), __float_as_uint(ta.y), 0x0040),
-                                 __byte_perm(__float_as_uint(tb.x), __float_as_uint(tb.y), 0x0040), 0x5410);
-        }
-        // float sums of the four kernels (elements 0-8, 9-17, 18-26, 27-35), for their signs
-        float ef[4];
-        {
-            const float2 s0 = __fadd2_rn(__fadd2_rn(P2[0], P2[1]), __fadd2_rn(P2[2], P2[3]));
-            const float2 s1 = __fadd2_rn(__fadd2_rn(P2[5], P2[6]), __fadd2_rn(P2[7], P2[8]));
-            const float2 s2p = __fadd2_rn(__fadd2_rn(P2[9], P2[10]), __fadd2_rn(P2[11], P2[12]));
-            const float2 s3 = __fadd2_rn(__fadd2_rn(P2[14], P2[15]), __fadd2_rn(P2[16], P2[17]));
-            ef[0] = __fadd_rn(__fadd_rn(s0.x, s0.y), P2[4].x);
-            ef[1] = __fadd_rn(__fadd_rn(s1.x, s1.y), P2[4].y);
-            ef[2] = __fadd_rn(__fadd_rn(s2p.x, s2p.y), P2[13].x);
-            ef[3] = __fadd_rn(__fadd_rn(s3.x, s3.y), P2[13].y);
-        }
-        // normalise every perturbation to the sign of its kernel's sum (pairs 4 and 13 straddle two kernels)
-        {
-            const float g0 = copysignf(1.0f, ef[0]), g1 = copysignf(1.0f, ef[1]);
-            const float g2 = copysignf(1.0f, ef[2]), g3 = copysignf(1.0f, ef[3]);
-            const float2 G0 = make_float2(g0, g0), G1 = make_float2(g1, g1), G2 = make_float2(g2, g2), G3 = make_float2(g3, g3);
-#pragma unroll
-            for (int p = 0; p < 4; ++p) {
-                P2[p] = __fmul2_rn(P2[p], G0);
-                P2[5 + p] = __fmul2_rn(P2[5 + p], G1);
-                P2[9 + p] = __fmul2_rn(P2[9 + p], G2);
-                P2[14 + p] = __fmul2_rn(P2[14 + p], G3);
-            }
-            P2[4] = __fmul2_rn(P2[4], make_float2(g0, g1));
-            P2[13] = __fmul2_rn(P2[13], make_float2(g2, g3));
-        }
-        int e4[4], v4[4];
-        unsigned i4 = 0;
-        unsigned char *cq = cbuf + Q * 36;
-#pragma unroll
-        for (int kq = 0; kq < 4; ++kq) {
-            float Pk[9];
-#pragma unroll
-            for (int i = 0; i < 9; ++i) {
-                const int el = 9 * kq + i;
-                Pk[i] = (el & 1) ? P2[el >> 1].y : P2[el >> 1].x;
-            }
-            unsigned idx;
-            if (kernel9_select(Pk, ef[kq], cq + 9 * kq, e4[kq], v4[kq], idx)) {   // rare: redone exactly later
-                const int pos = atomicAdd(redo_cnt, 1);
-                if (pos < redo_cap) redo[pos] = static_cast<unsigned short>(4 * Q + kq);
-            }
-            {   // candidate histogram; |v| < 2^30 for valid input, the mask keeps garbage in range (v = 0 adds nothing)
-                const int v = v4[kq];
-                atomicAdd(&hist[(abs(v) >> 22) & (kHistBins - 1)], v > 0 ? 1 : ((v >> 31) & 0x10000));
-            }
-            i4 |= idx << (8 * kq);
-        }
-        esum += static_cast<long long>(e4[0] + e4[1]) + (e4[2] + e4[3]);   // pairs fit 32 bits
-        reinterpret_cast<int4 *>(ev)[Q] = make_int4(e4[0], e4[1], e4[2], e4[3]);
-        reinterpret_cast<int4 *>(vv)[Q] = make_int4(v4[0], v4[1], v4[2], v4[3]);
-        reinterpret_cast<unsigned *>(vi)[Q] = i4;
-        if (kerr) {
-            float4 f;
-            f.x = __fmul_rn(__int2float_rn(e4[0]), 0x1p-30f);
-            f.y = __fmul_rn(__int2float_rn(e4[1]), 0x1p-30f);
-            f.z = __fmul_rn(__int2float_rn(e4[2]), 0x1p-30f);
-            f.w = __fmul_rn(__int2float_rn(e4[3]), 0x1p-30f);
-            if (kvec) __stcs(reinterpret_cast<float4 *>(kerr) + Q, f);
-            else { kerr[4 * Q] = f.x; kerr[4 * Q + 1] = f.y; kerr[4 * Q + 2] = f.z; kerr[4 * Q + 3] = f.w; }
-        }
-    }
-    return esum;
-}
-
-__device__ __forceinline__ void channel_body_k9_fast(const LayerDesc &L, int m, const Group &G,
-                                                     unsigned char *slice, float s, unsigned mode)
-{
-    const float s2 = __fmul_rn(s, 0x1p-30f);
-    const float y = __frcp_rn(s2);
-    const long long esum = k9_quantize(L, m, G, slice, s, s2, y);
-    float *kerr = L.kerr ? L.kerr + static_cast<size_t>(m) * L.N : nullptr;
-    finish_channel_hist<9>(L, m, G, slice, s, mode, esum, kerr, y, s2);
+    // ---- codes, scale, channel error (the perturbations are dead: scratch)
+    emit_channel(L, m, G, cbuf, slice, s, ec, mode);
 }
 
 // ---------------------------------------------------------------- channel body, 1x1 fast path
@@ -1534,7 +1239,7 @@ __device__ __forceinline__ void channel_body_k1_fast(const LayerDesc &L, int m, 
             else { kerr[4 * Q] = f.x; kerr[4 * Q + 1] = f.y; kerr[4 * Q + 2] = f.z; kerr[4 * Q + 3] = f.w; }
         }
     }
-    finish_channel_hist<1>(L, m, G, slice, s, mode, esum, kerr, y, s2);
+    finish_row_hist(L, m, G, slice, s, mode, esum, kerr);
 }
 
 // ---------------------------------------------------------------- self-check of the fast division
@@ -1657,7 +1362,7 @@ __device__ __forceinline__ void run_item(const LayerDesc &L, int ch0, unsigned c
     } else if ((L.N & 3) == 0 && s >= 0x1p-60f && s <= 0x1p60f) {
         channel_body_k1_fast(L, m, G, slice, s, mode);
     } else {
-        channel_body<1>(L, m, G, slice, s, mode);
+        channel_body_row(L, m, G, slice, s, mode);
     }
 }
 

@@ -1,13 +1,10 @@
-// Streaming kernel for layers of long 3x3 channels with plain int8 codes (no packed, no
-// dequantized output): the successor of the pipelined kernel on its most common case.
+// Streaming kernel for layers of long 3x3 channels: ONE persistent CTA per SM.
 //
-// In the pipelined kernel the quantizer warps of an SM walk through a channel's phases together
-// (wait, absmax, barrier, SQuant-E/K, sum) and four finisher warps run SQuant-C as a chain of
-// short barrier-separated steps over per-kernel arrays in shared memory; both chains are about
-// as long as the whole period, so neither can be shortened alone.  A chain of dependent
-// instructions is what costs here (twenty and more cycles per instruction beside fifteen busy
-// warps), so this kernel keeps the quantizer warps' step down to straight, independent work and
-// as few hand-overs as the method allows:
+// Run by one CTA from start to end, such a channel is a chain of phases (wait for its weights, absmax,
+// SQuant-E/K, channel sum, SQuant-C, stores) in which most warps wait for each other, and a chain of
+// dependent instructions is what costs here (twenty and more cycles per instruction beside fifteen busy
+// warps).  So this kernel keeps the quantizer warps' step down to straight, independent work and as few
+// hand-overs as the method allows, and gives every chain to a helper warp that has the time:
 //
 //   copy warp (one thread)   fetches channel c + 2 by a bulk asynchronous copy as soon as every
 //                            quantizer warp has read the weights of channel c; hands out the work
@@ -40,9 +37,25 @@
 
 #include <cstddef>
 
-#include "squant_pipe.cuh"
+#include "squant_conv.cuh"
 
 namespace sq {
+
+// Work counters, one slot per launch plan.  Launches that share a slot must not overlap; a slot
+// belongs to one plan, i.e. to one set of output buffers, for which overlapping launches would
+// race on the outputs anyway.
+constexpr int kTicketSlots = 1024;
+__device__ unsigned g_ticket[kTicketSlots];
+__device__ unsigned g_done[kTicketSlots];
+
+__device__ __forceinline__ int layer_of(const LaunchTable &tbl, int item)
+{
+    int layer = 0;   // last layer whose first item is <= item
+#pragma unroll 1
+    for (int step = tbl.top_step; step > 0; step >>= 1)
+        if (layer + step < tbl.n_layers && tbl.first_item[layer + step] <= item) layer += step;
+    return layer;
+}
 
 constexpr int kStreamQuantWarps = 16;
 constexpr int kStreamQuantThreads = 32 * kStreamQuantWarps;
@@ -51,7 +64,7 @@ constexpr int kStreamHelpThreads = 128;                     // channel warp, cop
 constexpr int kStreamThreads = kStreamHelpThreads + kStreamQuantThreads;
 constexpr int kStreamListCap = 128;                        // candidates ranked exactly inside the boundary bin
 constexpr int kStreamQueueCap = 128;                       // quantizer threads per channel that hand their flips to the channel warp
-constexpr int kStreamCtrlBytes = 3328;
+constexpr int kStreamCtrlBytes = 3456;
 
 // SQuant-C of one channel as the quantizers need it (sixteen bytes, read as one word).
 struct StreamDecision {
@@ -79,6 +92,13 @@ struct StreamSlot {
     long long pad;
 };
 
+// What the quantizers need to know of a channel three steps later, when they emit its further outputs.
+struct StreamEmit {
+    int layer, m;
+    float s;
+    int pad;
+};
+
 struct StreamCtrl {
     unsigned long long full[2];      // staged weights have arrived (copy -> quantizers)
     unsigned long long wread[2];     // every quantizer warp has the channel's weights in registers (quantizers -> copy)
@@ -101,6 +121,8 @@ struct StreamCtrl {
     int lcount[2];                   // entries in the boundary list
     int qcount[2];                   // entries in the queue of concerned threads
     unsigned short queue[2][kStreamQueueCap];   // quantizer threads with kernels to flip (or to rank)
+    StreamEmit emit[8];              // the channels whose further outputs are still to come, by step modulo eight (a warp
+                                     // may be a step behind when the writer starts the next but three)
     int abort;                       // a wait ran out: nobody waits any more
     unsigned amax[2];                // absmax of the staged channel (bit pattern), from the two scale warps
     int scratch[kStreamQuantWarps][12];                // nine words per quantizer warp for the exact routine
@@ -287,6 +309,66 @@ __device__ __forceinline__ void stream_flip_thread(int t, const StreamDecision &
     }
 }
 
+// Packed int4 codes and code * s (fp32, bfloat16) of one warp's run of a channel: its 1152 codes from code
+// e0 on, final, in shared memory at c.  Called by the whole warp.
+__device__ __forceinline__ void stream_emit(const LayerDesc &L, int m, float s, unsigned mode, const unsigned char *c, int e0)
+{
+    const int lane = threadIdx.x & 31;
+    const int n = min(L.NK - e0, 32 * 36);   // (N is a multiple of four: so is n)
+    if (n <= 0) return;
+    if (mode & kModePackInt4) {   // two codes per byte, low nibble = even flat index
+        unsigned char *row = reinterpret_cast<unsigned char *>(L.codes) + static_cast<size_t>(m) * (L.NK >> 1) + (e0 >> 1);
+        if ((reinterpret_cast<uintptr_t>(row) & 3) == 0) {
+#pragma unroll 1
+            for (int i = lane; i < (n >> 3); i += 32) {
+                const uint2 v = reinterpret_cast<const uint2 *>(c)[i];
+                const unsigned a = v.x & 0x0f0f0f0fu, b = v.y & 0x0f0f0f0fu;
+                __stcs(reinterpret_cast<unsigned *>(row) + i, __byte_perm(a | (a >> 4), b | (b >> 4), 0x6420));
+            }
+            if ((n & 4) && lane == 0) {
+                const unsigned a = reinterpret_cast<const unsigned *>(c)[(n >> 2) - 1] & 0x0f0f0f0fu;
+                *reinterpret_cast<unsigned short *>(row + (n >> 1) - 2) = static_cast<unsigned short>(__byte_perm(a | (a >> 4), 0u, 0x4420));
+            }
+        } else if ((reinterpret_cast<uintptr_t>(row) & 1) == 0) {
+#pragma unroll 2
+            for (int i = lane; i < (n >> 2); i += 32) {
+                const unsigned a = reinterpret_cast<const unsigned *>(c)[i] & 0x0f0f0f0fu;
+                reinterpret_cast<unsigned short *>(row)[i] = static_cast<unsigned short>(__byte_perm(a | (a >> 4), 0u, 0x4420));
+            }
+        } else {
+#pragma unroll 1
+            for (int i = lane; i < (n >> 1); i += 32) row[i] = static_cast<unsigned char>((c[2 * i] & 15) | (c[2 * i + 1] << 4));
+        }
+    }
+    if (L.deq) {
+        float *row = L.deq + static_cast<size_t>(m) * L.NK + e0;
+        const bool vec = (reinterpret_cast<uintptr_t>(row) & 15) == 0;
+#pragma unroll 2
+        for (int i = lane; i < (n >> 2); i += 32) {
+            const unsigned c4 = reinterpret_cast<const unsigned *>(c)[i];
+            const float4 d = make_float4(row_deq(c4, s), row_deq(c4 >> 8, s), row_deq(c4 >> 16, s), row_deq(c4 >> 24, s));
+            if (vec) __stcs(reinterpret_cast<float4 *>(row) + i, d);
+            else { row[4 * i] = d.x; row[4 * i + 1] = d.y; row[4 * i + 2] = d.z; row[4 * i + 3] = d.w; }
+        }
+    }
+    if (L.deq16) {
+        uint16_t *row = L.deq16 + static_cast<size_t>(m) * L.NK + e0;
+        const bool vec = (reinterpret_cast<uintptr_t>(row) & 7) == 0;
+#pragma unroll 2
+        for (int i = lane; i < (n >> 2); i += 32) {
+            const unsigned c4 = reinterpret_cast<const unsigned *>(c)[i];
+            const unsigned b0 = bf16_bits(row_deq(c4, s)), b1 = bf16_bits(row_deq(c4 >> 8, s));
+            const unsigned b2 = bf16_bits(row_deq(c4 >> 16, s)), b3 = bf16_bits(row_deq(c4 >> 24, s));
+            if (vec) {
+                __stcs(reinterpret_cast<uint2 *>(row) + i, make_uint2(b0 | (b1 << 16), b2 | (b3 << 16)));
+            } else {
+                row[4 * i] = static_cast<uint16_t>(b0); row[4 * i + 1] = static_cast<uint16_t>(b1);
+                row[4 * i + 2] = static_cast<uint16_t>(b2); row[4 * i + 3] = static_cast<uint16_t>(b3);
+            }
+        }
+    }
+}
+
 // One warp over 256 counts, highest bins first: lane l holds bins 8 (31 - l) .. 8 (31 - l) + 7 in c[0..7].
 // Finds the bin in which the want-th largest entry falls, want = min(kc, total): its index, its
 // count and how many of its entries are among the want largest.  Returns want (0: nothing there).
@@ -319,9 +401,14 @@ __device__ __forceinline__ int stream_boundary(const int (&c)[8], int lane, int 
     return want;
 }
 
-// Layers: 3x3, N a multiple of 4 and at most 4 * 512, SQuant-K on, absmax scales, int8 codes only.
+// Layers: 3x3, N a multiple of 4 and at most 4 * 512, SQuant-K on, absmax scales.  kOut = false: plain int8
+// codes.  kOut = true: packed int4 codes and / or code * s as well; the quantizer warps emit those three
+// steps after they have written a channel's codes: the decision they have just waited for says that
+// the channel's flips are done by then (see the four codes buffers), and a warp reads only the codes that
+// its own threads wrote and will overwrite next.
 // One item = one output channel; nk_max / n_max are the longest channel of the launch (weights /
 // kernels), from which every CTA derives the same layout.
+template <bool kOut>
 __global__ void __launch_bounds__(kStreamThreads, 1)
 squant_stream_kernel(const __grid_constant__ LaunchTable tbl, int qmax, unsigned mode, int n_items, int slot,
                      int nk_max, int n_max, unsigned char *held_scratch)
@@ -365,7 +452,7 @@ squant_stream_kernel(const __grid_constant__ LaunchTable tbl, int qmax, unsigned
                 ended = true;
                 return;
             }
-            sl.layer = pipe_layer_of(tbl, item);
+            sl.layer = layer_of(tbl, item);
             const LayerDesc &L = tbl.layers[sl.layer];
             sl.m = item - tbl.first_item[sl.layer];
             sl.quads = L.N >> 2;
@@ -509,6 +596,15 @@ squant_stream_kernel(const __grid_constant__ LaunchTable tbl, int qmax, unsigned
             }
         };
 
+        // further outputs of the channel of step k, whose codes are final
+        auto emit = [&](int k) {
+            if (k < 0) return;
+            const StreamEmit em = ctrl->emit[k & 7];
+            SQ_DBG(em.layer >= 0 && em.layer < tbl.n_layers, 25);
+            const LayerDesc &L = tbl.layers[em.layer];
+            stream_emit(L, em.m, em.s, mode, smem + lay.off_codes + static_cast<size_t>(k & 3) * lay.c_bytes + warp * (32 * 36), warp * (32 * 36));
+        };
+
         for (int i = 0;; ++i) {
             const int b = i & 1, u = i >> 1, j = i & 3;
             // the channel's scale (the scale warp has been over its weights during the previous step)
@@ -518,9 +614,15 @@ squant_stream_kernel(const __grid_constant__ LaunchTable tbl, int qmax, unsigned
             if (cur.item < 0) {
                 // the last channel's flips, then the end mark for the channel warp
                 if (held.have) apply(b ^ 1, static_cast<unsigned>((i - 1) >> 1) & 1u, (i + 3) & 3);
+                if (kOut) emit(i - 3);
                 if (qt == 0) ctrl->fin[b] = make_int4(-1, 0, 0, 0);
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&ctrl->qdone[b]);
+                if (kOut) {   // the channel warp's last word: everything is flipped
+                    stream_wait(ctrl, &ctrl->cdec[b], static_cast<unsigned>(u) & 1u);
+                    emit(i - 2);
+                    emit(i - 1);
+                }
                 break;
             }
             const bool active = qt < cur.quads;
@@ -533,6 +635,11 @@ squant_stream_kernel(const __grid_constant__ LaunchTable tbl, int qmax, unsigned
             if (qt == 0) {
                 ctrl->fin[b] = make_int4(cur.item, cur.layer, cur.m, __float_as_int(sc.x));
                 ctrl->kprev[j] = cur.kerr;
+                if (kOut) {
+                    StreamEmit em;
+                    em.layer = cur.layer; em.m = cur.m; em.s = sc.x; em.pad = 0;
+                    ctrl->emit[i & 7] = em;
+                }
             }
             int e4[4] = {0, 0, 0, 0}, v4[4] = {0, 0, 0, 0};
             unsigned i4 = 0u;
@@ -641,6 +748,7 @@ squant_stream_kernel(const __grid_constant__ LaunchTable tbl, int qmax, unsigned
             held.vmax = max(max(v4[0], v4[1]), max(v4[2], v4[3]));
             held.vmin = min(min(v4[0], v4[1]), min(v4[2], v4[3]));
             held.have = true;
+            if (kOut) emit(i - 3);
         }
         return;
     }
@@ -802,7 +910,9 @@ squant_stream_kernel(const __grid_constant__ LaunchTable tbl, int qmax, unsigned
             unsigned char *cg = reinterpret_cast<unsigned char *>(L.codes) + static_cast<size_t>(f_m) * L.NK;
             // a row that is not a whole number of 16-byte words, or does not start on one, leaves by plain stores
             bulk_prev = (reinterpret_cast<uintptr_t>(cg) & 15) == 0 && (L.NK & 15) == 0;
-            if (!bulk_prev) {
+            if (kOut && (mode & kModePackInt4)) {
+                bulk_prev = false;   // the quantizers emit the packed codes
+            } else if (!bulk_prev) {
                 if ((reinterpret_cast<uintptr_t>(cg) & 3) == 0) {   // N is a multiple of four: so is the row
                     for (int q = lane; q < (L.NK >> 2); q += 32)
                         reinterpret_cast<unsigned *>(cg)[q] = reinterpret_cast<const unsigned *>(codes)[q];
@@ -823,7 +933,10 @@ squant_stream_kernel(const __grid_constant__ LaunchTable tbl, int qmax, unsigned
         if (f_valid && bulk_prev && lane == 0) bulk_store_wait();
         __syncwarp();
         p_valid = item >= 0;
-        if (item < 0) break;
+        if (item < 0) {
+            if (kOut && lane == 0) mbar_arrive(&ctrl->cdec[b]);   // no decision, but every flip is done
+            break;
+        }
     }
 }
 

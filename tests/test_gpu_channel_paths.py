@@ -70,3 +70,29 @@ def test_channel_paths(kind, bits, mode, flags):
         check(ws, bits, mode, flags | sq.FLAG_PACK_INT4, start=3)
     check(ws, bits, mode, flags, start=2, clip=0.6)
     check(ws, bits, mode, flags, outputs=True, clip=0.9)
+
+
+@pytest.mark.parametrize("n", [1184, 1188, 1412, 2048])
+def test_long_channels_with_packed_and_dequantized_outputs(n):
+    """Long 3x3 channels with further outputs: one, two, three and many channels per persistent thread block
+    (the outputs follow three steps behind), partial last warps, rows that start on two-byte boundaries."""
+    for m in (1, 149, 297, 450, 700):
+        w = [adversarial_layer((m, n, 3, 3), seed=m + n)]
+        check(w, 4, flags=sq.FLAG_NARROW_RANGE | sq.FLAG_PACK_INT4, outputs=m < 400)
+        check(w, 6, outputs=True)
+
+
+def test_long_channels_with_packed_codes_in_a_capture():
+    """The first call of a plan inside a stream capture can allocate nothing: the grouped kernel takes it."""
+    w = adversarial_layer((40, 1536, 3, 3), seed=5)
+    b = sq.alloc_outputs(torch.from_numpy(w).cuda(), pack_int4=True)
+    flags = sq.FLAG_NARROW_RANGE | sq.FLAG_PACK_INT4
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        sq.squant_quantize_model([b], bits=4, flags=flags)
+    b.codes.fill_(-128)
+    graph.replay()
+    sq.squant_device_status()
+    r = oracle.quantize_layer(w, bits=4, flags=flags)
+    assert np.array_equal(b.codes.cpu().numpy(), r.codes)
+    assert np.array_equal(b.kernel_err.cpu().numpy().view(np.uint32), r.kernel_err.view(np.uint32))
