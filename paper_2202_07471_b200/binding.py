@@ -12,6 +12,11 @@ from typing import List, Optional, Sequence
 
 import torch
 
+try:   # host-side marshalling only; descriptors are written in Python where it has not been built
+    from . import _marshal
+except ImportError:
+    _marshal = None
+
 MODE_E, MODE_K, MODE_C = 1, 2, 4
 MODE_EKC = MODE_E | MODE_K | MODE_C
 FLAG_NARROW_RANGE = 1
@@ -46,6 +51,7 @@ class Layer(ctypes.Structure):
 
 
 _lib = None
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
 
 
 def load_library() -> ctypes.CDLL:
@@ -113,14 +119,23 @@ def alloc_outputs(w: torch.Tensor, kernel_err: bool = True, channel_err: bool = 
     kw = dict(device=w.device)
     if pin and not w.is_cuda:
         kw["pin_memory"] = True
-    m, n = w.shape[0], w.shape[1]
-    cshape = (m, (w[0].numel() + 1) // 2) if pack_int4 else w.shape
+    shape = w.shape
+    m, n = shape[0], shape[1]
+    cshape = (m, (w[0].numel() + 1) // 2) if pack_int4 else shape
+    if w.is_cuda and not pack_int4 and type(w) in (torch.Tensor, torch.nn.Parameter):   # the same tensors, sooner
+        like = dict(memory_format=torch.contiguous_format)
+        return LayerBuffers(
+            w, torch.empty_like(w, dtype=torch.int8, **like), w.new_empty(m),
+            w.new_empty((m, n)) if kernel_err else None, w.new_empty(m) if channel_err else None,
+            torch.empty_like(w, **like) if dequant else None, None,
+            torch.empty_like(w, dtype=torch.bfloat16, **like) if dequant_bf16 else None)
+    empty = torch.empty
     return LayerBuffers(
-        w, torch.empty(cshape, dtype=torch.int8, **kw), torch.empty(m, dtype=torch.float32, **kw),
-        torch.empty((m, n), dtype=torch.float32, **kw) if kernel_err else None,
-        torch.empty(m, dtype=torch.float32, **kw) if channel_err else None,
-        torch.empty(w.shape, dtype=torch.float32, **kw) if dequant else None, None,
-        torch.empty(w.shape, dtype=torch.bfloat16, **kw) if dequant_bf16 else None)
+        w, empty(cshape, dtype=torch.int8, **kw), empty(m, dtype=torch.float32, **kw),
+        empty((m, n), dtype=torch.float32, **kw) if kernel_err else None,
+        empty(m, dtype=torch.float32, **kw) if channel_err else None,
+        empty(shape, dtype=torch.float32, **kw) if dequant else None, None,
+        empty(shape, dtype=torch.bfloat16, **kw) if dequant_bf16 else None)
 
 
 def _descriptor(b: LayerBuffers) -> Layer:
@@ -142,11 +157,29 @@ def _descriptor(b: LayerBuffers) -> Layer:
                  ptr(b.dequant_bf16), ptr(b.scales_in))
 
 
+def _descriptors(buffers: List[LayerBuffers]):
+    """Descriptors of the layers as a ctypes array: by the native extension where it is built, element by
+    element in Python for what that leaves out (tensor subclasses, arguments to be rejected)."""
+    n = len(buffers)
+    array = (Layer * max(1, n))()
+    i = 0
+    while i < n:
+        if _marshal is not None:
+            i = _marshal.fill(buffers, i, ctypes.addressof(array))
+            if i == n:
+                break
+        array[i] = _descriptor(buffers[i])
+        i += 1
+    return array
+
+
 def _options(bits: int, mode: int, flags: int) -> Options:
     return Options(int(bits), int(mode), int(flags))
 
 
 def _stream_handle(stream: Optional[torch.cuda.Stream]) -> ctypes.c_void_p:
+    if stream is None and _raw_stream is not None and torch.cuda.is_initialized():   # a tenth of current_stream()'s time
+        return ctypes.c_void_p(_raw_stream(torch.cuda.current_device()))
     s = stream if stream is not None else torch.cuda.current_stream()
     return ctypes.c_void_p(s.cuda_stream)
 
@@ -158,7 +191,7 @@ class ModelCall:
                  flags: int = FLAG_NARROW_RANGE):
         self.buffers: List[LayerBuffers] = list(layers)
         self.n = len(self.buffers)
-        self.array = (Layer * max(1, self.n))(*[_descriptor(b) for b in self.buffers])
+        self.array = _descriptors(self.buffers)
         self.opt = _options(bits, mode, flags)
         self.on_device = bool(self.buffers and self.buffers[0].w.is_cuda)
 
@@ -195,9 +228,9 @@ def squant_quantize_layer(w: torch.Tensor, bits: int = 4, mode: int = MODE_EKC,
     if not w.is_cuda:
         raise ValueError("squant_quantize_layer needs a CUDA tensor")
     b = alloc_outputs(w)
-    d = _descriptor(b)
+    d = _descriptors([b])
     opt = _options(bits, mode, flags)
-    _check(load_library().squant_quantize_layer(ctypes.byref(d), ctypes.byref(opt), _stream_handle(stream)))
+    _check(load_library().squant_quantize_layer(d, ctypes.byref(opt), _stream_handle(stream)))
     return b
 
 

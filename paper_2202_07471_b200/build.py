@@ -45,6 +45,32 @@ def build(force: bool = False, verbose: bool = False, debug: bool = False) -> st
     return lib
 
 
+MARSHAL = os.path.join(HERE, "_marshal.so")            # Python extension: descriptors of LayerBuffers objects
+MARSHAL_SRC = os.path.join(CSRC, "marshal.cpp")
+
+
+def build_marshal(force: bool = False) -> str:
+    if not force and os.path.exists(MARSHAL) and all(
+            os.path.getmtime(MARSHAL) >= os.path.getmtime(d) for d in (MARSHAL_SRC, os.path.join(ROOT, "include", "squant.h"))):
+        return MARSHAL
+    import sysconfig
+    import torch
+    base = os.path.dirname(torch.__file__)
+    tmp = MARSHAL + f".tmp{os.getpid()}"
+    cmd = ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+           "-I", os.path.join(ROOT, "include"), "-I", sysconfig.get_paths()["include"],
+           "-isystem", os.path.join(base, "include"), "-isystem", os.path.join(base, "include", "torch", "csrc", "api", "include"),
+           "-o", tmp, MARSHAL_SRC, "-L", os.path.join(base, "lib"), "-lc10", "-ltorch_cpu", "-ltorch_python"]
+    res = subprocess.run(cmd, capture_output=True, text=True)
+    if res.returncode != 0:
+        print(res.stdout)
+        print(res.stderr)
+        raise RuntimeError("g++ failed building _marshal.so")
+    os.replace(tmp, MARSHAL)
+    return MARSHAL
+
+
 if __name__ == "__main__":
     print(build(force=True, verbose=True))
+    print(build_marshal(force=True))
     print(build(force=True, debug=True))
