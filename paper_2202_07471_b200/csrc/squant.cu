@@ -128,8 +128,9 @@ void layout_staged(const squant_layer &l, LayerDesc &d, unsigned mode)
 }
 
 // Device-side descriptor of one layer: group size and the layout of a group's shared-memory
-// slice.  Returns the dynamic shared memory one CTA needs for this layer.
-int64_t layout_layer(const squant_layer &l, LayerDesc &d, unsigned mode, unsigned flags)
+// slice.  Returns the dynamic shared memory one CTA needs for this layer.  spread_rows, spread_kernels: 1, 2 or
+// 4 times the threads per channel that use them best.
+int64_t layout_layer(const squant_layer &l, LayerDesc &d, unsigned mode, unsigned flags, int spread_rows = 1, int spread_kernels = 1)
 {
     d.w = l.w; d.codes = l.codes; d.scales = l.scales; d.kerr = l.kernel_err; d.cerr = l.channel_err; d.deq = l.dequant;
     d.sin = l.scales_in; d.deq16 = l.dequant_bf16;
@@ -150,8 +151,9 @@ int64_t layout_layer(const squant_layer &l, LayerDesc &d, unsigned mode, unsigne
     if (d.K == 1) {   // a channel that fits the registers of at most one thread block: no staging
         const int first = static_cast<int>((reinterpret_cast<uintptr_t>(l.w) >> 2) & 3);
         const int vecs = (d.N & 3) ? (d.N + 6) >> 2 : (d.N + first + 3) >> 2;   // of the most misaligned row
-        const int g = sq::row_group(vecs);
+        int g = sq::row_group(vecs);
         if (g) {
+            for (int s = 1; s < spread_rows && g < sq::kCtaThreads && 2 * g <= vecs; s *= 2) g *= 2;
             d.g = g;
             d.g_shift = 0;
             while ((1 << d.g_shift) < d.g) ++d.g_shift;
@@ -161,7 +163,7 @@ int64_t layout_layer(const squant_layer &l, LayerDesc &d, unsigned mode, unsigne
         }
     }
     if (d.K > 1 && !((mode & SQUANT_MODE_C) && !(mode & SQUANT_MODE_K))) {   // kernels: a thread settles up to four of them (larger than 3x3: two)
-        const int per = d.K <= 9 ? 4 : 2;
+        const int per = std::max((d.K <= 9 ? 4 : 2) / spread_kernels, 1);
         int g = 32;
         while (g < sq::kCtaThreads && (per * g < d.N || sq::kCtaThreads / g * sq::conv_bytes(g, d.NK, d.K) > kGroupedSmemGoal)) g *= 2;
         d.g = g;
@@ -284,7 +286,7 @@ int fill_table(sq::LaunchTable &t, const std::vector<LayerDesc> &descs, const in
 }
 
 int build_param_plan(const squant_layer *layers, int32_t n_layers, const squant_options &o,
-                     int max_smem, ParamPlan &p)
+                     int max_smem, int sms, ParamPlan &p)
 {
     p.qmax = (1 << (o.bits - 1)) - 1;
     p.mode = o.mode | ((o.flags & SQUANT_FLAG_PACK_INT4) ? sq::kModePackInt4 : 0u) |
@@ -361,6 +363,17 @@ int build_param_plan(const squant_layer *layers, int32_t n_layers, const squant_
             g_next_slot = (g_next_slot + 1) % sq::kTicketSlots;
         }
     }
+    // A launch whose warps do not fill the GPU takes the time of one channel, so its channels get twice or
+    // four times the threads (up to 32 warps per multiprocessor for 1x1 rows: 3531 rows of 461 weights
+    // 27.0 -> 17.2 us, MobileNetV2 shapes at half width 12.3 -> 7.8; half as many for larger kernels: 256x256x3x3
+    // 7.3 -> 6.4, whereas 512x512x3x3 is slower with twice the threads, 10.5 against 9.4 us).
+    int64_t warps = 0;
+    for (int i : order) warps += (static_cast<int64_t>(descs[i].M) * descs[i].g + 31) / 32;
+    int spread[2] = {1, 1};
+    for (int k = 0; k < 2; ++k)
+        while (spread[k] < 4 && 2 * spread[k] * warps <= static_cast<int64_t>(sms) * (k ? 16 : 32)) spread[k] *= 2;
+    if (spread[0] > 1)
+        for (int i : order) layout_layer(layers[i], descs[i], o.mode, o.flags, spread[0], spread[1]);
     // The grouped kernel takes the rest, layers of long channels in launches of their own: their CTAs need
     // shared memory that would cost the others their fourth CTA per multiprocessor.
     // Estimated duration of one CTA of the layer.  Kernel sizes without a body of their own take the
@@ -457,7 +470,7 @@ int get_plan(const squant_layer *layers, int32_t n_layers, const squant_options 
     CachedPlan cp;
     cp.device = device;
     cp.key = std::move(key);
-    rc = build_param_plan(layers, n_layers, o, limit, cp.plan);
+    rc = build_param_plan(layers, n_layers, o, limit, std::max(g_sm_count_by_device[device], 1), cp.plan);
     if (rc) return rc;
     if (g_plans.size() >= kMaxPlans) g_plans.pop_back();
     g_plans.push_front(std::move(cp));
