@@ -49,7 +49,7 @@ def algorithmic_bytes(shapes) -> float:
 
 def source_digest() -> str:
     h = hashlib.sha256()
-    for f in ("squant_device.cuh", "squant_pipe.cuh", "squant_stream.cuh"):   # the device code; squant.cu is host code only
+    for f in ("squant_device.cuh", "squant_stream.cuh"):   # the code of the streaming kernel, whose traffic was captured
         with open(os.path.join(ROOT, "paper_2202_07471_b200", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
@@ -369,8 +369,8 @@ def run_cuda(args):
         cfgs["large_layer_one_layer_E|C"] = {"layers": 1, "weights": one.numel(), "bits": BITS, "ms_cold": t["cold"], "ms_warm": t["warm"],
                                              "weights_per_s_cold": one.numel() / (t["cold"] * 1e-3), "channels": ch, "mismatches": bad[0],
                                              "note": "checker compared on the first 256 output channels"}
-        # packed int4 codes on the same layer (4 + 0.5 + 4/9 B per weight): long channels with packed or
-        # dequantized outputs take the pipelined kernel
+        # packed int4 codes on the same layer (4 + 0.5 + 4/9 B per weight): the streaming kernel's variant with
+        # further outputs
         pk = [sq.alloc_outputs(one, pack_int4=True)]
         pflags = sq.FLAG_NARROW_RANGE | sq.FLAG_PACK_INT4
         t = time_model(sq, torch, pk, BITS, sq.MODE_EKC, stream, flush, reps=7, flags=pflags)

@@ -57,3 +57,10 @@ def test_parity_checker_of_the_bench_counts_corrupted_channels():
     bad[1][3][8] = 0.125                # and the channel sum of the same channel: still one channel
     ch, mism, dt = bench.oracle_check_all(ws, [good, bad], 4, oracle.MODE_EKC, threads=3, slab=64)
     assert ch == 79 and mism == [0, 3] and dt > 0
+
+
+def test_traffic_record_covers_files_that_exist():
+    """The digest that ties the captured DRAM traffic to the streaming kernel's source reads its files."""
+    sys.path.insert(0, ROOT)
+    import bench
+    assert len(bench.source_digest()) == 16
