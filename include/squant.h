@@ -118,11 +118,11 @@ int squant_quantize_layer(const squant_layer *layer, const squant_options *opt, 
 
 /*
  * Algorithm 1 on every layer of a model in one pass (the paper sums per-layer times and notes
- * that layers could be quantized in parallel, Sec. 4.2): ONE grouped kernel launch for all
- * layers, plus one launch of a persistent kernel for those layers whose 3x3 output channels are
- * longer than 8192 weights (cin a multiple of 4 and at most 2048, SQuant-K on, absmax scales): the
- * streaming kernel when only int8 codes are wanted, the pipelined kernel for packed or
- * dequantized outputs.
+ * that layers could be quantized in parallel, Sec. 4.2): one launch of the grouped kernel for
+ * most models; layers of channels longer than 8192 weights take launches of their own: 3x3 channels
+ * of 1184 input channels and more (a multiple of 4, at most 2048; SQuant-K on, absmax scales) one of
+ * the persistent streaming kernel, 1x1 rows one of the row kernel, channels that do not fit one
+ * thread block's shared memory one of the cluster kernel per layer.
  *
  *   layers, n_layers  host array of descriptors holding DEVICE pointers; n_layers >= 0
  *   opt               bits / mode / flags shared by all layers; NULL means 4 bit, E|K|C, narrow
@@ -133,10 +133,11 @@ int squant_quantize_layer(const squant_layer *layer, const squant_options *opt, 
  * Host-side launch tables of recent calls are cached.  The only device memory the call ever
  * allocates is the streaming kernel's scratch area (72 KB per multiprocessor, about 11 MB on a
  * B200): at the FIRST call with given descriptors that has such layers, by cudaMalloc, kept with
- * the cached launch tables and freed with them (so that first call belongs outside any stream
- * capture; callers that cannot allocate at all: see squant_quantize_layer_noalloc).  Outputs are valid when the stream reaches the end of the
- * launches.  The persistent kernels hand out their channels through a counter in device memory
- * that, like the scratch area, belongs to the cached launch tables of these exact descriptors:
+ * the cached launch tables and freed when neither they nor a graph that captured such a call are
+ * left (so that first call belongs outside any stream capture; callers that cannot allocate at all:
+ * see squant_quantize_layer_noalloc).  Calls with packed or dequantized outputs take the grouped
+ * kernel where the area cannot be allocated.  Outputs are valid when the stream reaches the end of
+ * the launches.  The streaming kernel hands out its channels through a counter in device memory that, like the scratch area, belongs to the cached launch tables of these exact descriptors:
  * two calls with the SAME descriptors must not overlap on the GPU (they would race on the
  * outputs anyway); calls with different descriptors may.  All arguments are validated
  * on the host first; a failed call launches nothing and writes nothing.  Returns SQUANT_OK or a
@@ -160,8 +161,8 @@ int squant_quantize_model_host(const squant_layer *layers, int32_t n_layers,
 /*
  * Geometry of the grouped launch (one thread block per 256/g output channels) that covers
  * these descriptors, as squant_quantize_layer_noalloc issues it (pointers are not dereferenced
- * and may be NULL here).  squant_quantize_model itself sends layers of long 3x3 channels to its
- * pipelined kernel instead, whose grid is one block per multiprocessor.  Any output may be NULL.
+ * and may be NULL here).  squant_quantize_model itself sends layers of long channels to other
+ * kernels and may give the channels of a small launch more threads.  Any output may be NULL.
  */
 int squant_plan_info(const squant_layer *layers, int32_t n_layers, const squant_options *opt,
                      int32_t *grid_ctas, int32_t *cta_threads, int32_t *dynamic_smem_bytes);

@@ -8,7 +8,9 @@
 #include <cstdlib>
 #include <cstring>
 #include <list>
+#include <memory>
 #include <mutex>
+#include <new>
 #include <string>
 #include <vector>
 
@@ -209,6 +211,67 @@ int build_plan(const squant_layer *layers, int32_t n_layers, const squant_option
     return SQUANT_OK;
 }
 
+// Scratch memory of the streaming kernel is shared by the plan that launches with it and by every graph
+// that captured such a launch, and goes with the last of them.  A graph lets go inside a CUDA callback,
+// where no CUDA call is allowed: the memory is then listed here and freed by the next call that
+// is not being captured (cudaFree waits for the device, so no launch still uses it).
+struct DeadScratch {
+    std::mutex mutex;
+    std::vector<void *> list;
+    std::atomic<bool> any{false};
+};
+
+DeadScratch &dead_scratch()
+{
+    static DeadScratch *d = new DeadScratch;   // outlives graphs that are destroyed at exit
+    return *d;
+}
+
+void scratch_unused(void *p)
+{
+    DeadScratch &d = dead_scratch();
+    std::lock_guard<std::mutex> lock(d.mutex);
+    try {
+        d.list.push_back(p);
+        d.any.store(true, std::memory_order_release);
+    } catch (const std::bad_alloc &) {   // host memory is exhausted: left to the end of the process
+    }
+}
+
+void free_dead_scratch()
+{
+    DeadScratch &d = dead_scratch();
+    if (!d.any.load(std::memory_order_acquire)) return;
+    std::vector<void *> list;
+    {
+        std::lock_guard<std::mutex> lock(d.mutex);
+        list.swap(d.list);
+        d.any.store(false, std::memory_order_relaxed);
+    }
+    for (void *p : list) cudaFree(p);
+}
+
+void CUDART_CB release_scratch(void *p) { delete static_cast<std::shared_ptr<void> *>(p); }
+
+// The graph that is being captured takes a share in the scratch memory that its kernel node points to.
+int share_with_graph(const std::shared_ptr<void> &scratch, cudaGraph_t graph)
+{
+    auto *share = new (std::nothrow) std::shared_ptr<void>(scratch);
+    if (!share) return SQUANT_ERR_NOMEM;
+    cudaUserObject_t obj = nullptr;
+    const cudaError_t e = cudaUserObjectCreate(&obj, share, release_scratch, 1, cudaUserObjectNoDestructorSync);
+    if (e != cudaSuccess) {
+        delete share;
+        return cuda_fail(e, "cudaUserObjectCreate");
+    }
+    const cudaError_t r = cudaGraphRetainUserObject(graph, obj, 1, cudaGraphUserObjectMove);
+    if (r != cudaSuccess) {
+        cudaUserObjectRelease(obj, 1);
+        return cuda_fail(r, "cudaGraphRetainUserObject");
+    }
+    return SQUANT_OK;
+}
+
 // Launch tables for the parameter-space variant: layers ordered by the work of one of their
 // CTAs (heaviest first, so the tail of the launch is made of light CTAs), at most
 // kMaxParamLayers per launch.
@@ -226,27 +289,17 @@ struct ParamPlan {
     // streaming kernel (layers of long 3x3 channels): one item per output channel
     struct Stream {
         sq::LaunchTable table;
-        int items, nk_max, n_max, slot;
-        bool out;                     // packed or dequantized outputs wanted
+        int items = 0, nk_max = 0, n_max = 0, slot = 0;
+        bool out = false;                     // packed or dequantized outputs wanted
         // Scratch (what SQuant-C needs of every kernel one step later: four sets of 18 KB per thread block),
-        // allocated at the plan's first launch, freed with the plan.
-        void *scratch;
+        // allocated at the plan's first launch, freed when neither the plan nor a graph needs it.
+        std::shared_ptr<void> scratch;
         // Layers with packed or dequantized outputs can also go to the grouped kernel, which needs no scratch:
         // where it cannot be allocated (a full device, the plan's first launch inside a stream capture).
         sq::LaunchTable grouped;
-        int grouped_grid, grouped_smem;
+        int grouped_grid = 0, grouped_smem = 0;
     };
     mutable std::vector<Stream> streams;
-    ParamPlan() = default;
-    ParamPlan(ParamPlan &&) = default;
-    ParamPlan &operator=(ParamPlan &&) = default;
-    ParamPlan(const ParamPlan &) = delete;
-    ParamPlan &operator=(const ParamPlan &) = delete;
-    ~ParamPlan()
-    {
-        for (Stream &st : streams)
-            if (st.scratch) cudaFree(st.scratch);
-    }
     mutable bool slots_clean = false;   // the streams' work counters have been zeroed on the stream of the plan's first launch
 };
 
@@ -349,7 +402,6 @@ int build_param_plan(const squant_layer *layers, int32_t n_layers, const squant_
             const int n = static_cast<int>(std::min<size_t>(list.size() - base, sq::kMaxParamLayers));
             p.streams.emplace_back();
             ParamPlan::Stream &st = p.streams.back();
-            std::memset(&st, 0, sizeof(st));
             st.items = fill_table(st.table, descs, list.data() + base, n, false);
             st.grouped_grid = fill_table(st.grouped, descs, list.data() + base, n, true);
             for (int j = 0; j < n; ++j) {
@@ -508,25 +560,30 @@ int launch_plan(const ParamPlan &p, cudaStream_t stream)
         int device = 0;
         SQ_CUDA(cudaGetDevice(&device));
         const int sms = std::max(g_sm_count_by_device[device], 1);
-        if (!st.scratch) {
-            bool try_alloc = true;
-            if (st.out) {
-                cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-                SQ_CUDA(cudaStreamIsCapturing(stream, &cap));
-                try_alloc = cap == cudaStreamCaptureStatusNone;
-            }
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        cudaGraph_t graph = nullptr;
+        SQ_CUDA(cudaStreamGetCaptureInfo_v2(stream, &cap, nullptr, &graph, nullptr, nullptr));
+        const bool capturing = cap == cudaStreamCaptureStatusActive;
+        if (!capturing) free_dead_scratch();
+        if (!st.scratch && (!st.out || !capturing)) {
             const size_t bytes = static_cast<size_t>(sms) * sq::kStreamHeldSets * sq::kStreamHeldBytes;
-            if (try_alloc && cudaMalloc(&st.scratch, bytes) != cudaSuccess) {
+            void *ptr = nullptr;
+            if (cudaMalloc(&ptr, bytes) == cudaSuccess) {
+                st.scratch = std::shared_ptr<void>(ptr, scratch_unused);
+            } else {
                 cudaGetLastError();   // the failed allocation is reported by the return code, not left pending
-                st.scratch = nullptr;
                 if (!st.out) return SQUANT_ERR_NOMEM;
             }
+        }
+        if (st.scratch && capturing) {
+            const int rc = share_with_graph(st.scratch, graph);
+            if (rc) return rc;
         }
         if (st.scratch) {
             const int grid = std::min(st.items, sms), smem = sq::stream_layout(st.nk_max, st.n_max).total;
             auto kernel = st.out ? sq::squant_stream_kernel<true> : sq::squant_stream_kernel<false>;
             kernel<<<grid, sq::kStreamThreads, smem, stream>>>(st.table, p.qmax, p.mode, st.items, st.slot, st.nk_max, st.n_max,
-                                                               static_cast<unsigned char *>(st.scratch));
+                                                               static_cast<unsigned char *>(st.scratch.get()));
         } else {
             sq::squant_model_kernel<<<st.grouped_grid, sq::kCtaThreads, st.grouped_smem, stream>>>(st.grouped, p.qmax, p.mode);
         }

@@ -2,6 +2,8 @@
 1x1 rows around every group size and vector remainder, kernels of every specialised size around the
 group sizes, rows that start anywhere, all output forms, many flips and massive ties (the selection's
 exact search).  Whole numbers and raw float words must equal the checker's."""
+import time
+
 import numpy as np
 import pytest
 import torch
@@ -96,3 +98,51 @@ def test_long_channels_with_packed_codes_in_a_capture():
     r = oracle.quantize_layer(w, bits=4, flags=flags)
     assert np.array_equal(b.codes.cpu().numpy(), r.codes)
     assert np.array_equal(b.kernel_err.cpu().numpy().view(np.uint32), r.kernel_err.view(np.uint32))
+
+
+def test_scratch_of_a_captured_call_lives_as_long_as_the_graph():
+    """A graph keeps the scratch memory its streaming launch points to after the plan has left the cache."""
+    area = 70 << 10   # bytes per multiprocessor; 72 KB are allocated
+    area *= torch.cuda.get_device_properties(0).multi_processor_count
+    w = adversarial_layer((40, 1536, 3, 3), seed=6)
+    b = sq.alloc_outputs(torch.from_numpy(w).cuda(), pack_int4=True)
+    flags = sq.FLAG_NARROW_RANGE | sq.FLAG_PACK_INT4
+    small = [sq.alloc_outputs(torch.randn(1, 3, device="cuda")) for _ in range(66)]
+    again = sq.alloc_outputs(torch.from_numpy(w).cuda(), pack_int4=True)
+
+    def evict():   # the cache holds 64 plans; the last call is one that can free
+        for s in small:
+            sq.squant_quantize_model([s], bits=4)
+
+    evict()
+    sq.squant_quantize_model([again], bits=4, flags=flags)   # its own area, and what earlier tests left is freed
+    call = sq.ModelCall([b], bits=4, flags=flags)
+    call.run()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        call.run()
+    sq.squant_quantize_model([again], bits=4, flags=flags)
+    torch.cuda.synchronize()
+    free0 = torch.cuda.mem_get_info()[0]
+    for s in small[:62]:
+        sq.squant_quantize_model([s], bits=4)
+    sq.squant_quantize_model([again], bits=4, flags=flags)   # most recent: stays
+    for s in small[62:]:
+        sq.squant_quantize_model([s], bits=4)                # the captured plan has left by now
+    sq.squant_quantize_model([again], bits=4, flags=flags)
+    assert torch.cuda.mem_get_info()[0] < free0 + area       # (checked before the replay)
+    b.codes.fill_(-128)
+    graph.replay()
+    sq.squant_device_status()
+    r = oracle.quantize_layer(w, bits=4, flags=flags)
+    assert np.array_equal(b.codes.cpu().numpy(), r.codes)
+    assert np.array_equal(b.kernel_err.cpu().numpy().view(np.uint32), r.kernel_err.view(np.uint32))
+    free1 = torch.cuda.mem_get_info()[0]
+    del graph
+    torch.cuda.synchronize()
+    for _ in range(200):   # the graph's resources go in a callback of the driver
+        sq.squant_quantize_model([again], bits=4, flags=flags)
+        if torch.cuda.mem_get_info()[0] >= free1 + area:
+            break
+        time.sleep(0.01)
+    assert torch.cuda.mem_get_info()[0] >= free1 + area
