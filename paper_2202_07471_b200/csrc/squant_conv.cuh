@@ -8,7 +8,8 @@
 // What bounds it is the number of instructions: 9 loads, 30 for SQuant-E and about 90 for the selection
 // per 3x3 kernel.  A thread with four kernels at once (128-bit loads) needs fewer of them, but leaves half
 // of a short channel's threads idle, needs N to be a multiple of four and an aligned row, and its 1500
-// instructions of straight code are fetched anew by every warp; this body is a loop of about 170.
+// instructions of straight code are fetched anew by every warp; this body is a loop of about 170 (ResNet-18 shapes
+// 35.9 -> 31.3 us device time on a B200, with supplied scales 81 -> 58, mixed kernel sizes 57 -> 45).
 #pragma once
 
 #include "squant_rows.cuh"

@@ -16,6 +16,8 @@
 //     elements).  T0 is searched among the maxima, the elements from T0 on are listed, and those of
 //     the first k_c ranks are flipped.  What that cannot settle (k_c beyond the number of maxima, a
 //     full list) goes to an exact search over the 48-bit keys.
+// With squant_conv.cuh: ResNet-50 shapes 84.5 -> 65.6 us device time on a B200, 55 thread-instructions per weight;
+// five linear layers of 125 M weights at 8 bit 267 -> 252 us.
 #pragma once
 
 #include <cooperative_groups.h>

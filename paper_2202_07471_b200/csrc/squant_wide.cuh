@@ -10,6 +10,9 @@
 // the edge of the clip range (|w/s| a shade above qmax) can make it into a top-k; they run the bodies
 // that check every candidate against the range, as in the CPU definition: an element whose flipped code
 // would leave the range is no candidate.
+//
+// With the bodies of squant_rows.cuh and squant_conv.cuh, two thread blocks per multiprocessor where the channel
+// can be cut that small: 256 rows of 100,352, 128 of 65,541 and 64x8192x3x3 690 -> 224 us on a B200.
 #pragma once
 
 #include "squant_conv.cuh"
