@@ -127,6 +127,9 @@ struct StreamCtrl {
     unsigned amax[2];                // absmax of the staged channel (bit pattern), from the two scale warps
     int scratch[kStreamQuantWarps][12];                // nine words per quantizer warp for the exact routine
     int dummy[kStreamQuantWarps][12];                  // where lanes without kernels put their (void) code bytes
+#ifdef SQUANT_DEBUG_BOUNDS
+    int step[kStreamQuantWarps];                       // step that a lane of the warp has begun
+#endif
 };
 static_assert(sizeof(StreamCtrl) <= kStreamCtrlBytes, "control block too large");
 
@@ -405,7 +408,8 @@ __device__ __forceinline__ int stream_boundary(const int (&c)[8], int lane, int 
 // codes.  kOut = true: packed int4 codes and / or code * s as well; the quantizer warps emit those three
 // steps after they have written a channel's codes: the decision they have just waited for says that
 // the channel's flips are done by then (see the four codes buffers), and a warp reads only the codes that
-// its own threads wrote and will overwrite next.
+// its own threads wrote and will overwrite next - but a lane reads what other lanes own (words 32 apart of
+// the warp's run, whereas a lane's codes are 36 consecutive bytes), so a warp barrier ends the step.
 // One item = one output channel; nk_max / n_max are the longest channel of the launch (weights /
 // kernels), from which every CTA derives the same layout.
 template <bool kOut>
@@ -625,6 +629,9 @@ squant_stream_kernel(const __grid_constant__ LaunchTable tbl, int qmax, unsigned
                 }
                 break;
             }
+#ifdef SQUANT_DEBUG_BOUNDS
+            *reinterpret_cast<volatile int *>(&ctrl->step[warp]) = i;
+#endif
             const bool active = qt < cur.quads;
             const unsigned char *wbuf = smem + static_cast<size_t>(b) * lay.w_bytes;
             unsigned char *cq = active ? smem + lay.off_codes + static_cast<size_t>(j) * lay.c_bytes + qt * 36
@@ -748,7 +755,11 @@ squant_stream_kernel(const __grid_constant__ LaunchTable tbl, int qmax, unsigned
             held.vmax = max(max(v4[0], v4[1]), max(v4[2], v4[3]));
             held.vmin = min(min(v4[0], v4[1]), min(v4[2], v4[3]));
             held.have = true;
-            if (kOut) emit(i - 3);
+            if (kOut) {
+                emit(i - 3);
+                SQ_DBG(*reinterpret_cast<volatile int *>(&ctrl->step[warp]) == i, 26);   // no lane has gone on to the step that overwrites these codes
+                __syncwarp();   // the lanes have read each other's codes, which the next step overwrites
+            }
         }
         return;
     }

@@ -84,6 +84,28 @@ def test_long_channels_with_packed_and_dequantized_outputs(n):
         check(w, 6, outputs=True)
 
 
+@pytest.mark.parametrize("n", [1188, 1500, 2044])
+def test_no_lane_overtakes_the_further_outputs(n):
+    """The further outputs of a long channel are written by whole warps from codes that other lanes own and
+    overwrite in the next step.  The checked build sees a lane that begins the next step while another is still
+    reading (trip counts that differ by lane: 144 packed words over 32 lanes, the row's tail); many steps per
+    thread block, and the outputs must be right in either build."""
+    from paper_2202_07471_b200 import build as lib_build
+    ws = [adversarial_layer((1200, n, 3, 3), seed=n)]
+    flags = sq.FLAG_NARROW_RANGE | sq.FLAG_PACK_INT4
+    check(ws, 4, flags=flags)
+    sq.use_library(lib_build.LIB_DEBUG)
+    try:
+        sq.squant_debug_violations()
+        check(ws, 4, flags=flags)
+        check([w[:400] for w in ws], 4, flags=flags, outputs=True)
+        check([w[:400] for w in ws], 5, outputs=True)
+        checked, failed, site = sq.squant_debug_violations()
+        assert checked and failed == 0, (failed, site)
+    finally:
+        sq.use_library(None)
+
+
 def test_long_channels_with_packed_codes_in_a_capture():
     """The first call of a plan inside a stream capture can allocate nothing: the grouped kernel takes it."""
     w = adversarial_layer((40, 1536, 3, 3), seed=5)
