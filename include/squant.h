@@ -168,6 +168,18 @@ int squant_plan_info(const squant_layer *layers, int32_t n_layers, const squant_
                      int32_t *grid_ctas, int32_t *cta_threads, int32_t *dynamic_smem_bytes);
 
 /*
+ * Which kernel squant_quantize_model gives each layer to on a B200: kernels[i] (HOST array of n_layers)
+ * receives one of the values below.  No GPU is needed; the layers' pointers are not dereferenced, but their
+ * alignment and which of them are NULL count as in the call itself.  Returns what the call would return
+ * for these layers (SQUANT_ERR_TOO_WIDE for a channel that fits no kernel).  For tests and tools.
+ */
+#define SQUANT_KERNEL_GROUPED 1 /* many channels per thread block */
+#define SQUANT_KERNEL_ROW 2     /* long 1x1 rows, a thread block each */
+#define SQUANT_KERNEL_CLUSTER 3 /* channels wider than a thread block's shared memory */
+#define SQUANT_KERNEL_STREAM 4  /* long 3x3 channels, persistent thread blocks */
+int squant_plan_kernels(const squant_layer *layers, int32_t n_layers, const squant_options *opt, int32_t *kernels);
+
+/*
  * squant_quantize_layer without any device allocation.  (An addition of this library; the paper
  * has no counterpart.)
  *

@@ -28,7 +28,7 @@ LIB_PATH = os.path.join(_HERE, "libsquant.so")
 NOALLOC_MAX_CTAS = 32768
 
 EXPORTS = ("squant_quantize_layer", "squant_quantize_layer_noalloc", "squant_quantize_model", "squant_quantize_model_host",
-           "squant_plan_info", "squant_selfcheck_division", "squant_device_status", "squant_launch_count", "squant_strerror", "squant_last_cuda_error",
+           "squant_plan_info", "squant_plan_kernels", "squant_selfcheck_division", "squant_device_status", "squant_launch_count", "squant_strerror", "squant_last_cuda_error",
            "squant_shutdown", "squant_debug_set_status", "squant_debug_wait_expires", "squant_debug_violations")
 
 
@@ -70,9 +70,10 @@ def load_library() -> ctypes.CDLL:
     lib.squant_quantize_model.argtypes = [lp, ctypes.c_int32, op, vp]
     lib.squant_quantize_model_host.argtypes = [lp, ctypes.c_int32, op, vp]
     lib.squant_plan_info.argtypes = [lp, ctypes.c_int32, op, i32p, i32p, i32p]
+    lib.squant_plan_kernels.argtypes = [lp, ctypes.c_int32, op, i32p]
     lib.squant_selfcheck_division.argtypes = [ctypes.c_void_p, ctypes.c_int32, ctypes.c_int32, ctypes.c_void_p, vp]
     for f in ("squant_quantize_layer", "squant_quantize_layer_noalloc", "squant_quantize_model", "squant_quantize_model_host",
-              "squant_plan_info", "squant_selfcheck_division", "squant_device_status", "squant_shutdown"):
+              "squant_plan_info", "squant_plan_kernels", "squant_selfcheck_division", "squant_device_status", "squant_shutdown"):
         getattr(lib, f).restype = ctypes.c_int
     lib.squant_debug_violations.argtypes = [i32p, i32p]
     lib.squant_debug_violations.restype = ctypes.c_int
@@ -263,6 +264,19 @@ def squant_plan_info(shapes: Sequence[Sequence[int]], bits: int = 4, mode: int =
     _check(load_library().squant_plan_info(arr, len(shapes), ctypes.byref(opt), ctypes.byref(g),
                                            ctypes.byref(t), ctypes.byref(s)))
     return {"grid_ctas": g.value, "cta_threads": t.value, "dynamic_smem_bytes": s.value}
+
+
+def squant_plan_kernels(layers: Sequence, bits: int = 4, mode: int = MODE_EKC, flags: int = FLAG_NARROW_RANGE) -> List[str]:
+    """Which kernel squant_quantize_model gives each layer to: "grouped", "row", "cluster" or "stream" (no GPU
+    needed).  layers: LayerBuffers, or [cout, cin, kh, kw] shapes (aligned buffers, no optional outputs)."""
+    n = len(layers)
+    arr = (Layer * max(1, n))()
+    for i, l in enumerate(layers):
+        arr[i] = _descriptor(l) if isinstance(l, LayerBuffers) else Layer(None, *[int(x) for x in l])
+    out = (ctypes.c_int32 * max(1, n))()
+    opt = _options(bits, mode, flags)
+    _check(load_library().squant_plan_kernels(arr, n, ctypes.byref(opt), out))
+    return [("grouped", "row", "cluster", "stream")[k - 1] for k in out[:n]]
 
 
 def squant_selfcheck_division(scales, bits: int = 4):

@@ -338,8 +338,9 @@ int fill_table(sq::LaunchTable &t, const std::vector<LayerDesc> &descs, const in
     return items;
 }
 
+// kernels: SQUANT_KERNEL_* of every layer, or null.
 int build_param_plan(const squant_layer *layers, int32_t n_layers, const squant_options &o,
-                     int max_smem, int sms, ParamPlan &p)
+                     int max_smem, int sms, ParamPlan &p, int32_t *kernels = nullptr)
 {
     p.qmax = (1 << (o.bits - 1)) - 1;
     p.mode = o.mode | ((o.flags & SQUANT_FLAG_PACK_INT4) ? sq::kModePackInt4 : 0u) |
@@ -349,7 +350,8 @@ int build_param_plan(const squant_layer *layers, int32_t n_layers, const squant_
     for (int i = 0; i < n_layers; ++i) {
         const int64_t cta_smem = layout_layer(layers[i], descs[i], o.mode, o.flags);
         if (cta_smem > max_smem || descs[i].NK > kMaxChannelElems) {
-            // a cluster of 2, 4 or 8 CTAs per output channel, each with an even number of kernels
+            // a cluster of 2, 4 or 8 CTAs per output channel, each with an even number of kernels (packed codes of a
+            // run start on a byte), of 1x1 rows a multiple of four (a run starts on a vector)
             if ((o.mode & SQUANT_MODE_C) && !(o.mode & SQUANT_MODE_K) && descs[i].K > 1) return SQUANT_ERR_TOO_WIDE;   // E|C selects among elements: one CTA only
             // (the limit: what eight of them hold at 5 B a weight and 10 B a larger kernel)
             ParamPlan::Wide w{descs[i], 0, 0, 0};
@@ -360,7 +362,8 @@ int build_param_plan(const squant_layer *layers, int32_t n_layers, const squant_
             // weights or for its cluster the other works
             for (int goal = kWideSmemGoal;; goal = max_smem) {
                 for (int c = 2; c <= sq::kWideMaxCluster && !w.cluster; c *= 2) {
-                    const int kpc = (((descs[i].N + c - 1) / c) + 3) & ~3;
+                    const int unit = descs[i].K == 1 ? 4 : 2;
+                    const int kpc = ((descs[i].N + c - 1) / c + unit - 1) / unit * unit;
                     const int64_t bytes = sq::wide_bytes(kpc, descs[i].K);
                     if (bytes <= goal) { w.cluster = c; w.kpc = kpc; w.smem = static_cast<int>(bytes); }
                 }
@@ -369,18 +372,22 @@ int build_param_plan(const squant_layer *layers, int32_t n_layers, const squant_
             if (!w.cluster) return SQUANT_ERR_TOO_WIDE;
             w.d.off_vi = (w.kpc + 6) >> 2;
             p.wide.push_back(w);
+            if (kernels) kernels[i] = SQUANT_KERNEL_CLUSTER;
             continue;
         }
         if (stream_eligible(layers[i], descs[i], o, max_smem)) {
             const squant_layer &l = layers[i];
             streamed[l.dequant || l.dequant_bf16 || (o.flags & SQUANT_FLAG_PACK_INT4) ? 1 : 0].push_back(i);
+            if (kernels) kernels[i] = SQUANT_KERNEL_STREAM;
             continue;
         }
         if (descs[i].K == 1 && descs[i].off_hist != 0 && descs[i].N <= sq::kRowBlockElems) {   // too long for a group, 164 KB at most
             rows.push_back(i);
+            if (kernels) kernels[i] = SQUANT_KERNEL_ROW;
             continue;
         }
         order.push_back(i);
+        if (kernels) kernels[i] = SQUANT_KERNEL_GROUPED;
     }
     // long rows, longest first: a thread block per output channel
     std::stable_sort(rows.begin(), rows.end(), [&](int a, int b) { return descs[a].N > descs[b].N; });
@@ -866,6 +873,17 @@ int squant_plan_info(const squant_layer *layers, int32_t n_layers, const squant_
     if (cta_threads) *cta_threads = sq::kCtaThreads;
     if (dynamic_smem_bytes) *dynamic_smem_bytes = hp.smem_bytes;
     return SQUANT_OK;
+}
+
+int squant_plan_kernels(const squant_layer *layers, int32_t n_layers, const squant_options *opt, int32_t *kernels)
+{
+    squant_options o;
+    int rc = validate(layers, n_layers, opt, false, o);
+    if (rc) return rc;
+    if (n_layers > 0 && !kernels) return SQUANT_ERR_NULL;
+    std::lock_guard<std::mutex> lock(g_mutex);   // (plans draw work-counter slots)
+    ParamPlan plan;
+    return build_param_plan(layers, n_layers, o, kMaxSmemFallback, 148, plan, kernels);
 }
 
 int squant_selfcheck_division(const float *scales, int32_t n, int32_t bits, uint64_t *mismatches,

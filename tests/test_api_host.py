@@ -69,6 +69,45 @@ def test_valid_edge_arguments():
     assert _info([(2, 4000, 3, 3)])["grid_ctas"] == 2
 
 
+@pytest.mark.parametrize("shape", [(50, 1254, 17, 17), (700, 897, 20, 20), (8, 48, 1, 7600), (3, 16, 1, 20000), (4, 12, 120, 120), (3, 3, 150, 150)])
+def test_channels_of_few_large_kernels_fit_a_cluster(shape):
+    """Of kernels of more than one element each thread block of a cluster takes an even number, not a multiple of
+    four: rounding up further would cost such a channel the shared memory of up to two kernels more."""
+    assert sq.squant_plan_kernels([shape]) == ["cluster"]
+
+
+@pytest.mark.parametrize("k", [1, 9, 16, 25, 49, 81, 121, 169, 225, 289, 400, 1024, 2500, 7600, 14400, 22500])
+def test_limit_of_the_cluster_kernel(k):
+    """A channel is taken if an eighth of its kernels, rounded up to an even number, fits one thread block at 5 B a
+    weight and, of larger kernels, 10 B a kernel."""
+    up = lambda v: (v + 15) // 16 * 16
+    def fits(n):
+        n8 = ((n + 7) // 8 + 1) // 2 * 2
+        return up(4 * n8 * k) + up(n8 * k) + (2 * up(4 * n8) + up(2 * n8) if k > 1 else 0) + 2304 <= 232448
+    lo, hi = 1, 262143
+    while lo < hi:   # the widest channel that fits
+        mid = (lo + hi + 1) // 2
+        lo, hi = (mid, hi) if fits(mid) else (lo, mid - 1)
+    for n in {max(lo + d, 1) for d in (-40, -17, -16, -9, -8, -7, -5, -4, -3, -2, -1, 0, 1, 2, 3, 8, 15, 16, 17, 40)}:
+        if n > 262143:
+            continue
+        if fits(n):
+            assert sq.squant_plan_kernels([(3, n, 1, k)])[0] in ("cluster", "row", "grouped"), n
+        else:
+            with pytest.raises(sq.SquantError) as ei:
+                sq.squant_plan_kernels([(3, n, 1, k)])
+            assert ei.value.code == -6, n
+
+
+def test_kernel_of_a_layer():
+    shapes = [(64, 64, 3, 3), (8, 8192, 1, 1), (8, 8193, 1, 1), (8, 32768, 1, 1), (8, 40000, 1, 1), (8, 70000, 1, 1),
+              (8, 2048, 3, 3), (8, 2049, 3, 3), (8, 2052, 3, 3), (8, 600, 5, 5), (8, 8192, 3, 3)]
+    want = ["grouped", "grouped", "row", "row", "grouped", "cluster", "stream", "grouped", "grouped", "grouped", "cluster"]
+    assert sq.squant_plan_kernels(shapes) == want
+    assert sq.squant_plan_kernels([(8, 2048, 3, 3)], mode=sq.MODE_E) == ["grouped"]   # without SQuant-K
+    assert sq.squant_plan_kernels([]) == []
+
+
 def test_null_pointers_are_rejected_before_any_cuda_call():
     lib = sq.load_library()
     layer = binding.Layer(None, 4, 3, 3, 3, None, None, None, None, None, None, None)

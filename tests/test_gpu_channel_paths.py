@@ -74,6 +74,17 @@ def test_channel_paths(kind, bits, mode, flags):
     check(ws, bits, mode, flags, outputs=True, clip=0.9)
 
 
+@pytest.mark.parametrize("shape", [(3, 1254, 17, 17), (3, 897, 20, 20), (2, 11, 120, 120), (2, 16, 1, 20000), (2, 3, 150, 150)])
+def test_cluster_runs_of_an_even_number_of_kernels(shape):
+    """Channels of few large kernels whose thread blocks take a number of kernels that is no multiple of four."""
+    assert sq.squant_plan_kernels([shape]) == ["cluster"]
+    w = [adversarial_layer(shape, seed=shape[1])]
+    check(w, 4)
+    check(w, 4, mode=sq.MODE_E | sq.MODE_K, start=1, outputs=True)
+    check(w, 3, flags=sq.FLAG_NARROW_RANGE | sq.FLAG_PACK_INT4, start=2, outputs=True)
+    check(w, 8, flags=0, clip=0.98)
+
+
 @pytest.mark.parametrize("n", [1184, 1188, 1412, 2048])
 def test_long_channels_with_packed_and_dequantized_outputs(n):
     """Long 3x3 channels with further outputs: one, two, three and many channels per persistent thread block
