@@ -137,7 +137,9 @@ int squant_quantize_layer(const squant_layer *layer, const squant_options *opt, 
  * left (so that first call belongs outside any stream capture; callers that cannot allocate at all:
  * see squant_quantize_layer_noalloc).  Calls with packed or dequantized outputs take the grouped
  * kernel where the area cannot be allocated.  Outputs are valid when the stream reaches the end of
- * the launches.  The streaming kernel hands out its channels through a counter in device memory that, like the scratch area, belongs to the cached launch tables of these exact descriptors:
+ * the launches.  The streaming kernel hands out its channels through a counter in device memory, which is
+ * part of the scratch area and so belongs to the cached launch tables of these exact descriptors and the graphs
+ * captured with them:
  * two calls with the SAME descriptors must not overlap on the GPU (they would race on the
  * outputs anyway); calls with different descriptors may.  All arguments are validated
  * on the host first; a failed call launches nothing and writes nothing.  Returns SQUANT_OK or a

@@ -211,8 +211,9 @@ int build_plan(const squant_layer *layers, int32_t n_layers, const squant_option
     return SQUANT_OK;
 }
 
-// Scratch memory of the streaming kernel is shared by the plan that launches with it and by every graph
-// that captured such a launch, and goes with the last of them.  A graph lets go inside a CUDA callback,
+// Scratch memory of the streaming kernel (what SQuant-C needs of every kernel one step later: four sets of
+// 18 KB per thread block; the launch's work counters) is shared by the plan that launches with it and by every
+// graph that captured such a launch, and goes with the last of them.  A graph lets go inside a CUDA callback,
 // where no CUDA call is allowed: the memory is then listed here and freed by the next call that
 // is not being captured (cudaFree waits for the device, so no launch still uses it).
 struct DeadScratch {
@@ -251,12 +252,45 @@ void free_dead_scratch()
     for (void *p : list) cudaFree(p);
 }
 
-void CUDART_CB release_scratch(void *p) { delete static_cast<std::shared_ptr<void> *>(p); }
+struct StreamScratch {
+    unsigned char *mem;
+    size_t area;   // bytes before the work counters
+    int device;
+    StreamScratch(unsigned char *m, size_t a, int d) : mem(m), area(a), device(d) {}
+    StreamScratch(const StreamScratch &) = delete;
+    StreamScratch &operator=(const StreamScratch &) = delete;
+    ~StreamScratch() { scratch_unused(mem); }
+    unsigned *work() const { return reinterpret_cast<unsigned *>(mem + area); }
+};
+using ScratchRef = std::shared_ptr<StreamScratch>;
+
+std::vector<std::weak_ptr<StreamScratch>> g_scratch;   // every area in use; guarded by g_mutex
+
+// A new area on the current device; its work counters are zeroed in the order of `stream`.  Leaves `out` empty
+// where there is no memory.
+int new_scratch(int device, int sms, cudaStream_t stream, ScratchRef &out)
+{
+    const size_t area = static_cast<size_t>(sms) * sq::kStreamHeldSets * sq::kStreamHeldBytes;
+    void *mem = nullptr;
+    if (cudaMalloc(&mem, area + sq::kStreamWorkBytes) != cudaSuccess) {
+        cudaGetLastError();   // reported by the return code of the call, not left pending
+        return SQUANT_OK;
+    }
+    ScratchRef s = std::make_shared<StreamScratch>(static_cast<unsigned char *>(mem), area, device);
+    SQ_CUDA(cudaMemsetAsync(s->work(), 0, sq::kStreamWorkBytes, stream));
+    g_scratch.erase(std::remove_if(g_scratch.begin(), g_scratch.end(), [](const std::weak_ptr<StreamScratch> &w) { return w.expired(); }),
+                    g_scratch.end());
+    g_scratch.push_back(s);
+    out = std::move(s);
+    return SQUANT_OK;
+}
+
+void CUDART_CB release_scratch(void *p) { delete static_cast<ScratchRef *>(p); }
 
 // The graph that is being captured takes a share in the scratch memory that its kernel node points to.
-int share_with_graph(const std::shared_ptr<void> &scratch, cudaGraph_t graph)
+int share_with_graph(const ScratchRef &scratch, cudaGraph_t graph)
 {
-    auto *share = new (std::nothrow) std::shared_ptr<void>(scratch);
+    auto *share = new (std::nothrow) ScratchRef(scratch);
     if (!share) return SQUANT_ERR_NOMEM;
     cudaUserObject_t obj = nullptr;
     const cudaError_t e = cudaUserObjectCreate(&obj, share, release_scratch, 1, cudaUserObjectNoDestructorSync);
@@ -289,21 +323,16 @@ struct ParamPlan {
     // streaming kernel (layers of long 3x3 channels): one item per output channel
     struct Stream {
         sq::LaunchTable table;
-        int items = 0, nk_max = 0, n_max = 0, slot = 0;
+        int items = 0, nk_max = 0, n_max = 0;
         bool out = false;                     // packed or dequantized outputs wanted
-        // Scratch (what SQuant-C needs of every kernel one step later: four sets of 18 KB per thread block),
-        // allocated at the plan's first launch, freed when neither the plan nor a graph needs it.
-        std::shared_ptr<void> scratch;
+        ScratchRef scratch;                   // allocated at the plan's first launch outside a capture
         // Layers with packed or dequantized outputs can also go to the grouped kernel, which needs no scratch:
         // where it cannot be allocated (a full device, the plan's first launch inside a stream capture).
         sq::LaunchTable grouped;
         int grouped_grid = 0, grouped_smem = 0;
     };
     mutable std::vector<Stream> streams;
-    mutable bool slots_clean = false;   // the streams' work counters have been zeroed on the stream of the plan's first launch
 };
-
-int g_next_slot = 0;   // next work-counter slot of the streaming kernel; guarded by g_mutex
 
 // Layers the streaming kernel takes: 3x3 channels so long that no four CTAs of the grouped kernel fit a
 // multiprocessor (from 1184 input channels on: 2048 channels take 42.4 us in the grouped kernel and 59.8 us
@@ -418,8 +447,6 @@ int build_param_plan(const squant_layer *layers, int32_t n_layers, const squant_
                 st.grouped_smem = std::max(st.grouped_smem, sq::kCtaThreads / d.g * d.slice_bytes);
             }
             st.out = kind != 0;
-            st.slot = g_next_slot;
-            g_next_slot = (g_next_slot + 1) % sq::kTicketSlots;
         }
     }
     // A launch whose warps do not fill the GPU takes the time of one channel, so its channels get twice or
@@ -537,31 +564,8 @@ int get_plan(const squant_layer *layers, int32_t n_layers, const squant_options 
     return SQUANT_OK;
 }
 
-// Device address of a work counter (done = false) or of its "CTAs finished" twin (done = true).
-void *ticket_address(int slot, bool done)
-{
-    static std::vector<std::pair<unsigned *, unsigned *>> base;   // per device; guarded by g_mutex
-    int device = 0;
-    cudaGetDevice(&device);
-    if (static_cast<int>(base.size()) <= device) base.resize(device + 1, {nullptr, nullptr});
-    if (!base[device].first) {
-        cudaGetSymbolAddress(reinterpret_cast<void **>(&base[device].first), sq::g_ticket);
-        cudaGetSymbolAddress(reinterpret_cast<void **>(&base[device].second), sq::g_done);
-    }
-    return (done ? base[device].second : base[device].first) + slot;
-}
-
 int launch_plan(const ParamPlan &p, cudaStream_t stream)
 {
-    // A work-counter slot comes to a plan in an unknown state (a plan that was evicted, or a launch
-    // that failed, may have left it dirty): zero it in stream order before the plan's first launch.
-    if (!p.slots_clean) {
-        for (const ParamPlan::Stream &st : p.streams) {
-            SQ_CUDA(cudaMemsetAsync(ticket_address(st.slot, false), 0, sizeof(unsigned), stream));
-            SQ_CUDA(cudaMemsetAsync(ticket_address(st.slot, true), 0, sizeof(unsigned), stream));
-        }
-        p.slots_clean = true;
-    }
     // long 3x3 channels first: one persistent CTA per multiprocessor
     for (ParamPlan::Stream &st : p.streams) {
         int device = 0;
@@ -572,25 +576,21 @@ int launch_plan(const ParamPlan &p, cudaStream_t stream)
         SQ_CUDA(cudaStreamGetCaptureInfo_v2(stream, &cap, nullptr, &graph, nullptr, nullptr));
         const bool capturing = cap == cudaStreamCaptureStatusActive;
         if (!capturing) free_dead_scratch();
-        if (!st.scratch && (!st.out || !capturing)) {
-            const size_t bytes = static_cast<size_t>(sms) * sq::kStreamHeldSets * sq::kStreamHeldBytes;
-            void *ptr = nullptr;
-            if (cudaMalloc(&ptr, bytes) == cudaSuccess) {
-                st.scratch = std::shared_ptr<void>(ptr, scratch_unused);
-            } else {
-                cudaGetLastError();   // the failed allocation is reported by the return code, not left pending
-                if (!st.out) return SQUANT_ERR_NOMEM;
-            }
+        ScratchRef scratch = st.scratch;
+        if (!scratch && (!st.out || !capturing)) {
+            const int rc = new_scratch(device, sms, stream, scratch);
+            if (rc) return rc;
+            if (!scratch && !st.out) return SQUANT_ERR_NOMEM;
+            if (!capturing) st.scratch = scratch;   // (of a capture: zeroed by the graph, so the graph's alone)
         }
-        if (st.scratch && capturing) {
-            const int rc = share_with_graph(st.scratch, graph);
+        if (scratch && capturing) {
+            const int rc = share_with_graph(scratch, graph);
             if (rc) return rc;
         }
-        if (st.scratch) {
+        if (scratch) {
             const int grid = std::min(st.items, sms), smem = sq::stream_layout(st.nk_max, st.n_max).total;
             auto kernel = st.out ? sq::squant_stream_kernel<true> : sq::squant_stream_kernel<false>;
-            kernel<<<grid, sq::kStreamThreads, smem, stream>>>(st.table, p.qmax, p.mode, st.items, st.slot, st.nk_max, st.n_max,
-                                                               static_cast<unsigned char *>(st.scratch.get()));
+            kernel<<<grid, sq::kStreamThreads, smem, stream>>>(st.table, p.qmax, p.mode, st.items, st.nk_max, st.n_max, scratch->mem, scratch->work());
         } else {
             sq::squant_model_kernel<<<st.grouped_grid, sq::kCtaThreads, st.grouped_smem, stream>>>(st.grouped, p.qmax, p.mode);
         }
@@ -881,7 +881,6 @@ int squant_plan_kernels(const squant_layer *layers, int32_t n_layers, const squa
     int rc = validate(layers, n_layers, opt, false, o);
     if (rc) return rc;
     if (n_layers > 0 && !kernels) return SQUANT_ERR_NULL;
-    std::lock_guard<std::mutex> lock(g_mutex);   // (plans draw work-counter slots)
     ParamPlan plan;
     return build_param_plan(layers, n_layers, o, kMaxSmemFallback, 148, plan, kernels);
 }
@@ -924,9 +923,12 @@ int squant_device_status(void)
     if (st == 0) return SQUANT_OK;
     const int zero = 0;
     SQ_CUDA(cudaMemcpyToSymbol(sq::g_device_status, &zero, sizeof(int)));
-    // a launch that gave up may have left its work counter half drawn: all plans start clean again
-    SQ_CUDA(cudaMemset(ticket_address(0, false), 0, sizeof(unsigned) * sq::kTicketSlots));
-    SQ_CUDA(cudaMemset(ticket_address(0, true), 0, sizeof(unsigned) * sq::kTicketSlots));
+    // a launch that gave up may have left its work counters half drawn: all start clean again
+    int device = 0;
+    SQ_CUDA(cudaGetDevice(&device));
+    for (const std::weak_ptr<StreamScratch> &w : g_scratch)
+        if (const ScratchRef s = w.lock())
+            if (s->device == device) SQ_CUDA(cudaMemset(s->work(), 0, sq::kStreamWorkBytes));
     return SQUANT_ERR_TIMEOUT;
 }
 

@@ -41,13 +41,6 @@
 
 namespace sq {
 
-// Work counters, one slot per launch plan.  Launches that share a slot must not overlap; a slot
-// belongs to one plan, i.e. to one set of output buffers, for which overlapping launches would
-// race on the outputs anyway.
-constexpr int kTicketSlots = 1024;
-__device__ unsigned g_ticket[kTicketSlots];
-__device__ unsigned g_done[kTicketSlots];
-
 __device__ __forceinline__ int layer_of(const LaunchTable &tbl, int item)
 {
     int layer = 0;   // last layer whose first item is <= item
@@ -220,6 +213,11 @@ __device__ __noinline__ KernelOut kernel9_exact_smem(int *P, unsigned char *cb)
 constexpr int kStreamHeldBytes = kStreamQuantThreads * 36;   // one set
 constexpr int kStreamHeldSets = 4;   // by step modulo four, like the code buffers: a set is rewritten only after a wait
                                      // that implies the channel warp is done with it
+// Behind the sets of all thread blocks: the launch's work counter and its "thread blocks finished" twin, zero
+// before and after every launch.  They live as long as the area, which the launch plan shares with the graphs
+// that captured it, so no other launch ever draws from them; launches of the same plan must not overlap
+// (they would race on its output buffers anyway).
+constexpr int kStreamWorkBytes = 8;
 struct StreamHeld {
     int vmax, vmin;   // largest and smallest of the four candidates (0 where there are no kernels)
     bool have;        // a previous channel exists
@@ -414,8 +412,8 @@ __device__ __forceinline__ int stream_boundary(const int (&c)[8], int lane, int 
 // kernels), from which every CTA derives the same layout.
 template <bool kOut>
 __global__ void __launch_bounds__(kStreamThreads, 1)
-squant_stream_kernel(const __grid_constant__ LaunchTable tbl, int qmax, unsigned mode, int n_items, int slot,
-                     int nk_max, int n_max, unsigned char *held_scratch)
+squant_stream_kernel(const __grid_constant__ LaunchTable tbl, int qmax, unsigned mode, int n_items, int nk_max, int n_max,
+                     unsigned char *held_scratch, unsigned *work)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     const StreamLayout lay = stream_layout(nk_max, n_max);
@@ -467,7 +465,7 @@ squant_stream_kernel(const __grid_constant__ LaunchTable tbl, int qmax, unsigned
             bulk_load(smem + static_cast<size_t>(b) * lay.w_bytes, wg, static_cast<unsigned>(L.NK) * 4u, &ctrl->full[b]);
             ++issued;
             // the next channel is drawn now: the counter's latency passes during the waits
-            const unsigned t = gridDim.x + atomicAdd(&g_ticket[slot], 1u);
+            const unsigned t = gridDim.x + atomicAdd(&work[0], 1u);
             item = t < static_cast<unsigned>(n_items) ? static_cast<int>(t) : -1;
         };
         stage(0);
@@ -482,11 +480,11 @@ squant_stream_kernel(const __grid_constant__ LaunchTable tbl, int qmax, unsigned
             // CTA's shared memory; wait for them (bounded) before the CTA may end
             for (int j = max(issued - 2, 0); j < issued; ++j) mbar_wait(&ctrl->full[j & 1], static_cast<unsigned>(j >> 1) & 1u);
         }
-        // every ticket this CTA draws has been drawn: the last CTA to get here resets the slot
+        // every ticket this CTA draws has been drawn: the last CTA to get here resets the counters
         __threadfence();
-        if (atomicAdd(&g_done[slot], 1u) == gridDim.x - 1) {
-            g_ticket[slot] = 0;
-            g_done[slot] = 0;
+        if (atomicAdd(&work[1], 1u) == gridDim.x - 1) {
+            work[0] = 0;
+            work[1] = 0;
             __threadfence();
         }
         return;

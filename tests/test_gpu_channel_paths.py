@@ -179,3 +179,39 @@ def test_scratch_of_a_captured_call_lives_as_long_as_the_graph():
             break
         time.sleep(0.01)
     assert torch.cuda.mem_get_info()[0] >= free1 + area
+
+
+def test_a_captured_call_keeps_its_work_counter():
+    """A graph of a streaming launch and a call whose plan was made a thousand plans later overlap on the GPU:
+    each draws its channels from a counter of its own, so none is left out."""
+    shape = (700, 1536, 3, 3)
+    w = W.random_layer(shape, seed=15)
+    r = oracle.quantize_layer(w, bits=4)
+    t = torch.from_numpy(w).cuda()
+    a, *later = [sq.alloc_outputs(t.clone()) for _ in range(4)]
+    assert sq.squant_plan_kernels([a]) == ["stream"]
+    call = sq.ModelCall([a], bits=4)
+    call.run()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        call.run()
+    small = sq.alloc_outputs(torch.randn(1, 1184, 3, 3, device="cuda"))
+    base = torch.randn(10656 + 4 * 1024, device="cuda")
+    for i in range(1023):   # further plans: the same outputs, other weights
+        small.w = base[4 * i:4 * i + 10656].view(1, 1184, 3, 3)
+        sq.squant_quantize_model([small], bits=4)
+    other = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    for b in later * 2:
+        for x in (a, b):
+            x.codes.fill_(-128)
+            x.kernel_err.fill_(float("nan"))
+        torch.cuda.synchronize()
+        for _ in range(3):
+            graph.replay()
+            sq.squant_quantize_model([b], bits=4, stream=other)
+        sq.squant_device_status()
+        for x in (a, b):
+            assert np.array_equal(x.codes.cpu().numpy(), r.codes)
+            assert np.array_equal(x.kernel_err.cpu().numpy().view(np.uint32), r.kernel_err.view(np.uint32))
+            assert np.array_equal(x.channel_err.cpu().numpy().view(np.uint32), r.channel_err.view(np.uint32))
