@@ -133,13 +133,13 @@ int squant_quantize_layer(const squant_layer *layer, const squant_options *opt, 
  * Host-side launch tables of recent calls are cached.  The only device memory the call ever
  * allocates is the streaming kernel's scratch area (72 KB per multiprocessor, about 11 MB on a
  * B200): at the FIRST call with given descriptors that has such layers, by cudaMalloc, kept with
- * the cached launch tables and freed when neither they nor a graph that captured such a call are
- * left (so that first call belongs outside any stream capture; callers that cannot allocate at all:
- * see squant_quantize_layer_noalloc).  Calls with packed or dequantized outputs take the grouped
- * kernel where the area cannot be allocated.  Outputs are valid when the stream reaches the end of
- * the launches.  The streaming kernel hands out its channels through a counter in device memory, which is
- * part of the scratch area and so belongs to the cached launch tables of these exact descriptors and the graphs
- * captured with them:
+ * the cached launch tables and freed by the next call (or squant_shutdown) when neither they nor a
+ * graph that captured such a call are left (so that first call belongs outside any stream capture;
+ * callers that cannot allocate at all: see squant_quantize_layer_noalloc).  Calls with packed or
+ * dequantized outputs take the grouped kernel where the area cannot be allocated.  Outputs are valid
+ * when the stream reaches the end of the launches.  The streaming kernel hands out its channels through
+ * a counter in device memory, which is part of the scratch area and so belongs to the cached launch
+ * tables of these exact descriptors and the graphs captured with them:
  * two calls with the SAME descriptors must not overlap on the GPU (they would race on the
  * outputs anyway); calls with different descriptors may.  All arguments are validated
  * on the host first; a failed call launches nothing and writes nothing.  Returns SQUANT_OK or a
@@ -278,7 +278,10 @@ const char *squant_strerror(int code);
 /* Text of the CUDA error behind the calling thread's last SQUANT_ERR_CUDA ("" if none). */
 const char *squant_last_cuda_error(void);
 
-/* Frees cached plans and staging buffers on all devices.  Call with no work in flight. */
+/*
+ * Frees cached plans, their scratch areas and staging buffers on all devices.  Call with no work in flight.
+ * A scratch area that a captured graph still points to is freed by the first call after the graph has gone.
+ */
 int squant_shutdown(void);
 
 #ifdef __cplusplus

@@ -214,8 +214,9 @@ int build_plan(const squant_layer *layers, int32_t n_layers, const squant_option
 // Scratch memory of the streaming kernel (what SQuant-C needs of every kernel one step later: four sets of
 // 18 KB per thread block; the launch's work counters) is shared by the plan that launches with it and by every
 // graph that captured such a launch, and goes with the last of them.  A graph lets go inside a CUDA callback,
-// where no CUDA call is allowed: the memory is then listed here and freed by the next call that
-// is not being captured (cudaFree waits for the device, so no launch still uses it).
+// where no CUDA call is allowed: the memory is then listed here and freed by the next call that quantizes device
+// or host buffers and is not being captured, or by squant_shutdown (cudaFree waits for the device, so no launch
+// still uses it).
 struct DeadScratch {
     std::mutex mutex;
     std::vector<void *> list;
@@ -242,14 +243,31 @@ void scratch_unused(void *p)
 void free_dead_scratch()
 {
     DeadScratch &d = dead_scratch();
-    if (!d.any.load(std::memory_order_acquire)) return;
     std::vector<void *> list;
     {
         std::lock_guard<std::mutex> lock(d.mutex);
         list.swap(d.list);
         d.any.store(false, std::memory_order_relaxed);
     }
-    for (void *p : list) cudaFree(p);
+    // captures of other streams may be under way; they do not depend on this memory
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    for (void *p : list)
+        if (cudaFree(p) != cudaSuccess) {
+            cudaGetLastError();   // not the caller's error: it stays listed
+            scratch_unused(p);
+        }
+    cudaThreadExchangeStreamCaptureMode(&mode);
+}
+
+// The same unless `stream` is being captured; costs nothing where there is nothing to free.
+int free_dead_scratch(cudaStream_t stream)
+{
+    if (!dead_scratch().any.load(std::memory_order_acquire)) return SQUANT_OK;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    SQ_CUDA(cudaStreamIsCapturing(stream, &cap));
+    if (cap == cudaStreamCaptureStatusNone) free_dead_scratch();
+    return SQUANT_OK;
 }
 
 struct StreamScratch {
@@ -566,6 +584,8 @@ int get_plan(const squant_layer *layers, int32_t n_layers, const squant_options 
 
 int launch_plan(const ParamPlan &p, cudaStream_t stream)
 {
+    const int freed = free_dead_scratch(stream);   // of graphs and of plans that have left the cache
+    if (freed) return freed;
     // long 3x3 channels first: one persistent CTA per multiprocessor
     for (ParamPlan::Stream &st : p.streams) {
         int device = 0;
@@ -575,7 +595,6 @@ int launch_plan(const ParamPlan &p, cudaStream_t stream)
         cudaGraph_t graph = nullptr;
         SQ_CUDA(cudaStreamGetCaptureInfo_v2(stream, &cap, nullptr, &graph, nullptr, nullptr));
         const bool capturing = cap == cudaStreamCaptureStatusActive;
-        if (!capturing) free_dead_scratch();
         ScratchRef scratch = st.scratch;
         if (!scratch && (!st.out || !capturing)) {
             const int rc = new_scratch(device, sms, stream, scratch);
@@ -997,6 +1016,7 @@ int squant_shutdown(void)
     int cur = 0;
     const bool have = cudaGetDevice(&cur) == cudaSuccess;
     g_plans.clear();
+    free_dead_scratch();   // (areas that a graph still holds go with the graph)
     for (size_t d = 0; d < g_arenas.size(); ++d) {
         if (g_arenas[d].ptr) { cudaSetDevice(static_cast<int>(d)); cudaDeviceSynchronize(); cudaFree(g_arenas[d].ptr); }
     }

@@ -215,3 +215,80 @@ def test_a_captured_call_keeps_its_work_counter():
             assert np.array_equal(x.codes.cpu().numpy(), r.codes)
             assert np.array_equal(x.kernel_err.cpu().numpy().view(np.uint32), r.kernel_err.view(np.uint32))
             assert np.array_equal(x.channel_err.cpu().numpy().view(np.uint32), r.channel_err.view(np.uint32))
+
+
+def free_memory():
+    torch.cuda.synchronize()
+    return torch.cuda.mem_get_info()[0]
+
+
+def test_scratch_is_given_back():
+    """The streaming kernel's scratch memory (72 KB per multiprocessor) goes with its plan: at squant_shutdown, and
+    when the plan leaves the cache although no further streaming call follows."""
+    area = (70 << 10) * torch.cuda.get_device_properties(0).multi_processor_count
+    long_call = sq.ModelCall([sq.alloc_outputs(torch.randn(3, 1536, 3, 3, device="cuda"))])
+    small = [sq.ModelCall([sq.alloc_outputs(torch.randn(1, 3, device="cuda"))]) for _ in range(65)]
+    for call in [long_call] + small:   # loads what there is to load
+        call.run()
+    for again in range(2):
+        sq.squant_shutdown()
+        free0 = free_memory()
+        long_call.run()
+        assert free_memory() <= free0 - area
+        if again:
+            for call in small:         # the cache holds 64 plans
+                call.run()
+        else:
+            sq.squant_shutdown()
+        assert free_memory() >= free0
+
+
+def test_scratch_of_a_graph_survives_shutdown_and_goes_after_it():
+    area = (70 << 10) * torch.cuda.get_device_properties(0).multi_processor_count
+    w = adversarial_layer((40, 1536, 3, 3), seed=8)
+    b = sq.alloc_outputs(torch.from_numpy(w).cuda())
+    call = sq.ModelCall([b])
+    small = sq.ModelCall([sq.alloc_outputs(torch.randn(1, 3, device="cuda"))])
+    call.run()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        call.run()
+    sq.squant_shutdown()
+    small.run()
+    b.codes.fill_(-128)
+    graph.replay()
+    sq.squant_device_status()
+    assert np.array_equal(b.codes.cpu().numpy(), oracle.quantize_layer(w, bits=4).codes)
+    free0 = free_memory()
+    del graph
+    for _ in range(200):   # the graph's resources go in a callback of the driver
+        small.run()        # not a streaming call
+        if free_memory() >= free0 + area:
+            break
+        time.sleep(0.01)
+    assert free_memory() >= free0 + area
+
+
+def test_freeing_scratch_leaves_captures_of_other_streams_alone():
+    """A call that frees scratch memory of an evicted plan, on a stream that is not captured, while another stream is."""
+    long_call = sq.ModelCall([sq.alloc_outputs(torch.randn(3, 1536, 3, 3, device="cuda"))])
+    small = [sq.ModelCall([sq.alloc_outputs(torch.randn(1, 3, device="cuda"))]) for _ in range(66)]
+    w = W.random_layer((8, 64, 3, 3), seed=9)
+    b = sq.alloc_outputs(torch.from_numpy(w).cuda())
+    captured = sq.ModelCall([b])
+    side = torch.cuda.Stream()
+    for call in small:
+        call.run()
+    long_call.run()
+    captured.run()
+    free0 = free_memory()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        captured.run()
+        for call in small:   # the plan of long_call leaves the cache
+            call.run(side)
+    assert free_memory() > free0
+    b.codes.fill_(-128)
+    graph.replay()
+    sq.squant_device_status()
+    assert np.array_equal(b.codes.cpu().numpy(), oracle.quantize_layer(w, bits=4).codes)
