@@ -140,6 +140,8 @@ int64_t layout_layer(const squant_layer &l, LayerDesc &d, unsigned mode, unsigne
     d.g = group_size(d.NK);
     d.g_shift = 0;
     while ((1 << d.g_shift) < d.g) ++d.g_shift;
+    // No layout holds a channel in less than 5 B a weight; the sizes below are 32-bit numbers.
+    if (5ll * d.NK > kMaxSmemFallback) return 5ll * d.NK;
     // Depthwise layers (one kernel per output channel) with plain outputs: a whole channel per thread.
     // SQuant-C is void there once SQuant-K has run; without K (E|C) the channel step is real.
     if (d.N == 1 && d.K <= 64 && !l.scales_in && !l.dequant && !l.dequant_bf16 && !(flags & SQUANT_FLAG_PACK_INT4) &&
@@ -193,10 +195,11 @@ int build_plan(const squant_layer *layers, int32_t n_layers, const squant_option
     for (int i = 0; i < n_layers; ++i) {
         LayerDesc &d = p.layers[i];
         const int64_t cta_smem = layout_layer(layers[i], d, o.mode, o.flags);
+        if (cta_smem > max_smem) return SQUANT_ERR_TOO_WIDE;
         const int groups = sq::kCtaThreads / d.g;
         LayerDesc staged = d;
         layout_staged(layers[i], staged, o.mode);   // (the limit: a channel staged with its per-kernel arrays)
-        if (cta_smem > max_smem || static_cast<int64_t>(sq::kCtaThreads / staged.g) * staged.slice_bytes > max_smem) return SQUANT_ERR_TOO_WIDE;
+        if (static_cast<int64_t>(sq::kCtaThreads / staged.g) * staged.slice_bytes > max_smem) return SQUANT_ERR_TOO_WIDE;
         if (cta_smem > p.smem_bytes) p.smem_bytes = static_cast<int>(cta_smem);
         for (int c = 0; c < d.M; c += groups) {
             const int nch = (d.M - c < groups) ? d.M - c : groups;

@@ -61,6 +61,16 @@ def test_invalid_arguments_are_rejected(shape, kw, code):
     assert ei.value.code == code
 
 
+@pytest.mark.parametrize("n,k", [(13207, 65041), (13210, 65026), (13270, 64732), (262143, 3277), (16384, 52429), (16384, 65535)])
+def test_sizes_beyond_32_bits_are_rejected(n, k):
+    """5 B a weight of such a channel are a small number modulo 2^32."""
+    for mode in (sq.MODE_EKC, sq.MODE_E | sq.MODE_C, sq.MODE_E):
+        for plan in (sq.squant_plan_info, sq.squant_plan_kernels):
+            with pytest.raises(sq.SquantError) as ei:
+                plan([(1, n, 1, k)], mode=mode)
+            assert ei.value.code == -6, (plan, mode)
+
+
 def test_valid_edge_arguments():
     assert _info([], bits=4)["grid_ctas"] == 0
     assert _info([(4, 300, 1, 1)], mode=1 | 4)["grid_ctas"] >= 1      # E|C ablation mode
