@@ -29,7 +29,8 @@ NOALLOC_MAX_CTAS = 32768
 
 EXPORTS = ("squant_quantize_layer", "squant_quantize_layer_noalloc", "squant_quantize_model", "squant_quantize_model_host",
            "squant_plan_info", "squant_plan_kernels", "squant_selfcheck_division", "squant_device_status", "squant_launch_count", "squant_strerror", "squant_last_cuda_error",
-           "squant_shutdown", "squant_debug_set_status", "squant_debug_wait_expires", "squant_debug_violations")
+           "squant_shutdown", "squant_debug_set_status", "squant_debug_wait_expires", "squant_debug_violations",
+           "squant_debug_sums_checked")
 
 
 class SquantError(RuntimeError):
@@ -77,6 +78,7 @@ def load_library() -> ctypes.CDLL:
         getattr(lib, f).restype = ctypes.c_int
     lib.squant_debug_violations.argtypes = [i32p, i32p]
     lib.squant_debug_violations.restype = ctypes.c_int
+    lib.squant_debug_sums_checked.restype = ctypes.c_int64
     lib.squant_debug_set_status.argtypes = [ctypes.c_int]
     lib.squant_debug_set_status.restype = ctypes.c_int
     lib.squant_debug_wait_expires.argtypes = [ctypes.c_int32, vp]
@@ -309,6 +311,14 @@ def squant_debug_violations():
     if rc < 0:
         _check(rc)
     return bool(rc), n.value, site.value
+
+
+def squant_debug_sums_checked() -> int:
+    """Error sums the checked build has taken a second time since the last call (0 in the regular build)."""
+    n = int(load_library().squant_debug_sums_checked())
+    if n < 0:
+        _check(n)
+    return n
 
 
 def squant_debug_set_status(value: int) -> None:

@@ -974,6 +974,17 @@ int squant_debug_violations(int32_t *count, int32_t *first_site)
 #endif
 }
 
+int64_t squant_debug_sums_checked(void)
+{
+    std::lock_guard<std::mutex> lock(g_mutex);
+    SQ_CUDA(cudaDeviceSynchronize());
+    unsigned n = 0;
+    SQ_CUDA(cudaMemcpyFromSymbol(&n, sq::g_debug_sums, sizeof(n)));
+    const unsigned zero = 0;
+    SQ_CUDA(cudaMemcpyToSymbol(sq::g_debug_sums, &zero, sizeof(zero)));
+    return static_cast<int64_t>(n);
+}
+
 int squant_debug_set_status(int value)
 {
     std::lock_guard<std::mutex> lock(g_mutex);

@@ -139,6 +139,7 @@ __device__ __forceinline__ void emit_codes(const LayerDesc &L, size_t first, siz
             __stcs(reinterpret_cast<int4 *>(row + head) + i, reinterpret_cast<const int4 *>(cel + head)[i]);
         for (int i = G.t; i < head + (n - tail); i += G.g) {
             const int e = i < head ? i : tail + i - head;
+            SQ_DBG(tail <= n && e >= 0 && e < n, 17);
             row[e] = cel[e];
         }
     } else {   // two codes per byte, low nibble = even flat index
@@ -155,6 +156,7 @@ __device__ __forceinline__ void emit_codes(const LayerDesc &L, size_t first, siz
         }
         for (int i = G.t; i < head + ((n + 1) >> 1) - tail; i += G.g) {
             const int b = i < head ? i : tail + i - head;
+            SQ_DBG(2 * tail <= n && b >= 0 && 2 * b < n, 18);
             row[b] = static_cast<unsigned char>((cel[2 * b] & 15) | (2 * b + 1 < n ? cel[2 * b + 1] << 4 : 0));
         }
     }
@@ -164,6 +166,7 @@ __device__ __forceinline__ void emit_codes(const LayerDesc &L, size_t first, siz
         const bool words = ((reinterpret_cast<uintptr_t>(cel) - sp.r) & 3) == 0;
         for (int q = sp.q_lo + G.t; q < sp.q_hi; q += G.g) {
             const unsigned char *c = cel + (4 * q - sp.r);
+            SQ_DBG(4 * q - sp.r >= 0 && 4 * q - sp.r + 4 <= n, 19);
             const unsigned c4 = words ? *reinterpret_cast<const unsigned *>(c) : c[0] | (c[1] << 8) | (c[2] << 16) | (static_cast<unsigned>(c[3]) << 24);
             __stcs(reinterpret_cast<float4 *>(row + (4 * q - sp.r)), make_float4(row_deq(c4, s), row_deq(c4 >> 8, s), row_deq(c4 >> 16, s), row_deq(c4 >> 24, s)));
         }
@@ -183,6 +186,7 @@ __device__ __forceinline__ void emit_codes(const LayerDesc &L, size_t first, siz
         }
         for (int i = G.t; i < head + (n - tail); i += G.g) {
             const int e = i < head ? i : tail + i - head;
+            SQ_DBG(tail <= n && e >= 0 && e < n, 20);
             row[e] = static_cast<uint16_t>(bf16_bits(row_deq(cel[e], s)));
         }
     }
@@ -229,6 +233,7 @@ __device__ __forceinline__ void conv_body(const LayerDesc &L, int m, const Group
     {
         unsigned char *c0 = slice + sel_bytes(g, kOwn, K) + ((4 * NK + 12 + 15) & ~15);
         cel = c0 + ((reinterpret_cast<uintptr_t>(L.codes) + first) & 15);
+        SQ_DBG(reinterpret_cast<unsigned char *>(wel + NK) <= c0 && cel + NK <= slice + conv_bytes(g, NK, K, kOwn), 16);
     }
 
     // ---- scale
@@ -445,6 +450,9 @@ __device__ __forceinline__ void conv_body(const LayerDesc &L, int m, const Group
         }
     }
     G.sync();   // all codes are final
+#ifdef SQUANT_DEBUG_BOUNDS
+    if (!kClip && kOwn != kCluster && ((mode & 4u) || L.cerr)) debug_check_sum(G, wrow, cel, NK, s, ec, true, sc);
+#endif
 
     emit_codes(L, first, static_cast<size_t>(m) * ((L.NK + 1) >> 1) + ((static_cast<size_t>(n0) * K) >> 1), G, cel, NK, s, mode);
     if (G.t == 0 && n0 == 0) {

@@ -70,12 +70,13 @@ struct Group {
 
 // ---------------------------------------------------------------- checked build
 // Built with -DSQUANT_DEBUG_BOUNDS (a second library, for tests on small cases), the kernels check
-// the indices they form into shared memory and into the launch table against their bounds, and
-// recompute every channel's error sum from its final codes and staged weights; a failed check is
-// counted and its site recorded, the access it guards is skipped where it can be.  The regular
-// build compiles the checks away.
+// the indices they form into shared memory and into the launch table against their bounds, and row_body
+// and conv_body take the error sum of a channel with an absmax scale a second time, from its final codes
+// and the weights; a failed check is counted and its site recorded.  The regular build compiles the
+// checks away.
 __device__ unsigned g_debug_violations = 0;
 __device__ int g_debug_site = 0;
+__device__ unsigned g_debug_sums = 0;   // error sums taken a second time
 #ifdef SQUANT_DEBUG_BOUNDS
 __device__ __noinline__ void sq_debug_fail(int site)
 {
@@ -83,10 +84,16 @@ __device__ __noinline__ void sq_debug_fail(int site)
     atomicCAS(&g_debug_site, 0, site);
 }
 #define SQ_DBG(cond, site) do { if (!(cond)) sq_debug_fail(site); } while (0)
-#define SQ_DBG_OK(cond, site) ((cond) ? true : (sq_debug_fail(site), false))
+
+// What an element adds to the error sum: weight w, scale s, final code; by plain IEEE division (the difference
+// from the rounded quotient is exact, then whole steps for the flips).
+__device__ __forceinline__ long long debug_error(float w, float s, int code)
+{
+    const float x = __fdiv_rn(w, s), q = rintf(x);
+    return __float2ll_rn(__fmul_rn(__fsub_rn(q, x), 1073741824.0f)) + (static_cast<long long>(code) - __float2int_rn(q)) * kOne;
+}
 #else
 #define SQ_DBG(cond, site) ((void)0)
-#define SQ_DBG_OK(cond, site) (true)
 #endif
 
 __device__ __forceinline__ unsigned dynamic_smem_bytes()

@@ -142,6 +142,29 @@ __device__ __forceinline__ int cluster_sum(const int *w)
     return __reduce_add_sync(kFull, lane < static_cast<int>(cl.num_blocks()) ? remote(w, lane) : 0);
 }
 
+#ifdef SQUANT_DEBUG_BOUNDS
+// The channel's error sum from its final codes and the weights (global memory), compared with ec.  Called by
+// every thread of the group after the codes' last barrier; groups that share a warp come together.
+__device__ __forceinline__ void debug_check_sum(const Group &G, const float *w, const unsigned char *codes, int n, float s, long long ec, bool valid,
+                                                SelScratch *sc)
+{
+    long long e = 0;
+    for (int j = G.t; j < n; j += G.g) e += debug_error(w[j], s, static_cast<signed char>(codes[j]));
+    for (int o = min(G.g, 32) >> 1; o > 0; o >>= 1) e += __shfl_xor_sync(kFull, e, o);
+    if (G.g > 32) {
+        if (G.t == 0) sc->sum64 = 0ull;
+        G.sync();
+        if ((G.t & 31) == 0) atomicAdd(&sc->sum64, static_cast<unsigned long long>(e));
+        G.sync();
+        e = static_cast<long long>(sc->sum64);
+    }
+    if (G.t == 0 && valid) {
+        SQ_DBG(e == ec, 8);
+        atomicAdd(&g_debug_sums, 1u);
+    }
+}
+#endif
+
 // ---------------------------------------------------------------- SQuant-C: the k_c largest candidates
 // each(t, f) visits those of the calling thread's elements that reach t >= 1, f(a, n) with a = the
 // candidate's value in the direction of the flips and n its kernel index in the channel; m0, m1: the
@@ -211,6 +234,7 @@ __device__ __forceinline__ int select_top(const Group &G, Each each, Flip flip, 
     if (want && !slow && max(m0, m1) >= T0)
         each(T0, [&](int a, int n) {
             const int pos = atomicAdd(&sc->count, 1);
+            SQ_DBG(a >= 1 && a < top && n >= 0 && n < n_all, 12);
             if (pos < cap)
                 list[pos] = (static_cast<unsigned long long>(static_cast<unsigned>(a)) << kIdxBits) |
                             static_cast<unsigned long long>(((1 << kIdxBits) - 1) - n);
@@ -369,6 +393,7 @@ __device__ __forceinline__ void row_body(const LayerDesc &L, int m, const Group 
     const bool pack = (mode & kModePackInt4) != 0;
     const Span sp(pack ? 0 : static_cast<int>((reinterpret_cast<uintptr_t>(wrow) >> 2) & 3), N, G.t);
     const int r = sp.r, q_hi = sp.q_hi, rag = sp.rag, q0 = sp.q_lo + G.t;
+    SQ_DBG(N >= 0 && N + r <= 4 * L.off_vi && q_hi <= L.off_vi, 14);   // the vectors' places below
     int4 *Pbuf = reinterpret_cast<int4 *>(slice + sel_bytes(g, kOwn));              // what SQuant-C may choose from
     unsigned *cbuf = reinterpret_cast<unsigned *>(slice + sel_bytes(g, kOwn) + 16 * L.off_vi);   // codes, by vectors
     int *Pel = reinterpret_cast<int *>(Pbuf) + r;                                   // the same by elements
@@ -582,6 +607,7 @@ __device__ __forceinline__ void row_body(const LayerDesc &L, int m, const Group 
 #pragma unroll 1
                 for (; hit != 0u; hit &= hit - 1u) {
                     const int b = __ffs(hit) - 1, n = 4 * (qb + (b >> 2) * g) - r + (b & 3);
+                    SQ_DBG(n >= 0 && n < N, 15);
                     fn((Pel[n] ^ sx) - sx, n0 + n);
                 }
                 if (kOwn == kGroup) break;
@@ -603,6 +629,9 @@ __device__ __forceinline__ void row_body(const LayerDesc &L, int m, const Group 
         }
     }
     G.sync();   // all codes are final
+#ifdef SQUANT_DEBUG_BOUNDS
+    if (!kClip && kOwn != kCluster && ((mode & 4u) || L.cerr)) debug_check_sum(G, wrow, cel, N, s, ec, valid, sc);
+#endif
     if (!valid) return;
 
     // ---- codes, scale, channel error

@@ -117,6 +117,25 @@ def test_no_lane_overtakes_the_further_outputs(n):
         sq.use_library(None)
 
 
+def test_checked_build_takes_every_error_sum_a_second_time():
+    """Groups of 8 threads to a thread block, the row kernel, kernels of every body; each channel once."""
+    from paper_2202_07471_b200 import build as lib_build
+    shapes = [(37, 64, 3, 3), (33, 5, 1, 1), (9, 300, 1, 1), (5, 4097, 1, 1), (3, 9001, 1, 1), (4, 3, 5, 5), (6, 70, 1, 7), (11, 9, 3, 1), (3, 1100, 3, 3)]
+    ws = [adversarial_layer(s, seed=s[1]) for s in shapes]
+    sq.use_library(lib_build.LIB_DEBUG)
+    try:
+        sq.squant_debug_violations()
+        sq.squant_debug_sums_checked()
+        for bits, mode in ((4, sq.MODE_EKC), (8, sq.MODE_EKC), (3, sq.MODE_E | sq.MODE_K)):
+            check(ws, bits, mode, start=bits & 3)
+            assert sq.squant_debug_sums_checked() == sum(s[0] for s in shapes)
+            checked, failed, site = sq.squant_debug_violations()
+            assert checked and failed == 0, (failed, site)
+    finally:
+        sq.use_library(None)
+    assert sq.squant_debug_sums_checked() == 0   # the regular build takes none
+
+
 def test_long_channels_with_packed_codes_in_a_capture():
     """The first call of a plan inside a stream capture can allocate nothing: the grouped kernel takes it."""
     w = adversarial_layer((40, 1536, 3, 3), seed=5)
