@@ -16,17 +16,26 @@ namespace {
 
 PyObject *s_names[8];   // w, codes, scales, kernel_err, channel_err, dequant, dequant_bf16, scales_in
 
+// A reference that goes with its scope, also when data_ptr() throws.
+struct Held {
+    PyObject *p = nullptr;
+    Held() = default;
+    Held(const Held &) = delete;
+    Held &operator=(const Held &) = delete;
+    ~Held() { Py_XDECREF(p); }
+};
+
 // The tensor behind attribute i of o: 1 found, 0 None, -1 not a plain tensor (or no such attribute).
-int tensor_of(PyObject *o, int i, const at::Tensor *&t, PyObject *&held)
+int tensor_of(PyObject *o, int i, const at::Tensor *&t, Held &held)
 {
-    held = PyObject_GetAttr(o, s_names[i]);
-    if (!held) {
+    held.p = PyObject_GetAttr(o, s_names[i]);
+    if (!held.p) {
         PyErr_Clear();
         return -1;
     }
-    if (held == Py_None) return 0;
-    if (!THPVariable_CheckExact(held)) return -1;   // subclasses may have their own idea of data_ptr()
-    t = &THPVariable_Unpack(held);
+    if (held.p == Py_None) return 0;
+    if (!THPVariable_CheckExact(held.p)) return -1;   // subclasses may have their own idea of data_ptr()
+    t = &THPVariable_Unpack(held.p);
     return 1;
 }
 
@@ -36,7 +45,7 @@ bool descriptor(PyObject *o, squant_layer &l)
     void *ptr[8] = {};
     bool ok = true;
     const at::Tensor *w = nullptr;
-    PyObject *held[8] = {};
+    Held held[8];
     for (int i = 0; i < 8 && ok; ++i) {
         const at::Tensor *t = nullptr;
         const int kind = tensor_of(o, i, t, held[i]);
@@ -67,7 +76,6 @@ bool descriptor(PyObject *o, squant_layer &l)
         l.dequant_bf16 = static_cast<uint16_t *>(ptr[6]);
         l.scales_in = static_cast<const float *>(ptr[7]);
     }
-    for (PyObject *h : held) Py_XDECREF(h);
     return ok;
 }
 

@@ -1,6 +1,7 @@
 """Descriptors written by the native extension equal those of the Python code, and what the extension
 leaves out (tensor subclasses, wrong arguments) ends as it does in Python."""
 import ctypes
+import sys
 
 import pytest
 import torch
@@ -41,3 +42,16 @@ def test_wrong_arguments_are_rejected_as_before(bad):
     bad(b)
     with pytest.raises((ValueError, IndexError)):
         sq.ModelCall([sq.alloc_outputs(torch.randn(2, 2)), b])
+
+
+@pytest.mark.parametrize("name", ["w", "codes", "scales_in"])
+def test_no_reference_is_kept_of_a_tensor_without_storage(name):
+    """data_ptr() of a sparse tensor raises, here as in Python; the objects looked at before are released."""
+    b = sq.alloc_outputs(torch.randn(4, 3, 3, 3))
+    sparse = torch.zeros(4, 3, 3, 3).to_sparse()
+    setattr(b, name, sparse)
+    before = sys.getrefcount(sparse), sys.getrefcount(b.scales), sys.getrefcount(b.w)
+    for _ in range(50):
+        with pytest.raises((RuntimeError, ValueError)):
+            sq.ModelCall([b])
+    assert (sys.getrefcount(sparse), sys.getrefcount(b.scales), sys.getrefcount(b.w)) == before
