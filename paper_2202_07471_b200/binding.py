@@ -51,6 +51,14 @@ class Layer(ctypes.Structure):
                 ("scales_in", ctypes.c_void_p)]
 
 
+def _native(module):
+    """The descriptor extension if it was built with this layout of a descriptor, else None (a stale build would
+    write fields into the wrong places or past the array)."""
+    here = (ctypes.sizeof(Layer),) + tuple(getattr(Layer, name).offset for name, _ in Layer._fields_)
+    return module if getattr(module, "layout", None) == here else None
+
+
+_marshal = _native(_marshal)
 _lib = None
 _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
 

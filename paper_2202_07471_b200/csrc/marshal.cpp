@@ -8,6 +8,7 @@
 #include <ATen/PythonTorchFunctionTLS.h>
 #include <torch/csrc/autograd/python_variable.h>
 
+#include <cstddef>
 #include <limits>
 
 #include "squant.h"
@@ -114,5 +115,18 @@ PyMODINIT_FUNC PyInit__marshal(void)
         s_names[i] = PyUnicode_InternFromString(names[i]);
         if (!s_names[i]) return nullptr;
     }
-    return PyModule_Create(&module);
+    PyObject *m = PyModule_Create(&module);
+    if (!m) return nullptr;
+    // Size of a descriptor and the places of its fields as this extension was built with them, in the order of
+    // squant.h: the Python code compares them with its own before it hands over an array.
+    using L = squant_layer;
+    PyObject *layout = Py_BuildValue("(nnnnnnnnnnnnn)", sizeof(L), offsetof(L, w), offsetof(L, cout), offsetof(L, cin), offsetof(L, kh), offsetof(L, kw),
+                                     offsetof(L, codes), offsetof(L, scales), offsetof(L, kernel_err), offsetof(L, channel_err),
+                                     offsetof(L, dequant), offsetof(L, dequant_bf16), offsetof(L, scales_in));
+    if (!layout || PyModule_AddObject(m, "layout", layout) != 0) {
+        Py_XDECREF(layout);
+        Py_DECREF(m);
+        return nullptr;
+    }
+    return m;
 }

@@ -2,6 +2,7 @@
 leaves out (tensor subclasses, wrong arguments) ends as it does in Python."""
 import ctypes
 import sys
+import types
 
 import pytest
 import torch
@@ -55,3 +56,15 @@ def test_no_reference_is_kept_of_a_tensor_without_storage(name):
         with pytest.raises((RuntimeError, ValueError)):
             sq.ModelCall([b])
     assert (sys.getrefcount(sparse), sys.getrefcount(b.scales), sys.getrefcount(b.w)) == before
+
+
+def test_an_extension_with_another_layout_is_not_used():
+    built = binding._native(types.SimpleNamespace(layout=None, fill=None))
+    assert built is None and binding._native(None) is None
+    assert binding._native(types.SimpleNamespace(fill=None)) is None   # built before it told its layout
+    if binding._marshal is not None:
+        layout = binding._marshal.layout
+        assert binding._native(types.SimpleNamespace(layout=layout)) is not None
+        for i in range(len(layout)):   # a field elsewhere, another size
+            other = layout[:i] + (layout[i] + 8,) + layout[i + 1:]
+            assert binding._native(types.SimpleNamespace(layout=other)) is None
