@@ -24,6 +24,11 @@ def run_gpu(ws, bits, mode, flags=sq.FLAG_NARROW_RANGE):
     return bufs
 
 
+def assert_kernels(bufs, kernels, **kw):
+    """The kernels that take these layers, so that a test cannot miss the one it is about."""
+    assert sq.squant_plan_kernels(bufs, **kw) == kernels
+
+
 def assert_layer_equal(b, w, bits, mode, flags=oracle.FLAG_NARROW_RANGE, tag=""):
     r = oracle.quantize_layer(w, bits=bits, mode=mode, flags=flags)
     codes = b.codes.cpu().numpy()
@@ -112,16 +117,16 @@ def test_kernels_the_fast_selection_hands_back(bits):
 
 
 @pytest.mark.parametrize("bits,mode", [(4, EKC), (8, EKC), (3, EK)])
-def test_long_3x3_channels_pipelined_kernel(bits, mode):
-    """Layers of long 3x3 channels (more than 8192 weights each) take the streaming kernel (int8 codes only;
-    the pipelined kernel when packed or dequantized outputs are wanted, see the tests of those): several
+def test_long_3x3_channels_streaming_kernel(bits, mode):
+    """Layers of long 3x3 channels (1184 to 2048 input channels) take the streaming kernel: several
     such layers of different widths in one launch (one, a few and many more channels than the GPU
-    has multiprocessors), next to layers that stay with the grouped kernel, with special channels
+    has multiprocessors), next to layers that stay with other kernels, with special channels
     (zero, single non-zero, constant, scales far outside the reciprocal's range, ties)."""
-    shapes = [(1, 2048, 3, 3), (5, 1024, 3, 3), (333, 1000, 3, 3), (7, 1400, 3, 3), (40, 2048, 3, 3),
-              (9, 912, 3, 3), (6, 2044, 3, 3), (3, 2052, 3, 3), (4, 512, 3, 3), (11, 4100, 1, 1)]
+    shapes = [(1, 2048, 3, 3), (5, 1184, 3, 3), (333, 1200, 3, 3), (7, 1400, 3, 3), (40, 2048, 3, 3),
+              (9, 1188, 3, 3), (6, 2044, 3, 3), (3, 2052, 3, 3), (4, 512, 3, 3), (33, 1000, 3, 3), (7, 1180, 3, 3), (11, 9100, 1, 1)]
     ws = [adversarial_layer(s, seed=100 * bits + i) for i, s in enumerate(shapes)]
     bufs = run_gpu(ws, bits, mode)
+    assert_kernels(bufs, 7 * ["stream"] + 4 * ["grouped"] + ["row"], bits=bits, mode=mode)
     for i, (b, w) in enumerate(zip(bufs, ws)):
         assert_layer_equal(b, w, bits, mode, tag=f"shape{shapes[i]} mode{mode}")
     # the same buffers again: the work counter of the launch plan starts clean every time
@@ -142,9 +147,9 @@ def test_random_mixed_launches():
         for _ in range(int(rng.integers(1, 7))):
             kind = rng.integers(0, 4)
             if kind == 0:
-                shapes.append((int(rng.integers(1, 400)), int(rng.integers(228, 513)) * 4, 3, 3))
+                shapes.append((int(rng.integers(1, 400)), int(rng.integers(296, 513)) * 4, 3, 3))
             elif kind == 1:
-                shapes.append((int(rng.integers(1, 40)), int(rng.integers(1, 228)) * 4, 3, 3))
+                shapes.append((int(rng.integers(1, 40)), int(rng.integers(1, 296)) * 4, 3, 3))
             elif kind == 2:
                 shapes.append((int(rng.integers(1, 60)), int(rng.integers(1, 3000)), 1, 1))
             else:
@@ -249,10 +254,11 @@ def test_more_layers_than_one_launch_table_holds():
 
 def test_more_long_channel_layers_than_one_launch_table_holds():
     """The same for the streaming kernel: 101 layers of long 3x3 channels, two launches."""
-    shapes = [(1 + (i % 3), 912 + 4 * (i % 11), 3, 3) for i in range(101)]
+    shapes = [(1 + (i % 3), 1184 + 4 * (i % 11), 3, 3) for i in range(101)]
     ws = [W.random_layer(s, seed=3000 + i) for i, s in enumerate(shapes)]
     n0 = sq.squant_launch_count()
     bufs = run_gpu(ws, 4, EKC)
+    assert_kernels(bufs, 101 * ["stream"])
     assert sq.squant_launch_count() == n0 + 2
     for i, (b, w) in enumerate(zip(bufs, ws)):
         assert_layer_equal(b, w, 4, EKC, tag=f"layer {i} {shapes[i]}")
@@ -261,7 +267,7 @@ def test_more_long_channel_layers_than_one_launch_table_holds():
 def test_non_finite_inputs_do_not_disturb_other_channels():
     """NaN / Inf weights are outside the method's domain; their channels produce unspecified
     codes, but every index the kernel forms stays in bounds and finite channels are unaffected."""
-    for shape in [(8, 64, 3, 3), (8, 256, 1, 1), (8, 10, 5, 5), (8, 2048, 3, 3), (8, 1000, 3, 3), (300, 1024, 3, 3)]:
+    for shape in [(8, 64, 3, 3), (8, 256, 1, 1), (8, 10, 5, 5), (8, 2048, 3, 3), (8, 1000, 3, 3), (8, 1200, 3, 3), (300, 1184, 3, 3)]:
         w = W.random_layer(shape, seed=77)
         bad = w.copy()
         bad[1].reshape(-1)[3] = np.nan
@@ -296,25 +302,25 @@ def test_packed_int4_output(bits):
         sq.squant_quantize_model(bufs[:1], bits=8, flags=flags)
 
 
-@pytest.mark.parametrize("k", [1, 9])
-def test_boundary_bin_between_list_and_radix_capacity(k):
-    """SQuant-C boundary bins of every size class: taken whole, ranked from the short list
-    (<= 128 members), and the radix-select fallback (129..256 and thousands of tied members)."""
+@pytest.mark.parametrize("k,n,kernel", [(1, 1024, "grouped"), (9, 1024, "grouped"), (9, 1184, "stream"), (1, 9000, "row")])
+def test_boundary_bin_between_list_and_radix_capacity(k, n, kernel):
+    """Ties at the boundary of SQuant-C of every size class: taken whole, ranked from the short list (the
+    streaming kernel's holds 128 members), settled digit by digit or by counting beyond that."""
     for members in (40, 128, 129, 200, 256, 257, 700):
-        n = 1024
         w = np.zeros((2, n, k), dtype=np.float32)
         w[:, 0, 0] = 127.0                         # scale 1 with bits = 8
         w[:, 1:51, 0] = 0.45                       # 50 candidates at -0.45: taken whole
         w[:, 51:51 + members, 0] = 0.30            # `members` tied candidates at -0.30: boundary bin
         w[1] = -w[1]
         (b,) = run_gpu([w.reshape(2, n, 3, 3) if k == 9 else w.reshape(2, n, 1, 1)], 8, EKC)
+        assert_kernels([b], [kernel], bits=8)
         assert_layer_equal(b, w.reshape(2, n, 3, 3) if k == 9 else w.reshape(2, n, 1, 1), 8, EKC, tag=f"members {members}")
 
 
 def test_dequantized_output():
     """Optional outputs code * s (what Algorithm 1 returns) in fp32 and bfloat16, all paths - the
-    pipelined kernel for the long 3x3 channels included -, aligned and not, with int8 and packed codes."""
-    shapes = [(6, 64, 3, 3), (3, 2048, 3, 3), (150, 1000, 3, 3), (5, 256, 1, 1), (7, 33, 1, 1), (4, 3, 5, 5), (3, 7, 3, 3)]
+    streaming kernel for the long 3x3 channels included -, aligned and not, with int8 and packed codes."""
+    shapes = [(6, 64, 3, 3), (3, 2048, 3, 3), (160, 1200, 3, 3), (15, 1000, 3, 3), (5, 256, 1, 1), (7, 33, 1, 1), (4, 3, 5, 5), (3, 7, 3, 3)]
     ws = [adversarial_layer(s, seed=40 + i) for i, s in enumerate(shapes)]
     for flags, pack in ((sq.FLAG_NARROW_RANGE, False), (sq.FLAG_NARROW_RANGE | sq.FLAG_PACK_INT4, True)):
         bufs = [sq.alloc_outputs(torch.from_numpy(w).cuda(), dequant=True, pack_int4=pack, dequant_bf16=True) for w in ws]
@@ -364,13 +370,14 @@ def test_host_entry_point_several_chunks_against_the_checker():
 
 
 def test_one_call_three_kernels():
-    """One call whose layers go to three kernels: long 3x3 channels with plain codes (streaming kernel), long 3x3
-    channels with a dequantized output (pipelined kernel), short layers (grouped kernel); three launches per
+    """One call whose layers go to three kernels: long 3x3 channels with plain codes (streaming kernel), the same
+    with a dequantized output (its variant with further outputs), short layers (grouped kernel); three launches per
     call, every output compared with the checker, repeated (cached plans, work counters, scratch area)."""
-    shapes = [(300, 1024, 3, 3), (200, 2048, 3, 3), (64, 64, 3, 3), (100, 512, 1, 1), (37, 1400, 3, 3)]
+    shapes = [(300, 1200, 3, 3), (200, 2048, 3, 3), (64, 64, 3, 3), (100, 512, 1, 1), (37, 1400, 3, 3)]
     ws = [adversarial_layer(s, seed=31 + i) for i, s in enumerate(shapes)]
     for bits in (4, 8):
         bufs = [sq.alloc_outputs(torch.from_numpy(w).cuda(), dequant=(i in (1, 4)), dequant_bf16=(i == 4)) for i, w in enumerate(ws)]
+        assert_kernels(bufs, ["stream", "stream", "grouped", "grouped", "stream"], bits=bits)
         count0 = sq.squant_launch_count()
         for rep in range(3):
             for b in bufs:
@@ -386,12 +393,12 @@ def test_one_call_three_kernels():
         assert sq.squant_launch_count() - count0 == 9
 
 
-@pytest.mark.parametrize("n", [2048, 1500, 1028])
+@pytest.mark.parametrize("n", [2048, 1500, 1184, 1028])
 def test_streaming_kernel_hundreds_of_channel_flips(n):
     """Long 3x3 channels whose kernel sums all lean the same way: SQuant-C flips hundreds of kernels per
     channel, with candidates spread over many histogram bins - far more threads are concerned than the
     streaming kernel's queue holds (the rest do their own flips), and the boundary bin is ranked from the
-    list.  Weights sit on the 4-bit grid of scale 1/8 except one element per kernel, which is off the grid
+    list.  (1028 input channels: the grouped kernel.)  Weights sit on the 4-bit grid of scale 1/8 except one element per kernel, which is off the grid
     by 0.25 .. 0.49 of a step (downwards in the odd channels)."""
     rng = np.random.default_rng(n)
     m = 6
@@ -404,6 +411,7 @@ def test_streaming_kernel_hundreds_of_channel_flips(n):
     w[:, 0, 0] = 0.875   # absmax: scale 1/8 at 4 bit
     w = w.reshape(m, n, 3, 3)
     (b,) = run_gpu([w], 4, EKC)
+    assert_kernels([b], ["stream" if n >= 1184 else "grouped"])
     assert_layer_equal(b, w, 4, EKC, tag=f"n {n}")
     r = oracle.quantize_layer(w, bits=4, mode=EKC)
     flips = int(np.abs(np.rint((oracle.quantize_layer(w, bits=4, mode=EK).kernel_err.astype(np.float64).sum(axis=1)))).min())
@@ -412,14 +420,15 @@ def test_streaming_kernel_hundreds_of_channel_flips(n):
 
 
 @pytest.mark.parametrize("bits,flags", [(2, sq.FLAG_NARROW_RANGE), (6, sq.FLAG_NARROW_RANGE), (4, 0), (8, 0)])
-def test_pipelined_kernel_optional_outputs_and_ranges(bits, flags):
+def test_streaming_kernel_optional_outputs_and_ranges(bits, flags):
     """Long 3x3 channels (streaming kernel) without the optional outputs, at 2 and 6 bit, and
     without the narrow-range flag; one table holds a layer with fewer channels than the GPU has
     multiprocessors and one with many more."""
-    shapes = [(9, 1024, 3, 3), (700, 912, 3, 3), (33, 2048, 3, 3)]
+    shapes = [(9, 1188, 3, 3), (700, 1184, 3, 3), (33, 2048, 3, 3)]
     ws = [adversarial_layer(s, seed=50 * bits + i) for i, s in enumerate(shapes)]
     for variant in range(3):   # all outputs, no kernel sums, no sums at all
         bufs = [sq.alloc_outputs(torch.from_numpy(w).cuda(), kernel_err=variant == 0, channel_err=variant <= 1) for w in ws]
+        assert_kernels(bufs, 3 * ["stream"], bits=bits, flags=flags)
         for b in bufs:
             b.codes.fill_(-128)
         sq.squant_quantize_model(bufs, bits=bits, mode=EKC, flags=flags)
@@ -437,10 +446,11 @@ def test_pipelined_kernel_optional_outputs_and_ranges(bits, flags):
 def test_overlapping_calls_with_different_descriptors():
     """Calls with different descriptors may overlap on the GPU: two models (both with layers for
     the streaming kernel, each with its own work counter and scratch area) on two streams, several rounds."""
-    wa = [W.random_layer((200, 1024, 3, 3), seed=61), W.random_layer((50, 64, 3, 3), seed=62)]
-    wb = [W.random_layer((300, 912, 3, 3), seed=63), W.random_layer((64, 300, 1, 1), seed=64)]
+    wa = [W.random_layer((200, 1200, 3, 3), seed=61), W.random_layer((50, 64, 3, 3), seed=62)]
+    wb = [W.random_layer((300, 1184, 3, 3), seed=63), W.random_layer((64, 300, 1, 1), seed=64)]
     ba = [sq.alloc_outputs(torch.from_numpy(w).cuda()) for w in wa]
     bb = [sq.alloc_outputs(torch.from_numpy(w).cuda()) for w in wb]
+    assert_kernels(ba + bb, ["stream", "grouped", "stream", "grouped"])
     s1, s2 = torch.cuda.Stream(), torch.cuda.Stream()
     torch.cuda.synchronize()
     for _ in range(5):
@@ -474,9 +484,9 @@ def _clip_scales(w, bits, lo=1.5, hi=4.0, seed=0):
 def test_caller_supplied_scales(bits, flags):
     """Algorithm 1 with its scale as an input: the clip of Sec. 2.2 fires, clipped elements are
     never flipped outward and kernels / channels can run out of candidates.  All kernel sizes, long
-    3x3 channels included (they leave the persistent kernels), modes E, E|K, E|K|C and E|C on 1x1."""
+    3x3 channels included (they leave the streaming kernel), modes E, E|K, E|K|C and E|C on 1x1."""
     shapes = [(12, 64, 3, 3), (9, 7, 3, 3), (10, 300, 1, 1), (6, 2049, 1, 1), (8, 5, 5, 5), (16, 1, 3, 3), (5, 3, 7, 7),
-              (4, 1024, 3, 3), (3, 33, 2, 2)]
+              (4, 1200, 3, 3), (3, 33, 2, 2)]
     ws = [W.random_layer(s, seed=300 + i) for i, s in enumerate(shapes)]
     scs = [_clip_scales(w, bits, seed=i) for i, w in enumerate(ws)]
     for mode in (EKC, EK, E):
@@ -550,8 +560,16 @@ def test_failure_path_status_word_and_expiring_wait():
         sq.squant_device_status()
     assert ei.value.code == -10
     sq.squant_device_status()
-    w = W.random_layer((40, 1024, 3, 3), seed=12)      # streaming kernel: its work counters were reset with the status
+    w = W.random_layer((200, 1200, 3, 3), seed=12)     # streaming kernel: its work counters are reset with the status
     (b,) = run_gpu([w], 4, EKC)
+    assert_kernels([b], ["stream"])
+    assert_layer_equal(b, w, 4, EKC)
+    sq.squant_debug_set_status(1)
+    with pytest.raises(sq.SquantError):
+        sq.squant_device_status()
+    b.codes.fill_(-128)
+    sq.squant_quantize_model([b], bits=4)
+    sq.squant_device_status()
     assert_layer_equal(b, w, 4, EKC)
 
 
@@ -615,8 +633,8 @@ def test_channels_wider_than_one_thread_block():
 
 
 def test_checked_build_finds_no_violation_on_small_cases():
-    """The checked build of the library (every shared-memory / table index verified, each 3x3
-    channel's error sum taken a second time from its final codes by plain division) runs the
+    """The checked build of the library (shared-memory and table indexes verified, the error sums of
+    the grouped and row kernels taken a second time from the final codes by plain division) runs the
     sweep of small shapes, the 3x3 cases the fast selection hands back, long 3x3 channels through the
     streaming kernel, and a cluster case: no check fails, and its results are the regular build's."""
     from paper_2202_07471_b200 import build as lib_build
@@ -625,8 +643,9 @@ def test_checked_build_finds_no_violation_on_small_cases():
         pytest.skip("libsquant_debug.so has not been built")
     ws = [adversarial_layer(s, seed=9 + i) for i, s in enumerate(SWEEP_SHAPES)] + [redo_layer(64, 4, seed=4), redo_layer(2048, 4)]
     # long 3x3 channels (streaming kernel): special channels, heavy ties (digit-by-digit selection), a partial last warp
-    ws += [adversarial_layer((150, 1000, 3, 3), seed=77), coarse(W.random_layer((5, 2048, 3, 3), seed=78), steps=24, div=4)]
+    ws += [adversarial_layer((150, 1200, 3, 3), seed=77), adversarial_layer((15, 1000, 3, 3), seed=79), coarse(W.random_layer((5, 2048, 3, 3), seed=78), steps=24, div=4)]
     ref = run_gpu(ws, 4, EKC)
+    assert_kernels(ref[-3:], ["stream", "grouped", "stream"])
     sq.use_library(lib_build.LIB_DEBUG)
     try:
         checked, n, site = sq.squant_debug_violations()
