@@ -198,8 +198,8 @@ int squant_plan_kernels(const squant_layer *layers, int32_t n_layers, const squa
  *   layer, opt, cuda_stream   as for squant_quantize_layer; DEVICE pointers, caller-owned
  *
  * Limits: one layer per call, and the layer's launch must need at most SQUANT_NOALLOC_MAX_CTAS
- * thread blocks (one block handles 256/g output channels, g = 32..256 threads per channel by
- * channel length; squant_plan_info reports the count).  A larger layer is rejected with
+ * thread blocks (one block handles 256/g output channels, g = 8..256 threads per channel by
+ * channel length, 256 depthwise channels; squant_plan_info reports the count).  A larger layer is rejected with
  * SQUANT_ERR_LIMIT before anything is launched; split it by output-channel range and call once
  * per part.
  *

@@ -30,8 +30,8 @@ constexpr int64_t kMaxChannelElems = 65535; // one-CTA paths: keeps the clamp-ed
 constexpr int64_t kMaxKernels = (1 << sq::kIdxBits) - 1;   // kernels per channel: the select keys hold 18 index bits
 constexpr size_t kMaxPlans = 64;
 constexpr int kLongChannel = 8192;           // weights: longer channels are launched apart from the others
-constexpr int kWideSmemGoal = 112 << 10;     // the same of a cluster's thread block: two of them
 constexpr int kGroupedSmemGoal = 55 << 10;   // shared memory of a grouped CTA with which four of them share a multiprocessor
+constexpr int kWideSmemGoal = 112 << 10;     // the same of a cluster's thread block: two of them
 
 std::mutex g_mutex;
 std::atomic<int64_t> g_launches{0};
@@ -356,10 +356,16 @@ struct ParamPlan {
 };
 
 // Layers the streaming kernel takes: 3x3 channels so long that no four CTAs of the grouped kernel fit a
-// multiprocessor (from 1184 input channels on: 2048 channels take 42.4 us in the grouped kernel and 59.8 us
-// in this one at N = 1028, 46.5 and 52.7 us at 1152, 55.0 and 53.1 us at 1280, 89.0 and 57.5 us at 2048; with
-// packed codes 44 and 59, 58 and 60, 94 and 68 us at 1028, 1280, 2048), input channels a multiple of four and one quad of kernels per
+// multiprocessor (1184 input channels on), input channels a multiple of four and one quad of kernels per
 // quantizer thread, SQuant-K on, absmax scales, and its buffers fit the shared memory of one SM.
+// Grouped / streaming kernel in us, cold and with the events' own time, at 1152, 1184, 1280, 1408 and 2048 input channels:
+//   2048 output channels, plain codes   56 / 60, 58 / 60, 67 / 60, 71 / 63, 99 / 69
+//                         packed codes          60 / 69, 69 / 71, 74 / 70, 106 / 79
+//                         bf16 output           68 / 78, 75 / 78, 81 / 79, 118 / 89
+//   512 output channels,  plain codes   25 / 28, 25 / 27, 32 / 28, 34 / 28, 40 / 32
+//                         packed codes          28 / 30, 32 / 32, 33 / 31, 42 / 36
+//   148 output channels   plain codes   19 / 17, 20 / 17, 20 / 17, 20 / 20, 22 / 20
+// (with further outputs both kernels are even at about 1350; the line is the plain codes').
 bool stream_eligible(const squant_layer &l, const LayerDesc &d, const squant_options &o, int max_smem)
 {
     if (d.K != 9 || (d.N & 3) != 0 || sq::conv_bytes(sq::kCtaThreads, d.NK, d.K) <= kGroupedSmemGoal) return false;
@@ -472,7 +478,7 @@ int build_param_plan(const squant_layer *layers, int32_t n_layers, const squant_
     }
     // A launch whose warps do not fill the GPU takes the time of one channel, so its channels get twice or
     // four times the threads (up to 32 warps per multiprocessor for 1x1 rows: 3531 rows of 461 weights
-    // 27.0 -> 17.2 us, MobileNetV2 shapes at half width 12.3 -> 7.8; half as many for larger kernels: 256x256x3x3
+    // 27.0 -> 17.4 us, MobileNetV2 shapes at half width 12.3 -> 8.0; half as many for larger kernels: 256x256x3x3
     // 7.3 -> 6.4, whereas 512x512x3x3 is slower with twice the threads, 10.5 against 9.4 us).
     int64_t warps = 0;
     for (int i : order) warps += (static_cast<int64_t>(descs[i].M) * descs[i].g + 31) / 32;

@@ -1,10 +1,12 @@
 // Device code of the SQuant solver for sm_100a.
 //
-// One cooperative thread group (a warp, or 64..512 threads joined by a named barrier) owns one
-// output channel: it stages the channel's N*K weights in shared memory while taking their
-// absmax, then every thread quantizes whole kernels (SQuant-E, SQuant-K and the candidate of
-// Algorithm 3 are thread-local), and the group finishes with the channel step (SQuant-C): an
-// exact integer sum and a radix select over the kernels' candidate keys.
+// One cooperative thread group (8 to 256 threads of a thread block in the grouped kernel, a whole thread block
+// or a cluster in the kernels for longer channels) owns one output channel: it brings the channel's N*K
+// weights to shared memory and takes their absmax, then every thread quantizes whole kernels (SQuant-E,
+// SQuant-K and the candidate of Algorithm 3 are thread-local), and the group finishes with the channel step
+// (SQuant-C): an exact integer sum and the choice of the largest candidates.  Here: the steps that the
+// kernels share, the bodies for staged channels (E|C on larger kernels, the longest 1x1 rows), depthwise
+// channels, and the grouped kernel.
 //
 // All decisions after the fp32 division are integer arithmetic on perturbations in units of
 // 2^-30, so the result does not depend on how the work is split over threads.
@@ -33,7 +35,7 @@ struct LayerDesc {
     const float *sin;     // caller-supplied scales, or null: absmax scales
     uint16_t *deq16;      // bfloat16 code * s, or null
     int32_t M, N, K, NK;
-    int32_t g;            // threads per channel group: 32, 64, 128 or 256
+    int32_t g;            // threads per channel: a power of two, 8 to 256 (1: depthwise)
     int32_t g_shift;      // log2(g)
     int32_t slice_bytes;  // shared memory per group
     int32_t off_codes, off_ev, off_vv, off_vi, off_hist, off_red;   // 1x1 layers (off_hist = 0): off_vi = vectors of a row
