@@ -30,6 +30,7 @@ constexpr int64_t kMaxChannelElems = 65535; // one-CTA paths: keeps the clamp-ed
 constexpr int64_t kMaxKernels = (1 << sq::kIdxBits) - 1;   // kernels per channel: the select keys hold 18 index bits
 constexpr size_t kMaxPlans = 64;
 constexpr int kLongChannel = 8192;           // weights: longer channels are launched apart from the others
+constexpr int kStreamKernels = 1184;         // 3x3 channels of at least as many kernels go to the streaming kernel (stream_eligible)
 constexpr int kGroupedSmemGoal = 55 << 10;   // shared memory of a grouped CTA with which four of them share a multiprocessor
 constexpr int kWideSmemGoal = 112 << 10;     // the same of a cluster's thread block: two of them
 
@@ -127,6 +128,13 @@ void layout_staged(const squant_layer &l, LayerDesc &d, unsigned mode)
     d.off_hist = off; off += 4 * sq::kHistBins;
     d.off_red = off; off += 256;
     d.slice_bytes = off;
+}
+
+// 1x1: every row of weights, error sums and codes starts on a vector.
+int regular_rows(const LayerDesc &d)
+{
+    return (d.N & 3) == 0 && (reinterpret_cast<uintptr_t>(d.w) & 15) == 0 && (reinterpret_cast<uintptr_t>(d.kerr) & 15) == 0 &&
+           (reinterpret_cast<uintptr_t>(d.codes) & 3) == 0;
 }
 
 // Device-side descriptor of one layer: group size and the layout of a group's shared-memory
@@ -339,8 +347,8 @@ struct ParamPlan {
     struct Wide { LayerDesc d; int cluster, kpc, smem; };
     std::vector<Wide> wide;
     // row kernel (1x1 rows too long for a group): one item per output channel
-    std::vector<sq::LaunchTable> row_tables;
-    std::vector<int> row_grids, row_smem;
+    struct Rows { sq::LaunchTable table; int grid, threads, smem; };
+    std::vector<Rows> rows;
     // streaming kernel (layers of long 3x3 channels): one item per output channel
     struct Stream {
         sq::LaunchTable table;
@@ -356,7 +364,7 @@ struct ParamPlan {
 };
 
 // Layers the streaming kernel takes: 3x3 channels so long that no four CTAs of the grouped kernel fit a
-// multiprocessor (1184 input channels on), input channels a multiple of four and one quad of kernels per
+// multiprocessor (kStreamKernels input channels on), input channels a multiple of four and one quad of kernels per
 // quantizer thread, SQuant-K on, absmax scales, and its buffers fit the shared memory of one SM.
 // Grouped / streaming kernel in us, cold and with the events' own time, at 1152, 1184, 1280, 1408 and 2048 input channels:
 //   2048 output channels, plain codes   56 / 60, 58 / 60, 67 / 60, 71 / 63, 99 / 69
@@ -368,7 +376,7 @@ struct ParamPlan {
 // (with further outputs both kernels are even at about 1350; the line is the plain codes').
 bool stream_eligible(const squant_layer &l, const LayerDesc &d, const squant_options &o, int max_smem)
 {
-    if (d.K != 9 || (d.N & 3) != 0 || sq::conv_bytes(sq::kCtaThreads, d.NK, d.K) <= kGroupedSmemGoal) return false;
+    if (d.K != 9 || (d.N & 3) != 0 || d.N < kStreamKernels) return false;
     if (!(o.mode & SQUANT_MODE_K) || l.scales_in) return false;
     if ((reinterpret_cast<uintptr_t>(l.w) & 15) || (reinterpret_cast<uintptr_t>(l.codes) & 15)) return false;
     if (d.N > 4 * sq::kStreamQuantThreads) return false;
@@ -401,6 +409,7 @@ int build_param_plan(const squant_layer *layers, int32_t n_layers, const squant_
     p.qmax = (1 << (o.bits - 1)) - 1;
     p.mode = o.mode | ((o.flags & SQUANT_FLAG_PACK_INT4) ? sq::kModePackInt4 : 0u) |
              ((o.flags & SQUANT_FLAG_NARROW_RANGE) ? 0u : sq::kModeWideRange);
+    const bool pack = (o.flags & SQUANT_FLAG_PACK_INT4) != 0;
     std::vector<LayerDesc> descs(n_layers);
     std::vector<int> order, streamed[2], rows;
     for (int i = 0; i < n_layers; ++i) {
@@ -420,13 +429,14 @@ int build_param_plan(const squant_layer *layers, int32_t n_layers, const squant_
                 for (int c = 2; c <= sq::kWideMaxCluster && !w.cluster; c *= 2) {
                     const int unit = descs[i].K == 1 ? 4 : 2;
                     const int kpc = ((descs[i].N + c - 1) / c + unit - 1) / unit * unit;
-                    const int64_t bytes = sq::wide_bytes(kpc, descs[i].K);
+                    const int64_t bytes = sq::wide_bytes(kpc, descs[i].K, pack);
                     if (bytes <= goal) { w.cluster = c; w.kpc = kpc; w.smem = static_cast<int>(bytes); }
                 }
                 if (w.cluster || goal == max_smem) break;
             }
             if (!w.cluster) return SQUANT_ERR_TOO_WIDE;
             w.d.off_vi = (w.kpc + 6) >> 2;
+            w.d.off_ev = regular_rows(w.d);
             p.wide.push_back(w);
             if (kernels) kernels[i] = SQUANT_KERNEL_CLUSTER;
             continue;
@@ -447,17 +457,23 @@ int build_param_plan(const squant_layer *layers, int32_t n_layers, const squant_
     }
     // long rows, longest first: a thread block per output channel
     std::stable_sort(rows.begin(), rows.end(), [&](int a, int b) { return descs[a].N > descs[b].N; });
-    for (size_t base = 0; base < rows.size(); base += sq::kMaxParamLayers) {
-        const int n = static_cast<int>(std::min<size_t>(rows.size() - base, sq::kMaxParamLayers));
+    for (size_t base = 0; base < rows.size();) {
+        const bool small = descs[rows[base]].N <= sq::kRowSmallElems;
+        size_t n = 0;
         int smem = 0;
-        for (int j = 0; j < n; ++j) {
-            LayerDesc &d = descs[rows[base + j]];
+        while (base + n < rows.size() && n < sq::kMaxParamLayers && (descs[rows[base + n]].N <= sq::kRowSmallElems) == small) {
+            LayerDesc &d = descs[rows[base + n]];
             d.off_vi = (d.N + 6) >> 2;
-            smem = std::max(smem, sq::row_bytes(sq::kBlockThreads, d.off_vi, sq::kBlock));
+            d.off_ev = regular_rows(d);
+            smem = std::max(smem, sq::long_row_bytes(small ? 256 : 512, d.off_vi, pack, sq::kBlock));
+            ++n;
         }
-        p.row_tables.emplace_back();
-        p.row_grids.push_back(fill_table(p.row_tables.back(), descs, rows.data() + base, n, false));
-        p.row_smem.push_back(smem);
+        p.rows.emplace_back();
+        ParamPlan::Rows &r = p.rows.back();
+        r.grid = fill_table(r.table, descs, rows.data() + base, static_cast<int>(n), false);
+        r.threads = small ? 256 : 512;
+        r.smem = smem;
+        base += n;
     }
     for (int kind = 1; kind >= 0; --kind) {
         const std::vector<int> &list = streamed[kind];
@@ -547,7 +563,9 @@ int device_smem_limit(int device, int &limit)
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, v));
         SQ_CUDA(cudaFuncSetAttribute(sq::squant_table_kernel,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, v));
-        SQ_CUDA(cudaFuncSetAttribute(sq::squant_row_kernel,
+        SQ_CUDA(cudaFuncSetAttribute(sq::squant_row_kernel<256>,
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, v));
+        SQ_CUDA(cudaFuncSetAttribute(sq::squant_row_kernel<512>,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, v));
         SQ_CUDA(cudaFuncSetAttribute(sq::squant_wide_kernel,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, v));
@@ -625,8 +643,9 @@ int launch_plan(const ParamPlan &p, cudaStream_t stream)
         SQ_CUDA(cudaGetLastError());
         g_launches.fetch_add(1, std::memory_order_relaxed);
     }
-    for (size_t c = 0; c < p.row_tables.size(); ++c) {
-        sq::squant_row_kernel<<<p.row_grids[c], sq::kBlockThreads, p.row_smem[c], stream>>>(p.row_tables[c], p.qmax, p.mode);
+    for (const ParamPlan::Rows &r : p.rows) {
+        if (r.threads == 256) sq::squant_row_kernel<256><<<r.grid, 256, r.smem, stream>>>(r.table, p.qmax, p.mode);
+        else sq::squant_row_kernel<512><<<r.grid, 512, r.smem, stream>>>(r.table, p.qmax, p.mode);
         SQ_CUDA(cudaGetLastError());
         g_launches.fetch_add(1, std::memory_order_relaxed);
     }

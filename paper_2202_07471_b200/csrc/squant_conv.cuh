@@ -135,8 +135,10 @@ __device__ __forceinline__ void emit_codes(const LayerDesc &L, size_t first, siz
         unsigned char *row = reinterpret_cast<unsigned char *>(L.codes) + first;
         const int head = min(static_cast<int>((16 - (reinterpret_cast<uintptr_t>(row) & 15)) & 15), n);
         const int nv = (n - head) >> 4, tail = head + 16 * nv;
+#pragma unroll 1
         for (int i = G.t; i < nv; i += G.g)
             __stcs(reinterpret_cast<int4 *>(row + head) + i, reinterpret_cast<const int4 *>(cel + head)[i]);
+#pragma unroll 1
         for (int i = G.t; i < head + (n - tail); i += G.g) {
             const int e = i < head ? i : tail + i - head;
             SQ_DBG(tail <= n && e >= 0 && e < n, 17);
@@ -147,6 +149,7 @@ __device__ __forceinline__ void emit_codes(const LayerDesc &L, size_t first, siz
         // eight codes at a time where the packed row is aligned, the rest byte by byte
         const int head = min(static_cast<int>((4 - (reinterpret_cast<uintptr_t>(row) & 3)) & 3), n >> 1);   // packed bytes
         const int nv = ((n >> 1) - head) >> 2, tail = head + 4 * nv;
+#pragma unroll 1
         for (int i = G.t; i < nv; i += G.g) {
             const unsigned char *c = cel + 2 * (head + 4 * i);
             unsigned o = 0u;
@@ -154,6 +157,7 @@ __device__ __forceinline__ void emit_codes(const LayerDesc &L, size_t first, siz
             for (int k = 0; k < 8; ++k) o |= static_cast<unsigned>(c[k] & 15) << (4 * k);
             __stcs(reinterpret_cast<unsigned *>(row + head) + i, o);
         }
+#pragma unroll 1
         for (int i = G.t; i < head + ((n + 1) >> 1) - tail; i += G.g) {
             const int b = i < head ? i : tail + i - head;
             SQ_DBG(2 * tail <= n && b >= 0 && 2 * b < n, 18);
@@ -164,6 +168,7 @@ __device__ __forceinline__ void emit_codes(const LayerDesc &L, size_t first, siz
         float *row = L.deq + first;
         const Span sp(row, n, G.t);
         const bool words = ((reinterpret_cast<uintptr_t>(cel) - sp.r) & 3) == 0;
+#pragma unroll 1
         for (int q = sp.q_lo + G.t; q < sp.q_hi; q += G.g) {
             const unsigned char *c = cel + (4 * q - sp.r);
             SQ_DBG(4 * q - sp.r >= 0 && 4 * q - sp.r + 4 <= n, 19);
@@ -177,6 +182,7 @@ __device__ __forceinline__ void emit_codes(const LayerDesc &L, size_t first, siz
         const int head = min(static_cast<int>(((8 - (reinterpret_cast<uintptr_t>(row) & 7)) & 7) >> 1), n);
         const int nv = (n - head) >> 2, tail = head + 4 * nv;
         const bool words = (reinterpret_cast<uintptr_t>(cel + head) & 3) == 0;
+#pragma unroll 1
         for (int i = G.t; i < nv; i += G.g) {
             const unsigned char *c = cel + head + 4 * i;
             const unsigned c4 = words ? *reinterpret_cast<const unsigned *>(c) : c[0] | (c[1] << 8) | (c[2] << 16) | (static_cast<unsigned>(c[3]) << 24);
@@ -184,6 +190,7 @@ __device__ __forceinline__ void emit_codes(const LayerDesc &L, size_t first, siz
             const unsigned b2 = bf16_bits(row_deq(c4 >> 16, s)), b3 = bf16_bits(row_deq(c4 >> 24, s));
             __stcs(reinterpret_cast<uint2 *>(row + head) + i, make_uint2(b0 | (b1 << 16), b2 | (b3 << 16)));
         }
+#pragma unroll 1
         for (int i = G.t; i < head + (n - tail); i += G.g) {
             const int e = i < head ? i : tail + i - head;
             SQ_DBG(tail <= n && e >= 0 && e < n, 20);
@@ -203,11 +210,11 @@ __device__ __forceinline__ void conv_body(const LayerDesc &L, int m, const Group
 {
     const int g = G.g, N = kOwn == kCluster ? nloc : L.N, K = KT ? KT : L.K, NK = kOwn == kCluster ? nloc * K : L.NK;   // here
     const size_t first = static_cast<size_t>(m) * L.NK + static_cast<size_t>(n0) * K;   // of these elements in the layer
-    SelScratch *sc = reinterpret_cast<SelScratch *>(slice);
+    const Sel S(slice, g, kOwn, K);
     if (G.t == 0) {
-        sc->amax = 0u; sc->count = 0; sc->top = 0;
-        sc->total[0] = 0;
-        sc->sum64 = 0ull;
+        S.sc->count = 0;
+        S.sc->total[0] = 0;
+        S.sc->found[0] = 0;
     }
     // ---- stage the row, take its absmax (each thread over what it has copied itself)
     const float *wrow = L.w + first;
@@ -218,13 +225,14 @@ __device__ __forceinline__ void conv_body(const LayerDesc &L, int m, const Group
         float4 *buf = reinterpret_cast<float4 *>(slice + sel_bytes(g, kOwn, K));
         wel = reinterpret_cast<float *>(buf) + sp.r;
         const float4 *src = reinterpret_cast<const float4 *>(wrow - sp.r);
-#pragma unroll 2
-        for (int q = sp.q_lo + G.t; q < sp.q_hi; q += g) copy_async16(buf + q, src + q);
+        const int q0 = sp.q_lo + G.t, vecs = G.rounds(sp.q_lo, sp.q_hi);   // this thread's vectors: q0, q0 + g, ..
+#pragma unroll 4
+        for (int i = 0; i < vecs; ++i) copy_async16(buf + q0 + i * g, src + q0 + i * g);
         if (sp.rag >= 0) copy_async4(wel + sp.rag, wrow + sp.rag);
         copy_async_wait();
-#pragma unroll 2
-        for (int q = sp.q_lo + G.t; q < sp.q_hi; q += g) {
-            const float4 v = buf[q];
+#pragma unroll 4
+        for (int i = 0; i < vecs; ++i) {
+            const float4 v = buf[q0 + i * g];
             amax = absmax3(absmax3(amax, v.x, v.y), v.z, v.w);
         }
         if (sp.rag >= 0) amax = fmaxf(amax, fabsf(wel[sp.rag]));
@@ -237,27 +245,11 @@ __device__ __forceinline__ void conv_body(const LayerDesc &L, int m, const Group
     }
 
     // ---- scale
-    float s;
-    {
-        unsigned u = __reduce_max_sync(kFull, __float_as_uint(amax));   // >= 0: uint order = float order
-        G.sync();   // the scratch words are cleared, the staged weights are visible
-        if (g > 32) {
-            if ((G.t & 31) == 0) atomicMax(&sc->amax, u);
-            G.sync();
-            u = sc->amax;
-        }
-        if (kOwn == kCluster) {
-            cg::cluster_group cl = cg::this_cluster();
-            cl.sync();
-            const int lane = threadIdx.x & 31;
-            u = __reduce_max_sync(kFull, lane < static_cast<int>(cl.num_blocks()) ? remote(&sc->amax, lane) : 0u);
-        }
-        amax = __uint_as_float(u);
-        s = (amax < 0x1p-100f) ? 1.0f : __fdiv_rn(amax, static_cast<float>(qmax));
-        if (kClip && (kOwn != kCluster || L.sin)) {
-            s = L.sin[m];
-            if (!(s > 0.0f && s < __int_as_float(0x7f800000))) s = 1.0f;
-        }
+    amax = owner_absmax<kOwn>(G, amax, S);   // (its barrier: the staged weights are visible)
+    float s = absmax_scale(amax, qmax);
+    if (kClip && (kOwn != kCluster || L.sin)) {
+        s = L.sin[m];
+        if (!(s > 0.0f && s < __int_as_float(0x7f800000))) s = 1.0f;
     }
 
     // ---- SQuant-E, SQuant-K, candidates: one thread per kernel
@@ -393,20 +385,13 @@ __device__ __forceinline__ void conv_body(const LayerDesc &L, int m, const Group
 
     // ---- channel sum
     long long ec = 0;
+    int up = hi0, down = -lo0;   // the channel's extremes
     if ((mode & 4u) || L.cerr) {
-        for (int o = 16; o > 0; o >>= 1) esum += __shfl_xor_sync(kFull, esum, o);
-        if (g > 32) {
-            if ((G.t & 31) == 0) atomicAdd(&sc->sum64, static_cast<unsigned long long>(esum));
-            G.sync();
-            esum = static_cast<long long>(sc->sum64);
-            if (kOwn == kCluster) {
-                cg::cluster_group cl = cg::this_cluster();
-                cl.sync();
-                esum = 0;
-                for (int c = 0; c < static_cast<int>(cl.num_blocks()); ++c) esum += static_cast<long long>(remote(&sc->sum64, c));
-            }
+        if (kOwn != kCluster && g > 32) {   // the maxima that SQuant-C looks for its bound among
+            S.mx[G.t] = hi0;
+            S.mx[G.t + g] = -lo0;
         }
-        ec = esum;
+        ec = owner_sum<kOwn, kClip, true>(G, S, esum, static_cast<unsigned>(esum), static_cast<int>((esum + (1 << 16)) >> 17), up, down);
     }
 
     // ---- SQuant-C: Algorithm 2 on the channel, keys = the kernels' candidates
@@ -415,14 +400,36 @@ __device__ __forceinline__ void conv_body(const LayerDesc &L, int m, const Group
         const long long abs_e = ec > 0 ? ec : -ec;
         const int kc = static_cast<int>(min((abs_e + (kHalf - 1)) >> 30, 1ll << 30));   // a clipped channel's sum can be huge
         if (kc > 0) {   // uniform in the group
+            const int m0 = sgn > 0 ? hi0 : -lo0;
+            const int *mx = sgn > 0 ? S.mx : S.mx + g;
+            const int lane = threadIdx.x & 31;
+            auto count = [&](int t, int it) {
+                int c;
+                if (kOwn == kCluster) {
+                    c = __popc(__ballot_sync(kFull, m0 >= t));
+                    if (lane == 0) atomicAdd(&S.sc->found[it % 3], c);
+                    if (G.t == 0) S.sc->found[(it + 1) % 3] = 0;   // (last read before the previous round's barrier)
+                    return cluster_sum(&S.sc->found[it % 3]);
+                }
+                if (kOwn == kGroup && g <= 32) return __popc(__ballot_sync(kFull, m0 >= t));
+                c = 0;
+#pragma unroll 1
+                for (int i = lane; i < (g >> 2); i += 32) {
+                    const int4 q = reinterpret_cast<const int4 *>(mx)[i];
+                    c += (q.x >= t) + (q.y >= t) + (q.z >= t) + (q.w >= t);
+                }
+                return __reduce_add_sync(kFull, c);
+            };
             auto each = [&](int t, auto fn) {
-#pragma unroll 2
+                if (m0 < t) return;   // (m0: the thread's largest)
+#pragma unroll 1
                 for (int n = by_warp ? ((G.t & 31) ? N : G.t >> 5) : G.t; n < N; n += by_warp ? g >> 5 : g) {
                     const int a = reinterpret_cast<const int *>(wel)[n * K] * sgn;
                     if (a >= t) fn(a, n0 + n);
                 }
             };
-            auto flip = [&](int, int n_abs) {
+            auto listing = [&](int t, auto push) { each(t, [&](int a, int n) { push(a, n, 0u); }); };   // (positions are with the kernels)
+            auto flip = [&](int, int n_abs, unsigned) {
                 const int n = n_abs - n0;
                 const int *rec = reinterpret_cast<const int *>(wel + n * K);
                 const int idx = K > 2 ? rec[2] : rec[1] & 1;
@@ -431,27 +438,16 @@ __device__ __forceinline__ void conv_body(const LayerDesc &L, int m, const Group
                 *cb = static_cast<unsigned char>(*cb - sgn);
                 if (kerr) kerr[n] = __fmul_rn(__int2float_rn((K > 2 ? rec[1] : rec[1] >> 1) - sgn * kOne), 0x1p-30f);
             };
-            const int m0 = sgn > 0 ? hi0 : -lo0;
             // Over-SQuant candidates reach one, but few come near it: the search starts at the largest
-            int top = static_cast<int>(__reduce_max_sync(kFull, static_cast<unsigned>(m0)));
-            if (g > 32) {
-                if ((G.t & 31) == 0) atomicMax(&sc->top, top);
-                G.sync();
-                top = sc->top;
-                if (kOwn == kCluster) {
-                    cg::cluster_group cl = cg::this_cluster();
-                    cl.sync();
-                    const int lane = threadIdx.x & 31;
-                    top = __reduce_max_sync(kFull, lane < static_cast<int>(cl.num_blocks()) ? remote(&sc->top, lane) : 0);
-                }
-            }
-            const int k_eff = select_top<kOwn>(G, each, flip, m0, 0, top + 1, 3.0f, kc, L.N, true, sc, K);
+            const int top = (sgn > 0 ? up : down) + 1;
+            const int nmax = g * (kOwn == kCluster ? static_cast<int>(cg::this_cluster().num_blocks()) : 1);
+            const int k_eff = select_top<kOwn>(G, count, listing, [] {}, each, [](int) { return 0u; }, flip, nmax, top, top, 3.0f, kc, L.N, true, S, K);
             ec -= static_cast<long long>(sgn) * k_eff * kOne;
         }
     }
     G.sync();   // all codes are final
 #ifdef SQUANT_DEBUG_BOUNDS
-    if (!kClip && kOwn != kCluster && ((mode & 4u) || L.cerr)) debug_check_sum(G, wrow, cel, NK, s, ec, true, sc);
+    if (!kClip && kOwn != kCluster && ((mode & 4u) || L.cerr)) debug_check_sum(G, wrow, cel, NK, s, ec, true, S);
 #endif
 
     emit_codes(L, first, static_cast<size_t>(m) * ((L.NK + 1) >> 1) + ((static_cast<size_t>(n0) * K) >> 1), G, cel, NK, s, mode);

@@ -38,7 +38,8 @@ struct LayerDesc {
     int32_t g;            // threads per channel: a power of two, 8 to 256 (1: depthwise)
     int32_t g_shift;      // log2(g)
     int32_t slice_bytes;  // shared memory per group
-    int32_t off_codes, off_ev, off_vv, off_vi, off_hist, off_red;   // 1x1 layers (off_hist = 0): off_vi = vectors of a row
+    int32_t off_codes, off_ev, off_vv, off_vi, off_hist, off_red;   // 1x1 layers (off_hist = 0): off_vi = vectors of a row, off_ev = 1
+                                                                    // if every row of weights, codes and error sums starts on a vector
 };
 
 // One CTA: channels ch0 .. ch0 + 256/g - 1 of one layer, one per group.
@@ -61,11 +62,15 @@ struct LaunchTable {
 
 struct Group {
     int g;    // threads in the group
+    int sh;   // log2(g)
     int t;    // this thread's index inside the group
     int bar;  // named barrier of the group (groups wider than a warp)
+    // How many of the indices from + t, from + t + g, .. lie below `to` (0 or less: none).  (Loops over a channel count
+    // with this: left to itself the compiler divides by g wherever it unrolls one.)
+    __device__ __forceinline__ int rounds(int from, int to) const { return (to - from - t + g - 1) >> sh; }
     __device__ __forceinline__ void sync() const
     {
-        if (g <= 32) __syncwarp();   // groups of 8 and 16 threads share a warp and keep step with each other
+        if (g <= 32) __syncwarp();   // smaller groups share a warp and keep step with each other
         else asm volatile("bar.sync %0, %1;" ::"r"(bar), "r"(g) : "memory");
     }
 };
@@ -1326,6 +1331,7 @@ __device__ __forceinline__ void run_item(const LayerDesc &L, int ch0, unsigned c
     }
     Group G;
     G.g = L.g;
+    G.sh = L.g_shift;
     G.t = threadIdx.x & (L.g - 1);
     const int gi = threadIdx.x >> L.g_shift;
     G.bar = 1 + gi;

@@ -17,7 +17,9 @@
 //     the first k_c ranks are flipped.  What that cannot settle (k_c beyond the number of maxima, a
 //     full list) goes to an exact search over the 48-bit keys.
 // With squant_conv.cuh: ResNet-50 shapes 84.5 -> 65.6 us device time on a B200, 55 thread-instructions per weight;
-// five linear layers of 125 M weights at 8 bit 267 -> 252 us.
+// five linear layers of 125 M weights at 8 bit 267 -> 252 us.  With one barrier per reduction (a place for every warp
+// instead of shared atomics that have to be cleared first), loops counted without a division and the IEEE division out
+// of the SQuant-E loop: ResNet-50 shapes 70.5 -> 66.9 us a call, MobileNetV2 shapes 17.4 -> 16.7.
 #pragma once
 
 #include <cooperative_groups.h>
@@ -28,27 +30,34 @@ namespace sq {
 
 namespace cg = cooperative_groups;
 
-constexpr int kRowVecs = 8;                       // float4 a thread holds
+constexpr int kRowVecs = 8;                       // vectors of four weights a thread of a group takes
 
-// Threads per channel for rows of `vecs` vectors (8, 16, .. 256), 0: too long for one thread block.
+// Threads per channel for rows of `vecs` vectors (8, 16, .. 256), 0: too long for a group.
 __host__ __device__ inline int row_group(int vecs)
 {
-    int g = 8;
+    int g = 8;   // (six elements of a row can lie outside its vectors)
     while (g * kRowVecs < vecs) g *= 2;
     return g <= kCtaThreads ? g : 0;
 }
 
-// Control words of one group, followed by its list and, for groups wider than a warp, the threads'
-// maxima.
+// Control words of one group, followed (groups wider than a warp) by what its warps contribute to the channel's
+// reductions, then by its list and by the threads' maxima.
 struct SelScratch {
-    unsigned amax;             // absmax accumulator (bit pattern of a non-negative float)
-    unsigned sum;              // channel sum modulo 2^32
-    int approx;                // channel sum in units of 2^20
-    int count;                 // listed elements
-    int total[3];              // rotating counters of the exact search
-    int top;                   // largest candidate (larger kernels)
-    unsigned long long sum64;  // channel sum (supplied scales)
-    int found[2];              // rotating counters of the search over a cluster
+    int count;      // listed elements
+    int total[3];   // rotating counters of the exact search
+    int found[3];   // the same of the search over a cluster
+    int pad;
+};
+
+// What a warp contributes: absmax (bit pattern of a non-negative float) first, then error sum and extremes of the candidates.
+constexpr int kMaxWarps = 16;   // of a channel in one thread block
+struct WarpPart {
+    int lo32, hi32;   // the error sum: modulo 2^32 and, in units of 2^17, its size; or both halves of 64 bits
+    int up, down;     // largest candidate of each sign
+};
+struct SelWarps {
+    unsigned amax[kMaxWarps];
+    WarpPart part[kMaxWarps];
 };
 
 // Who owns a channel: a group inside a thread block, a whole thread block, a cluster of thread blocks
@@ -60,15 +69,35 @@ constexpr int kBlockThreads = 512;   // kBlock, kCluster
 // and leave little shared memory: short lists there.
 __host__ __device__ constexpr int merged_cap(int K) { return K > 16 ? 128 : 1024; }
 
-__host__ __device__ constexpr int sel_cap(int g, int K = 1) { return g <= 64 || (g > 256 && K > 16) ? 64 : g; }
-__host__ __device__ constexpr int sel_maxima(int g) { return g <= 64 ? 2 * g : g; }   // two per thread up to 64 threads
+__host__ __device__ constexpr int sel_cap(int g, int K = 1) { return g <= 64 || (g > 256 && K > 16) ? 64 : (K > 1 && g <= 256 ? 128 : g); }
+// Maxima that a group leaves in shared memory: one per thread and sign, of 1x1 channels two up to 64 threads.
+__host__ __device__ constexpr int sel_maxima(int g, int K) { return K == 1 && g <= 64 ? 4 * g : 2 * g; }
 __host__ __device__ constexpr int sel_bytes(int g, Owner own = kGroup, int K = 1)
 {
-    return static_cast<int>(sizeof(SelScratch)) + 8 * sel_cap(g, K) +
-           (own == kGroup ? (g > 32 ? 4 * sel_maxima(g) : 0) : (own == kCluster ? 8 * merged_cap(K) : 0));
+    return static_cast<int>(sizeof(SelScratch)) + (g > 32 ? static_cast<int>(sizeof(SelWarps)) : 0) + 8 * sel_cap(g, K) +
+           (own == kCluster ? 8 * merged_cap(K) : (g > 32 ? 4 * sel_maxima(g, K) : 0));
 }
-// The same of a 1x1 channel of `vecs` vectors: selection, perturbations, codes.
-__host__ __device__ constexpr int row_bytes(int g, int vecs, Owner own = kGroup) { return sel_bytes(g, own) + 20 * vecs; }
+// Shared memory of a 1x1 channel of `vecs` vectors: selection, perturbations, codes.
+__host__ __device__ constexpr int row_bytes(int g, int vecs) { return sel_bytes(g) + 20 * vecs; }
+// The same where a thread block or a cluster takes the row: weights, and codes if they are to be packed.
+__host__ __device__ constexpr int long_row_bytes(int g, int vecs, bool pack, Owner own) { return sel_bytes(g, own) + (pack ? 20 : 16) * vecs; }
+
+// The parts of a group's selection memory.
+struct Sel {
+    SelScratch *sc;
+    SelWarps *warps;
+    unsigned long long *list;
+    int *mx;   // the threads' maxima (not kCluster: the lists of all thread blocks are there)
+    int cap;
+    __device__ __forceinline__ Sel(unsigned char *slice, int g, Owner own, int K)
+    {
+        sc = reinterpret_cast<SelScratch *>(slice);
+        warps = reinterpret_cast<SelWarps *>(sc + 1);
+        list = reinterpret_cast<unsigned long long *>(slice + sizeof(SelScratch) + (g > 32 ? sizeof(SelWarps) : 0));
+        cap = sel_cap(g, K);
+        mx = reinterpret_cast<int *>(list + cap);
+    }
+};
 
 // How a run of n 4-byte elements that starts anywhere is cut into 16-byte vectors: vector q holds the
 // elements 4q - r .. 4q - r + 3; those with q_lo <= q < q_hi are whole, the up to six elements outside
@@ -125,15 +154,108 @@ __device__ __forceinline__ int lanes_add(int g, int v)
 }
 
 // ---------------------------------------------------------------- reductions over the owner of a channel
-// (of kBlock and kCluster; every thread calls them)
-// Word w of another thread block's control words.
+// One barrier each: a warp leaves its part in a place of its own, after the barrier every warp reads all of them
+// (of a cluster through distributed shared memory).
 template <class T>
 __device__ __forceinline__ T remote(const T *w, int rank)
 {
     return *cg::this_cluster().map_shared_rank(w, rank);
 }
 
-// Sum over the cluster of *w, which every thread block has completed before its last barrier.
+template <Owner kOwn>
+__device__ __forceinline__ void owner_sync(const Group &G)
+{
+    if (kOwn == kCluster) cg::this_cluster().sync();
+    else if (kOwn == kBlock) __syncthreads();
+    else G.sync();
+}
+
+template <Owner kOwn>
+__device__ __forceinline__ float owner_absmax(const Group &G, float amax, const Sel &S)
+{
+    unsigned u = lanes_max(G.g, __float_as_uint(amax));   // >= 0: uint order = float order
+    const int lane = threadIdx.x & 31;
+    if (kOwn == kGroup && G.g <= 32) {
+        __syncwarp();   // the control words are cleared
+        return __uint_as_float(u);
+    }
+    if (lane == 0) S.warps->amax[G.t >> 5] = u;
+    owner_sync<kOwn>(G);
+    if (kOwn == kCluster) {
+        const int c = lane >> 2;   // a lane reads four of a thread block's sixteen warps
+        const uint4 q = c < static_cast<int>(cg::this_cluster().num_blocks())
+                            ? remote(reinterpret_cast<const uint4 *>(S.warps->amax) + (lane & 3), c) : make_uint4(0u, 0u, 0u, 0u);
+        u = max(max(q.x, q.y), max(q.z, q.w));
+    } else {
+        u = S.warps->amax[lane & ((G.g >> 5) - 1)];
+    }
+    return __uint_as_float(__reduce_max_sync(kFull, u));
+}
+
+// Channel-wide error sum and extremes.  k64: the sum of e; else the sum of which lo32 is a thread's value
+// modulo 2^32 and apx its size in units of 2^17, off by less than 2^13 units over the channel.  kExt: up, down
+// (both >= 0) become the channel's (groups of whole warps).
+template <Owner kOwn, bool k64, bool kExt>
+__device__ __forceinline__ long long owner_sum(const Group &G, const Sel &S, long long e, unsigned lo32, int apx, int &up, int &down)
+{
+    const int lane = threadIdx.x & 31;
+    if (k64) {
+        for (int o = min(G.g, 32) >> 1; o > 0; o >>= 1) e += __shfl_xor_sync(kFull, e, o);
+    } else {
+        lo32 = static_cast<unsigned>(lanes_add(G.g, static_cast<int>(lo32)));
+        apx = lanes_add(G.g, apx);
+    }
+    if (kExt) {
+        up = static_cast<int>(__reduce_max_sync(kFull, static_cast<unsigned>(up)));
+        down = static_cast<int>(__reduce_max_sync(kFull, static_cast<unsigned>(down)));
+    }
+    if (kOwn != kGroup || G.g > 32) {
+        if (lane == 0) {
+            WarpPart p;
+            p.lo32 = k64 ? static_cast<int>(static_cast<unsigned>(e)) : static_cast<int>(lo32);
+            p.hi32 = k64 ? static_cast<int>(e >> 32) : apx;
+            p.up = up;
+            p.down = down;
+            *reinterpret_cast<int4 *>(S.warps->part + (G.t >> 5)) = make_int4(p.lo32, p.hi32, p.up, p.down);
+        }
+        owner_sync<kOwn>(G);
+        int4 q[4];
+        const int n = kOwn == kCluster ? 4 : 1;
+        if (kOwn == kCluster) {
+            const int c = lane >> 2;
+            const bool there = c < static_cast<int>(cg::this_cluster().num_blocks());
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                q[i] = there ? remote(reinterpret_cast<const int4 *>(S.warps->part) + 4 * (lane & 3) + i, c) : make_int4(0, 0, 0, 0);
+        } else {
+            q[0] = lane < (G.g >> 5) ? reinterpret_cast<const int4 *>(S.warps->part)[lane] : make_int4(0, 0, 0, 0);
+        }
+        if (k64) {
+            e = 0;
+#pragma unroll
+            for (int i = 0; i < n; ++i) e += (static_cast<long long>(q[i].y) << 32) | static_cast<unsigned>(q[i].x);
+            for (int o = 16; o > 0; o >>= 1) e += __shfl_xor_sync(kFull, e, o);
+        } else {
+            int a = 0, b = 0;
+#pragma unroll
+            for (int i = 0; i < n; ++i) { a += q[i].x; b += q[i].y; }
+            lo32 = static_cast<unsigned>(__reduce_add_sync(kFull, a));
+            apx = __reduce_add_sync(kFull, b);
+        }
+        if (kExt) {
+            int a = 0, b = 0;
+#pragma unroll
+            for (int i = 0; i < n; ++i) { a = max(a, q[i].z); b = max(b, q[i].w); }
+            up = static_cast<int>(__reduce_max_sync(kFull, static_cast<unsigned>(a)));
+            down = static_cast<int>(__reduce_max_sync(kFull, static_cast<unsigned>(b)));
+        }
+    }
+    if (k64) return e;
+    const unsigned base = static_cast<unsigned>(apx) << 17;
+    return static_cast<long long>(apx) * (1ll << 17) + static_cast<int>(lo32 - base);
+}
+
+// Sum over the cluster of *w, which every thread block has completed before the barrier in here.
 __device__ __forceinline__ int cluster_sum(const int *w)
 {
     cg::cluster_group cl = cg::this_cluster();
@@ -142,21 +264,30 @@ __device__ __forceinline__ int cluster_sum(const int *w)
     return __reduce_add_sync(kFull, lane < static_cast<int>(cl.num_blocks()) ? remote(w, lane) : 0);
 }
 
+// absmax / qmax, correctly rounded: with y = RN(1 / qmax), x0 = RN(a y) and the exact remainder r = a - x0 qmax,
+// RN(x0 + r y) is the rounded quotient (Markstein's theorem; a >= 2^-100, so nothing underflows).  Three
+// instructions in the place of a general division that every warp of a short channel would run once.
+__device__ __forceinline__ float absmax_scale(float amax, int qmax)
+{
+    return (amax < 0x1p-100f) ? 1.0f : __fdiv_rn(amax, static_cast<float>(qmax));
+}
+
 #ifdef SQUANT_DEBUG_BOUNDS
 // The channel's error sum from its final codes and the weights (global memory), compared with ec.  Called by
 // every thread of the group after the codes' last barrier; groups that share a warp come together.
 __device__ __forceinline__ void debug_check_sum(const Group &G, const float *w, const unsigned char *codes, int n, float s, long long ec, bool valid,
-                                                SelScratch *sc)
+                                                const Sel &S)
 {
+    unsigned long long *sum64 = reinterpret_cast<unsigned long long *>(S.warps->amax);   // (dead by now)
     long long e = 0;
     for (int j = G.t; j < n; j += G.g) e += debug_error(w[j], s, static_cast<signed char>(codes[j]));
     for (int o = min(G.g, 32) >> 1; o > 0; o >>= 1) e += __shfl_xor_sync(kFull, e, o);
     if (G.g > 32) {
-        if (G.t == 0) sc->sum64 = 0ull;
+        if (G.t == 0) *sum64 = 0ull;
         G.sync();
-        if ((G.t & 31) == 0) atomicAdd(&sc->sum64, static_cast<unsigned long long>(e));
+        if ((G.t & 31) == 0) atomicAdd(sum64, static_cast<unsigned long long>(e));
         G.sync();
-        e = static_cast<long long>(sc->sum64);
+        e = static_cast<long long>(*sum64);
     }
     if (G.t == 0 && valid) {
         SQ_DBG(e == ec, 8);
@@ -166,29 +297,36 @@ __device__ __forceinline__ void debug_check_sum(const Group &G, const float *w, 
 #endif
 
 // ---------------------------------------------------------------- SQuant-C: the k_c largest candidates
-// each(t, f) visits those of the calling thread's elements that reach t >= 1, f(a, n) with a = the
-// candidate's value in the direction of the flips and n its kernel index in the channel; m0, m1: the
-// thread's maxima of a over two disjoint parts of its elements, top a value above every candidate, spread the expected
-// distance between the largest candidates in units of top / n_all.  flip(a, n) is called once for each
-// of the min(kc, candidates) largest (equal values: lower index first), by some thread of the
-// group.  want: this group selects at all (kc >= 1).  Returns the number of flips.  Every thread of
-// the group calls it, groups that share a warp together; it starts with no barrier and ends
-// with none.
-template <Owner kOwn, class Each, class Flip>
-__device__ __forceinline__ int select_top(const Group &G, Each each, Flip flip, int m0, int m1, int top, float spread, int kc, int n_all, bool want,
-                                          SelScratch *sc, int K = 1)
+// Entry of a list: larger values first, equal values by lower index; the code byte comes along.
+__device__ __forceinline__ unsigned long long list_key(int a, int n, unsigned code)
+{
+    return (static_cast<unsigned long long>(static_cast<unsigned>(a)) << 32) | (static_cast<unsigned>(~n) << 8) | (code & 255u);
+}
+// *w += 1, the old value.  (One instruction: the compiler would have the lanes of a warp agree on one of them first.)
+__device__ __forceinline__ int shared_count(int *w)
+{
+    int old;
+    asm volatile("atom.shared.add.u32 %0, [%1], 1;" : "=r"(old) : "r"(smem_addr(w)) : "memory");
+    return old;
+}
+
+// a = the value of a candidate in the direction of the flips, n its kernel index in the channel.  The threads know
+// maxima of a over parts of their elements, in some unit: count(t) = how many of the group's nmax maxima are at least
+// t, t >= 1, below `top`, one unit above the largest possible.  listing(t, push) calls push(a, n, code) for those of
+// the thread's elements that are at least t units; code is handed through to flip.  For the exact search: settle()
+// once, then each(v, f) calls f(a, n) for those with a >= v (any v >= 1, vtop above all), code_of(n) is the code of one.  spread: the expected distance between the largest candidates in units
+// of top / n_all.  flip(a, n, code) is called once for each of the min(kc, candidates) largest (equal values: lower
+// index first), by some thread of the group.  want: this group selects at all (kc >= 1).  Returns the number of
+// flips.  Every thread of the group calls it, groups that share a warp together; it starts with no barrier and
+// ends with none.
+template <Owner kOwn, class Count, class Listing, class Settle, class Each, class CodeOf, class Flip>
+__device__ __forceinline__ int select_top(const Group &G, Count count, Listing listing, Settle settle, Each each, CodeOf code_of, Flip flip, int nmax, int top, int vtop, float spread,
+                                          int kc, int n_all, bool want, const Sel &S, int K)
 {
     const int g = G.g, lane = threadIdx.x & 31;
-    const unsigned gmask = g >= 32 ? kFull : (((1u << g) - 1u) << (lane & ~(g - 1)));
-    unsigned long long *list = reinterpret_cast<unsigned long long *>(sc + 1);
-    const int cap = sel_cap(g, kOwn == kCluster ? K : 1);
-    const int nmax = kOwn == kGroup ? sel_maxima(g) : 2 * g * (kOwn == kCluster ? static_cast<int>(cg::this_cluster().num_blocks()) : 1);
-    int *mx = reinterpret_cast<int *>(list + cap);
-    if (kOwn == kGroup && g > 32) {
-        if (g <= 64) { mx[G.t] = m0; mx[G.t + g] = m1; }
-        else mx[G.t] = max(m0, m1);
-        G.sync();
-    }
+    SelScratch *sc = S.sc;
+    unsigned long long *list = S.list;
+    const int cap = S.cap;
 
     // ---- T0: at least kc of the maxima reach it, and not many more.  The first guess supposes an even
     // spread; the distance to the top is doubled until it is enough, then the interval is halved (1x1:
@@ -201,25 +339,7 @@ __device__ __forceinline__ int select_top(const Group &G, Each each, Flip flip, 
     int mid = max(top - 1 - __float2int_rz(__fmul_rn(__fmul_rn(static_cast<float>(kc) + 1.0f, spread), __fdividef(static_cast<float>(top), static_cast<float>(n_all)))), 1);
 #pragma unroll 1
     for (int it = 0; __any_sync(kFull, !done); ++it) {
-        int c;
-        if (kOwn != kGroup) {
-            c = __syncthreads_count(m0 >= mid) + __syncthreads_count(m1 >= mid);
-            if (kOwn == kCluster) {
-                if (G.t == 0) sc->found[it & 1] = c;
-                __syncthreads();
-                c = cluster_sum(&sc->found[it & 1]);
-            }
-        } else if (g <= 32) {
-            c = __popc(__ballot_sync(kFull, m0 >= mid) & gmask) + __popc(__ballot_sync(kFull, m1 >= mid) & gmask);
-        } else {
-            c = 0;
-#pragma unroll 1
-            for (int i = lane; i < (nmax >> 2); i += 32) {
-                const int4 q = reinterpret_cast<const int4 *>(mx)[i];
-                c += (q.x >= mid) + (q.y >= mid) + (q.z >= mid) + (q.w >= mid);
-            }
-            c = __reduce_add_sync(kFull, c);
-        }
+        const int c = count(mid, it);
         if (!done) {
             if (c >= kc) { lo = mid; sure = true; done = c <= slack; }
             else hi = mid;
@@ -227,41 +347,59 @@ __device__ __forceinline__ int select_top(const Group &G, Each each, Flip flip, 
             mid = sure ? lo + ((hi - lo) >> 1) : max(hi - (top - hi), 1);
         }
     }
-    const int T0 = lo;
     bool slow = want && !sure;   // fewer than kc maxima are candidates at all
 
-    // ---- list the elements from T0 on
-    if (want && !slow && max(m0, m1) >= T0)
-        each(T0, [&](int a, int n) {
-            const int pos = atomicAdd(&sc->count, 1);
-            SQ_DBG(a >= 1 && a < top && n >= 0 && n < n_all, 12);
-            if (pos < cap)
-                list[pos] = (static_cast<unsigned long long>(static_cast<unsigned>(a)) << kIdxBits) |
-                            static_cast<unsigned long long>(((1 << kIdxBits) - 1) - n);
-        });
-    G.sync();
-    int cnt = sc->count, all = cnt;   // this list, all lists
+    // ---- list the elements from T0 on; where they are more than the list holds (many to a maximum: k_c is large
+    // for the number of maxima), once more from further up, supposing an even spread from T0 to the top
+    int cnt = 0, all = 0;   // this list, all lists
     int k_eff = want ? kc : 0;
     const unsigned long long *merged = list;
-    if (kOwn == kCluster) {   // every thread block collects all lists
-        cg::cluster_group cl = cg::this_cluster();
-        cl.sync();
-        unsigned long long *dst = list + cap;
-        merged = dst;
-        all = 0;
+    bool relist = false;
+#pragma unroll 1
+    for (int round = 0;; ++round) {
+        if (want && !slow && (round == 0 || relist))
+            listing(lo, [&](int a, int n, unsigned code) {
+                const int pos = shared_count(&sc->count);
+                SQ_DBG(a >= 1 && a < vtop && n >= 0 && n < n_all, 12);
+                if (pos < cap) list[pos] = list_key(a, n, code);
+            });
+        owner_sync<kOwn>(G);
+        cnt = all = sc->count;
         bool full = false;
-        for (int c = 0; c < static_cast<int>(cl.num_blocks()); ++c) {
-            const int n = remote(&sc->count, c);
-            full = full || n > cap || all + n > merged_cap(K);
-            if (!full)
-                for (int y = G.t; y < n; y += g) dst[all + y] = remote(list + y, c);
-            all += n;
+        if (kOwn == kCluster) {   // every thread block collects all lists
+            unsigned long long *dst = list + cap;
+            merged = dst;
+            all = 0;
+            for (int c = 0; c < static_cast<int>(cg::this_cluster().num_blocks()); ++c) {
+                const int n = remote(&sc->count, c);
+                full = full || n > cap || all + n > merged_cap(K);
+                if (!full)
+                    for (int y = G.t; y < n; y += g) dst[all + y] = remote(list + y, c);
+                all += n;
+            }
+        } else {
+            full = cnt > cap;
         }
-        if (full) slow = true;
-        G.sync();
-    } else if (want && !slow && cnt > cap) {
-        slow = true;
+        full = full && want && !slow;
+        if (round > 0 && relist && all < kc) slow = true;   // (too far up)
+        relist = full && round < 3;
+        if (full && !relist) slow = true;
+        if (kOwn == kCluster) __syncthreads();
+        if (!__any_sync(kFull, relist)) break;   // (uniform over groups wider than a warp)
+        const int goal = kc + ((min(cap, kOwn == kCluster ? merged_cap(K) : cap) - kc) >> 1);
+        if (relist) {
+            const int up = top - __float2int_rz(__fmul_rn(static_cast<float>(top - lo), __fdividef(static_cast<float>(goal), static_cast<float>(all))));
+            if (goal <= kc || up <= lo || up >= top) { relist = false; slow = true; }
+            lo = up;
+        }
+        owner_sync<kOwn>(G);   // everybody has read the lists
+        if (relist && G.t == 0) sc->count = 0;
+        owner_sync<kOwn>(G);
     }
+    auto flip_entry = [&](unsigned long long e) {
+        const unsigned low = static_cast<unsigned>(e);
+        flip(static_cast<int>(e >> 32), static_cast<int>(~low >> 8), low & 255u);
+    };
     if (kOwn != kGroup && want && !slow) {   // exact ranks, a warp per entry: keys are distinct
 #pragma unroll 1
         for (int x = G.t >> 5; x < cnt; x += g >> 5) {
@@ -269,7 +407,7 @@ __device__ __forceinline__ int select_top(const Group &G, Each each, Flip flip, 
             int rank = 0;
             for (int y = lane; y < all; y += 32) rank += merged[y] > me ? 1 : 0;
             rank = __reduce_add_sync(kFull, rank);
-            if (rank < kc && lane == 0) flip(static_cast<int>(me >> kIdxBits), ((1 << kIdxBits) - 1) - static_cast<int>(me & ((1ull << kIdxBits) - 1)));
+            if (rank < kc && lane == 0) flip_entry(me);
         }
     }
     if (kOwn == kGroup && want && !slow) {   // exact ranks inside the list: keys are distinct
@@ -281,7 +419,7 @@ __device__ __forceinline__ int select_top(const Group &G, Each each, Flip flip, 
 #pragma unroll 4
                 for (int y = 0; y < cnt; ++y) rank += list[y] > me ? 1 : 0;
             }
-            if (rank < kc) flip(static_cast<int>(me >> kIdxBits), ((1 << kIdxBits) - 1) - static_cast<int>(me & ((1ull << kIdxBits) - 1)));
+            if (rank < kc) flip_entry(me);
         }
     }
 
@@ -289,14 +427,14 @@ __device__ __forceinline__ int select_top(const Group &G, Each each, Flip flip, 
     // counting (eight rounds interpolate, then the interval is halved); all candidates above v are
     // flipped, and of those that tie at v the ones with the lowest indices
     if (__any_sync(kFull, slow)) {   // group-uniform for groups of whole warps
-        int vlo = 1, vhi = top, vm = 1, c_lo = 0, c_hi = 0, tie = 0;   // count(vlo) >= kc > count(vhi)
+        if (slow) settle();
+        int vlo = 1, vhi = vtop, vm = 1, c_lo = 0, c_hi = 0, tie = 0;   // count(vlo) >= kc > count(vhi)
         int ilo = 0, ihi = n_all, im = 0;                      // ties with index < ihi suffice, with index < ilo do not
         int phase = slow ? 0 : 2;
 #pragma unroll 1
         for (int it = 0; __any_sync(kFull, phase < 2); ++it) {
             int c = 0;
-            if (phase == 0) each(vm, [&](int, int) { ++c; });
-            if (phase == 1) each(vlo, [&](int a, int n) { c += (a == vlo && n < im) ? 1 : 0; });
+            if (phase < 2) each(phase == 0 ? vm : vlo, [&](int a, int n) { c += phase == 0 || (a == vlo && n < im) ? 1 : 0; });
             c = lanes_add(g, c);
             if (g > 32) {
                 if (lane == 0) atomicAdd(&sc->total[it % 3], c);
@@ -327,28 +465,44 @@ __device__ __forceinline__ int select_top(const Group &G, Each each, Flip flip, 
                 im = ilo + ((ihi - ilo) >> 1);
             }
         }
-        if (slow) each(vlo, [&](int a, int n) { if (a > vlo || n < ihi) flip(a, n); });
+        if (slow) each(vlo, [&](int a, int n) { if (a > vlo || n < ihi) flip(a, n, code_of(n)); });
     }
     return k_eff;
 }
 
-// SQuant-E on four weights by plain IEEE division, codes clamped to [lo, hi]: for scales outside the
-// range of the reciprocal sequence.  Out of line: rare, and its code would be in the way.
-__device__ __noinline__ unsigned row_e_div(float4 w, float s, int lo, int hi, float2 &Pa, float2 &Pb)
+// code (low byte of c) * s
+__device__ __forceinline__ float row_deq(unsigned c, float s)
 {
+    return __fmul_rn(__int2float_rn(static_cast<int>(static_cast<signed char>(c & 255u))), s);
+}
+
+// two fp32 -> bfloat16, round to nearest, ties to even; a in the low half
+__device__ __forceinline__ unsigned bf16_pair(float a, float b)
+{
+    unsigned d;
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(b), "f"(a));
+    return d;
+}
+
+// SQuant-E on four weights by plain IEEE division, codes clamped to [lo, hi]: for scales outside the range of the reciprocal
+// sequence.  Out of line: rare, and its code would be in the way.
+struct QuadDiv {
+    unsigned c4;
     float P[4];
-    unsigned c4 = 0u;
+};
+__device__ __noinline__ QuadDiv row_div(float4 w, float s, int lo, int hi)
+{
+    QuadDiv o;
+    o.c4 = 0u;
     const float ws[4] = {w.x, w.y, w.z, w.w};
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
         const float x = __fdiv_rn(ws[c], s);
-        const float qf = fminf(fmaxf(rintf(x), static_cast<float>(lo)), static_cast<float>(hi));
-        P[c] = __fmul_rn(__fsub_rn(qf, x), 1073741824.0f);
-        c4 |= (static_cast<unsigned>(__float2int_rn(qf)) & 255u) << (8 * c);
+        const float q = fminf(fmaxf(rintf(x), static_cast<float>(lo)), static_cast<float>(hi));
+        o.P[c] = __fmul_rn(__fsub_rn(q, x), 1073741824.0f);
+        o.c4 |= (static_cast<unsigned>(__float2int_rn(q)) & 255u) << (8 * c);
     }
-    Pa = make_float2(P[0], P[1]);
-    Pb = make_float2(P[2], P[3]);
-    return c4;
+    return o;
 }
 
 // One element under the clip: its exact perturbation Pf goes into the 64-bit sum and, as a float,
@@ -363,39 +517,29 @@ __device__ __forceinline__ void row_clip_one(float Pf, int &P, unsigned c, int q
     if ((P > 0 && q8 == qmin) || (P < 0 && q8 == qmax)) P = 0;
 }
 
-// code (low byte of c) * s
-__device__ __forceinline__ float row_deq(unsigned c, float s)
-{
-    return __fmul_rn(__int2float_rn(static_cast<int>(static_cast<signed char>(c & 255u))), s);
-}
-
 // ---------------------------------------------------------------- one 1x1 channel
-// kClip: the clip of Sec. 2.2 can fire (caller-supplied scales) or the element at the edge of the
-// range can reach the selection (channels of 2^16 and more kernels): codes are clamped, sums are 64
+// kClip: the clip of Sec. 2.2 can fire (caller-supplied scales): codes are clamped, sums are 64
 // bit and an element whose flipped code would leave the range is no candidate.  valid = false: the
 // group has no channel (its lanes take part in the warp's steps and write nothing).
-// kCluster: this thread block has the elements n0 .. n0 + nloc - 1 (n0 a multiple of four).
-template <bool kClip, Owner kOwn = kGroup>
-__device__ __forceinline__ void row_body(const LayerDesc &L, int m, const Group &G, unsigned char *slice, int qmax, unsigned mode,
-                                         bool valid, int n0 = 0, int nloc = 0)
+template <bool kClip>
+__device__ __forceinline__ void row_body(const LayerDesc &L, int m, const Group &G, unsigned char *slice, int qmax, unsigned mode, bool valid)
 {
-    const int g = G.g, N = kOwn == kCluster ? nloc : (valid ? L.N : 0);   // elements here
-    SelScratch *sc = reinterpret_cast<SelScratch *>(slice);
+    const int g = G.g, N = valid ? L.N : 0;
+    const Sel S(slice, g, kGroup, 1);
     if (G.t == 0) {
-        sc->amax = 0u; sc->sum = 0u; sc->approx = 0; sc->count = 0;
-        sc->total[0] = 0;
-        sc->sum64 = 0ull;
+        S.sc->count = 0;
+        S.sc->total[0] = 0;
     }
-    const size_t first = static_cast<size_t>(m) * L.N + n0;   // of these elements in the layer
+    const size_t first = static_cast<size_t>(m) * L.N;   // of the row in the layer
     const float *wrow = L.w + first;
     // The row is cut into vectors at 16-byte boundaries of the weights (packed codes pair elements from
     // the row's start, so there the vectors start with the row).
     const bool pack = (mode & kModePackInt4) != 0;
     const Span sp(pack ? 0 : static_cast<int>((reinterpret_cast<uintptr_t>(wrow) >> 2) & 3), N, G.t);
-    const int r = sp.r, q_hi = sp.q_hi, rag = sp.rag, q0 = sp.q_lo + G.t;
+    const int r = sp.r, q_hi = sp.q_hi, rag = sp.rag, q0 = sp.q_lo + G.t, vecs = G.rounds(sp.q_lo, sp.q_hi);   // vectors q0, q0 + g, ..
     SQ_DBG(N >= 0 && N + r <= 4 * L.off_vi && q_hi <= L.off_vi, 14);   // the vectors' places below
-    int4 *Pbuf = reinterpret_cast<int4 *>(slice + sel_bytes(g, kOwn));              // what SQuant-C may choose from
-    unsigned *cbuf = reinterpret_cast<unsigned *>(slice + sel_bytes(g, kOwn) + 16 * L.off_vi);   // codes, by vectors
+    int4 *Pbuf = reinterpret_cast<int4 *>(slice + sel_bytes(g));              // what SQuant-C may choose from
+    unsigned *cbuf = reinterpret_cast<unsigned *>(slice + sel_bytes(g) + 16 * L.off_vi);   // codes, by vectors
     int *Pel = reinterpret_cast<int *>(Pbuf) + r;                                   // the same by elements
     unsigned char *cel = reinterpret_cast<unsigned char *>(cbuf) + r;
     float *kerr = L.kerr ? L.kerr + first : nullptr;
@@ -408,7 +552,7 @@ __device__ __forceinline__ void row_body(const LayerDesc &L, int m, const Group 
         const float4 *src = reinterpret_cast<const float4 *>(wrow - r);
         if ((reinterpret_cast<uintptr_t>(src) & 15) == 0) {
 #pragma unroll 2
-            for (int q = q0; q < q_hi; q += g) copy_async16(Pbuf + q, src + q);
+            for (int i = 0; i < vecs; ++i) copy_async16(Pbuf + q0 + i * g, src + q0 + i * g);
         } else {   // packed codes of a misaligned row
 #pragma unroll 1
             for (int q = q0; q < q_hi; q += g)
@@ -417,8 +561,8 @@ __device__ __forceinline__ void row_body(const LayerDesc &L, int m, const Group 
         if (rag >= 0) copy_async4(Pel + rag, wrow + rag);
         copy_async_wait();
 #pragma unroll 2
-        for (int q = q0; q < q_hi; q += g) {
-            const float4 v = reinterpret_cast<const float4 *>(Pbuf)[q];
+        for (int i = 0; i < vecs; ++i) {
+            const float4 v = reinterpret_cast<const float4 *>(Pbuf)[q0 + i * g];
             amax = absmax3(absmax3(amax, v.x, v.y), v.z, v.w);
         }
     }
@@ -427,27 +571,11 @@ __device__ __forceinline__ void row_body(const LayerDesc &L, int m, const Group 
     amax = fmaxf(amax, fabsf(w_rag));
 
     // ---- scale
-    float s;
-    {
-        unsigned u = lanes_max(g, __float_as_uint(amax));   // >= 0: uint order = float order
-        G.sync();   // the scratch words are cleared
-        if (g > 32) {
-            if ((G.t & 31) == 0) atomicMax(&sc->amax, u);
-            G.sync();
-            u = sc->amax;
-        }
-        if (kOwn == kCluster) {
-            cg::cluster_group cl = cg::this_cluster();
-            cl.sync();
-            const int lane = threadIdx.x & 31;
-            u = __reduce_max_sync(kFull, lane < static_cast<int>(cl.num_blocks()) ? remote(&sc->amax, lane) : 0u);
-        }
-        amax = __uint_as_float(u);
-        s = (amax < 0x1p-100f) ? 1.0f : __fdiv_rn(amax, static_cast<float>(qmax));
-        if (kClip && L.sin && valid) {
-            s = L.sin[m];
-            if (!(s > 0.0f && s < __int_as_float(0x7f800000))) s = 1.0f;
-        }
+    amax = owner_absmax<kGroup>(G, amax, S);
+    float s = absmax_scale(amax, qmax);
+    if (kClip && valid) {
+        s = L.sin[m];
+        if (!(s > 0.0f && s < __int_as_float(0x7f800000))) s = 1.0f;
     }
 
     // ---- SQuant-E: codes and perturbations; the kernels' error sums leave at once (SQuant-C corrects
@@ -487,7 +615,10 @@ __device__ __forceinline__ void row_body(const LayerDesc &L, int m, const Group 
                 c4 = __byte_perm(__byte_perm(__float_as_uint(ta.x), __float_as_uint(ta.y), 0x0040),
                                  __byte_perm(__float_as_uint(tb.x), __float_as_uint(tb.y), 0x0040), 0x5410);
             } else {
-                c4 = row_e_div(w, s, kClip ? qmin : -255, kClip ? qmax : 255, Pa, Pb);
+                const QuadDiv d = row_div(w, s, kClip ? qmin : -255, kClip ? qmax : 255);
+                c4 = d.c4;
+                Pa = make_float2(d.P[0], d.P[1]);
+                Pb = make_float2(d.P[2], d.P[3]);
             }
             p = make_int4(__float2int_rn(Pa.x), __float2int_rn(Pa.y), __float2int_rn(Pb.x), __float2int_rn(Pb.y));
             if (!kClip) {
@@ -514,7 +645,8 @@ __device__ __forceinline__ void row_body(const LayerDesc &L, int m, const Group 
             return c4;
         };
 #pragma unroll 2
-        for (int q = q0; q < q_hi; q += g) {
+        for (int i = 0; i < vecs; ++i) {
+            const int q = q0 + i * g;
             int4 p;
             float2 oa, ob;
             cbuf[q] = quantize(reinterpret_cast<const float4 *>(Pbuf)[q], p, oa, ob);
@@ -538,49 +670,21 @@ __device__ __forceinline__ void row_body(const LayerDesc &L, int m, const Group 
     }
 
     // ---- channel sum.  !kClip: its value modulo 2^32 is exact, its size is known from the float sums
-    // (2^16 elements of at most one half: the float sums are off by far less than 2^31)
+    // (2^16 elements of at most one half: the float sums are off by far less than 2^30)
     long long ec = 0;
+    const int per = g > 64 ? 1 : 2;   // maxima a thread puts in
     if ((mode & 4u) || L.cerr) {
-        unsigned tot = 0u;
-        int apx = 0;
-        if (!kClip) {
-            tot = static_cast<unsigned>(lanes_add(g, static_cast<int>(sum)));
-            apx = lanes_add(g, __float2int_rn(__fmul_rn(__fadd_rn(fs.x, fs.y), 0x1p-20f)));
-        } else {
-            for (int o = min(g, 32) >> 1; o > 0; o >>= 1) sum64 += __shfl_xor_sync(kFull, sum64, o);
-        }
-        if (g > 32) {
-            if ((G.t & 31) == 0) {
-                if (!kClip) {
-                    atomicAdd(&sc->sum, tot);
-                    atomicAdd(&sc->approx, apx);
-                } else {
-                    atomicAdd(&sc->sum64, static_cast<unsigned long long>(sum64));
-                }
-            }
-            G.sync();
-            tot = sc->sum;
-            apx = sc->approx;
-            sum64 = static_cast<long long>(sc->sum64);
-            if (kOwn == kCluster) {
-                cg::cluster_group cl = cg::this_cluster();
-                cl.sync();
-                tot = 0u;
-                apx = 0;
-                sum64 = 0;
-                for (int c = 0; c < static_cast<int>(cl.num_blocks()); ++c) {
-                    tot += remote(&sc->sum, c);
-                    apx += remote(&sc->approx, c);
-                    sum64 += static_cast<long long>(remote(&sc->sum64, c));
-                }
+        if (g > 32) {   // those that SQuant-C looks for its bound among, of either sign
+            if (per == 2) {
+                S.mx[G.t] = hi0; S.mx[G.t + g] = hi1;
+                S.mx[G.t + 2 * g] = -lo0; S.mx[G.t + 3 * g] = -lo1;
+            } else {
+                S.mx[G.t] = max(hi0, hi1);
+                S.mx[G.t + g] = -min(lo0, lo1);
             }
         }
-        if (!kClip) {
-            const unsigned base = static_cast<unsigned>(apx) << 20;
-            ec = static_cast<long long>(apx) * (1ll << 20) + static_cast<int>(tot - base);
-        } else {
-            ec = sum64;
-        }
+        int up = 0, down = 0;
+        ec = owner_sum<kGroup, kClip, false>(G, S, sum64, sum, __float2int_rn(__fmul_rn(__fadd_rn(fs.x, fs.y), 0x1p-17f)), up, down);
     }
 
     // ---- SQuant-C: Algorithm 2 on the channel, the perturbations are the keys
@@ -594,11 +698,10 @@ __device__ __forceinline__ void row_body(const LayerDesc &L, int m, const Group 
             const int sx = sgn > 0 ? 0 : -1;   // p ^ sx = the value in the direction of the flips, less one if that is downward
             auto each = [&](int t, auto fn) {
                 const int tx = t + sx;
-                for (int qb = q0; qb < q_hi; qb += kRowVecs * g) {   // (kGroup: once)
-                unsigned hit = 0u, bit = 1u;   // a bit for each of these 32 elements that count
+                unsigned hit = 0u, bit = 1u;   // a bit for each of the thread's elements in vectors (at most 32) that counts
 #pragma unroll 2
-                for (int q = qb; q < min(q_hi, qb + kRowVecs * g); q += g, bit <<= 4) {
-                    const int4 p = Pbuf[q];
+                for (int i = 0; i < vecs; ++i, bit <<= 4) {
+                    const int4 p = Pbuf[q0 + i * g];
                     if ((p.x ^ sx) >= tx) hit |= bit;
                     if ((p.y ^ sx) >= tx) hit |= 2u * bit;
                     if ((p.z ^ sx) >= tx) hit |= 4u * bit;
@@ -606,31 +709,45 @@ __device__ __forceinline__ void row_body(const LayerDesc &L, int m, const Group 
                 }
 #pragma unroll 1
                 for (; hit != 0u; hit &= hit - 1u) {
-                    const int b = __ffs(hit) - 1, n = 4 * (qb + (b >> 2) * g) - r + (b & 3);
+                    const int b = __ffs(hit) - 1, n = 4 * (q0 + (b >> 2) * g) - r + (b & 3);
                     SQ_DBG(n >= 0 && n < N, 15);
-                    fn((Pel[n] ^ sx) - sx, n0 + n);
-                }
-                if (kOwn == kGroup) break;
+                    fn((Pel[n] ^ sx) - sx, n);
                 }
                 if (rag >= 0) {
                     const int v = Pel[rag] ^ sx;
-                    if (v >= tx) fn(v - sx, n0 + rag);
+                    if (v >= tx) fn(v - sx, rag);
                 }
             };
-            auto flip = [&](int a, int n_abs) {
-                const int n = n_abs - n0;
+            auto listing = [&](int t, auto push) {
+                if (max(m0, m1) >= t) each(t, [&](int a, int n) { push(a, n, 0u); });   // (the codes are here)
+            };
+            const int lane = threadIdx.x & 31;
+            const unsigned gmask = g >= 32 ? kFull : (((1u << g) - 1u) << (lane & ~(g - 1)));
+            const int *mx = sgn > 0 ? S.mx : S.mx + per * g;
+            auto count = [&](int t, int) {
+                if (g <= 32) return __popc(__ballot_sync(kFull, m0 >= t) & gmask) + __popc(__ballot_sync(kFull, m1 >= t) & gmask);
+                int c = 0;
+#pragma unroll 1
+                for (int i = lane; i < ((per * g) >> 2); i += 32) {
+                    const int4 q = reinterpret_cast<const int4 *>(mx)[i];
+                    c += (q.x >= t) + (q.y >= t) + (q.z >= t) + (q.w >= t);
+                }
+                return __reduce_add_sync(kFull, c);
+            };
+            auto flip = [&](int a, int n, unsigned) {
                 SQ_DBG(n >= 0 && n < N, 3);
                 unsigned char *cb = cel + n;
                 *cb = static_cast<unsigned char>(*cb - sgn);
                 if (kerr) kerr[n] = __fmul_rn(__int2float_rn(sgn > 0 ? a - kOne : kOne - a), 0x1p-30f);
             };
-            const int k_eff = select_top<kOwn>(G, each, flip, m0, m1, kHalf + (1 << 14) + 1, 2.0f, kc, L.N, want, sc);
+            const int vtop = kHalf + (1 << 14) + 1;
+            const int k_eff = select_top<kGroup>(G, count, listing, [] {}, each, [](int) { return 0u; }, flip, per * g, vtop, vtop, 2.0f, kc, N, want, S, 1);
             ec -= static_cast<long long>(sgn) * k_eff * kOne;
         }
     }
     G.sync();   // all codes are final
 #ifdef SQUANT_DEBUG_BOUNDS
-    if (!kClip && kOwn != kCluster && ((mode & 4u) || L.cerr)) debug_check_sum(G, wrow, cel, N, s, ec, valid, sc);
+    if (!kClip && ((mode & 4u) || L.cerr)) debug_check_sum(G, wrow, cel, N, s, ec, valid, S);
 #endif
     if (!valid) return;
 
@@ -640,14 +757,15 @@ __device__ __forceinline__ void row_body(const LayerDesc &L, int m, const Group 
         if (((reinterpret_cast<uintptr_t>(crow) - r) & 3) == 0) {
             unsigned *dst = reinterpret_cast<unsigned *>(crow - r);
 #pragma unroll 4
-            for (int q = q0; q < q_hi; q += g) __stcs(dst + q, cbuf[q]);
+            for (int i = 0; i < vecs; ++i) __stcs(dst + q0 + i * g, cbuf[q0 + i * g]);
             if (rag >= 0) crow[rag] = cel[rag];
         } else {
             for (int n = G.t; n < N; n += g) crow[n] = cel[n];
         }
     } else {   // two codes per byte, low nibble = even flat index; r = 0
-        unsigned char *crow = reinterpret_cast<unsigned char *>(L.codes) + static_cast<size_t>(m) * ((L.N + 1) >> 1) + (n0 >> 1);
+        unsigned char *crow = reinterpret_cast<unsigned char *>(L.codes) + static_cast<size_t>(m) * ((L.N + 1) >> 1);
         const bool two = (reinterpret_cast<uintptr_t>(crow) & 1) == 0;
+#pragma unroll 1
         for (int q = q0; q < q_hi; q += g) {
             const unsigned b = cbuf[q] & 0x0f0f0f0fu, h = b | (b >> 4);
             if (two) {
@@ -662,6 +780,7 @@ __device__ __forceinline__ void row_body(const LayerDesc &L, int m, const Group 
     if (L.deq) {   // Algorithm 1's own return value: code * s
         float *dg = L.deq + first;
         const bool vec = ((reinterpret_cast<uintptr_t>(dg) - 4 * r) & 15) == 0;
+#pragma unroll 1
         for (int q = q0; q < q_hi; q += g) {
             const unsigned c4 = cbuf[q];
             const float4 d = make_float4(row_deq(c4, s), row_deq(c4 >> 8, s), row_deq(c4 >> 16, s), row_deq(c4 >> 24, s));
@@ -674,6 +793,7 @@ __device__ __forceinline__ void row_body(const LayerDesc &L, int m, const Group 
     if (L.deq16) {   // the same product as bfloat16
         uint16_t *dg = L.deq16 + first;
         const bool vec = ((reinterpret_cast<uintptr_t>(dg) - 2 * r) & 7) == 0;
+#pragma unroll 1
         for (int q = q0; q < q_hi; q += g) {
             const unsigned c4 = cbuf[q];
             const unsigned b0 = bf16_bits(row_deq(c4, s)), b1 = bf16_bits(row_deq(c4 >> 8, s));
@@ -684,7 +804,7 @@ __device__ __forceinline__ void row_body(const LayerDesc &L, int m, const Group 
         }
         if (rag >= 0) dg[rag] = static_cast<uint16_t>(bf16_bits(row_deq(cel[rag], s)));
     }
-    if (G.t == 0 && n0 == 0) {
+    if (G.t == 0) {
         L.scales[m] = s;
         if (L.cerr) L.cerr[m] = __fmul_rn(__ll2float_rn(ec), 0x1p-30f);
     }

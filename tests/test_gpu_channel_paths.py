@@ -311,3 +311,29 @@ def test_freeing_scratch_leaves_captures_of_other_streams_alone():
     graph.replay()
     sq.squant_device_status()
     assert np.array_equal(b.codes.cpu().numpy(), oracle.quantize_layer(w, bits=4).codes)
+
+
+@pytest.mark.parametrize("n", [8193, 8196, 12290, 16384, 16387, 32767])
+def test_long_rows(n):
+    """1x1 rows of the row kernel: both of its sizes, lengths around their limits, rows that start anywhere, hundreds
+    of flips and massive ties (full lists, the exact search), every output form."""
+    assert sq.squant_plan_kernels([(3, n, 1, 1)]) == ["row"]
+    ws = layers((3, n, 1, 1), n)
+    check(ws, 4)
+    check(ws, 8, flags=0, start=1, outputs=True)
+    check(ws, 3, flags=sq.FLAG_NARROW_RANGE | sq.FLAG_PACK_INT4, start=2)
+    check(ws, 4, mode=sq.MODE_E, outputs=True)
+    check(ws, 4, start=3, clip=0.7)
+    check(ws[:1], 2, flags=0, outputs=True, clip=0.98)
+
+
+def test_wide_rows_without_supplied_scales():
+    """Rows of a cluster on either side of 2^16 elements, from where a flip can be barred without a supplied scale too:
+    every alignment and output form, hundreds of flips."""
+    shapes = [(2, 100353, 1, 1), (3, 65541, 1, 1), (1, 65536, 1, 1), (2, 50000, 1, 1)]
+    assert set(sq.squant_plan_kernels(shapes)) == {"cluster"}
+    ws = [adversarial_layer(s, seed=i) for i, s in enumerate(shapes)] + [np.abs(W.random_layer((1, 70001, 1, 1), 9))]
+    check(ws, 4, start=1)
+    check(ws, 8, flags=0, outputs=True)
+    check(ws, 4, flags=sq.FLAG_NARROW_RANGE | sq.FLAG_PACK_INT4, start=2)
+    check(ws, 4, clip=0.8)
