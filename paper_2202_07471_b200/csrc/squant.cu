@@ -447,10 +447,7 @@ int build_param_plan(const squant_layer *layers, int32_t n_layers, const squant_
             if (kernels) kernels[i] = SQUANT_KERNEL_STREAM;
             continue;
         }
-        // rows too long for a group, as far as a thread block's shared memory holds them with codes to be packed (44.7 K weights;
-        // the staged body of the grouped kernel takes five times as long: 1024 rows of 40,000 weights 472 us against 102 here,
-        // 16 of them 76 against 27)
-        if (descs[i].K == 1 && descs[i].off_hist != 0 && sq::long_row_bytes(sq::kBlockThreads, (descs[i].N + 6) >> 2, true, sq::kBlock) <= max_smem) {
+        if (descs[i].K == 1 && descs[i].off_hist != 0 && descs[i].N <= sq::kRowBlockElems) {   // too long for a group, 164 KB at most
             rows.push_back(i);
             if (kernels) kernels[i] = SQUANT_KERNEL_ROW;
             continue;

@@ -20,6 +20,10 @@ namespace sq {
 
 static_assert(kBlockThreads == 1 << 9, "");
 constexpr int kWideMaxCluster = 8;
+// Longest row of the row kernel (164 KB of shared memory); up to here it was laid out and compared with the staged
+// body of the grouped kernel.  Longer rows that fit one thread block still take that body, which is the slower one
+// there: 1024 rows of 32,772 weights 318 us against 99 in this kernel, of 40,000 480 against 116, 16 rows of 40,000 83 against 22.
+constexpr int kRowBlockElems = 32768;
 
 // ---------------------------------------------------------------- SQuant-E on four weights of a 1x1 row
 struct Quad {

@@ -337,13 +337,3 @@ def test_wide_rows_without_supplied_scales():
     check(ws, 8, flags=0, outputs=True)
     check(ws, 4, flags=sq.FLAG_NARROW_RANGE | sq.FLAG_PACK_INT4, start=2)
     check(ws, 4, clip=0.8)
-
-
-@pytest.mark.parametrize("n", [32769, 40000, 44001, 44700])
-def test_rows_up_to_one_thread_blocks_shared_memory(n):
-    """The longest rows of the row kernel."""
-    assert sq.squant_plan_kernels([(2, n, 1, 1)]) == ["row"]
-    ws = [adversarial_layer((2, n, 1, 1), seed=n)]
-    check(ws, 4)
-    check(ws, 6, flags=0, start=1, outputs=True, clip=0.9)
-    check(ws, 4, flags=sq.FLAG_NARROW_RANGE | sq.FLAG_PACK_INT4, start=3)
