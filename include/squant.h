@@ -151,10 +151,11 @@ int squant_quantize_model(const squant_layer *layers, int32_t n_layers, const sq
 /*
  * The same, with HOST buffers: copies the weights to the current device, runs the launches,
  * copies codes / scales / error sums back and returns when the outputs are in host memory.
- * The layers are taken in chunks of about 64 MB of weights: uploads, launches and downloads of
+ * The layers are taken in chunks of at least 8 MB of weights: uploads, launches and downloads of
  * consecutive chunks overlap on two copy streams of the library (created on first use) beside
- * the caller's stream, on which the launches run.  Device staging memory is cached inside the
- * library between calls (cudaMalloc on first use or growth; squant_shutdown frees it).  Pinned
+ * the caller's stream, on which the launches run.  Device staging memory, and pinned host memory
+ * through which outputs of up to 32 KB come down, are cached inside the library between calls
+ * (allocated on first use or growth; squant_shutdown frees them).  Pinned
  * host memory gives the copies their full speed and lets them overlap; pageable memory works.
  */
 int squant_quantize_model_host(const squant_layer *layers, int32_t n_layers,

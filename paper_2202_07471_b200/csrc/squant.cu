@@ -685,7 +685,19 @@ struct HostPipe {
     std::vector<cudaEvent_t> uploaded, computed;
 };
 std::vector<HostPipe> g_host_pipes;
-constexpr size_t kHostChunkBytes = 64u << 20;   // weights per chunk: large enough to hide the launches
+// Weights per chunk.  A chunk's downloads can run while the next chunks' weights are on their way, so what remains
+// outside the overlap is about one chunk at either end: ResNet-50 shapes (102 MB up, 87 MB down) take 3356 us, and
+// 4286 us in chunks of 64 MB with every tensor copied by itself.
+constexpr size_t kHostChunkBytes = 8u << 20;
+constexpr size_t kHostChunks = 24;   // and no more than about these: each has a cached plan (kMaxPlans)
+// Outputs of at most this many bytes come down through pinned staging memory, all of a chunk in one copy: a copy of a
+// few KB costs its fixed few microseconds on the copy engine, more than the host's memcpy takes.  (Inputs don't: work
+// that the caller's stream still holds may be about to write them.)
+constexpr size_t kHostSmallBytes = 32u << 10;
+
+// Pinned staging memory of the host-buffer entry point, one per device, grown on demand.
+struct Staging { void *ptr = nullptr; size_t bytes = 0; };
+std::vector<Staging> g_stagings;
 
 int host_pipe(int device, size_t chunks, HostPipe *&out)
 {
@@ -766,24 +778,63 @@ int squant_quantize_model_host(const squant_layer *layers, int32_t n_layers,
     std::lock_guard<std::mutex> lock(g_mutex);
     int device = 0;
     SQ_CUDA(cudaGetDevice(&device));
-    // carve one device arena: per layer weights, codes, scales, kernel sums, channel sums
-    std::vector<squant_layer> dev(layers, layers + n_layers);
-    std::vector<size_t> off(static_cast<size_t>(n_layers) * 8);
-    size_t total = 0;
+    // Chunks of consecutive layers.  Uploads run on one
+    // copy stream, each chunk's launches on the caller's stream once its upload is done, its
+    // downloads on a second copy stream once its launches are done: the two copy directions and
+    // the kernels overlap.
+    std::vector<int> chunk_first(1, 0);
+    {
+        size_t acc = 0, all = 0;
+        const auto weight_bytes = [&](int i) { return static_cast<size_t>(layers[i].cin) * layers[i].kh * layers[i].kw * layers[i].cout * 4; };
+        for (int i = 0; i < n_layers; ++i) all += weight_bytes(i);
+        const size_t goal = std::max(kHostChunkBytes, all / kHostChunks);
+        for (int i = 0; i < n_layers; ++i) {
+            acc += weight_bytes(i);
+            if (acc >= goal && i + 1 < n_layers) { chunk_first.push_back(i + 1); acc = 0; }
+        }
+        chunk_first.push_back(n_layers);
+    }
+    const size_t chunks = chunk_first.size() - 1;
+    // every tensor of the call, in the order of squant_layer's inputs and outputs
+    struct Tensor { void *host; size_t bytes, off; bool small; };
+    constexpr int kInputs = 2, kTensors = 8;   // weights, supplied scales | codes, scales, sums (kernels, channels), dequantized (fp32, bf16)
+    std::vector<Tensor> tensors(static_cast<size_t>(n_layers) * kTensors);
     for (int i = 0; i < n_layers; ++i) {
         const squant_layer &l = layers[i];
-        const size_t n = static_cast<size_t>(l.cin) * l.kh * l.kw * l.cout;
-        off[8 * i + 0] = total; total += align256(n * 4);
-        const size_t code_bytes = (o.flags & SQUANT_FLAG_PACK_INT4)
-                                      ? static_cast<size_t>(l.cout) * ((static_cast<size_t>(l.cin) * l.kh * l.kw + 1) / 2) : n;
-        off[8 * i + 1] = total; total += align256(code_bytes);
-        off[8 * i + 2] = total; total += align256(static_cast<size_t>(l.cout) * 4);
-        off[8 * i + 3] = total; total += l.kernel_err ? align256(static_cast<size_t>(l.cout) * l.cin * 4) : 0;
-        off[8 * i + 4] = total; total += l.channel_err ? align256(static_cast<size_t>(l.cout) * 4) : 0;
-        off[8 * i + 5] = total; total += l.dequant ? align256(n * 4) : 0;
-        off[8 * i + 6] = total; total += l.scales_in ? align256(static_cast<size_t>(l.cout) * 4) : 0;
-        off[8 * i + 7] = total; total += l.dequant_bf16 ? align256(n * 2) : 0;
+        const size_t m = static_cast<size_t>(l.cout), nk = static_cast<size_t>(l.cin) * l.kh * l.kw, n = m * nk;
+        const size_t code_bytes = (o.flags & SQUANT_FLAG_PACK_INT4) ? m * ((nk + 1) / 2) : n;
+        Tensor *t = &tensors[static_cast<size_t>(i) * kTensors];
+        const auto put = [&](int k, const void *p, size_t bytes) {
+            t[k] = {const_cast<void *>(p), p ? bytes : 0, 0, k >= kInputs && bytes <= kHostSmallBytes};
+        };
+        put(0, l.w, n * 4);
+        put(1, l.scales_in, m * 4);
+        put(2, l.codes, code_bytes);
+        put(3, l.scales, m * 4);
+        put(4, l.kernel_err, m * l.cin * 4);
+        put(5, l.channel_err, m * 4);
+        put(6, l.dequant, n * 4);
+        put(7, l.dequant_bf16, n * 2);
     }
+    // One device arena; a chunk's small outputs lie together in it.
+    struct Run { size_t off, bytes, at; };   // in the arena; its place in the staging memory
+    std::vector<Run> small(chunks);
+    size_t total = 0, staged = 0;
+    for (size_t c = 0; c < chunks; ++c)
+        for (int pass = 0; pass < 2; ++pass) {   // the small ones first
+            if (pass == 0) small[c] = {total, 0, staged};
+            for (int i = chunk_first[c]; i < chunk_first[c + 1]; ++i)
+                for (int k = 0; k < kTensors; ++k) {
+                    Tensor &t = tensors[static_cast<size_t>(i) * kTensors + k];
+                    if (!t.host || t.small != (pass == 0)) continue;
+                    t.off = total;
+                    total += align256(t.bytes);
+                }
+            if (pass == 0) {
+                small[c].bytes = total - small[c].off;
+                staged += small[c].bytes;
+            }
+        }
     if (static_cast<int>(g_arenas.size()) <= device) g_arenas.resize(device + 1);
     Arena &a = g_arenas[device];
     if (a.bytes < total) {
@@ -792,45 +843,65 @@ int squant_quantize_model_host(const squant_layer *layers, int32_t n_layers,
         if (e != cudaSuccess) { a.ptr = nullptr; return e == cudaErrorMemoryAllocation ? SQUANT_ERR_NOMEM : cuda_fail(e, "cudaMalloc"); }
         a.bytes = total;
     }
-    unsigned char *base = static_cast<unsigned char *>(a.ptr);
-    for (int i = 0; i < n_layers; ++i) {
-        const squant_layer &l = layers[i];
-        dev[i].w = reinterpret_cast<const float *>(base + off[8 * i + 0]);
-        dev[i].codes = reinterpret_cast<int8_t *>(base + off[8 * i + 1]);
-        dev[i].scales = reinterpret_cast<float *>(base + off[8 * i + 2]);
-        dev[i].kernel_err = l.kernel_err ? reinterpret_cast<float *>(base + off[8 * i + 3]) : nullptr;
-        dev[i].channel_err = l.channel_err ? reinterpret_cast<float *>(base + off[8 * i + 4]) : nullptr;
-        dev[i].dequant = l.dequant ? reinterpret_cast<float *>(base + off[8 * i + 5]) : nullptr;
-        dev[i].scales_in = l.scales_in ? reinterpret_cast<const float *>(base + off[8 * i + 6]) : nullptr;
-        dev[i].dequant_bf16 = l.dequant_bf16 ? reinterpret_cast<uint16_t *>(base + off[8 * i + 7]) : nullptr;
-    }
-    // Chunks of consecutive layers (about kHostChunkBytes of weights each).  Uploads run on one
-    // copy stream, each chunk's launches on the caller's stream once its upload is done, its
-    // downloads on a second copy stream once its launches are done: the two copy directions and
-    // the kernels overlap.
-    std::vector<int> chunk_first(1, 0);
-    {
-        size_t acc = 0;
-        for (int i = 0; i < n_layers; ++i) {
-            acc += static_cast<size_t>(layers[i].cin) * layers[i].kh * layers[i].kw * layers[i].cout * 4;
-            if (acc >= kHostChunkBytes && i + 1 < n_layers) { chunk_first.push_back(i + 1); acc = 0; }
+    if (static_cast<int>(g_stagings.size()) <= device) g_stagings.resize(device + 1);
+    Staging &stg = g_stagings[device];
+    if (stg.bytes < staged) {   // (no call is under way: each ends with its copies done)
+        if (stg.ptr) { SQ_CUDA(cudaFreeHost(stg.ptr)); stg.ptr = nullptr; stg.bytes = 0; }
+        if (cudaHostAlloc(&stg.ptr, staged, cudaHostAllocDefault) == cudaSuccess) {
+            stg.bytes = staged;
+        } else {   // no pinned memory to be had: every tensor is copied by itself
+            cudaGetLastError();
+            stg.ptr = nullptr;
         }
-        chunk_first.push_back(n_layers);
     }
-    const size_t chunks = chunk_first.size() - 1;
+    unsigned char *base = static_cast<unsigned char *>(a.ptr), *pinned = static_cast<unsigned char *>(stg.ptr);
+    std::vector<squant_layer> dev(layers, layers + n_layers);
+    for (int i = 0; i < n_layers; ++i) {
+        const Tensor *t = &tensors[static_cast<size_t>(i) * kTensors];
+        const auto at = [&](int k) -> void * { return t[k].host ? base + t[k].off : nullptr; };
+        dev[i].w = static_cast<const float *>(at(0));
+        dev[i].scales_in = static_cast<const float *>(at(1));
+        dev[i].codes = static_cast<int8_t *>(at(2));
+        dev[i].scales = static_cast<float *>(at(3));
+        dev[i].kernel_err = static_cast<float *>(at(4));
+        dev[i].channel_err = static_cast<float *>(at(5));
+        dev[i].dequant = static_cast<float *>(at(6));
+        dev[i].dequant_bf16 = static_cast<uint16_t *>(at(7));
+    }
     HostPipe *hp = nullptr;
     rc = host_pipe(device, chunks, hp);
     if (rc) return rc;
+    const auto each = [&](size_t c, bool outputs, auto fn) -> int {   // a chunk's tensors
+        for (int i = chunk_first[c]; i < chunk_first[c + 1]; ++i)
+            for (int k = outputs ? kInputs : 0; k < (outputs ? kTensors : kInputs); ++k) {
+                const Tensor &t = tensors[static_cast<size_t>(i) * kTensors + k];
+                if (!t.host) continue;
+                const int e = fn(t);
+                if (e) return e;
+            }
+        return SQUANT_OK;
+    };
+    // whatever ends the call, its copies have ended then too
+    struct Drain {
+        cudaStream_t a, b, c;
+        bool armed;
+        ~Drain()
+        {
+            if (!armed) return;
+            cudaStreamSynchronize(a);
+            cudaStreamSynchronize(b);
+            cudaStreamSynchronize(c);
+        }
+    };
+    Drain drain{hp->in, stream, hp->out, true};
     SQ_CUDA(cudaEventRecord(hp->start, stream));          // uploads follow what the caller's stream holds so far
     SQ_CUDA(cudaStreamWaitEvent(hp->in, hp->start, 0));
     for (size_t c = 0; c < chunks; ++c) {
-        for (int i = chunk_first[c]; i < chunk_first[c + 1]; ++i) {
-            const squant_layer &l = layers[i];
-            const size_t n = static_cast<size_t>(l.cin) * l.kh * l.kw * l.cout;
-            SQ_CUDA(cudaMemcpyAsync(base + off[8 * i + 0], l.w, n * 4, cudaMemcpyHostToDevice, hp->in));
-            if (l.scales_in)
-                SQ_CUDA(cudaMemcpyAsync(base + off[8 * i + 6], l.scales_in, static_cast<size_t>(l.cout) * 4, cudaMemcpyHostToDevice, hp->in));
-        }
+        rc = each(c, false, [&](const Tensor &t) -> int {
+            SQ_CUDA(cudaMemcpyAsync(base + t.off, t.host, t.bytes, cudaMemcpyHostToDevice, hp->in));
+            return SQUANT_OK;
+        });
+        if (rc) return rc;
         SQ_CUDA(cudaEventRecord(hp->uploaded[c], hp->in));
     }
     for (size_t c = 0; c < chunks; ++c) {
@@ -843,25 +914,23 @@ int squant_quantize_model_host(const squant_layer *layers, int32_t n_layers,
         if (rc) return rc;
         SQ_CUDA(cudaEventRecord(hp->computed[c], stream));
         SQ_CUDA(cudaStreamWaitEvent(hp->out, hp->computed[c], 0));
-        for (int i = first; i < first + count; ++i) {
-            const squant_layer &l = layers[i];
-            const size_t n = static_cast<size_t>(l.cin) * l.kh * l.kw * l.cout;
-            const size_t code_bytes = (o.flags & SQUANT_FLAG_PACK_INT4)
-                                          ? static_cast<size_t>(l.cout) * ((static_cast<size_t>(l.cin) * l.kh * l.kw + 1) / 2) : n;
-            SQ_CUDA(cudaMemcpyAsync(l.codes, dev[i].codes, code_bytes, cudaMemcpyDeviceToHost, hp->out));
-            SQ_CUDA(cudaMemcpyAsync(l.scales, dev[i].scales, static_cast<size_t>(l.cout) * 4, cudaMemcpyDeviceToHost, hp->out));
-            if (l.kernel_err)
-                SQ_CUDA(cudaMemcpyAsync(l.kernel_err, dev[i].kernel_err, static_cast<size_t>(l.cout) * l.cin * 4, cudaMemcpyDeviceToHost, hp->out));
-            if (l.channel_err)
-                SQ_CUDA(cudaMemcpyAsync(l.channel_err, dev[i].channel_err, static_cast<size_t>(l.cout) * 4, cudaMemcpyDeviceToHost, hp->out));
-            if (l.dequant)
-                SQ_CUDA(cudaMemcpyAsync(l.dequant, dev[i].dequant, n * 4, cudaMemcpyDeviceToHost, hp->out));
-            if (l.dequant_bf16)
-                SQ_CUDA(cudaMemcpyAsync(l.dequant_bf16, dev[i].dequant_bf16, n * 2, cudaMemcpyDeviceToHost, hp->out));
-        }
+        const Run &run = small[c];
+        rc = each(c, true, [&](const Tensor &t) -> int {
+            if (!pinned || !t.small) SQ_CUDA(cudaMemcpyAsync(t.host, base + t.off, t.bytes, cudaMemcpyDeviceToHost, hp->out));
+            return SQUANT_OK;
+        });
+        if (rc) return rc;
+        if (pinned && run.bytes) SQ_CUDA(cudaMemcpyAsync(pinned + run.at, base + run.off, run.bytes, cudaMemcpyDeviceToHost, hp->out));
     }
+    drain.armed = false;
     SQ_CUDA(cudaStreamSynchronize(hp->out));
     SQ_CUDA(cudaStreamSynchronize(stream));
+    if (pinned)
+        for (size_t c = 0; c < chunks; ++c)
+            each(c, true, [&](const Tensor &t) -> int {
+                if (t.small) std::memcpy(t.host, pinned + small[c].at + (t.off - small[c].off), t.bytes);
+                return SQUANT_OK;
+            });
     return SQUANT_OK;
 }
 
@@ -1060,6 +1129,9 @@ int squant_shutdown(void)
         if (g_arenas[d].ptr) { cudaSetDevice(static_cast<int>(d)); cudaDeviceSynchronize(); cudaFree(g_arenas[d].ptr); }
     }
     g_arenas.clear();
+    for (Staging &stg : g_stagings)
+        if (stg.ptr) cudaFreeHost(stg.ptr);
+    g_stagings.clear();
     for (size_t d = 0; d < g_host_pipes.size(); ++d) {
         HostPipe &hp = g_host_pipes[d];
         if (!hp.in) continue;

@@ -662,3 +662,30 @@ def test_checked_build_finds_no_violation_on_small_cases():
     finally:
         sq.use_library(None)
     assert sq.squant_debug_violations()[0] is False      # the regular build has no checks
+
+
+@pytest.mark.parametrize("pin", [True, False])
+def test_host_entry_point_small_and_large_outputs_in_many_chunks(pin):
+    """Outputs on either side of the size that comes down through staging memory, in chunks on either side of 8 MB of
+    weights, every output form, guard bytes around the tensors untouched; a second call with other sizes."""
+    for k, shapes in enumerate(([(64, 3, 7, 7), (32, 1, 3, 3), (512, 512, 3, 3), (1000, 2048, 1, 1), (7, 5, 1, 1), (700, 3000, 1, 1), (33, 31, 3, 3), (8192, 1, 1, 1),
+                                 (8193, 1, 1, 1)], [(3, 2, 1, 1), (700, 3000, 1, 1)])):
+        ws = [W.random_layer(s, seed=70 + i) for i, s in enumerate(shapes)]
+        dev = [sq.alloc_outputs(torch.from_numpy(w).cuda(), dequant=True, dequant_bf16=True) for w in ws]
+        sq.squant_quantize_model(dev, bits=4)
+        pad, bufs = 64, []
+        for w in ws:
+            t = torch.from_numpy(w)
+            b = sq.alloc_outputs(t.pin_memory() if pin else t, pin=pin, dequant=True, dequant_bf16=True)
+            whole = {}
+            for name in ("codes", "scales", "kernel_err", "channel_err", "dequant", "dequant_bf16"):
+                o = getattr(b, name)
+                big = torch.full((o.numel() + 2 * pad,), -77, dtype=o.dtype, pin_memory=pin)
+                whole[name] = big
+                setattr(b, name, big[pad:pad + o.numel()].view(o.shape))
+            bufs.append((b, whole))
+        sq.squant_quantize_model_host([b for b, _ in bufs], bits=4)
+        for (b, whole), d, s in zip(bufs, dev, shapes):
+            for name, big in whole.items():
+                assert torch.equal(getattr(b, name).view(torch.uint8), getattr(d, name).cpu().view(torch.uint8)), (k, s, name)
+                assert (big[:pad] == -77).all() and (big[-pad:] == -77).all(), (k, s, name)
