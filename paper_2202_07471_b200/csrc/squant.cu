@@ -456,12 +456,18 @@ int build_param_plan(const squant_layer *layers, int32_t n_layers, const squant_
         if (kernels) kernels[i] = SQUANT_KERNEL_GROUPED;
     }
     // long rows, longest first: a thread block per output channel
+    // Rows of up to 16 K weights take 256 threads if they are more than one wave of such thread blocks (four per
+    // multiprocessor), else 512: fewer rows take the time of one row's chain (512 rows of 16,000 weights 30.2 us with 256 threads,
+    // 25.4 with 512; of 12,000 24.8, 23.3; 1000 of 12,000 33.1, 37.3; 2000 of 10,000 50.0, 63.5).
     std::stable_sort(rows.begin(), rows.end(), [&](int a, int b) { return descs[a].N > descs[b].N; });
+    int64_t short_rows = 0;
+    for (int i : rows) short_rows += descs[i].N <= sq::kRowSmallElems ? descs[i].M : 0;
+    const int small_limit = short_rows > 4ll * sms ? sq::kRowSmallElems : 0;
     for (size_t base = 0; base < rows.size();) {
-        const bool small = descs[rows[base]].N <= sq::kRowSmallElems;
+        const bool small = descs[rows[base]].N <= small_limit;
         size_t n = 0;
         int smem = 0;
-        while (base + n < rows.size() && n < sq::kMaxParamLayers && (descs[rows[base + n]].N <= sq::kRowSmallElems) == small) {
+        while (base + n < rows.size() && n < sq::kMaxParamLayers && (descs[rows[base + n]].N <= small_limit) == small) {
             LayerDesc &d = descs[rows[base + n]];
             d.off_vi = (d.N + 6) >> 2;
             d.off_ev = regular_rows(d);

@@ -457,7 +457,7 @@ __device__ __forceinline__ void long_row_body(const LayerDesc &L, int m, const G
 }
 
 // Rows of more than 8 K weights, one thread block per output channel.
-// kThreads = 256 for rows of up to 16 K weights, 512 beyond: about eleven vectors a thread, over which the code that
+// kThreads = 256 for many rows of up to 16 K weights, 512 else: about eleven vectors a thread, over which the code that
 // runs once is spread (4096 rows of 11,008 weights at 8 bit:
 // 85 us, 115 with 512 threads).
 constexpr int kRowSmallElems = 16384;

@@ -319,7 +319,7 @@ def test_long_rows(n):
     of flips and massive ties (full lists, the exact search), every output form."""
     assert sq.squant_plan_kernels([(3, n, 1, 1)]) == ["row"]
     ws = layers((3, n, 1, 1), n)
-    check(ws, 4)
+    check(ws + ([adversarial_layer((600, n, 1, 1), seed=1)] if n <= 16384 else []), 4)   # more than one wave: the smaller thread blocks
     check(ws, 8, flags=0, start=1, outputs=True)
     check(ws, 3, flags=sq.FLAG_NARROW_RANGE | sq.FLAG_PACK_INT4, start=2)
     check(ws, 4, mode=sq.MODE_E, outputs=True)
