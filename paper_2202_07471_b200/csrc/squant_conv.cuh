@@ -384,10 +384,11 @@ __device__ __forceinline__ void conv_body(const LayerDesc &L, int m, const Group
     }
 
     // ---- channel sum
+    const bool late = KT == 0 && kOwn != kCluster && g > 32 && late_maxima(K);
     long long ec = 0;
     int up = hi0, down = -lo0;   // the channel's extremes
     if ((mode & 4u) || L.cerr) {
-        if (kOwn != kCluster && g > 32) {   // the maxima that SQuant-C looks for its bound among
+        if (kOwn != kCluster && g > 32 && !late) {   // the maxima that SQuant-C looks for its bound among
             S.mx[G.t] = hi0;
             S.mx[G.t + g] = -lo0;
         }
@@ -401,8 +402,12 @@ __device__ __forceinline__ void conv_body(const LayerDesc &L, int m, const Group
         const int kc = static_cast<int>(min((abs_e + (kHalf - 1)) >> 30, 1ll << 30));   // a clipped channel's sum can be huge
         if (kc > 0) {   // uniform in the group
             const int m0 = sgn > 0 ? hi0 : -lo0;
-            const int *mx = sgn > 0 ? S.mx : S.mx + g;
+            const int *mx = sgn > 0 || late ? S.mx : S.mx + g;
             const int lane = threadIdx.x & 31;
+            if (late) {
+                S.mx[G.t] = m0;
+                G.sync();
+            }
             auto count = [&](int t, int it) {
                 int c;
                 if (kOwn == kCluster) {

@@ -55,10 +55,6 @@ struct WarpPart {
     int lo32, hi32;   // the error sum: modulo 2^32 and, in units of 2^17, its size; or both halves of 64 bits
     int up, down;     // largest candidate of each sign
 };
-struct SelWarps {
-    unsigned amax[kMaxWarps];
-    WarpPart part[kMaxWarps];
-};
 
 // Who owns a channel: a group inside a thread block, a whole thread block, a cluster of thread blocks
 // (each a run of the channel's kernels; they read each other's control words and lists through
@@ -69,12 +65,28 @@ constexpr int kBlockThreads = 512;   // kBlock, kCluster
 // and leave little shared memory: short lists there.
 __host__ __device__ constexpr int merged_cap(int K) { return K > 16 ? 128 : 1024; }
 
-__host__ __device__ constexpr int sel_cap(int g, int K = 1) { return g <= 64 || (g > 256 && K > 16) ? 64 : (K > 1 && g <= 256 ? 128 : g); }
+// Warps that have a place for their parts.
+__host__ __device__ constexpr int sel_warps(int g, Owner own, int K) { return g <= 32 ? 0 : (own == kGroup && K > 1 ? g >> 5 : kMaxWarps); }
+// Kernels of more than nine elements: a thread's maximum is put in when the direction of the flips is known, one word
+// instead of two and a barrier more, which the few kernels of such a channel hardly notice.
+__host__ __device__ constexpr bool late_maxima(int K) { return K > 9; }
+// Entries of a list.  Groups of 64, 128 and 256 threads on larger kernels: as many as make the group's selection memory
+// 1,072, 2,160 and 3,120 B, with late maxima 1,072, 1,584 and 3,120 B.  The last figure is part of the longest
+// channel that a thread block takes; the others decide how many channels share one (512 channels of 106 7x7 kernels,
+// four layers: two channels to a thread block 49.6 us on a B200, one 70.9).
+__host__ __device__ constexpr int sel_cap(int g, int K = 1)
+{
+    return K == 1 ? (g <= 64 ? 64 : g)
+         : g > 256 ? (K > 16 ? 64 : g)
+         : g <= 32 ? 64
+         : late_maxima(K) ? (g == 64 ? 93 : (g == 128 ? 120 : 238))
+                          : (g == 64 ? 61 : (g == 128 ? 128 : 110));
+}
 // Maxima that a group leaves in shared memory: one per thread and sign, of 1x1 channels two up to 64 threads.
-__host__ __device__ constexpr int sel_maxima(int g, int K) { return K == 1 && g <= 64 ? 4 * g : 2 * g; }
+__host__ __device__ constexpr int sel_maxima(int g, int K) { return K == 1 && g <= 64 ? 4 * g : (late_maxima(K) ? g : 2 * g); }
 __host__ __device__ constexpr int sel_bytes(int g, Owner own = kGroup, int K = 1)
 {
-    return static_cast<int>(sizeof(SelScratch)) + (g > 32 ? static_cast<int>(sizeof(SelWarps)) : 0) + 8 * sel_cap(g, K) +
+    return static_cast<int>(sizeof(SelScratch)) + 20 * sel_warps(g, own, K) + 8 * sel_cap(g, K) +
            (own == kCluster ? 8 * merged_cap(K) : (g > 32 ? 4 * sel_maxima(g, K) : 0));
 }
 // Shared memory of a 1x1 channel of `vecs` vectors: selection, perturbations, codes.
@@ -85,15 +97,18 @@ __host__ __device__ constexpr int long_row_bytes(int g, int vecs, bool pack, Own
 // The parts of a group's selection memory.
 struct Sel {
     SelScratch *sc;
-    SelWarps *warps;
+    WarpPart *part;   // of every warp
+    unsigned *amax;   // the same
     unsigned long long *list;
     int *mx;   // the threads' maxima (not kCluster: the lists of all thread blocks are there)
     int cap;
     __device__ __forceinline__ Sel(unsigned char *slice, int g, Owner own, int K)
     {
+        const int warps = sel_warps(g, own, K);
         sc = reinterpret_cast<SelScratch *>(slice);
-        warps = reinterpret_cast<SelWarps *>(sc + 1);
-        list = reinterpret_cast<unsigned long long *>(slice + sizeof(SelScratch) + (g > 32 ? sizeof(SelWarps) : 0));
+        part = reinterpret_cast<WarpPart *>(sc + 1);
+        amax = reinterpret_cast<unsigned *>(part + warps);
+        list = reinterpret_cast<unsigned long long *>(amax + warps);
         cap = sel_cap(g, K);
         mx = reinterpret_cast<int *>(list + cap);
     }
@@ -179,15 +194,15 @@ __device__ __forceinline__ float owner_absmax(const Group &G, float amax, const 
         __syncwarp();   // the control words are cleared
         return __uint_as_float(u);
     }
-    if (lane == 0) S.warps->amax[G.t >> 5] = u;
+    if (lane == 0) S.amax[G.t >> 5] = u;
     owner_sync<kOwn>(G);
     if (kOwn == kCluster) {
         const int c = lane >> 2;   // a lane reads four of a thread block's sixteen warps
         const uint4 q = c < static_cast<int>(cg::this_cluster().num_blocks())
-                            ? remote(reinterpret_cast<const uint4 *>(S.warps->amax) + (lane & 3), c) : make_uint4(0u, 0u, 0u, 0u);
+                            ? remote(reinterpret_cast<const uint4 *>(S.amax) + (lane & 3), c) : make_uint4(0u, 0u, 0u, 0u);
         u = max(max(q.x, q.y), max(q.z, q.w));
     } else {
-        u = S.warps->amax[lane & ((G.g >> 5) - 1)];
+        u = S.amax[lane & ((G.g >> 5) - 1)];
     }
     return __uint_as_float(__reduce_max_sync(kFull, u));
 }
@@ -216,7 +231,7 @@ __device__ __forceinline__ long long owner_sum(const Group &G, const Sel &S, lon
             p.hi32 = k64 ? static_cast<int>(e >> 32) : apx;
             p.up = up;
             p.down = down;
-            *reinterpret_cast<int4 *>(S.warps->part + (G.t >> 5)) = make_int4(p.lo32, p.hi32, p.up, p.down);
+            *reinterpret_cast<int4 *>(S.part + (G.t >> 5)) = make_int4(p.lo32, p.hi32, p.up, p.down);
         }
         owner_sync<kOwn>(G);
         int4 q[4];
@@ -226,9 +241,9 @@ __device__ __forceinline__ long long owner_sum(const Group &G, const Sel &S, lon
             const bool there = c < static_cast<int>(cg::this_cluster().num_blocks());
 #pragma unroll
             for (int i = 0; i < 4; ++i)
-                q[i] = there ? remote(reinterpret_cast<const int4 *>(S.warps->part) + 4 * (lane & 3) + i, c) : make_int4(0, 0, 0, 0);
+                q[i] = there ? remote(reinterpret_cast<const int4 *>(S.part) + 4 * (lane & 3) + i, c) : make_int4(0, 0, 0, 0);
         } else {
-            q[0] = lane < (G.g >> 5) ? reinterpret_cast<const int4 *>(S.warps->part)[lane] : make_int4(0, 0, 0, 0);
+            q[0] = lane < (G.g >> 5) ? reinterpret_cast<const int4 *>(S.part)[lane] : make_int4(0, 0, 0, 0);
         }
         if (k64) {
             e = 0;
@@ -278,7 +293,7 @@ __device__ __forceinline__ float absmax_scale(float amax, int qmax)
 __device__ __forceinline__ void debug_check_sum(const Group &G, const float *w, const unsigned char *codes, int n, float s, long long ec, bool valid,
                                                 const Sel &S)
 {
-    unsigned long long *sum64 = reinterpret_cast<unsigned long long *>(S.warps->amax);   // (dead by now)
+    unsigned long long *sum64 = reinterpret_cast<unsigned long long *>(S.amax);   // (dead by now)
     long long e = 0;
     for (int j = G.t; j < n; j += G.g) e += debug_error(w[j], s, static_cast<signed char>(codes[j]));
     for (int o = min(G.g, 32) >> 1; o > 0; o >>= 1) e += __shfl_xor_sync(kFull, e, o);

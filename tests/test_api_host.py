@@ -109,6 +109,25 @@ def test_limit_of_the_cluster_kernel(k):
             assert ei.value.code == -6, n
 
 
+@pytest.mark.parametrize("n,k", [(1, 45857), (2, 22928), (3, 15285), (9, 5095), (17, 2697), (191, 240), (200, 229)])
+def test_limit_of_few_large_kernels_in_one_thread_block(n, k):
+    """Channels of few large kernels are taken up to these sizes: what a thread block holds at 5 B a weight beside
+    3,120 B for the selection."""
+    for mode in (sq.MODE_EKC, sq.MODE_E | sq.MODE_K):
+        assert _info([(2, n, 1, k)], mode=mode)["grid_ctas"] == 2
+        assert len(sq.squant_plan_kernels([(2, n, 1, k)], mode=mode)) == 1
+    with pytest.raises(sq.SquantError) as ei:
+        _info([(2, n, 1, k + 1)])
+    assert ei.value.code == -6
+
+
+@pytest.mark.parametrize("n,kh,kw,groups", [(106, 7, 7, 2), (108, 7, 7, 2), (212, 5, 5, 2), (13, 20, 20, 2), (18, 17, 17, 2),
+                                            (52, 7, 7, 4), (103, 5, 5, 4), (109, 7, 7, 1), (213, 5, 5, 1), (54, 7, 7, 2)])
+def test_channels_of_larger_kernels_that_share_a_thread_block(n, kh, kw, groups):
+    """As many channels of larger kernels share a thread block as leave room for four blocks on a multiprocessor."""
+    assert _info([(16, n, kh, kw)])["grid_ctas"] == 16 // groups
+
+
 def test_kernel_of_a_layer():
     shapes = [(64, 64, 3, 3), (8, 8192, 1, 1), (8, 8193, 1, 1), (8, 32768, 1, 1), (8, 40000, 1, 1), (8, 70000, 1, 1),
               (8, 2048, 3, 3), (8, 2049, 3, 3), (8, 2052, 3, 3), (8, 600, 5, 5), (8, 8192, 3, 3)]

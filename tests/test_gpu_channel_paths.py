@@ -85,6 +85,23 @@ def test_cluster_runs_of_an_even_number_of_kernels(shape):
     check(w, 8, flags=0, clip=0.98)
 
 
+@pytest.mark.parametrize("shape", [(2, 1, 1, 45857), (3, 2, 1, 22928), (2, 9, 1, 5095), (2, 200, 1, 229), (5, 106, 7, 7), (9, 52, 7, 7), (9, 103, 5, 5)])
+def test_larger_kernels_at_the_sizes_that_share_a_thread_block(shape):
+    """The longest channels of few large kernels that one thread block, or two and four channels that share one, hold;
+    in the table variant too."""
+    assert sq.squant_plan_kernels([shape]) == ["grouped"]
+    w = [adversarial_layer(shape, seed=shape[1])]
+    check(w, 4)
+    check(w, 8, flags=0, start=1, outputs=True)
+    check(w, 4, mode=sq.MODE_E | sq.MODE_K, start=3, clip=0.8)
+    b = sq.alloc_outputs(torch.from_numpy(w[0]).cuda())
+    sq.squant_quantize_layer_noalloc(b, bits=4)
+    sq.squant_device_status()
+    r = oracle.quantize_layer(w[0], bits=4)
+    assert np.array_equal(b.codes.cpu().numpy(), r.codes)
+    assert np.array_equal(b.kernel_err.cpu().numpy().view(np.uint32), r.kernel_err.view(np.uint32))
+
+
 @pytest.mark.parametrize("n", [1184, 1188, 1412, 2048])
 def test_long_channels_with_packed_and_dequantized_outputs(n):
     """Long 3x3 channels with further outputs: one, two, three and many channels per persistent thread block
