@@ -15,7 +15,7 @@
 //     distribution, and few other elements reach it (with k_c of m maxima about m ln(m / (m - k_c))
 //     elements).  T0 is searched among the maxima, the elements from T0 on are listed, and those of
 //     the first k_c ranks are flipped.  What that cannot settle (k_c beyond the number of maxima, a
-//     full list) goes to an exact search over the 48-bit keys.
+//     full list) goes to an exact search by counting.
 // With squant_conv.cuh: ResNet-50 shapes 84.5 -> 65.6 us device time on a B200, 55 thread-instructions per weight;
 // five linear layers of 125 M weights at 8 bit 267 -> 252 us.  With one barrier per reduction (a place for every warp
 // instead of shared atomics that have to be cleared first), loops counted without a division and the IEEE division out
@@ -365,7 +365,10 @@ __device__ __forceinline__ int select_top(const Group &G, Count count, Listing l
     bool slow = want && !sure;   // fewer than kc maxima are candidates at all
 
     // ---- list the elements from T0 on; where they are more than the list holds (many to a maximum: k_c is large
-    // for the number of maxima), once more from further up, supposing an even spread from T0 to the top
+    // for the number of maxima), once more from further up, supposing an even spread from T0 to the top.  Groups that
+    // share a warp go to the exact search at once, which takes them 8 to 10 k cycles where the other groups' lists, made again
+    // too, bring a second list to 16 to 24 k (ResNet-18 shapes with such a row among the last: 39.0 us on a B200, 36.5).
+    // From a warp a channel on the second list is the shorter way (4096 rows of 2048 weights 24.7 us, 28.0).
     int cnt = 0, all = 0;   // this list, all lists
     int k_eff = want ? kc : 0;
     const unsigned long long *merged = list;
@@ -396,6 +399,10 @@ __device__ __forceinline__ int select_top(const Group &G, Count count, Listing l
             full = cnt > cap;
         }
         full = full && want && !slow;
+        if (kOwn == kGroup && g < 32) {
+            slow = slow || full;
+            break;
+        }
         if (round > 0 && relist && all < kc) slow = true;   // (too far up)
         relist = full && round < 3;
         if (full && !relist) slow = true;
@@ -449,7 +456,8 @@ __device__ __forceinline__ int select_top(const Group &G, Count count, Listing l
 #pragma unroll 1
         for (int it = 0; __any_sync(kFull, phase < 2); ++it) {
             int c = 0;
-            if (phase < 2) each(phase == 0 ? vm : vlo, [&](int a, int n) { c += phase == 0 || (a == vlo && n < im) ? 1 : 0; });
+            if (phase == 0) each(vm, [&](int, int) { ++c; });
+            if (phase == 1) each(vlo, [&](int a, int n) { c += (a == vlo && n < im) ? 1 : 0; });
             c = lanes_add(g, c);
             if (g > 32) {
                 if (lane == 0) atomicAdd(&sc->total[it % 3], c);

@@ -85,6 +85,16 @@ def test_cluster_runs_of_an_even_number_of_kernels(shape):
     check(w, 8, flags=0, clip=0.98)
 
 
+@pytest.mark.parametrize("shape", [(4096, 250, 1, 1), (2048, 512, 1, 1), (1024, 1024, 1, 1), (300, 2048, 1, 1)])
+def test_rows_with_full_lists(shape):
+    """So many rows of normal weights that some have more candidates above the bound than their list holds: groups
+    that share a warp, of one warp and of two."""
+    w = W.random_layer(shape, seed=shape[1])
+    check([w, np.sign(w) * np.abs(w) ** np.float32(1.5)], 4)
+    check([w], 8, flags=0, start=1)
+    check([w], 4, start=2, clip=0.9)
+
+
 @pytest.mark.parametrize("shape", [(2, 1, 1, 45857), (3, 2, 1, 22928), (2, 9, 1, 5095), (2, 200, 1, 229), (5, 106, 7, 7), (9, 52, 7, 7), (9, 103, 5, 5)])
 def test_larger_kernels_at_the_sizes_that_share_a_thread_block(shape):
     """The longest channels of few large kernels that one thread block, or two and four channels that share one, hold;
