@@ -214,7 +214,7 @@ __device__ __forceinline__ void conv_body(const LayerDesc &L, int m, const Group
     if (G.t == 0) {
         S.sc->count = 0;
         S.sc->total[0] = 0;
-        S.sc->found[0] = 0;
+        clear_parts<kOwn>(S);
     }
     // ---- stage the row, take its absmax (each thread over what it has copied itself)
     const float *wrow = L.w + first;

@@ -131,7 +131,7 @@ __device__ __forceinline__ void long_row_body(const LayerDesc &L, int m, const G
     if (G.t == 0) {
         S.sc->count = 0;
         S.sc->total[0] = 0;
-        S.sc->found[0] = 0;
+        clear_parts<kOwn>(S);
     }
     const size_t first = static_cast<size_t>(m) * L.N + n0;   // of these elements in the layer
     const float *wrow = L.w + first;
