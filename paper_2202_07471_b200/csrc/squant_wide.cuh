@@ -222,7 +222,7 @@ __device__ __forceinline__ void long_row_body(const LayerDesc &L, int m, const G
     // error sum of an element: its perturbation rounded to units of 2^-30 (beyond 2^23 units the float is whole)
     auto esum_of = [&](float Pf) { return __fmul_rn(fabsf(Pf) < 0x1p30f ? __int2float_rn(__float2int_rn(Pf)) : Pf, 0x1p-30f); };
     const bool plain = R.fast && !pack && !deq && !deq16 &&
-                       (regular || (((reinterpret_cast<uintptr_t>(crow) - r) & 3) == 0 && ((reinterpret_cast<uintptr_t>(kerr) - 4 * r) & 15) == 0));
+                       (regular || (((reinterpret_cast<uintptr_t>(crow) - r) & 3) == 0 && (!kerr || ((reinterpret_cast<uintptr_t>(kerr) - 4 * r) & 15) == 0)));
     {
         unsigned *const cdst = reinterpret_cast<unsigned *>(crow - r) + q0;
         const float2 k30 = make_float2(0x1p-30f, 0x1p-30f);

@@ -28,15 +28,16 @@ def layers(shape, seed):
     return out
 
 
-def check(ws, bits, mode=sq.MODE_EKC, flags=sq.FLAG_NARROW_RANGE, start=0, outputs=False, clip=None):
+def check(ws, bits, mode=sq.MODE_EKC, flags=sq.FLAG_NARROW_RANGE, start=0, outputs=False, clip=None, sums=True):
     pack = bool(flags & sq.FLAG_PACK_INT4)
     bufs, scales = [], []
     for i, w in enumerate(ws):
         t = torch.zeros(w.size + 4, device="cuda")[start:start + w.size].view(w.shape)
         t.copy_(torch.from_numpy(w))
-        b = sq.alloc_outputs(t, pack_int4=pack, dequant=outputs, dequant_bf16=outputs)
+        b = sq.alloc_outputs(t, pack_int4=pack, dequant=outputs, dequant_bf16=outputs, kernel_err=sums, channel_err=sums)
         b.codes.fill_(-128)
-        b.kernel_err.fill_(float("nan"))
+        if sums:
+            b.kernel_err.fill_(float("nan"))
         sc = None
         if clip:
             a = np.abs(w).reshape(w.shape[0], -1).max(1)
@@ -48,7 +49,9 @@ def check(ws, bits, mode=sq.MODE_EKC, flags=sq.FLAG_NARROW_RANGE, start=0, outpu
     sq.squant_device_status()
     for b, w, sc in zip(bufs, ws, scales):
         r = oracle.quantize_layer(w, bits=bits, mode=mode, flags=flags, details=True, scales_in=sc)
-        pairs = [(b.codes, r.codes), (b.scales, r.scales), (b.kernel_err, r.kernel_err), (b.channel_err, r.channel_err)]
+        pairs = [(b.codes, r.codes), (b.scales, r.scales)]
+        if sums:
+            pairs += [(b.kernel_err, r.kernel_err), (b.channel_err, r.channel_err)]
         if outputs:
             pairs += [(b.dequant, r.dequant), (b.dequant_bf16.view(torch.int16), r.dequant_bf16.view(np.int16))]
         for k, (got, want) in enumerate(pairs):
@@ -364,3 +367,20 @@ def test_wide_rows_without_supplied_scales():
     check(ws, 8, flags=0, outputs=True)
     check(ws, 4, flags=sq.FLAG_NARROW_RANGE | sq.FLAG_PACK_INT4, start=2)
     check(ws, 4, clip=0.8)
+
+
+@pytest.mark.parametrize("n", [8193, 8196, 9001, 16387, 25002, 32767, 46501, 65535, 65541, 100352])
+def test_long_and_wide_rows_without_sums(n):
+    """Codes and scales only (rows of the row and the cluster kernel): every start of a row, packed codes, supplied
+    scales; many rows and few."""
+    assert sq.squant_plan_kernels([(3, n, 1, 1)]) == ["row" if n <= 32768 else "cluster"]
+    ws = layers((3, n, 1, 1), n)
+    m = 12 * torch.cuda.get_device_properties(0).multi_processor_count + 8
+    if n < 10000:   # more rows than four waves of the smaller thread blocks, both sides of a vector's start
+        check([W.random_layer((m, n, 1, 1), seed=2)], 4, sums=False, start=n & 3)
+    for start in (0, 1, 2, 3):
+        check(ws, 4, start=start, sums=False)
+    check(ws, 8, flags=0, sums=False)
+    check(ws, 4, flags=sq.FLAG_NARROW_RANGE | sq.FLAG_PACK_INT4, start=1, sums=False)
+    check(ws, 3, flags=sq.FLAG_NARROW_RANGE | sq.FLAG_PACK_INT4, outputs=True, sums=False)
+    check(ws, 4, clip=0.7, sums=False)
