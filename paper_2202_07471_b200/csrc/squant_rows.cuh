@@ -71,16 +71,17 @@ __host__ __device__ constexpr int sel_warps(int g, Owner own, int K) { return g 
 // instead of two and a barrier more, which the few kernels of such a channel hardly notice.
 __host__ __device__ constexpr bool late_maxima(int K) { return K > 9; }
 // Entries of a list.  Groups of 64, 128 and 256 threads on larger kernels: as many as make the group's selection memory
-// 1,072, 2,160 and 3,120 B, with late maxima 1,072, 1,584 and 3,120 B.  The last figure is part of the longest
-// channel that a thread block takes; the others decide how many channels share one (512 channels of 106 7x7 kernels,
-// four layers: two channels to a thread block 49.6 us on a B200, one 70.9).
+// 1,056, 2,144 and 3,104 B, with late maxima 1,056, 1,568 and 3,120 B.  The last figure is part of the longest
+// channel of few kernels that a thread block takes; the others decide how many channels share one (512 channels of 106
+// 7x7 kernels, four layers: two channels to a thread block 49.6 us on a B200, one 70.9).  The weights follow, so a multiple of 32 B: rows of
+// whole 32-byte sectors copied to an odd multiple of 16 cost 2000 rows of 21,000 weights 98.0 us instead of 91.8.
 __host__ __device__ constexpr int sel_cap(int g, int K = 1)
 {
     return K == 1 ? (g <= 64 ? 64 : g)
          : g > 256 ? (K > 16 ? 64 : g)
          : g <= 32 ? 64
-         : late_maxima(K) ? (g == 64 ? 93 : (g == 128 ? 120 : 238))
-                          : (g == 64 ? 61 : (g == 128 ? 128 : 110));
+         : late_maxima(K) ? (g == 64 ? 91 : (g == 128 ? 118 : 238))
+                          : (g == 64 ? 59 : (g == 128 ? 126 : 108));
 }
 // Maxima that a group leaves in shared memory: one per thread and sign, of 1x1 channels two up to 64 threads.
 __host__ __device__ constexpr int sel_maxima(int g, int K) { return K == 1 && g <= 64 ? 4 * g : (late_maxima(K) ? g : 2 * g); }
