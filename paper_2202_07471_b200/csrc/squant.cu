@@ -32,6 +32,9 @@ constexpr size_t kMaxPlans = 64;
 constexpr int kLongChannel = 8192;           // weights: longer channels are launched apart from the others
 constexpr int kStreamKernels = 1184;         // 3x3 channels of at least as many kernels go to the streaming kernel (stream_eligible)
 constexpr int kGroupedSmemGoal = 55 << 10;   // shared memory of a grouped CTA with which four of them share a multiprocessor
+constexpr int kLongRow512 = 22000;           // weights: see build_param_plan
+constexpr int kSmSmem = 228 << 10;           // shared memory of a multiprocessor; every thread block takes 1 KB of it for the system
+constexpr int kBlockSmemReserved = 1 << 10;
 constexpr int kWideSmemGoal = 112 << 10;     // the same of a cluster's thread block: two of them
 
 std::mutex g_mutex;
@@ -347,7 +350,8 @@ struct ParamPlan {
     struct Wide { LayerDesc d; int cluster, kpc, smem; };
     std::vector<Wide> wide;
     // row kernel (1x1 rows too long for a group): one item per output channel
-    struct Rows { sq::LaunchTable table; int grid, threads, smem; };
+    enum RowForm { kRow512, kLong512, kLong256 };   // row_body with 512 threads, long_row_body with 512, with 256
+    struct Rows { sq::LaunchTable table; RowForm form; int grid, smem; };
     std::vector<Rows> rows;
     // streaming kernel (layers of long 3x3 channels): one item per output channel
     struct Stream {
@@ -447,7 +451,7 @@ int build_param_plan(const squant_layer *layers, int32_t n_layers, const squant_
             if (kernels) kernels[i] = SQUANT_KERNEL_STREAM;
             continue;
         }
-        if (descs[i].K == 1 && descs[i].off_hist != 0 && descs[i].N <= sq::kRowBlockElems) {   // too long for a group, 164 KB at most
+        if (descs[i].K == 1 && descs[i].off_hist != 0 && descs[i].N <= sq::kRowBlockElems) {   // too long for a group
             rows.push_back(i);
             if (kernels) kernels[i] = SQUANT_KERNEL_ROW;
             continue;
@@ -455,29 +459,56 @@ int build_param_plan(const squant_layer *layers, int32_t n_layers, const squant_
         order.push_back(i);
         if (kernels) kernels[i] = SQUANT_KERNEL_GROUPED;
     }
-    // long rows, longest first: a thread block per output channel
-    // Rows of up to 16 K weights take 256 threads if they are more than one wave of such thread blocks (four per
-    // multiprocessor), else 512: fewer rows take the time of one row's chain (512 rows of 16,000 weights 30.2 us with 256 threads,
-    // 25.4 with 512; of 12,000 24.8, 23.3; 1000 of 12,000 33.1, 37.3; 2000 of 10,000 50.0, 63.5).
-    std::stable_sort(rows.begin(), rows.end(), [&](int a, int b) { return descs[a].N > descs[b].N; });
-    int64_t short_rows = 0;
-    for (int i : rows) short_rows += descs[i].N <= sq::kRowSmallElems ? descs[i].M : 0;
-    const int small_limit = short_rows > 4ll * sms ? sq::kRowSmallElems : 0;
+    // Long rows, a thread block per output channel, in one of three forms.  row_body holds 5 B of shared memory a weight,
+    // long_row_body 4 (5 of packed codes).  What counts is how many threads a multiprocessor holds and over how many
+    // vectors a thread spreads the code that runs once.  us a call on a B200, row_body / long_row_body:
+    //   - Many rows of up to 16 K weights: long_row_body with 256 threads.  Where four such thread blocks fit a multiprocessor
+    //     (13 K weights) the line is at one and a half waves of them: rows of 12,000 weights 700 28.8 / 29.9, 1000 37.9 / 35.7, 1500 49.9 / 46.9,
+    //     4096 119.5 / 96.9; with packed codes (10 K weights) at two: rows of 9000 1000 30.7 / 31.6, 1500 41.3 / 41.2, 2000 52.1 / 48.6.
+    //     Where three fit, at four, and not with packed codes or supplied scales: rows of 15,001 1000 42.9 / 47.3, 1500 59.6 / 58.9,
+    //     2000 75.2 / 72.9, 4096 143.7 / 133.4; 2000 of 13,500 with packed codes 63.0 / 71.9.
+    //   - More rows of over 22 K weights than multiprocessors, neither packed codes nor supplied scales: long_row_body with 512
+    //     threads, of which two blocks fit a multiprocessor up to 26 K weights and of row_body one (2000 rows of 17,000 78.2 / 81.4, of
+    //     20,000 86.1 / 88.9, of 25,001 143.4 / 109.4, of 32,768 157.4 / 155.1; 300 of 25,001 32.3 / 30.1; 16 of 25,001 14.3 / 15.7).
+    //   - All others row_body: few rows take the time of one row's chain, which is shorter there (16 rows of 9000 8.2 / 10.3, 1000 of
+    //     16,384 42.6 / 48.4, with packed codes 39.1 / 58.4).
+    const auto small_blocks = [&](int i) {   // of 256 threads on a multiprocessor
+        const int bytes = sq::long_row_bytes(256, (descs[i].N + 6) >> 2, pack, sq::kBlock);
+        return descs[i].N > sq::kRowSmallElems ? 0 : std::min(4, kSmSmem / (bytes + kBlockSmemReserved));
+    };
+    const auto codes_only = [&](int i) { return !pack && !descs[i].sin; };
+    int64_t four = 0, three = 0, longer = 0;   // rows
+    for (int i : rows) {
+        const int small = small_blocks(i);
+        if (small == 4) four += descs[i].M;
+        if (small == 3 && codes_only(i)) three += descs[i].M;
+        if (descs[i].N > kLongRow512 && codes_only(i)) longer += descs[i].M;
+    }
+    const auto form_of = [&](int i) {
+        const int small = small_blocks(i);
+        if (small == 4 && four > (pack ? 8ll : 6ll) * sms) return ParamPlan::kLong256;
+        if (small == 3 && codes_only(i) && three > 12ll * sms) return ParamPlan::kLong256;
+        return descs[i].N > kLongRow512 && codes_only(i) && longer > sms ? ParamPlan::kLong512 : ParamPlan::kRow512;
+    };
+    std::stable_sort(rows.begin(), rows.end(), [&](int a, int b) {   // by form, longest first
+        return form_of(a) != form_of(b) ? form_of(a) < form_of(b) : descs[a].N > descs[b].N;
+    });
     for (size_t base = 0; base < rows.size();) {
-        const bool small = descs[rows[base]].N <= small_limit;
+        const ParamPlan::RowForm form = form_of(rows[base]);
         size_t n = 0;
         int smem = 0;
-        while (base + n < rows.size() && n < sq::kMaxParamLayers && (descs[rows[base + n]].N <= small_limit) == small) {
+        while (base + n < rows.size() && n < sq::kMaxParamLayers && form_of(rows[base + n]) == form) {
             LayerDesc &d = descs[rows[base + n]];
             d.off_vi = (d.N + 6) >> 2;
             d.off_ev = regular_rows(d);
-            smem = std::max(smem, sq::long_row_bytes(small ? 256 : 512, d.off_vi, pack, sq::kBlock));
+            smem = std::max(smem, form == ParamPlan::kRow512 ? sq::row_bytes(512, d.off_vi, sq::kBlock)
+                                                             : sq::long_row_bytes(form == ParamPlan::kLong512 ? 512 : 256, d.off_vi, pack, sq::kBlock));
             ++n;
         }
         p.rows.emplace_back();
         ParamPlan::Rows &r = p.rows.back();
         r.grid = fill_table(r.table, descs, rows.data() + base, static_cast<int>(n), false);
-        r.threads = small ? 256 : 512;
+        r.form = form;
         r.smem = smem;
         base += n;
     }
@@ -569,9 +600,11 @@ int device_smem_limit(int device, int &limit)
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, v));
         SQ_CUDA(cudaFuncSetAttribute(sq::squant_table_kernel,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, v));
-        SQ_CUDA(cudaFuncSetAttribute(sq::squant_row_kernel<256>,
+        SQ_CUDA(cudaFuncSetAttribute((sq::squant_row_kernel<256, true>),
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, v));
-        SQ_CUDA(cudaFuncSetAttribute(sq::squant_row_kernel<512>,
+        SQ_CUDA(cudaFuncSetAttribute((sq::squant_row_kernel<512, true>),
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, v));
+        SQ_CUDA(cudaFuncSetAttribute((sq::squant_row_kernel<512, false>),
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, v));
         SQ_CUDA(cudaFuncSetAttribute(sq::squant_wide_kernel,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, v));
@@ -650,8 +683,9 @@ int launch_plan(const ParamPlan &p, cudaStream_t stream)
         g_launches.fetch_add(1, std::memory_order_relaxed);
     }
     for (const ParamPlan::Rows &r : p.rows) {
-        if (r.threads == 256) sq::squant_row_kernel<256><<<r.grid, 256, r.smem, stream>>>(r.table, p.qmax, p.mode);
-        else sq::squant_row_kernel<512><<<r.grid, 512, r.smem, stream>>>(r.table, p.qmax, p.mode);
+        if (r.form == ParamPlan::kRow512) sq::squant_row_kernel<512, false><<<r.grid, 512, r.smem, stream>>>(r.table, p.qmax, p.mode);
+        else if (r.form == ParamPlan::kLong512) sq::squant_row_kernel<512, true><<<r.grid, 512, r.smem, stream>>>(r.table, p.qmax, p.mode);
+        else sq::squant_row_kernel<256, true><<<r.grid, 256, r.smem, stream>>>(r.table, p.qmax, p.mode);
         SQ_CUDA(cudaGetLastError());
         g_launches.fetch_add(1, std::memory_order_relaxed);
     }

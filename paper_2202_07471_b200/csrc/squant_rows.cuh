@@ -1,5 +1,5 @@
 // 1x1 layers (fully connected and pointwise): a group of 8 to 256 threads takes a whole output
-// channel, up to 32 weights a thread.
+// channel, up to 32 weights a thread, or a thread block of 512 threads a longer one.
 //
 // Every element is its own kernel, so SQuant-K is a no-op (Sec. 3.4) and the work is absmax,
 // SQuant-E, the channel sum and SQuant-C's choice of the k_c largest perturbations of one sign.
@@ -77,7 +77,7 @@ __host__ __device__ constexpr bool late_maxima(int K) { return K > 9; }
 // whole 32-byte sectors copied to an odd multiple of 16 cost 2000 rows of 21,000 weights 98.0 us instead of 91.8.
 __host__ __device__ constexpr int sel_cap(int g, int K = 1)
 {
-    return K == 1 ? (g <= 64 ? 64 : g)
+    return K == 1 ? (g <= 64 ? 64 : (g > 256 ? 472 : g))   // (472: 4,128 B with the parts)
          : g > 256 ? (K > 16 ? 64 : g)
          : g <= 32 ? 64
          : late_maxima(K) ? (g == 64 ? 91 : (g == 128 ? 118 : 238))
@@ -85,13 +85,14 @@ __host__ __device__ constexpr int sel_cap(int g, int K = 1)
 }
 // Maxima that a group leaves in shared memory: one per thread and sign, of 1x1 channels two up to 64 threads.
 __host__ __device__ constexpr int sel_maxima(int g, int K) { return K == 1 && g <= 64 ? 4 * g : (late_maxima(K) ? g : 2 * g); }
+__host__ __device__ constexpr int sel_list_bytes(int g, Owner own, int K) { return static_cast<int>(sizeof(SelScratch)) + 20 * sel_warps(g, own, K) + 8 * sel_cap(g, K); }
 __host__ __device__ constexpr int sel_bytes(int g, Owner own = kGroup, int K = 1)
 {
-    return static_cast<int>(sizeof(SelScratch)) + 20 * sel_warps(g, own, K) + 8 * sel_cap(g, K) +
+    return sel_list_bytes(g, own, K) +
            (own == kCluster ? 8 * merged_cap(K) : (g > 32 ? 4 * sel_maxima(g, K) : 0));
 }
 // Shared memory of a 1x1 channel of `vecs` vectors: selection, perturbations, codes.
-__host__ __device__ constexpr int row_bytes(int g, int vecs) { return sel_bytes(g) + 20 * vecs; }
+__host__ __device__ constexpr int row_bytes(int g, int vecs, Owner own = kGroup) { return (own == kBlock ? sel_list_bytes(g, own, 1) : sel_bytes(g, own)) + 20 * vecs; }
 // The same where a thread block or a cluster takes the row: weights, and codes if they are to be packed.
 __host__ __device__ constexpr int long_row_bytes(int g, int vecs, bool pack, Owner own) { return sel_bytes(g, own) + (pack ? 20 : 16) * vecs; }
 
@@ -550,12 +551,14 @@ __device__ __forceinline__ void row_clip_one(float Pf, int &P, unsigned c, int q
 // ---------------------------------------------------------------- one 1x1 channel
 // kClip: the clip of Sec. 2.2 can fire (caller-supplied scales): codes are clamped, sums are 64
 // bit and an element whose flipped code would leave the range is no candidate.  valid = false: the
-// group has no channel (its lanes take part in the warp's steps and write nothing).
-template <bool kClip>
+// group has no channel (its lanes take part in the warp's steps and write nothing).  kBlock: a row of the row kernel
+// (see build_param_plan); the search then counts the threads' two maxima by barriers.
+template <bool kClip, Owner kOwn = kGroup>
 __device__ __forceinline__ void row_body(const LayerDesc &L, int m, const Group &G, unsigned char *slice, int qmax, unsigned mode, bool valid)
 {
+    static_assert(kOwn != kCluster, "");
     const int g = G.g, N = valid ? L.N : 0;
-    const Sel S(slice, g, kGroup, 1);
+    const Sel S(slice, g, kOwn, 1);
     if (G.t == 0) {
         S.sc->count = 0;
         S.sc->total[0] = 0;
@@ -568,8 +571,9 @@ __device__ __forceinline__ void row_body(const LayerDesc &L, int m, const Group 
     const Span sp(pack ? 0 : static_cast<int>((reinterpret_cast<uintptr_t>(wrow) >> 2) & 3), N, G.t);
     const int r = sp.r, q_hi = sp.q_hi, rag = sp.rag, q0 = sp.q_lo + G.t, vecs = G.rounds(sp.q_lo, sp.q_hi);   // vectors q0, q0 + g, ..
     SQ_DBG(N >= 0 && N + r <= 4 * L.off_vi && q_hi <= L.off_vi, 14);   // the vectors' places below
-    int4 *Pbuf = reinterpret_cast<int4 *>(slice + sel_bytes(g));              // what SQuant-C may choose from
-    unsigned *cbuf = reinterpret_cast<unsigned *>(slice + sel_bytes(g) + 16 * L.off_vi);   // codes, by vectors
+    const int sel = kOwn == kBlock ? sel_list_bytes(g, kOwn, 1) : sel_bytes(g);   // (a thread block keeps no maxima in shared memory)
+    int4 *Pbuf = reinterpret_cast<int4 *>(slice + sel);              // what SQuant-C may choose from
+    unsigned *cbuf = reinterpret_cast<unsigned *>(slice + sel + 16 * L.off_vi);   // codes, by vectors
     int *Pel = reinterpret_cast<int *>(Pbuf) + r;                                   // the same by elements
     unsigned char *cel = reinterpret_cast<unsigned char *>(cbuf) + r;
     float *kerr = L.kerr ? L.kerr + first : nullptr;
@@ -601,7 +605,7 @@ __device__ __forceinline__ void row_body(const LayerDesc &L, int m, const Group 
     amax = fmaxf(amax, fabsf(w_rag));
 
     // ---- scale
-    amax = owner_absmax<kGroup>(G, amax, S);
+    amax = owner_absmax<kOwn>(G, amax, S);
     float s = absmax_scale(amax, qmax);
     if (kClip && valid) {
         s = L.sin[m];
@@ -704,7 +708,7 @@ __device__ __forceinline__ void row_body(const LayerDesc &L, int m, const Group 
     long long ec = 0;
     const int per = g > 64 ? 1 : 2;   // maxima a thread puts in
     if ((mode & 4u) || L.cerr) {
-        if (g > 32) {   // those that SQuant-C looks for its bound among, of either sign
+        if (kOwn == kGroup && g > 32) {   // those that SQuant-C looks for its bound among, of either sign
             if (per == 2) {
                 S.mx[G.t] = hi0; S.mx[G.t + g] = hi1;
                 S.mx[G.t + 2 * g] = -lo0; S.mx[G.t + 3 * g] = -lo1;
@@ -714,7 +718,7 @@ __device__ __forceinline__ void row_body(const LayerDesc &L, int m, const Group 
             }
         }
         int up = 0, down = 0;
-        ec = owner_sum<kGroup, kClip, false>(G, S, sum64, sum, __float2int_rn(__fmul_rn(__fadd_rn(fs.x, fs.y), 0x1p-17f)), up, down);
+        ec = owner_sum<kOwn, kClip, false>(G, S, sum64, sum, __float2int_rn(__fmul_rn(__fadd_rn(fs.x, fs.y), 0x1p-17f)), up, down);
     }
 
     // ---- SQuant-C: Algorithm 2 on the channel, the perturbations are the keys
@@ -728,20 +732,24 @@ __device__ __forceinline__ void row_body(const LayerDesc &L, int m, const Group 
             const int sx = sgn > 0 ? 0 : -1;   // p ^ sx = the value in the direction of the flips, less one if that is downward
             auto each = [&](int t, auto fn) {
                 const int tx = t + sx;
-                unsigned hit = 0u, bit = 1u;   // a bit for each of the thread's elements in vectors (at most 32) that counts
-#pragma unroll 2
-                for (int i = 0; i < vecs; ++i, bit <<= 4) {
-                    const int4 p = Pbuf[q0 + i * g];
-                    if ((p.x ^ sx) >= tx) hit |= bit;
-                    if ((p.y ^ sx) >= tx) hit |= 2u * bit;
-                    if ((p.z ^ sx) >= tx) hit |= 4u * bit;
-                    if ((p.w ^ sx) >= tx) hit |= 8u * bit;
-                }
 #pragma unroll 1
-                for (; hit != 0u; hit &= hit - 1u) {
-                    const int b = __ffs(hit) - 1, n = 4 * (q0 + (b >> 2) * g) - r + (b & 3);
-                    SQ_DBG(n >= 0 && n < N, 15);
-                    fn((Pel[n] ^ sx) - sx, n);
+                for (int ib = 0; ib < vecs; ib += kRowVecs) {   // (groups: once)
+                    unsigned hit = 0u, bit = 1u;   // a bit for each of these (at most 32) elements that counts
+#pragma unroll 2
+                    for (int i = ib; i < min(vecs, ib + kRowVecs); ++i, bit <<= 4) {
+                        const int4 p = Pbuf[q0 + i * g];
+                        if ((p.x ^ sx) >= tx) hit |= bit;
+                        if ((p.y ^ sx) >= tx) hit |= 2u * bit;
+                        if ((p.z ^ sx) >= tx) hit |= 4u * bit;
+                        if ((p.w ^ sx) >= tx) hit |= 8u * bit;
+                    }
+#pragma unroll 1
+                    for (; hit != 0u; hit &= hit - 1u) {
+                        const int b = __ffs(hit) - 1, n = 4 * (q0 + (ib + (b >> 2)) * g) - r + (b & 3);
+                        SQ_DBG(n >= 0 && n < N, 15);
+                        fn((Pel[n] ^ sx) - sx, n);
+                    }
+                    if (kOwn == kGroup) break;
                 }
                 if (rag >= 0) {
                     const int v = Pel[rag] ^ sx;
@@ -755,6 +763,7 @@ __device__ __forceinline__ void row_body(const LayerDesc &L, int m, const Group 
             const unsigned gmask = g >= 32 ? kFull : (((1u << g) - 1u) << (lane & ~(g - 1)));
             const int *mx = sgn > 0 ? S.mx : S.mx + per * g;
             auto count = [&](int t, int) {
+                if (kOwn == kBlock) return __syncthreads_count(m0 >= t) + __syncthreads_count(m1 >= t);
                 if (g <= 32) return __popc(__ballot_sync(kFull, m0 >= t) & gmask) + __popc(__ballot_sync(kFull, m1 >= t) & gmask);
                 int c = 0;
 #pragma unroll 1
@@ -771,7 +780,7 @@ __device__ __forceinline__ void row_body(const LayerDesc &L, int m, const Group 
                 if (kerr) kerr[n] = __fmul_rn(__int2float_rn(sgn > 0 ? a - kOne : kOne - a), 0x1p-30f);
             };
             const int vtop = kHalf + (1 << 14) + 1;
-            const int k_eff = select_top<kGroup>(G, count, listing, [] {}, each, [](int) { return 0u; }, flip, per * g, vtop, vtop, 2.0f, kc, N, want, S, 1);
+            const int k_eff = select_top<kOwn>(G, count, listing, [] {}, each, [](int) { return 0u; }, flip, kOwn == kBlock ? 2 * g : per * g, vtop, vtop, 2.0f, kc, N, want, S, 1);
             ec -= static_cast<long long>(sgn) * k_eff * kOne;
         }
     }

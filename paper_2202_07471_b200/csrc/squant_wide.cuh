@@ -20,7 +20,7 @@ namespace sq {
 
 static_assert(kBlockThreads == 1 << 9, "");
 constexpr int kWideMaxCluster = 8;
-// Longest row of the row kernel (164 KB of shared memory); up to here it was laid out and compared with the staged
+// Longest row of the row kernel (168 KB of shared memory with packed codes or in row_body); up to here it was laid out and compared with the staged
 // body of the grouped kernel.  Longer rows that fit one thread block still take that body, which is the slower one
 // there: 1024 rows of 32,772 weights 318 us against 99 in this kernel, of 40,000 480 against 116, 16 rows of 40,000 83 against 22.
 constexpr int kRowBlockElems = 32768;
@@ -456,12 +456,10 @@ __device__ __forceinline__ void long_row_body(const LayerDesc &L, int m, const G
     }
 }
 
-// Rows of more than 8 K weights, one thread block per output channel.
-// kThreads = 256 for many rows of up to 16 K weights, 512 else: about eleven vectors a thread, over which the code that
-// runs once is spread (4096 rows of 11,008 weights at 8 bit:
-// 85 us, 115 with 512 threads).
-constexpr int kRowSmallElems = 16384;
-template <int kThreads>
+// Rows of more than 8 K weights, one thread block per output channel.  kLong: by long_row_body, else by row_body.
+// Which form a row takes: build_param_plan.
+constexpr int kRowSmallElems = 16384;   // longest row of 256 threads
+template <int kThreads, bool kLong>
 __global__ void __launch_bounds__(kThreads, 1024 / kThreads)
 squant_row_kernel(const __grid_constant__ LaunchTable tbl, int qmax, unsigned mode)
 {
@@ -477,9 +475,16 @@ squant_row_kernel(const __grid_constant__ LaunchTable tbl, int qmax, unsigned mo
     G.sh = kThreads == 256 ? 8 : 9;
     G.t = threadIdx.x;
     G.bar = 0;
-    SQ_DBG(long_row_bytes(kThreads, L.off_vi, (mode & kModePackInt4) != 0, kBlock) <= static_cast<int>(dynamic_smem_bytes()), 10);
-    if (L.sin) long_row_body<true, kBlock>(L, item - tbl.first_item[layer], G, smem, qmax, mode);
-    else long_row_body<false, kBlock>(L, item - tbl.first_item[layer], G, smem, qmax, mode);
+    const int m = item - tbl.first_item[layer];
+    if (kLong) {
+        SQ_DBG(long_row_bytes(kThreads, L.off_vi, (mode & kModePackInt4) != 0, kBlock) <= static_cast<int>(dynamic_smem_bytes()), 10);
+        if (L.sin) long_row_body<true, kBlock>(L, m, G, smem, qmax, mode);
+        else long_row_body<false, kBlock>(L, m, G, smem, qmax, mode);
+    } else {
+        SQ_DBG(row_bytes(kThreads, L.off_vi, kBlock) <= static_cast<int>(dynamic_smem_bytes()), 10);
+        if (L.sin) row_body<true, kBlock>(L, m, G, smem, qmax, mode, true);
+        else row_body<false, kBlock>(L, m, G, smem, qmax, mode, true);
+    }
 }
 
 // Shared memory of one of a cluster's thread blocks that has `kpc` kernels of K weights.

@@ -384,3 +384,28 @@ def test_long_and_wide_rows_without_sums(n):
     check(ws, 4, flags=sq.FLAG_NARROW_RANGE | sq.FLAG_PACK_INT4, start=1, sums=False)
     check(ws, 3, flags=sq.FLAG_NARROW_RANGE | sq.FLAG_PACK_INT4, outputs=True, sums=False)
     check(ws, 4, clip=0.7, sums=False)
+
+
+@pytest.mark.parametrize("n,waves", [(8200, 6), (8193, 8), (10001, 8), (12290, 6), (13100, 6), (13500, 12), (16384, 12), (16387, 1), (22001, 1), (26500, 1)])
+def test_forms_of_long_rows(n, waves):
+    """Rows of the row kernel on either side of the numbers, in rows a multiprocessor, from which they take another form:
+    every output form in each, and a call of all forms."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    w = adversarial_layer((waves * sms + 1, n, 1, 1), seed=n)
+    check([w], 4)
+    check([w[1:]], 4)
+    check([w], 4, sums=False, start=1)
+    check([w], 4, flags=sq.FLAG_NARROW_RANGE | sq.FLAG_PACK_INT4, start=2)
+    if n in (8193, 16384, 22001):
+        check([w], 8, flags=0, outputs=True, start=3)
+        check([w], 4, clip=0.8)
+        check([w], 3, mode=sq.MODE_E | sq.MODE_C)
+
+
+def test_call_with_every_form_of_long_rows():
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    shapes = [(12 * sms + 1, 13500, 1, 1), (6 * sms, 8201, 1, 1), (5, 12000, 1, 1), (sms, 22100, 1, 1), (7, 32768, 1, 1), (11, 17000, 1, 1), (3, 50000, 1, 1), (40, 64, 3, 3)]
+    ws = [adversarial_layer(s, seed=s[1]) for s in shapes]
+    n0 = sq.squant_launch_count()
+    check(ws, 4, start=1)
+    assert sq.squant_launch_count() - n0 == 3 + 1 + 1   # the forms, the wide layer, the grouped launch
