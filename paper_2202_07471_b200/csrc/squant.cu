@@ -908,6 +908,12 @@ int squant_quantize_model_host(const squant_layer *layers, int32_t n_layers,
         dev[i].dequant = static_cast<float *>(at(6));
         dev[i].dequant_bf16 = static_cast<uint16_t *>(at(7));
     }
+    // every chunk's plan first: a call that is refused has copied and launched nothing
+    for (size_t c = 0; c < chunks; ++c) {
+        const ParamPlan *pp = nullptr;
+        rc = get_plan(dev.data() + chunk_first[c], chunk_first[c + 1] - chunk_first[c], o, pp);
+        if (rc) return rc;
+    }
     HostPipe *hp = nullptr;
     rc = host_pipe(device, chunks, hp);
     if (rc) return rc;

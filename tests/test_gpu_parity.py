@@ -689,3 +689,21 @@ def test_host_entry_point_small_and_large_outputs_in_many_chunks(pin):
             for name, big in whole.items():
                 assert torch.equal(getattr(b, name).view(torch.uint8), getattr(d, name).cpu().view(torch.uint8)), (k, s, name)
                 assert (big[:pad] == -77).all() and (big[-pad:] == -77).all(), (k, s, name)
+
+
+def test_refused_host_call_writes_nothing():
+    """A layer that no kernel takes, in a later chunk of a host-buffer call: refused before anything is launched or written."""
+    shapes = [(1024, 2048, 1, 1), (1024, 2049, 1, 1), (1, 80000, 3, 3)]
+    bufs = [sq.alloc_outputs(torch.zeros(s).pin_memory(), pin=True) for s in shapes]
+    for b in bufs:
+        b.codes.fill_(-77)
+        b.scales.fill_(-77)
+    n0 = sq.squant_launch_count()
+    with pytest.raises(sq.SquantError) as ei:
+        sq.squant_quantize_model_host(bufs, bits=4)
+    torch.cuda.synchronize()
+    assert ei.value.code == -6 and sq.squant_launch_count() == n0
+    for b in bufs:
+        assert (b.codes == -77).all() and (b.scales == -77).all()
+    sq.squant_quantize_model_host(bufs[:2], bits=4)
+    assert (bufs[1].codes == 0).all()
