@@ -153,8 +153,9 @@ int squant_quantize_model(const squant_layer *layers, int32_t n_layers, const sq
  * copies codes / scales / error sums back and returns when the outputs are in host memory.
  * The layers are taken in chunks of at least 8 MB of weights: uploads, launches and downloads of
  * consecutive chunks overlap on two copy streams of the library (created on first use) beside
- * the caller's stream, on which the launches run.  Device staging memory, and pinned host memory
- * through which outputs of up to 32 KB come down, are cached inside the library between calls
+ * the caller's stream, on which the launches run.  Device staging memory, one scratch area of the streaming
+ * kernel per device, pinned host memory through which outputs of up to 32 KB come down and the launch tables of the last
+ * eight calls (apart from those of device calls) are kept inside the library between calls
  * (allocated on first use or growth; squant_shutdown frees them).  Pinned
  * host memory gives the copies their full speed and lets them overlap; pageable memory works.
  */

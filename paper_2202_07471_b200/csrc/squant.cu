@@ -648,6 +648,45 @@ int get_plan(const squant_layer *layers, int32_t n_layers, const squant_options 
     return SQUANT_OK;
 }
 
+// Plans of a host-buffer call, one per chunk of layers; apart from those of device calls, of which a few large models in
+// host memory would leave none cached.  The chunks run one after the other and every call ends with its work done, so one
+// scratch area per device serves all of them.
+struct HostCall {
+    int device = -1;
+    std::string key;
+    std::vector<ParamPlan> chunks;
+};
+constexpr size_t kMaxHostCalls = 8;
+std::list<HostCall> g_host_calls;         // most recently used first
+std::vector<ScratchRef> g_host_scratch;   // per device
+
+int get_host_plans(const std::vector<squant_layer> &layers, const std::vector<int> &chunk_first, const squant_options &o, int device, HostCall *&out)
+{
+    std::string key = plan_key(layers.data(), static_cast<int32_t>(layers.size()), o);   // (the chunks follow from the sizes)
+    for (auto it = g_host_calls.begin(); it != g_host_calls.end(); ++it)
+        if (it->device == device && it->key == key) {
+            g_host_calls.splice(g_host_calls.begin(), g_host_calls, it);
+            out = &g_host_calls.front();
+            return SQUANT_OK;
+        }
+    int limit = 0;
+    int rc = device_smem_limit(device, limit);
+    if (rc) return rc;
+    HostCall hc;
+    hc.device = device;
+    hc.key = std::move(key);
+    hc.chunks.resize(chunk_first.size() - 1);
+    for (size_t c = 0; c < hc.chunks.size(); ++c) {
+        rc = build_param_plan(layers.data() + chunk_first[c], chunk_first[c + 1] - chunk_first[c], o, limit,
+                              std::max(g_sm_count_by_device[device], 1), hc.chunks[c]);
+        if (rc) return rc;
+    }
+    if (g_host_calls.size() >= kMaxHostCalls) g_host_calls.pop_back();
+    g_host_calls.push_front(std::move(hc));
+    out = &g_host_calls.front();
+    return SQUANT_OK;
+}
+
 int launch_plan(const ParamPlan &p, cudaStream_t stream)
 {
     const int freed = free_dead_scratch(stream);   // of graphs and of plans that have left the cache
@@ -729,7 +768,7 @@ std::vector<HostPipe> g_host_pipes;
 // outside the overlap is about one chunk at either end: ResNet-50 shapes (102 MB up, 87 MB down) take 3356 us, and
 // 4286 us in chunks of 64 MB with every tensor copied by itself.
 constexpr size_t kHostChunkBytes = 8u << 20;
-constexpr size_t kHostChunks = 24;   // and no more than about these: each has a cached plan (kMaxPlans)
+constexpr size_t kHostChunks = 24;   // and no more than about these: each has a plan of its own
 // Outputs of at most this many bytes come down through pinned staging memory, all of a chunk in one copy: a copy of a
 // few KB costs its fixed few microseconds on the copy engine, more than the host's memcpy takes.  (Inputs don't: work
 // that the caller's stream still holds may be about to write them.)
@@ -909,11 +948,17 @@ int squant_quantize_model_host(const squant_layer *layers, int32_t n_layers,
         dev[i].dequant_bf16 = static_cast<uint16_t *>(at(7));
     }
     // every chunk's plan first: a call that is refused has copied and launched nothing
-    for (size_t c = 0; c < chunks; ++c) {
-        const ParamPlan *pp = nullptr;
-        rc = get_plan(dev.data() + chunk_first[c], chunk_first[c + 1] - chunk_first[c], o, pp);
-        if (rc) return rc;
-    }
+    HostCall *plans = nullptr;
+    rc = get_host_plans(dev, chunk_first, o, device, plans);
+    if (rc) return rc;
+    if (static_cast<int>(g_host_scratch.size()) <= device) g_host_scratch.resize(device + 1);
+    for (const ParamPlan &plan : plans->chunks)
+        for (ParamPlan::Stream &st : plan.streams) {
+            ScratchRef &shared = g_host_scratch[device];
+            if (!shared) rc = new_scratch(device, std::max(g_sm_count_by_device[device], 1), stream, shared);   // (none to be had: launch_plan's to settle)
+            if (rc) return rc;
+            st.scratch = shared;
+        }
     HostPipe *hp = nullptr;
     rc = host_pipe(device, chunks, hp);
     if (rc) return rc;
@@ -951,12 +996,8 @@ int squant_quantize_model_host(const squant_layer *layers, int32_t n_layers,
         SQ_CUDA(cudaEventRecord(hp->uploaded[c], hp->in));
     }
     for (size_t c = 0; c < chunks; ++c) {
-        const int first = chunk_first[c], count = chunk_first[c + 1] - first;
         SQ_CUDA(cudaStreamWaitEvent(stream, hp->uploaded[c], 0));
-        const ParamPlan *pp = nullptr;
-        rc = get_plan(dev.data() + first, count, o, pp);
-        if (rc) return rc;
-        rc = launch_plan(*pp, stream);
+        rc = launch_plan(plans->chunks[c], stream);
         if (rc) return rc;
         SQ_CUDA(cudaEventRecord(hp->computed[c], stream));
         SQ_CUDA(cudaStreamWaitEvent(hp->out, hp->computed[c], 0));
@@ -1170,6 +1211,8 @@ int squant_shutdown(void)
     int cur = 0;
     const bool have = cudaGetDevice(&cur) == cudaSuccess;
     g_plans.clear();
+    g_host_calls.clear();
+    g_host_scratch.clear();
     free_dead_scratch();   // (areas that a graph still holds go with the graph)
     for (size_t d = 0; d < g_arenas.size(); ++d) {
         if (g_arenas[d].ptr) { cudaSetDevice(static_cast<int>(d)); cudaDeviceSynchronize(); cudaFree(g_arenas[d].ptr); }

@@ -707,3 +707,32 @@ def test_refused_host_call_writes_nothing():
         assert (b.codes == -77).all() and (b.scales == -77).all()
     sq.squant_quantize_model_host(bufs[:2], bits=4)
     assert (bufs[1].codes == 0).all()
+
+def test_host_calls_leave_the_plans_of_device_calls_alone():
+    """Host-buffer calls of many chunks, more than the cache of device calls has places: a device call whose scratch memory
+    goes with its cached plan can still be captured (nothing may be allocated there), and the results are right."""
+    w = W.random_layer((40, 1536, 3, 3), seed=16)
+    b = sq.alloc_outputs(torch.from_numpy(w).cuda())
+    assert_kernels([b], ["stream"])
+    call = sq.ModelCall([b])
+    call.run()
+    shapes = 14 * [(1024, 2048, 1, 1)] + 3 * [(130, 2048, 3, 3)]
+    ws = [torch.from_numpy(W.random_layer(s, seed=i)) for i, s in enumerate(shapes[12:])]
+    ws = 12 * [ws[0]] + ws
+    host = [sq.alloc_outputs(t.pin_memory(), pin=True) for t in ws]
+    dev = [sq.alloc_outputs(t.cuda()) for t in ws[12:]]
+    for rep in range(2):
+        for bits in (4, 3, 5, 6, 8):   # 16 or so chunks each
+            sq.squant_quantize_model_host(host, bits=bits)
+            if rep == 0:
+                sq.squant_quantize_model(dev, bits=bits)
+                for h, d in zip(host[12:], dev):
+                    assert torch.equal(h.codes, d.codes.cpu()) and torch.equal(h.scales, d.scales.cpu())
+                    assert torch.equal(h.kernel_err, d.kernel_err.cpu()) and torch.equal(h.channel_err, d.channel_err.cpu())
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        call.run()
+    b.codes.fill_(-128)
+    graph.replay()
+    sq.squant_device_status()
+    assert_layer_equal(b, w, 4, EKC)
