@@ -428,9 +428,11 @@ int build_param_plan(const squant_layer *layers, int32_t n_layers, const squant_
             if (align16_64(4 * k8 * descs[i].K) + align16_64(k8 * descs[i].K) + (descs[i].K > 1 ? 2 * align16_64(4 * k8) + align16_64(2 * k8) : 0) + 2304 > max_smem)
                 return SQUANT_ERR_TOO_WIDE;
             // two thread blocks per multiprocessor if the channel can be cut that small: while one waits for its
-            // weights or for its cluster the other works
+            // weights or for its cluster the other works.  Few 1x1 rows take clusters of four at least (46,500 weights, in
+            // clusters of two / four: 16 rows 17.8 / 14.4 us on a B200, 64 18.5 / 18.0, 74 18.5 / 23.9, 200 39.9 / 47.2).
+            const int least = descs[i].K == 1 && 16ll * descs[i].M <= 7ll * sms ? 4 : 2;
             for (int goal = kWideSmemGoal;; goal = max_smem) {
-                for (int c = 2; c <= sq::kWideMaxCluster && !w.cluster; c *= 2) {
+                for (int c = least; c <= sq::kWideMaxCluster && !w.cluster; c *= 2) {
                     const int unit = descs[i].K == 1 ? 4 : 2;
                     const int kpc = ((descs[i].N + c - 1) / c + unit - 1) / unit * unit;
                     const int64_t bytes = sq::wide_bytes(kpc, descs[i].K, pack);

@@ -409,3 +409,16 @@ def test_call_with_every_form_of_long_rows():
     n0 = sq.squant_launch_count()
     check(ws, 4, start=1)
     assert sq.squant_launch_count() - n0 == 3 + 1 + 1   # the forms, the wide layer, the grouped launch
+
+
+@pytest.mark.parametrize("n", [46501, 48000, 50999])
+def test_wide_rows_in_clusters_of_two_and_four(n):
+    """On either side of the number of rows up to which clusters of two are not taken."""
+    m = 7 * torch.cuda.get_device_properties(0).multi_processor_count // 16
+    w = adversarial_layer((m + 1, n, 1, 1), seed=n)
+    assert sq.squant_plan_kernels([w.shape]) == ["cluster"]
+    for part in (w, w[1:]):
+        check([part], 4)
+        check([part], 4, sums=False, start=1)
+        check([part], 4, flags=sq.FLAG_NARROW_RANGE | sq.FLAG_PACK_INT4, start=3)
+    check([w[:9]], 8, flags=0, outputs=True, clip=0.9)
