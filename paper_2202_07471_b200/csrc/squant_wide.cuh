@@ -1,5 +1,5 @@
 // Output channels that are too long for a group of the grouped kernel: 1x1 rows of more than 8 K weights
-// get a thread block of 256 or 512 threads each, and channels that do not fit one thread block's shared memory a
+// get a thread block of 256 or 512 threads each (by long_row_body here or by row_body, see build_param_plan), and channels that do not fit one thread block's shared memory a
 // cluster of 2, 4 or 8 of them, each with a contiguous run of the channel's kernels.  What a channel needs
 // as a whole travels through distributed shared memory (plain loads from the other thread blocks' shared
 // memory; no multicast anywhere): absmax, error sum, the counts of SQuant-C's search and the short lists
@@ -9,7 +9,7 @@
 // Channels this wide can hold 2^16 and more kernels, the size from which the one element that sits on
 // the edge of the clip range (|w/s| a shade above qmax) can make it into a top-k: an element whose flipped
 // code would leave the range is no candidate.  Rows look for it where it can matter, among candidates of at most
-// 2^16 units of 2^-30, which only the exact search takes; larger kernels run the body that checks every candidate.
+// 2^16 units of 2^-30, which only the exact search takes (rows of the row kernel are shorter); larger kernels run the body that checks every candidate.
 //
 // Two thread blocks per multiprocessor where the channel can be cut that small.
 #pragma once
@@ -119,8 +119,8 @@ __device__ __forceinline__ unsigned row_extremes(const int4 p)
 //     anew, which yields the code of what is flipped too;
 //   - only codes that are to be packed wait in shared memory.
 // Against the body of the groups, with which these rows shared their code before: 256 rows of 100,352 weights 156 -> 83 us
-// on a B200 (the checked body of supplied scales until then), 4096 rows of 11,008 at 8 bit 105 -> 85.  In groups of up to
-// 256 threads it is the slower one (65,536 rows of 256 weights 54 -> 63 us): there the code that runs once counts most.
+// on a B200 (the checked body of supplied scales until then), 4096 rows of 12,000 123.0 -> 96.9.  In groups of up to
+// 256 threads it is the slower one (65,536 rows of 256 weights 54 -> 63 us), and for few rows: there the code that runs once counts most.
 template <bool kClip, Owner kOwn>
 __device__ __forceinline__ void long_row_body(const LayerDesc &L, int m, const Group &G, unsigned char *slice, int qmax, unsigned mode,
                                               int n0 = 0, int nloc = 0)
@@ -310,8 +310,8 @@ __device__ __forceinline__ void long_row_body(const LayerDesc &L, int m, const G
     }
 
     // ---- channel sum.  !kClip: its value modulo 2^32 is exact, its size is known from the float sums
-    // (a thread's fewer than 2^8 elements of at most one half are off by less than 2^18, a channel's 2^18 by less
-    // than 2^29, and by 2^28 for the rounding to units of 2^17)
+    // (a thread's fewer than 2^7 elements of at most one half give partial sums below 2^36, each addition off by at most 2^11, so
+    // its sum by less than 2^18; those of at most 2^12 threads by less than 2^30, and by 2^28 for the rounding to units of 2^17)
     long long ec = 0;
     if ((mode & 4u) || L.cerr) {
         if (kOwn != kCluster) S.mx[G.t] = static_cast<int>(__vmaxu2(__vmaxu2(e0, e1), __vmaxu2(e2, e3)));   // SQuant-C looks for its bound among these
