@@ -290,7 +290,7 @@ __device__ __forceinline__ void conv_body(const LayerDesc &L, int m, const Group
                         const float2 x0 = __fmul2_rn(w2, c2.y);
                         const float2 X = __ffma2_rn(__ffma2_rn(x0, c2.ns2, w2), c2.y, x0);
                         t = __fadd2_rn(X, c2.magic);
-                        P2[p] = __ffma2_rn(X, c2.neg1, __fadd2_rn(t, c2.nmagic));
+                        P2[p] = __ffma2_rn(X, c2.neg1, __ffma2_rn(c2.magic, c2.neg1, t));
                         const float lim_hi = (static_cast<float>(qmax) - 0.5f) * 1073741824.0f, lim_lo = (static_cast<float>(qmin) + 0.5f) * 1073741824.0f;
                         edge |= (X.x < lim_hi && X.x > lim_lo && X.y < lim_hi && X.y > lim_lo) ? 0u : 1u;
                     }
@@ -402,6 +402,7 @@ __device__ __forceinline__ void conv_body(const LayerDesc &L, int m, const Group
         const int kc = static_cast<int>(min((abs_e + (kHalf - 1)) >> 30, 1ll << 30));   // a clipped channel's sum can be huge
         if (kc > 0) {   // uniform in the group
             const int m0 = sgn > 0 ? hi0 : -lo0;
+            const Sel S(again(slice), g, kOwn, K);
             const int *mx = sgn > 0 || late ? S.mx : S.mx + g;
             const int lane = threadIdx.x & 31;
             if (late) {
@@ -446,7 +447,7 @@ __device__ __forceinline__ void conv_body(const LayerDesc &L, int m, const Group
             // Over-SQuant candidates reach one, but few come near it: the search starts at the largest
             const int top = (sgn > 0 ? up : down) + 1;
             const int nmax = g * (kOwn == kCluster ? static_cast<int>(cg::this_cluster().num_blocks()) : 1);
-            const int k_eff = select_top<kOwn>(G, count, listing, [] {}, each, [](int) { return 0u; }, flip, nmax, top, top, 3.0f, kc, L.N, true, S, K);
+            const int k_eff = select_top<kOwn>(G, [] {}, count, listing, [] {}, each, [](int) { return 0u; }, flip, nmax, false, 0, top, top, 3.0f, kc, L.N, true, S, K);
             ec -= static_cast<long long>(sgn) * k_eff * kOne;
         }
     }
@@ -455,7 +456,8 @@ __device__ __forceinline__ void conv_body(const LayerDesc &L, int m, const Group
     if (!kClip && kOwn != kCluster && ((mode & 4u) || L.cerr)) debug_check_sum(G, wrow, cel, NK, s, ec, true, S);
 #endif
 
-    emit_codes(L, first, static_cast<size_t>(m) * ((L.NK + 1) >> 1) + ((static_cast<size_t>(n0) * K) >> 1), G, cel, NK, s, mode);
+    const size_t ch = static_cast<size_t>(again(m)), k0 = kOwn == kCluster ? static_cast<size_t>(again(n0)) * K : 0;
+    emit_codes(L, ch * L.NK + k0, ch * ((L.NK + 1) >> 1) + (k0 >> 1), G, cel, NK, s, mode);
     if (G.t == 0 && n0 == 0) {
         L.scales[m] = s;
         if (L.cerr) L.cerr[m] = __fmul_rn(__ll2float_rn(ec), 0x1p-30f);

@@ -406,7 +406,7 @@ __device__ __forceinline__ void squant_e_fast(float w, float y, float s2, unsign
 // yields two IEEE round-to-nearest results, identical to the scalar sequence above, for one
 // issue slot.  E2 holds the channel's constants as pairs.
 struct E2 {
-    float2 y, ns2, magic, nmagic, neg1;
+    float2 y, ns2, magic, neg1;   // (neg1: differences by fused multiply-add, which needs no second constant)
 };
 
 __device__ __forceinline__ E2 make_e2(float y, float s2)
@@ -415,7 +415,6 @@ __device__ __forceinline__ E2 make_e2(float y, float s2)
     c.y = make_float2(y, y);
     c.ns2 = make_float2(-s2, -s2);
     c.magic = make_float2(kMagic, kMagic);
-    c.nmagic = make_float2(-kMagic, -kMagic);
     c.neg1 = make_float2(-1.0f, -1.0f);
     return c;
 }
@@ -426,7 +425,7 @@ __device__ __forceinline__ void squant_e_fast2(float2 w, const E2 &c, float2 &t,
     const float2 r = __ffma2_rn(x0, c.ns2, w);      // w - x0 * s2, exact
     const float2 X = __ffma2_rn(r, c.y, x0);        // RN(w / s2)
     t = __fadd2_rn(X, c.magic);
-    const float2 qX = __fadd2_rn(t, c.nmagic);
+    const float2 qX = __ffma2_rn(c.magic, c.neg1, t);
     Pf = __ffma2_rn(X, c.neg1, qX);                 // qX - X, exact
 }
 
@@ -1321,6 +1320,7 @@ namespace sq {
 #ifndef SQ_MIN_CTAS
 #define SQ_MIN_CTAS 4
 #endif
+template <bool kClip>
 __device__ __forceinline__ void run_item(const LayerDesc &L, int ch0, unsigned char *smem, int qmax,
                                          unsigned mode)
 {
@@ -1341,8 +1341,10 @@ __device__ __forceinline__ void run_item(const LayerDesc &L, int ch0, unsigned c
         SQ_DBG(ch0 >= 0 && L.g >= 8 && (1 << L.g_shift) == L.g && row_bytes(L.g, L.off_vi) <= L.slice_bytes &&
                static_cast<size_t>(gi + 1) * L.slice_bytes <= dynamic_smem_bytes(), 5);
         if (L.g >= 32 && m >= L.M) return;
-        if (L.sin) row_body<true>(L, m, G, slice, qmax, mode, m < L.M);
-        else row_body<false>(L, m, G, slice, qmax, mode, m < L.M);
+        if (kClip && L.sin) row_body<true, kGroup, 0>(L, m, G, slice, qmax, mode, m < L.M);
+        else if (L.g == 8) row_body<false, kGroup, 8>(L, m, G, slice, qmax, mode, m < L.M);
+        else if (L.g == 16) row_body<false, kGroup, 16>(L, m, G, slice, qmax, mode, m < L.M);
+        else row_body<false, kGroup, 32>(L, m, G, slice, qmax, mode, true);
         return;
     }
     if (m >= L.M) return;   // the whole group leaves together; it shares no barrier with others
@@ -1350,9 +1352,9 @@ __device__ __forceinline__ void run_item(const LayerDesc &L, int ch0, unsigned c
         SQ_DBG(ch0 >= 0 && L.g >= 32 && (1 << L.g_shift) == L.g && conv_bytes(L.g, L.NK, L.K) <= L.slice_bytes &&
                static_cast<size_t>(gi + 1) * L.slice_bytes <= dynamic_smem_bytes(), 6);
         if (L.K == 9 && (mode & 2u)) {
-            if (L.sin) conv_body<9, true>(L, m, G, slice, qmax, mode);
+            if (kClip && L.sin) conv_body<9, true>(L, m, G, slice, qmax, mode);
             else conv_body<9, false>(L, m, G, slice, qmax, mode);
-        } else if (L.sin) {
+        } else if (kClip && L.sin) {
             conv_body<0, true>(L, m, G, slice, qmax, mode);
         } else if (L.K == 7 && (mode & 2u)) {
             conv_body<7, false>(L, m, G, slice, qmax, mode);
@@ -1370,7 +1372,7 @@ __device__ __forceinline__ void run_item(const LayerDesc &L, int ch0, unsigned c
     if (s == 0.0f) return;   // staging wait ran out (status word set); nothing is written
     if (L.K > 1) {   // E + C without K
         channel_body_ec(L, m, G, slice, s, mode);
-    } else if (L.sin) {   // 1x1 rows too long for the registers of one thread block
+    } else if (kClip && L.sin) {   // 1x1 rows too long for the registers of one thread block
         float sc = L.sin[m];
         if (!(sc > 0.0f && sc < __int_as_float(0x7f800000))) sc = 1.0f;
         channel_body_clip(L, m, G, slice, sc, mode, qmax);
@@ -1381,6 +1383,10 @@ __device__ __forceinline__ void run_item(const LayerDesc &L, int ch0, unsigned c
     }
 }
 
+// kClip: layers of the launch have scales of their own.  (Without the bodies for these the others keep their values in
+// registers.  A spilled one comes back from L2, the L1 being shared memory: with 968 B of spill loads in a kernel for both four
+// 512x512x3x3 layers took 28.6 us on a B200, with 396 B 24.8.)
+template <bool kClip>
 __global__ void __launch_bounds__(kCtaThreads, SQ_MIN_CTAS)
 squant_model_kernel(const __grid_constant__ LaunchTable tbl, int qmax, unsigned mode)
 {
@@ -1392,7 +1398,7 @@ squant_model_kernel(const __grid_constant__ LaunchTable tbl, int qmax, unsigned 
         if (layer + step < tbl.n_layers && tbl.first_item[layer + step] <= item) layer += step;
     const LayerDesc &L = tbl.layers[layer];
     const int ch0 = (item - tbl.first_item[layer]) * (kCtaThreads >> L.g_shift);
-    run_item(L, ch0, smem, qmax, mode);
+    run_item<kClip>(L, ch0, smem, qmax, mode);
 }
 
 // The same with the descriptors in a table in global memory (used by the entry point whose
@@ -1404,7 +1410,7 @@ squant_table_kernel(const LayerDesc *__restrict__ layers, const Item *__restrict
     extern __shared__ __align__(16) unsigned char smem[];
     const Item it = items[blockIdx.x];
     const LayerDesc L = layers[it.layer];
-    run_item(L, it.ch0, smem, qmax, mode);
+    run_item<true>(L, it.ch0, smem, qmax, mode);
 }
 
 }  // namespace sq

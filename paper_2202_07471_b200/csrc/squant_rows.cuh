@@ -16,10 +16,10 @@
 //     elements).  T0 is searched among the maxima, the elements from T0 on are listed, and those of
 //     the first k_c ranks are flipped.  What that cannot settle (k_c beyond the number of maxima, a
 //     full list) goes to an exact search by counting.
-// With squant_conv.cuh: ResNet-50 shapes 84.5 -> 65.6 us device time on a B200, 55 thread-instructions per weight;
-// five linear layers of 125 M weights at 8 bit 267 -> 252 us.  With one barrier per reduction (a place for every warp
-// instead of shared atomics that have to be cleared first), loops counted without a division and the IEEE division out
-// of the SQuant-E loop: ResNet-50 shapes 69.8 -> 66.3 us a call, ResNet-18 shapes 36.4 -> 35.7, MobileNetV2 shapes 16.6 -> 16.4.
+// With squant_conv.cuh: ResNet-50 shapes 84.5 -> 65.6 us device time on a B200.  With loops of constant strides over a thread's vectors (a
+// warp of a longer row has a contiguous run of them), 22 instead of 30 thread-instructions a weight for SQuant-E in rows of 4096, and a list
+// that is made at a guessed bound before any search: 2 x 4096 rows of 4096 weights at 8 bit 65.5 -> 53.0 us a call, 16,384 of 512 29.2 -> 23.8,
+// 32,768 of 256 35.9 -> 28.9.
 #pragma once
 
 #include <cooperative_groups.h>
@@ -70,14 +70,16 @@ __host__ __device__ constexpr int sel_warps(int g, Owner own, int K) { return g 
 // Kernels of more than nine elements: a thread's maximum is put in when the direction of the flips is known, one word
 // instead of two and a barrier more, which the few kernels of such a channel hardly notice.
 __host__ __device__ constexpr bool late_maxima(int K) { return K > 9; }
-// Entries of a list.  Groups of 64, 128 and 256 threads on larger kernels: as many as make the group's selection memory
+// Entries of a list.  Groups of eight threads: 40, with which four thread blocks with 32 rows of 256 weights each share a multiprocessor
+// (with 64 three: ResNet-50 shapes 62.3 us on a B200, 57.4 with 40; mixed kernel sizes 47.1, 41.9; 65,536 rows of 192 weights alone
+// 38.3, 41.1, a matter of their last wave).  Groups of 64, 128 and 256 threads on larger kernels: as many as make the group's selection memory
 // 1,056, 2,144 and 3,104 B, with late maxima 1,056, 1,568 and 3,120 B.  The last figure is part of the longest
 // channel of few kernels that a thread block takes; the others decide how many channels share one (512 channels of 106
 // 7x7 kernels, four layers: two channels to a thread block 49.6 us on a B200, one 70.9).  The weights follow, so a multiple of 32 B: rows of
 // whole 32-byte sectors copied to an odd multiple of 16 cost 2000 rows of 21,000 weights 98.0 us instead of 91.8.
 __host__ __device__ constexpr int sel_cap(int g, int K = 1)
 {
-    return K == 1 ? (g <= 64 ? 64 : (g > 256 ? 472 : g))   // (472: 4,128 B with the parts)
+    return K == 1 ? (g == 8 ? 40 : g <= 64 ? 64 : (g > 256 ? 472 : g))   // (472: 4,128 B with the parts)
          : g > 256 ? (K > 16 ? 64 : g)
          : g <= 32 ? 64
          : late_maxima(K) ? (g == 64 ? 91 : (g == 128 ? 118 : 238))
@@ -153,6 +155,19 @@ __device__ __forceinline__ float absmax3(float a, float x, float y)
     float d;
     asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(fabsf(x)), "f"(fabsf(y)));
     return d;
+}
+
+// The same value, of which the compiler knows nothing: what follows from it is computed anew where it is used instead
+// of being kept in registers through the loops before.
+__device__ __forceinline__ int again(int v)
+{
+    asm volatile("" : "+r"(v));
+    return v;
+}
+extern __shared__ __align__(16) unsigned char g_smem[];
+__device__ __forceinline__ unsigned char *again(unsigned char *shared)
+{
+    return g_smem + again(static_cast<int>(smem_addr(shared) - smem_addr(g_smem)));
 }
 
 // ---------------------------------------------------------------- reductions inside a warp's group
@@ -331,98 +346,114 @@ __device__ __forceinline__ int shared_count(int *w)
     return old;
 }
 
-// a = the value of a candidate in the direction of the flips, n its kernel index in the channel.  The threads know
-// maxima of a over parts of their elements, in some unit: count(t) = how many of the group's nmax maxima are at least
-// t, t >= 1, below `top`, one unit above the largest possible.  listing(t, push) calls push(a, n, code) for those of
-// the thread's elements that are at least t units; code is handed through to flip.  For the exact search: settle()
-// once, then each(v, f) calls f(a, n) for those with a >= v (any v >= 1, vtop above all), code_of(n) is the code of one.  spread: the expected distance between the largest candidates in units
+// a = the value of a candidate in the direction of the flips, n its kernel index in the channel.  listing(t, push) calls
+// push(a, n, code) for those of the thread's elements that are at least t units, 1 <= t < top (`top` is one unit above
+// the largest possible); code is handed through to flip.  direct: from `start` on somewhat more than kc candidates are expected,
+// which are listed without a search.  If there is no such list or it will not do, the bound is searched: the threads know maxima of a
+// over parts of their elements, count(t) = how many of the group's nmax maxima are at least t (direct: prepare() once before, it may
+// write to shared memory).  For
+// the exact search: settle() once, then each(v, f) calls f(a, n) for those with a >= v (any v >= 1, vtop above all),
+// code_of(n) is the code of one.  spread: the expected distance between the largest candidates in units
 // of top / n_all.  flip(a, n, code) is called once for each of the min(kc, candidates) largest (equal values: lower
 // index first), by some thread of the group.  want: this group selects at all (kc >= 1).  Returns the number of
 // flips.  Every thread of the group calls it, groups that share a warp together; it starts with no barrier and
 // ends with none.
-template <Owner kOwn, class Count, class Listing, class Settle, class Each, class CodeOf, class Flip>
-__device__ __forceinline__ int select_top(const Group &G, Count count, Listing listing, Settle settle, Each each, CodeOf code_of, Flip flip, int nmax, int top, int vtop, float spread,
-                                          int kc, int n_all, bool want, const Sel &S, int K)
+template <Owner kOwn, class Prepare, class Count, class Listing, class Settle, class Each, class CodeOf, class Flip>
+__device__ __forceinline__ int select_top(const Group &G, Prepare prepare, Count count, Listing listing, Settle settle, Each each, CodeOf code_of, Flip flip, int nmax, bool direct, int start,
+                                          int top, int vtop, float spread, int kc, int n_all, bool want, const Sel &S, int K)
 {
     const int g = G.g, lane = threadIdx.x & 31;
     SelScratch *sc = S.sc;
     unsigned long long *list = S.list;
     const int cap = S.cap;
 
-    // ---- T0: at least kc of the maxima reach it, and not many more.  The first guess supposes an even
-    // spread; the distance to the top is doubled until it is enough, then the interval is halved (1x1:
-    // 1.1 rounds on normal and heavy-tailed weights of 4 and 8 bit, 3x3: 1.3 to 2.6; the list holds about
-    // kc + 3 elements for small, 1.6 kc for large kc).
-    int lo = 1, hi = top;
-    bool sure = false;   // lo has been counted
-    bool done = !want || kc > nmax;
-    const int slack = kc + (kc >> 1) + 6;
-    int mid = max(top - 1 - __float2int_rz(__fmul_rn(__fmul_rn(static_cast<float>(kc) + 1.0f, spread), __fdividef(static_cast<float>(top), static_cast<float>(n_all)))), 1);
-#pragma unroll 1
-    for (int it = 0; __any_sync(kFull, !done); ++it) {
-        const int c = count(mid, it);
-        if (!done) {
-            if (c >= kc) { lo = mid; sure = true; done = c <= slack; }
-            else hi = mid;
-            done = done || hi - lo <= 1;
-            mid = sure ? lo + ((hi - lo) >> 1) : max(hi - (top - hi), 1);
-        }
-    }
-    bool slow = want && !sure;   // fewer than kc maxima are candidates at all
-
-    // ---- list the elements from T0 on; where they are more than the list holds (many to a maximum: k_c is large
-    // for the number of maxima), once more from further up, supposing an even spread from T0 to the top.  Groups that
-    // share a warp go to the exact search at once, which takes them 8 to 10 k cycles where the other groups' lists, made again
-    // too, bring a second list to 16 to 24 k (ResNet-18 shapes with such a row among the last: 39.0 us on a B200, 36.5).
-    // From a warp a channel on the second list is the shorter way (4096 rows of 2048 weights 24.7 us, 28.0).
+    // ---- the elements from `lo` on are listed.  Round 0: from `start` on.  Where those are too few or more than the list
+    // holds, round 1 lists from a bound that the search has found: at least kc elements.  Where they are still more than the list
+    // holds (many to a maximum: k_c is large for the number of maxima), once more from further up, supposing an even
+    // spread from there to the top.  Groups that share a warp go to the exact search at once, which takes them 8 to 10 k cycles where
+    // the other groups' lists, made again too, bring a second list to 16 to 24 k (ResNet-18 shapes with such a row among the last:
+    // 39.0 us on a B200, 36.5).  From a warp a channel on the second list is the shorter way (4096 rows of 2048 weights 24.7 us, 28.0).
     int cnt = 0, all = 0;   // this list, all lists
-    int k_eff = want ? kc : 0;
+    int k_eff = want ? kc : 0, lo = max(start, 1);
     const unsigned long long *merged = list;
-    bool relist = false;
+    bool slow = false, todo = want;
+    auto search = [&] {
+        // T0: at least kc of the maxima reach it, and not many more.  The first guess supposes an even
+        // spread; the distance to the top is doubled until it is enough, then the interval is halved (1x1:
+        // 1.1 rounds on normal and heavy-tailed weights of 4 and 8 bit, 3x3: 1.3 to 2.6; the list holds about
+        // kc + 3 elements for small, 1.6 kc for large kc).
+        int hi = top;
+        bool sure = false;   // lo has been counted
+        bool done = !todo || kc > nmax;
+        const int slack = kc + (kc >> 1) + 6;
+        lo = 1;
+        int mid = max(top - 1 - __float2int_rz(__fmul_rn(__fmul_rn(static_cast<float>(kc) + 1.0f, spread), __fdividef(static_cast<float>(top), static_cast<float>(n_all)))), 1);
+#pragma unroll 1
+        for (int it = 0; __any_sync(kFull, !done); ++it) {
+            const int c = count(mid, it);
+            if (!done) {
+                if (c >= kc) { lo = mid; sure = true; done = c <= slack; }
+                else hi = mid;
+                done = done || hi - lo <= 1;
+                mid = sure ? lo + ((hi - lo) >> 1) : max(hi - (top - hi), 1);
+            }
+        }
+        slow = todo && !sure;   // fewer than kc maxima are candidates at all
+        todo = todo && sure;
+    };
 #pragma unroll 1
     for (int round = 0;; ++round) {
-        if (want && !slow && (round == 0 || relist))
-            listing(lo, [&](int a, int n, unsigned code) {
-                const int pos = shared_count(&sc->count);
-                SQ_DBG(a >= 1 && a < vtop && n >= 0 && n < n_all, 12);
-                if (pos < cap) list[pos] = list_key(a, n, code);
-            });
-        owner_sync<kOwn>(G);
-        cnt = all = sc->count;
-        bool full = false;
-        if (kOwn == kCluster) {   // every thread block collects all lists
-            unsigned long long *dst = list + cap;
-            merged = dst;
-            all = 0;
-            for (int c = 0; c < static_cast<int>(cg::this_cluster().num_blocks()); ++c) {
-                const int n = remote(&sc->count, c);
-                full = full || n > cap || all + n > merged_cap(K);
-                if (!full)
-                    for (int y = G.t; y < n; y += g) dst[all + y] = remote(list + y, c);
-                all += n;
+        if (round > 0 || direct) {
+            if (todo && (round > 0 || kc < cap))
+                listing(lo, [&](int a, int n, unsigned code) {
+                    const int pos = shared_count(&sc->count);
+                    SQ_DBG(a >= 1 && a < vtop && n >= 0 && n < n_all, 12);
+                    if (pos < cap) list[pos] = list_key(a, n, code);
+                });
+            owner_sync<kOwn>(G);
+            if (todo) cnt = all = sc->count;
+            bool full = false;
+            if (kOwn == kCluster) {   // every thread block collects all lists
+                unsigned long long *dst = list + cap;
+                merged = dst;
+                all = 0;
+                for (int c = 0; c < static_cast<int>(cg::this_cluster().num_blocks()); ++c) {
+                    const int n = remote(&sc->count, c);
+                    full = full || n > cap || all + n > merged_cap(K);
+                    if (!full)
+                        for (int y = G.t; y < n; y += g) dst[all + y] = remote(list + y, c);
+                    all += n;
+                }
+            } else {
+                full = cnt > cap;
             }
-        } else {
-            full = cnt > cap;
+            full = full && todo;
+            bool again = todo && (full || all < kc);
+            if (round > 0) {
+                if (kOwn == kGroup && g < 32) {
+                    slow = slow || full;
+                    break;
+                }
+                if (again && (!full || round > 3)) {   // (fewer than kc: too far up)
+                    slow = true;
+                    again = false;
+                }
+            }
+            if (kOwn == kCluster) __syncthreads();
+            if (!__any_sync(kFull, again)) break;   // (uniform over groups wider than a warp)
+            if (round > 0) {
+                const int goal = kc + ((min(cap, kOwn == kCluster ? merged_cap(K) : cap) - kc) >> 1);
+                const int up = top - __float2int_rz(__fmul_rn(static_cast<float>(top - lo), __fdividef(static_cast<float>(goal), static_cast<float>(all))));
+                if (goal <= kc || up <= lo || up >= top) { again = false; slow = true; }
+                lo = up;
+            }
+            owner_sync<kOwn>(G);   // everybody has read the lists
+            if (again && G.t == 0) sc->count = 0;
+            if (round == 0 && again) prepare();
+            owner_sync<kOwn>(G);
+            todo = again;
         }
-        full = full && want && !slow;
-        if (kOwn == kGroup && g < 32) {
-            slow = slow || full;
-            break;
-        }
-        if (round > 0 && relist && all < kc) slow = true;   // (too far up)
-        relist = full && round < 3;
-        if (full && !relist) slow = true;
-        if (kOwn == kCluster) __syncthreads();
-        if (!__any_sync(kFull, relist)) break;   // (uniform over groups wider than a warp)
-        const int goal = kc + ((min(cap, kOwn == kCluster ? merged_cap(K) : cap) - kc) >> 1);
-        if (relist) {
-            const int up = top - __float2int_rz(__fmul_rn(static_cast<float>(top - lo), __fdividef(static_cast<float>(goal), static_cast<float>(all))));
-            if (goal <= kc || up <= lo || up >= top) { relist = false; slow = true; }
-            lo = up;
-        }
-        owner_sync<kOwn>(G);   // everybody has read the lists
-        if (relist && G.t == 0) sc->count = 0;
-        owner_sync<kOwn>(G);
+        if (round == 0) search();
     }
     auto flip_entry = [&](unsigned long long e) {
         const unsigned low = static_cast<unsigned>(e);
@@ -547,14 +578,107 @@ __device__ __forceinline__ void row_clip_one(float Pf, int &P, unsigned c, int q
 }
 
 // ---------------------------------------------------------------- one 1x1 channel
+// Where a list for SQuant-C starts: from there on kc + kc / 4 + 6 of n_all values that are spread evenly from -top / 2 * spread
+// to top / 2 * spread are expected (2 to 3 % of such lists are too short).
+__device__ __forceinline__ int list_start(int kc, float spread, int top, int n_all)
+{
+    const float goal = static_cast<float>(kc) + static_cast<float>(kc >> 2) + 6.0f;
+    return top - 1 - __float2int_rz(__fmul_rn(__fmul_rn(goal, spread), __fdividef(static_cast<float>(top), static_cast<float>(n_all))));
+}
+
+// Weights: SQuant-C of shorter rows (which groups of at most a warp take) searches its bound first, since the guess takes in too many of their elements (the guess /
+// the search first, us on a B200: 131,072 rows of 64 49.2 / 45.0, 65,536 of 96 31.9 / 30.0, of 128 33.0 / 32.4, of 160 37.1 / 36.9, of 192 39.1 / 41.1,
+// 32,768 of 256 29.7 / 34.4).
+constexpr int kRowDirect = 176;
+
+// What a thread knows of the perturbations it has made: their sum modulo 2^32 and as floats, the extremes over
+// every other vector.
+struct RowSums {
+    unsigned sum;
+    float2 fs;
+    int hi[2], lo[2];
+};
+
+// SQuant-E on one vector by the reciprocal sequence.  Returns the codes as packed bytes.
+__device__ __forceinline__ unsigned row_vector(const float4 w, const E2 &c2, RowSums &R, int which, int4 &p)
+{
+    float2 ta, tb, Pa, Pb;
+    squant_e_fast2(make_float2(w.x, w.y), c2, ta, Pa);
+    squant_e_fast2(make_float2(w.z, w.w), c2, tb, Pb);
+    p = make_int4(__float2int_rn(Pa.x), __float2int_rn(Pa.y), __float2int_rn(Pb.x), __float2int_rn(Pb.y));
+    R.fs = __fadd2_rn(R.fs, Pa);
+    R.fs = __fadd2_rn(R.fs, Pb);
+    R.sum += static_cast<unsigned>(p.x) + static_cast<unsigned>(p.y);
+    R.sum += static_cast<unsigned>(p.z) + static_cast<unsigned>(p.w);
+    R.hi[which] = __vimax3_s32(__vimax3_s32(R.hi[which], p.x, p.y), p.z, p.w);
+    R.lo[which] = __vimin3_s32(__vimin3_s32(R.lo[which], p.x, p.y), p.z, p.w);
+    return __byte_perm(__byte_perm(__float_as_uint(ta.x), __float_as_uint(ta.y), 0x0040),
+                       __byte_perm(__float_as_uint(tb.x), __float_as_uint(tb.y), 0x0040), 0x5410);
+}
+__device__ __forceinline__ float4 row_error_sums(const int4 p)
+{
+    const float2 k30 = make_float2(0x1p-30f, 0x1p-30f);
+    const float2 a = __fmul2_rn(make_float2(__int2float_rn(p.x), __int2float_rn(p.y)), k30);
+    const float2 b = __fmul2_rn(make_float2(__int2float_rn(p.z), __int2float_rn(p.w)), k30);
+    return make_float4(a.x, a.y, b.x, b.y);
+}
+
+// The loops over a thread's vectors, which lie kStep vectors apart (a constant: the addresses of a step are immediates).
+template <int kStep>
+__device__ __forceinline__ float row_stage(float4 *w, const float4 *src, int vecs)
+{
+    float amax = 0.0f;
+#pragma unroll 4
+    for (int i = 0; i < vecs; ++i) copy_async16(w + i * kStep, src + i * kStep);
+    copy_async_wait();
+#pragma unroll 4
+    for (int i = 0; i < vecs; ++i) {
+        const float4 v = w[i * kStep];
+        amax = absmax3(absmax3(amax, v.x, v.y), v.z, v.w);
+    }
+    return amax;
+}
+template <int kStep, bool kErr>
+__device__ __forceinline__ void row_quantize(float4 *w, unsigned *codes, float4 *kerr, int vecs, const E2 &c2, RowSums &R)
+{
+#pragma unroll 1
+    for (; vecs > 1; vecs -= 2) {
+        const float4 w0 = w[0], w1 = w[kStep];
+        int4 p0, p1;
+        codes[0] = row_vector(w0, c2, R, 0, p0);
+        codes[kStep] = row_vector(w1, c2, R, 1, p1);
+        reinterpret_cast<int4 *>(w)[0] = p0;
+        reinterpret_cast<int4 *>(w)[kStep] = p1;
+        if (kErr) {
+            __stcs(kerr, row_error_sums(p0));
+            __stcs(kerr + kStep, row_error_sums(p1));
+            kerr += 2 * kStep;
+        }
+        w += 2 * kStep;
+        codes += 2 * kStep;
+    }
+    if (vecs > 0) {
+        int4 p;
+        codes[0] = row_vector(w[0], c2, R, 0, p);
+        reinterpret_cast<int4 *>(w)[0] = p;
+        if (kErr) __stcs(kerr, row_error_sums(p));
+    }
+}
+
 // kClip: the clip of Sec. 2.2 can fire (caller-supplied scales): codes are clamped, sums are 64
 // bit and an element whose flipped code would leave the range is no candidate.  valid = false: the
 // group has no channel (its lanes take part in the warp's steps and write nothing).  kBlock: a row of the row kernel
-// (see build_param_plan); the search then counts the threads' two maxima by barriers.
-template <bool kClip, Owner kOwn = kGroup>
-__device__ __forceinline__ void row_body(const LayerDesc &L, int m, const Group &G, unsigned char *slice, int qmax, unsigned mode, bool valid)
+// (see build_param_plan).  kLanes: lanes of a warp that share the row - 8 or 16: the whole group; 32: a warp or more, each warp has a
+// contiguous run of vectors; 0: any of these.
+template <bool kClip, Owner kOwn, int kLanes>
+__device__ __forceinline__ void row_body(const LayerDesc &L, int m, const Group &group, unsigned char *slice, int qmax, unsigned mode, bool valid)
 {
-    static_assert(kOwn != kCluster, "");
+    static_assert(kOwn != kCluster && (kOwn == kGroup || kLanes == 32), "");
+    Group G = group;
+    if (kLanes != 0 && kLanes < 32) {
+        G.g = kLanes;
+        G.sh = kLanes == 8 ? 3 : 4;
+    }
     const int g = G.g, N = valid ? L.N : 0;
     const Sel S(slice, g, kOwn, 1);
     if (G.t == 0) {
@@ -567,7 +691,12 @@ __device__ __forceinline__ void row_body(const LayerDesc &L, int m, const Group 
     // the row's start, so there the vectors start with the row).
     const bool pack = (mode & kModePackInt4) != 0;
     const Span sp(pack ? 0 : static_cast<int>((reinterpret_cast<uintptr_t>(wrow) >> 2) & 3), N, G.t);
-    const int r = sp.r, q_hi = sp.q_hi, rag = sp.rag, q0 = sp.q_lo + G.t, vecs = G.rounds(sp.q_lo, sp.q_hi);   // vectors q0, q0 + g, ..
+    const int r = sp.r, q_hi = sp.q_hi, rag = sp.rag;
+    // this thread's vectors: q0, q0 + step, .., `vecs` of them
+    const int sh = kLanes == 8 ? 3 : (kLanes == 16 ? 4 : (kLanes == 32 ? 5 : min(G.sh, 5))), step = 1 << sh;
+    const int run = kLanes != 0 && kLanes < 32 ? 0 : (G.t >> 5) * (((q_hi - sp.q_lo + g - 1) >> G.sh) << 5);   // of the warps before this one
+    const int q0 = sp.q_lo + run + (G.t & (step - 1));
+    const int vecs = kLanes != 0 && kLanes < 32 ? (q_hi - q0 + step - 1) >> sh : min((q_hi - q0 + step - 1) >> sh, (q_hi - sp.q_lo + g - 1) >> G.sh);
     SQ_DBG(N >= 0 && N + r <= 4 * L.off_vi && q_hi <= L.off_vi, 14);   // the vectors' places below
     const int sel = kOwn == kBlock ? sel_list_bytes(g, kOwn, 1) : sel_bytes(g);   // (a thread block keeps no maxima in shared memory)
     int4 *Pbuf = reinterpret_cast<int4 *>(slice + sel);              // what SQuant-C may choose from
@@ -581,21 +710,25 @@ __device__ __forceinline__ void row_body(const LayerDesc &L, int m, const Group 
     // faster than the old one, because code that every warp runs through once waits for its instructions.)
     float amax = 0.0f;
     {
-        const float4 *src = reinterpret_cast<const float4 *>(wrow - r);
-        if ((reinterpret_cast<uintptr_t>(src) & 15) == 0) {
-#pragma unroll 2
-            for (int i = 0; i < vecs; ++i) copy_async16(Pbuf + q0 + i * g, src + q0 + i * g);
-        } else {   // packed codes of a misaligned row
-#pragma unroll 1
-            for (int q = q0; q < q_hi; q += g)
-                for (int c = 0; c < 4; ++c) copy_async4(Pel + 4 * q + c, wrow + 4 * q + c);
-        }
+        float4 *w = reinterpret_cast<float4 *>(Pbuf) + q0;
+        const float4 *src = reinterpret_cast<const float4 *>(wrow - r) + q0;
         if (rag >= 0) copy_async4(Pel + rag, wrow + rag);
-        copy_async_wait();
+        if (kLanes != 0 && (!pack || (reinterpret_cast<uintptr_t>(src) & 15) == 0)) {
+            amax = row_stage<kLanes ? kLanes : 1>(w, src, vecs);
+        } else {
+            const bool whole = (reinterpret_cast<uintptr_t>(src) & 15) == 0;   // (packed codes of a misaligned row)
+#pragma unroll 1
+            for (int i = 0; i < vecs; ++i) {
+                if (whole) copy_async16(w + i * step, src + i * step);
+                else
+                    for (int c = 0; c < 4; ++c) copy_async4(reinterpret_cast<float *>(w + i * step) + c, reinterpret_cast<const float *>(src + i * step) + c);
+            }
+            copy_async_wait();
 #pragma unroll 2
-        for (int i = 0; i < vecs; ++i) {
-            const float4 v = reinterpret_cast<const float4 *>(Pbuf)[q0 + i * g];
-            amax = absmax3(absmax3(amax, v.x, v.y), v.z, v.w);
+            for (int i = 0; i < vecs; ++i) {
+                const float4 v = w[i * step];
+                amax = absmax3(absmax3(amax, v.x, v.y), v.z, v.w);
+            }
         }
     }
     float w_rag = 0.0f;
@@ -614,16 +747,17 @@ __device__ __forceinline__ void row_body(const LayerDesc &L, int m, const Group 
     // the few it flips)
     const bool fast = s >= 0x1p-60f && s <= 0x1p60f;
     const int qmin = (mode & kModeWideRange) ? -qmax - 1 : -qmax;
-    unsigned sum = 0u;
-    float2 fs = make_float2(0.0f, 0.0f);
+    RowSums R;
+    R.sum = 0u;
+    R.fs = make_float2(0.0f, 0.0f);
+    R.hi[0] = R.hi[1] = R.lo[0] = R.lo[1] = 0;   // of the even and the odd ones of the thread's vectors
     long long sum64 = 0;
-    int hi0 = 0, hi1 = 0, lo0 = 0, lo1 = 0;   // extremes over every other vector
     {
         const float s2 = fast ? __fmul_rn(s, 0x1p-30f) : 0.0f;
         const E2 c2 = make_e2(fast ? __frcp_rn(s2) : 0.0f, s2);
         const float tmin = kMagic + static_cast<float>(qmin) * 1073741824.0f, tmax = kMagic + static_cast<float>(qmax) * 1073741824.0f;
         const bool kvec = ((reinterpret_cast<uintptr_t>(kerr) - 4 * r) & 15) == 0;
-        auto quantize = [&](const float4 w, int4 &p, float2 &oa, float2 &ob) -> unsigned {
+        auto quantize = [&](const float4 w, int4 &p, float2 &oa, float2 &ob, int which) -> unsigned {
             float2 Pa, Pb;
             unsigned c4;
             if (fast) {
@@ -641,8 +775,8 @@ __device__ __forceinline__ void row_body(const LayerDesc &L, int m, const Group 
                     ta.y = fminf(fmaxf(ta.y, tmin), tmax);
                     tb.x = fminf(fmaxf(tb.x, tmin), tmax);
                     tb.y = fminf(fmaxf(tb.y, tmin), tmax);
-                    Pa = __ffma2_rn(Xa, c2.neg1, __fadd2_rn(ta, c2.nmagic));
-                    Pb = __ffma2_rn(Xb, c2.neg1, __fadd2_rn(tb, c2.nmagic));
+                    Pa = __ffma2_rn(Xa, c2.neg1, __ffma2_rn(c2.magic, c2.neg1, ta));
+                    Pb = __ffma2_rn(Xb, c2.neg1, __ffma2_rn(c2.magic, c2.neg1, tb));
                 }
                 c4 = __byte_perm(__byte_perm(__float_as_uint(ta.x), __float_as_uint(ta.y), 0x0040),
                                  __byte_perm(__float_as_uint(tb.x), __float_as_uint(tb.y), 0x0040), 0x5410);
@@ -654,10 +788,10 @@ __device__ __forceinline__ void row_body(const LayerDesc &L, int m, const Group 
             }
             p = make_int4(__float2int_rn(Pa.x), __float2int_rn(Pa.y), __float2int_rn(Pb.x), __float2int_rn(Pb.y));
             if (!kClip) {
-                fs = __fadd2_rn(fs, Pa);
-                fs = __fadd2_rn(fs, Pb);
-                sum += static_cast<unsigned>(p.x) + static_cast<unsigned>(p.y);
-                sum += static_cast<unsigned>(p.z) + static_cast<unsigned>(p.w);
+                R.fs = __fadd2_rn(R.fs, Pa);
+                R.fs = __fadd2_rn(R.fs, Pb);
+                R.sum += static_cast<unsigned>(p.x) + static_cast<unsigned>(p.y);
+                R.sum += static_cast<unsigned>(p.z) + static_cast<unsigned>(p.w);
                 oa = make_float2(__int2float_rn(p.x), __int2float_rn(p.y));
                 ob = make_float2(__int2float_rn(p.z), __int2float_rn(p.w));
             } else {
@@ -666,33 +800,37 @@ __device__ __forceinline__ void row_body(const LayerDesc &L, int m, const Group 
                 row_clip_one(Pb.x, p.z, c4 >> 16, qmin, qmax, sum64, ob.x);
                 row_clip_one(Pb.y, p.w, c4 >> 24, qmin, qmax, sum64, ob.y);
             }
-            if (mode & 4u) {   // the extremes change places with those of the thread's other vectors
-                const int h1 = __vimax3_s32(hi0, p.x, p.y), l1 = __vimin3_s32(lo0, p.x, p.y);
-                hi0 = hi1; lo0 = lo1;
-                hi1 = __vimax3_s32(h1, p.z, p.w); lo1 = __vimin3_s32(l1, p.z, p.w);
-            }
+            const int h = __vimax3_s32(__vimax3_s32(p.x, p.y, p.z), p.w, 0), l = __vimin3_s32(__vimin3_s32(p.x, p.y, p.z), p.w, 0);
+            if (which == 0) { R.hi[0] = max(R.hi[0], h); R.lo[0] = min(R.lo[0], l); }
+            else { R.hi[1] = max(R.hi[1], h); R.lo[1] = min(R.lo[1], l); }
             const float2 k30 = make_float2(0x1p-30f, 0x1p-30f);
             oa = __fmul2_rn(oa, k30);
             ob = __fmul2_rn(ob, k30);
             return c4;
         };
-#pragma unroll 2
-        for (int i = 0; i < vecs; ++i) {
-            const int q = q0 + i * g;
-            int4 p;
-            float2 oa, ob;
-            cbuf[q] = quantize(reinterpret_cast<const float4 *>(Pbuf)[q], p, oa, ob);
-            Pbuf[q] = p;
-            if (kerr) {
-                float *ke = kerr + (4 * q - r);
-                if (kvec) __stcs(reinterpret_cast<float4 *>(ke), make_float4(oa.x, oa.y, ob.x, ob.y));
-                else { ke[0] = oa.x; ke[1] = oa.y; ke[2] = ob.x; ke[3] = ob.y; }
+        if (!kClip && kLanes != 0 && __all_sync(kFull, fast && (!kerr || kvec))) {   // (uniform for groups of whole warps)
+            constexpr int kStep = kLanes ? kLanes : 1;
+            if (kerr) row_quantize<kStep, true>(reinterpret_cast<float4 *>(Pbuf) + q0, cbuf + q0, reinterpret_cast<float4 *>(kerr - r) + q0, vecs, c2, R);
+            else row_quantize<kStep, false>(reinterpret_cast<float4 *>(Pbuf) + q0, cbuf + q0, nullptr, vecs, c2, R);
+        } else {
+#pragma unroll 1
+            for (int i = 0; i < vecs; ++i) {
+                const int q = q0 + i * step;
+                int4 p;
+                float2 oa, ob;
+                cbuf[q] = quantize(reinterpret_cast<const float4 *>(Pbuf)[q], p, oa, ob, i & 1);
+                Pbuf[q] = p;
+                if (kerr) {
+                    float *ke = kerr + (4 * q - r);
+                    if (kvec) __stcs(reinterpret_cast<float4 *>(ke), make_float4(oa.x, oa.y, ob.x, ob.y));
+                    else { ke[0] = oa.x; ke[1] = oa.y; ke[2] = ob.x; ke[3] = ob.y; }
+                }
             }
         }
         if (sp.ragged) {
             int4 p;
             float2 oa, ob;
-            const unsigned c4 = quantize(make_float4(w_rag, 0.0f, 0.0f, 0.0f), p, oa, ob);
+            const unsigned c4 = quantize(make_float4(w_rag, 0.0f, 0.0f, 0.0f), p, oa, ob, 0);
             if (rag >= 0) {
                 cel[rag] = static_cast<unsigned char>(c4);
                 Pel[rag] = p.x;
@@ -704,19 +842,9 @@ __device__ __forceinline__ void row_body(const LayerDesc &L, int m, const Group 
     // ---- channel sum.  !kClip: its value modulo 2^32 is exact, its size is known from the float sums
     // (2^16 elements of at most one half: the float sums are off by far less than 2^30)
     long long ec = 0;
-    const int per = g > 64 ? 1 : 2;   // maxima a thread puts in
     if ((mode & 4u) || L.cerr) {
-        if (kOwn == kGroup && g > 32) {   // those that SQuant-C looks for its bound among, of either sign
-            if (per == 2) {
-                S.mx[G.t] = hi0; S.mx[G.t + g] = hi1;
-                S.mx[G.t + 2 * g] = -lo0; S.mx[G.t + 3 * g] = -lo1;
-            } else {
-                S.mx[G.t] = max(hi0, hi1);
-                S.mx[G.t + g] = -min(lo0, lo1);
-            }
-        }
         int up = 0, down = 0;
-        ec = owner_sum<kOwn, kClip, false>(G, S, sum64, sum, __float2int_rn(__fmul_rn(__fadd_rn(fs.x, fs.y), 0x1p-17f)), up, down);
+        ec = owner_sum<kOwn, kClip, false>(G, S, sum64, R.sum, __float2int_rn(__fmul_rn(__fadd_rn(R.fs.x, R.fs.y), 0x1p-17f)), up, down);
     }
 
     // ---- SQuant-C: Algorithm 2 on the channel, the perturbations are the keys
@@ -726,16 +854,18 @@ __device__ __forceinline__ void row_body(const LayerDesc &L, int m, const Group 
         const int kc = static_cast<int>(min((abs_e + (kHalf - 1)) >> 30, 1ll << 30));
         const bool want = kc > 0;
         if (g <= 32 ? __any_sync(kFull, want) : want) {
-            const int m0 = sgn > 0 ? hi0 : -lo0, m1 = sgn > 0 ? hi1 : -lo1;
+            const int m0 = sgn > 0 ? R.hi[0] : -R.lo[0], m1 = sgn > 0 ? R.hi[1] : -R.lo[1];
             const int sx = sgn > 0 ? 0 : -1;   // p ^ sx = the value in the direction of the flips, less one if that is downward
-            auto each = [&](int t, auto fn) {
+            // the elements of value t and more, in the vectors of `halves` (bit 0: the even ones, bit 1: the odd ones)
+            auto visit = [&](int t, unsigned halves, auto fn) {
                 const int tx = t + sx;
 #pragma unroll 1
-                for (int ib = 0; ib < vecs; ib += kRowVecs) {   // (groups: once)
+                for (; halves != 0u; halves &= halves - 1u) {
+                    const int odd = __ffs(halves) - 1;
                     unsigned hit = 0u, bit = 1u;   // a bit for each of these (at most 32) elements that counts
 #pragma unroll 2
-                    for (int i = ib; i < min(vecs, ib + kRowVecs); ++i, bit <<= 4) {
-                        const int4 p = Pbuf[q0 + i * g];
+                    for (int i = odd; i < vecs; i += 2, bit <<= 4) {
+                        const int4 p = Pbuf[q0 + i * step];
                         if ((p.x ^ sx) >= tx) hit |= bit;
                         if ((p.y ^ sx) >= tx) hit |= 2u * bit;
                         if ((p.z ^ sx) >= tx) hit |= 4u * bit;
@@ -743,30 +873,37 @@ __device__ __forceinline__ void row_body(const LayerDesc &L, int m, const Group 
                     }
 #pragma unroll 1
                     for (; hit != 0u; hit &= hit - 1u) {
-                        const int b = __ffs(hit) - 1, n = 4 * (q0 + (ib + (b >> 2)) * g) - r + (b & 3);
+                        const int b = __ffs(hit) - 1, n = 4 * (q0 + (odd + 2 * (b >> 2)) * step) - r + (b & 3);
                         SQ_DBG(n >= 0 && n < N, 15);
                         fn((Pel[n] ^ sx) - sx, n);
                     }
-                    if (kOwn == kGroup) break;
                 }
                 if (rag >= 0) {
                     const int v = Pel[rag] ^ sx;
                     if (v >= tx) fn(v - sx, rag);
                 }
             };
-            auto listing = [&](int t, auto push) {
-                if (max(m0, m1) >= t) each(t, [&](int a, int n) { push(a, n, 0u); });   // (the codes are here)
-            };
+            auto each = [&](int t, auto fn) { visit(t, 3u, fn); };
+            auto listing = [&](int t, auto push) { visit(t, (m0 >= t ? 1u : 0u) | (m1 >= t ? 2u : 0u), [&](int a, int n) { push(a, n, 0u); }); };   // (the codes are here)
             const int lane = threadIdx.x & 31;
             const unsigned gmask = g >= 32 ? kFull : (((1u << g) - 1u) << (lane & ~(g - 1)));
-            const int *mx = sgn > 0 ? S.mx : S.mx + per * g;
+            const int per = g > 64 ? 1 : 2;   // maxima a thread puts in
+            auto prepare = [&] {
+                if (kOwn == kBlock || g <= 32) return;
+                if (per == 2) {
+                    S.mx[G.t] = m0;
+                    S.mx[G.t + g] = m1;
+                } else {
+                    S.mx[G.t] = max(m0, m1);
+                }
+            };
             auto count = [&](int t, int) {
                 if (kOwn == kBlock) return __syncthreads_count(m0 >= t) + __syncthreads_count(m1 >= t);
                 if (g <= 32) return __popc(__ballot_sync(kFull, m0 >= t) & gmask) + __popc(__ballot_sync(kFull, m1 >= t) & gmask);
                 int c = 0;
 #pragma unroll 1
                 for (int i = lane; i < ((per * g) >> 2); i += 32) {
-                    const int4 q = reinterpret_cast<const int4 *>(mx)[i];
+                    const int4 q = reinterpret_cast<const int4 *>(S.mx)[i];
                     c += (q.x >= t) + (q.y >= t) + (q.z >= t) + (q.w >= t);
                 }
                 return __reduce_add_sync(kFull, c);
@@ -778,7 +915,8 @@ __device__ __forceinline__ void row_body(const LayerDesc &L, int m, const Group 
                 if (kerr) kerr[n] = __fmul_rn(__int2float_rn(sgn > 0 ? a - kOne : kOne - a), 0x1p-30f);
             };
             const int vtop = kHalf + (1 << 14) + 1;
-            const int k_eff = select_top<kOwn>(G, count, listing, [] {}, each, [](int) { return 0u; }, flip, kOwn == kBlock ? 2 * g : per * g, vtop, vtop, 2.0f, kc, N, want, S, 1);
+            const int k_eff = select_top<kOwn>(G, prepare, count, listing, [] {}, each, [](int) { return 0u; }, flip, kOwn == kBlock ? 2 * g : per * g, L.N >= kRowDirect,
+                                               list_start(kc, 2.0f, vtop, max(N, 1)), vtop, vtop, 2.0f, kc, N, want, S, 1);
             ec -= static_cast<long long>(sgn) * k_eff * kOne;
         }
     }
@@ -789,13 +927,19 @@ __device__ __forceinline__ void row_body(const LayerDesc &L, int m, const Group 
     if (!valid) return;
 
     // ---- codes, scale, channel error
+    const size_t first_code = static_cast<size_t>(again(m)) * L.N;
     if (!pack) {
-        unsigned char *crow = reinterpret_cast<unsigned char *>(L.codes) + first;
+        unsigned char *crow = reinterpret_cast<unsigned char *>(L.codes) + first_code;
         if (((reinterpret_cast<uintptr_t>(crow) - r) & 3) == 0) {
             unsigned *dst = reinterpret_cast<unsigned *>(crow - r);
+            if (((reinterpret_cast<uintptr_t>(crow) | static_cast<unsigned>(N) | (4u * r)) & 15) == 0) {   // the whole row in words of 16 bytes
+#pragma unroll 2
+                for (int i = G.t; i < (N >> 4); i += g) __stcs(reinterpret_cast<int4 *>(dst) + i, reinterpret_cast<const int4 *>(cbuf)[i]);
+            } else {
 #pragma unroll 4
-            for (int i = 0; i < vecs; ++i) __stcs(dst + q0 + i * g, cbuf[q0 + i * g]);
-            if (rag >= 0) crow[rag] = cel[rag];
+                for (int i = 0; i < vecs; ++i) __stcs(dst + q0 + i * step, cbuf[q0 + i * step]);
+                if (rag >= 0) crow[rag] = cel[rag];
+            }
         } else {
             for (int n = G.t; n < N; n += g) crow[n] = cel[n];
         }
@@ -803,7 +947,8 @@ __device__ __forceinline__ void row_body(const LayerDesc &L, int m, const Group 
         unsigned char *crow = reinterpret_cast<unsigned char *>(L.codes) + static_cast<size_t>(m) * ((L.N + 1) >> 1);
         const bool two = (reinterpret_cast<uintptr_t>(crow) & 1) == 0;
 #pragma unroll 1
-        for (int q = q0; q < q_hi; q += g) {
+        for (int i = 0; i < vecs; ++i) {
+            const int q = q0 + i * step;
             const unsigned b = cbuf[q] & 0x0f0f0f0fu, h = b | (b >> 4);
             if (two) {
                 *reinterpret_cast<unsigned short *>(crow + 2 * q) = static_cast<unsigned short>((h & 255u) | ((h >> 8) & 0xff00u));
@@ -815,10 +960,11 @@ __device__ __forceinline__ void row_body(const LayerDesc &L, int m, const Group 
         if (rag >= 0 && (rag & 1) == 0) crow[rag >> 1] = static_cast<unsigned char>((cel[rag] & 15) | (rag + 1 < N ? cel[rag + 1] << 4 : 0));
     }
     if (L.deq) {   // Algorithm 1's own return value: code * s
-        float *dg = L.deq + first;
+        float *dg = L.deq + first_code;
         const bool vec = ((reinterpret_cast<uintptr_t>(dg) - 4 * r) & 15) == 0;
 #pragma unroll 1
-        for (int q = q0; q < q_hi; q += g) {
+        for (int i = 0; i < vecs; ++i) {
+            const int q = q0 + i * step;
             const unsigned c4 = cbuf[q];
             const float4 d = make_float4(row_deq(c4, s), row_deq(c4 >> 8, s), row_deq(c4 >> 16, s), row_deq(c4 >> 24, s));
             float *o = dg + (4 * q - r);
@@ -828,10 +974,11 @@ __device__ __forceinline__ void row_body(const LayerDesc &L, int m, const Group 
         if (rag >= 0) dg[rag] = row_deq(cel[rag], s);
     }
     if (L.deq16) {   // the same product as bfloat16
-        uint16_t *dg = L.deq16 + first;
+        uint16_t *dg = L.deq16 + first_code;
         const bool vec = ((reinterpret_cast<uintptr_t>(dg) - 2 * r) & 7) == 0;
 #pragma unroll 1
-        for (int q = q0; q < q_hi; q += g) {
+        for (int i = 0; i < vecs; ++i) {
+            const int q = q0 + i * step;
             const unsigned c4 = cbuf[q];
             const unsigned b0 = bf16_bits(row_deq(c4, s)), b1 = bf16_bits(row_deq(c4 >> 8, s));
             const unsigned b2 = bf16_bits(row_deq(c4 >> 16, s)), b3 = bf16_bits(row_deq(c4 >> 24, s));

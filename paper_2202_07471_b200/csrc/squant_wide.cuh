@@ -84,8 +84,8 @@ __device__ __forceinline__ void row_quad(const float4 w, const RowQuant &R, Quad
             tb.y = fminf(fmaxf(tb.y, tmin), tmax);
         }
     }
-    o.qa = __fadd2_rn(ta, R.c2.nmagic);
-    o.qb = __fadd2_rn(tb, R.c2.nmagic);
+    o.qa = __ffma2_rn(R.c2.magic, R.c2.neg1, ta);
+    o.qb = __ffma2_rn(R.c2.magic, R.c2.neg1, tb);
     o.Pa = __ffma2_rn(Xa, R.c2.neg1, o.qa);
     o.Pb = __ffma2_rn(Xb, R.c2.neg1, o.qb);
     o.c4 = __byte_perm(__byte_perm(__float_as_uint(ta.x), __float_as_uint(ta.y), 0x0040),
@@ -423,7 +423,7 @@ __device__ __forceinline__ void long_row_body(const LayerDesc &L, int m, const G
                 if (deq16) deq16[n] = static_cast<uint16_t>(bf16_bits(row_deq(c, s)));
             };
             const int nmax = kOwn == kCluster ? 4 * g * static_cast<int>(cg::this_cluster().num_blocks()) : g;
-            const int k_eff = select_top<kOwn>(G, count, listing, settle, each, code_of, flip, nmax, (kHalf >> 16) + 1, kHalf + (1 << 14) + 1, 2.0f, kc, L.N, want, S, 1);
+            const int k_eff = select_top<kOwn>(G, [] {}, count, listing, settle, each, code_of, flip, nmax, false, 0, (kHalf >> 16) + 1, kHalf + (1 << 14) + 1, 2.0f, kc, L.N, want, S, 1);
             ec -= static_cast<long long>(sgn) * k_eff * kOne;
         }
     }
@@ -482,8 +482,8 @@ squant_row_kernel(const __grid_constant__ LaunchTable tbl, int qmax, unsigned mo
         else long_row_body<false, kBlock>(L, m, G, smem, qmax, mode);
     } else {
         SQ_DBG(row_bytes(kThreads, L.off_vi, kBlock) <= static_cast<int>(dynamic_smem_bytes()), 10);
-        if (L.sin) row_body<true, kBlock>(L, m, G, smem, qmax, mode, true);
-        else row_body<false, kBlock>(L, m, G, smem, qmax, mode, true);
+        if (L.sin) row_body<true, kBlock, 32>(L, m, G, smem, qmax, mode, true);
+        else row_body<false, kBlock, 32>(L, m, G, smem, qmax, mode, true);
     }
 }
 

@@ -98,6 +98,17 @@ def test_rows_with_full_lists(shape):
     check([w], 4, start=2, clip=0.9)
 
 
+@pytest.mark.parametrize("n", [64, 175, 176, 177, 255, 258, 513, 1030, 4100])
+def test_rows_whose_list_starts_at_a_guess(n):
+    """SQuant-C of rows from 176 weights on lists from a guessed bound first: rows for which the guess is good, too high
+    (two bits and outliers: few candidates come near one half) and too low (one-signed weights, ties: a full list)."""
+    shape = (400 if n < 1000 else 100, n, 1, 1)
+    w = W.random_layer(shape, seed=n)
+    ws = [w, np.where(W.random_layer(shape, seed=n + 1) > 2.0 * w.std(), 8 * w, w)] + layers((5,) + shape[1:], n)
+    for bits in (2, 4, 8):
+        check(ws, bits, start=bits % 3)
+
+
 @pytest.mark.parametrize("shape", [(2, 1, 1, 45857), (3, 2, 1, 22928), (2, 9, 1, 5095), (2, 200, 1, 229), (5, 106, 7, 7), (9, 52, 7, 7), (9, 103, 5, 5)])
 def test_larger_kernels_at_the_sizes_that_share_a_thread_block(shape):
     """The longest channels of few large kernels that one thread block, or two and four channels that share one, hold;
