@@ -342,7 +342,7 @@ int share_with_graph(const ScratchRef &scratch, cudaGraph_t graph)
 // CTAs (heaviest first, so the tail of the launch is made of light CTAs), at most
 // kMaxParamLayers per launch.
 struct ParamPlan {
-    struct Grouped { sq::LaunchTable table; int grid, smem; bool clip; };   // clip: some layer has scales of its own
+    struct Grouped { sq::LaunchTable table; int grid, smem; sq::Scales scales; };
     std::vector<Grouped> grouped;   // grouped kernel: one CTA per item
     int qmax = 0;
     unsigned mode = 0;
@@ -562,12 +562,13 @@ int build_param_plan(const squant_layer *layers, int32_t n_layers, const squant_
         p.grouped.emplace_back();
         ParamPlan::Grouped &gl = p.grouped.back();
         gl.smem = 0;
-        gl.clip = false;
+        size_t own = 0;   // layers with scales of their own
         for (size_t j = 0; j < n; ++j) {
             const LayerDesc &d = descs[order[base + j]];
-            gl.clip = gl.clip || d.sin;
+            own += d.sin ? 1 : 0;
             gl.smem = std::max(gl.smem, sq::kCtaThreads / d.g * d.slice_bytes);
         }
+        gl.scales = own == 0 ? sq::kAbsmax : (own == n ? sq::kOwnScales : sq::kEither);
         gl.grid = fill_table(gl.table, descs, order.data() + base, static_cast<int>(n), true);
         base += n;
     }
@@ -600,10 +601,8 @@ int device_smem_limit(int device, int &limit)
     if (g_smem_limit_by_device[device] == 0) {
         int v = 0;
         SQ_CUDA(cudaDeviceGetAttribute(&v, cudaDevAttrMaxSharedMemoryPerBlockOptin, device));
-        SQ_CUDA(cudaFuncSetAttribute(sq::squant_model_kernel<false>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, v));
-        SQ_CUDA(cudaFuncSetAttribute(sq::squant_model_kernel<true>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, v));
+        for (auto kernel : {sq::squant_model_kernel<sq::kAbsmax>, sq::squant_model_kernel<sq::kOwnScales>, sq::squant_model_kernel<sq::kEither>})
+            SQ_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, v));
         SQ_CUDA(cudaFuncSetAttribute(sq::squant_table_kernel,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, v));
         SQ_CUDA(cudaFuncSetAttribute((sq::squant_row_kernel<256, true>),
@@ -722,7 +721,7 @@ int launch_plan(const ParamPlan &p, cudaStream_t stream)
             auto kernel = st.out ? sq::squant_stream_kernel<true> : sq::squant_stream_kernel<false>;
             kernel<<<grid, sq::kStreamThreads, smem, stream>>>(st.table, p.qmax, p.mode, st.items, st.nk_max, st.n_max, scratch->mem, scratch->work());
         } else {
-            sq::squant_model_kernel<false><<<st.grouped_grid, sq::kCtaThreads, st.grouped_smem, stream>>>(st.grouped, p.qmax, p.mode);
+            sq::squant_model_kernel<sq::kAbsmax><<<st.grouped_grid, sq::kCtaThreads, st.grouped_smem, stream>>>(st.grouped, p.qmax, p.mode);
         }
         SQ_CUDA(cudaGetLastError());
         g_launches.fetch_add(1, std::memory_order_relaxed);
@@ -735,7 +734,8 @@ int launch_plan(const ParamPlan &p, cudaStream_t stream)
         g_launches.fetch_add(1, std::memory_order_relaxed);
     }
     for (const ParamPlan::Grouped &gl : p.grouped) {
-        auto kernel = gl.clip ? sq::squant_model_kernel<true> : sq::squant_model_kernel<false>;
+        auto kernel = gl.scales == sq::kAbsmax ? sq::squant_model_kernel<sq::kAbsmax>
+                      : gl.scales == sq::kOwnScales ? sq::squant_model_kernel<sq::kOwnScales> : sq::squant_model_kernel<sq::kEither>;
         kernel<<<gl.grid, sq::kCtaThreads, gl.smem, stream>>>(gl.table, p.qmax, p.mode);
         SQ_CUDA(cudaGetLastError());
         g_launches.fetch_add(1, std::memory_order_relaxed);

@@ -124,6 +124,43 @@ __device__ __noinline__ KernelOut64 kernel_clip_out(float *wk, int K, float s, b
     return o;
 }
 
+// A 3x3 kernel under the clip that the straight-line selection does not settle, from its weights, scale in the range of the
+// reciprocal sequence (y, s2: as in squant_e_fast).  Most have elements that lie two codes and more beyond the range, and every
+// candidate is flipped.  Out of line.  (Four 512x512x3x3 layers with scales of 0.7 absmax: 59.5 us on a B200 with every kernel that has codes on the edge of
+// the range settled by kernel_clip, 41.1 with all but these in line.)
+__device__ __noinline__ KernelOut64 kernel9_beyond(float *wk, float y, float s2, int qmin, int qmax, unsigned char *ck)
+{
+    const float xmin = static_cast<float>(qmin) * 1073741824.0f, xmax = static_cast<float>(qmax) * 1073741824.0f;
+    unsigned up = 0u, down = 0u;   // candidates
+    long long e = 0;
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+        const float X = div_scaled(wk[i], y, s2), Xc = fminf(fmaxf(X, xmin), xmax), t = __fadd_rn(Xc, kMagic);
+        const int P = __float2int_rn(__fsub_rn(__fsub_rn(t, kMagic), Xc));
+        e += P;
+        if (Xc != X) e += __float2ll_rn(__fsub_rn(Xc, X));
+        reinterpret_cast<int *>(wk)[i] = P;
+        up |= P > 0 ? 1u << i : 0u;
+        down |= P < 0 ? 1u << i : 0u;
+        ck[i] = static_cast<unsigned char>(__float_as_uint(t));
+    }
+    const int sgn = e < 0 ? -1 : 1;
+    unsigned left = sgn > 0 ? up : down;
+    const long long all = static_cast<long long>(__popc(left)) << 30;
+    if (e * sgn < all) return kernel_flip(reinterpret_cast<int *>(wk), ck, 9, true, e);
+    // at least as many flips are wanted as there are candidates, and none is one too many
+#pragma unroll 1
+    for (; left != 0u; left &= left - 1u) {
+        unsigned char *c = ck + __ffs(left) - 1;
+        *c = static_cast<unsigned char>(*c - sgn);
+    }
+    KernelOut64 o;
+    o.e = e - sgn * all;
+    o.v = 0;
+    o.idx = 0;
+    return o;
+}
+
 // ---------------------------------------------------------------- codes and their products to global memory
 // The n codes at cel (shared memory, visible to the whole group), which are those from element `first` of
 // the layer on: int8 or packed int4 (from byte first4 on), and code * s as fp32 and bfloat16.  cel has the
@@ -274,7 +311,9 @@ __device__ __forceinline__ void conv_body(const LayerDesc &L, int m, const Group
             if ((G.t & 31) != 0) continue;
         } else if (KT == 9 && fast) {
             float2 P2[5];
-            unsigned edge = 0u;
+            unsigned beyond = 0u;    // kClip: what clipped elements add to the kernel's sum, modulo 2^32
+            float2 rests = make_float2(0.0f, 0.0f);   // the same as floats
+            float size = 0.0f;       // and without signs
             {
                 float w[9];
 #pragma unroll
@@ -286,20 +325,26 @@ __device__ __forceinline__ void conv_body(const LayerDesc &L, int m, const Group
                     if (!kClip) {
                         squant_e_fast2(w2, c2, t, P2[p]);
                     } else {
-                        // the codes on the edge of the range and the clipped ones: a flip can be barred there
+                        // A flip is barred exactly where w/s lies beyond the last code: at the last code itself the perturbation
+                        // is 0 and the element no candidate; the rest of its perturbation only adds to the sum.
                         const float2 x0 = __fmul2_rn(w2, c2.y);
                         const float2 X = __ffma2_rn(__ffma2_rn(x0, c2.ns2, w2), c2.y, x0);
-                        t = __fadd2_rn(X, c2.magic);
-                        P2[p] = __ffma2_rn(X, c2.neg1, __ffma2_rn(c2.magic, c2.neg1, t));
-                        const float lim_hi = (static_cast<float>(qmax) - 0.5f) * 1073741824.0f, lim_lo = (static_cast<float>(qmin) + 0.5f) * 1073741824.0f;
-                        edge |= (X.x < lim_hi && X.x > lim_lo && X.y < lim_hi && X.y > lim_lo) ? 0u : 1u;
+                        const float xmax = static_cast<float>(qmax) * 1073741824.0f, xmin = static_cast<float>(qmin) * 1073741824.0f;
+                        const float2 Xc = make_float2(fminf(fmaxf(X.x, xmin), xmax), fminf(fmaxf(X.y, xmin), xmax));
+                        const float2 rest = __ffma2_rn(X, c2.neg1, Xc);
+                        beyond += static_cast<unsigned>(__float2int_rn(rest.x)) + static_cast<unsigned>(__float2int_rn(rest.y));
+                        rests = __fadd2_rn(rests, rest);
+                        size = __fadd_rn(__fadd_rn(size, fabsf(rest.x)), fabsf(rest.y));
+                        t = __fadd2_rn(Xc, c2.magic);
+                        P2[p] = __ffma2_rn(Xc, c2.neg1, __ffma2_rn(c2.magic, c2.neg1, t));
                     }
                     ck[2 * p] = static_cast<unsigned char>(__float_as_uint(t.x));
                     if (p < 4) ck[2 * p + 1] = static_cast<unsigned char>(__float_as_uint(t.y));
                 }
             }
             const float2 s01 = __fadd2_rn(__fadd2_rn(P2[0], P2[1]), __fadd2_rn(P2[2], P2[3]));
-            const float ef = __fadd_rn(__fadd_rn(s01.x, s01.y), P2[4].x);
+            float ef = __fadd_rn(__fadd_rn(s01.x, s01.y), P2[4].x);
+            if (kClip) ef = size < 0x1p31f ? __fadd_rn(ef, __fadd_rn(rests.x, rests.y)) : 0x1p40f;   // (further beyond: not settled here)
             const float gs = copysignf(1.0f, ef);
             const float2 G2 = make_float2(gs, gs);
             float Pk[9];
@@ -311,11 +356,11 @@ __device__ __forceinline__ void conv_body(const LayerDesc &L, int m, const Group
             }
             int e32;
             unsigned ix;
-            if (kClip && edge != 0u) {
-                const KernelOut64 o = kernel_clip_out(wk, 9, s, true, qmin, qmax, reinterpret_cast<int8_t *>(ck));
-                e = o.e; v = o.v; idx = o.idx;
-            } else {
-                if (kernel9_select(Pk, ef, ck, e32, v, ix)) {   // about one in 10^5: settled exactly
+            if (kernel9_select(Pk, ef, ck, e32, v, ix, beyond)) {   // without the clip about one in 10^5: settled exactly
+                if (kClip) {
+                    const KernelOut64 o = kernel9_beyond(wk, c2.y.x, s2, qmin, qmax, ck);
+                    e = o.e; v = o.v; idx = o.idx;
+                } else {
                     int *P = reinterpret_cast<int *>(wk);
                     const int gi = (__float_as_int(ef) >> 31) | 1;
 #pragma unroll
@@ -324,8 +369,9 @@ __device__ __forceinline__ void conv_body(const LayerDesc &L, int m, const Group
 #pragma unroll
                     for (int i = 0; i < 9; ++i) e64 += P[i];
                     const KernelOut64 o = kernel_flip(P, ck, 9, true, e64);
-                    e32 = static_cast<int>(o.e); v = o.v; ix = static_cast<unsigned>(o.idx);
+                    e = static_cast<int>(o.e); v = o.v; idx = o.idx;
                 }
+            } else {
                 e = e32;
                 idx = static_cast<int>(ix);
             }

@@ -523,13 +523,15 @@ __device__ __noinline__ KernelOut kernel9_exact_t(const float *wk, float y, floa
 // reported.  The four largest keys come from a 3x3 sorting tableau: sort each triple (rows), then
 // the columns; an entry in row i, column j has at least i * j - 1 entries above it, so the top
 // four of nine lie in row 1, column 1 and position (2, 2) (28 operations).
+//
+// beyond: what clipped elements add to the sum (their perturbations here are 0: they are no candidates).
 __device__ __forceinline__ bool kernel9_select(const float (&Psf)[9], float ef, unsigned char *cb,
-                                               int &e_out, int &v_out, unsigned &idx_out)
+                                               int &e_out, int &v_out, unsigned &idx_out, unsigned beyond = 0u)
 {
     // Psf[i] = Pf[i] * copysign(1, ef): the perturbations normalised to the sign of the float sum
     const int sgn = (__float_as_int(ef) >> 31) | 1;
     int a[9];
-    unsigned eabs = 0;   // |e| mod 2^32
+    unsigned eabs = beyond * static_cast<unsigned>(sgn);   // |e| mod 2^32
 #pragma unroll
     for (int i = 0; i < 9; ++i) {
         const int Ps = __float2int_rn(Psf[i]);
@@ -1320,7 +1322,9 @@ namespace sq {
 #ifndef SQ_MIN_CTAS
 #define SQ_MIN_CTAS 4
 #endif
-template <bool kClip>
+// Scales of the layers of a launch: absmax, all of them their own, or both.
+enum Scales { kAbsmax, kOwnScales, kEither };
+template <Scales kScales>
 __device__ __forceinline__ void run_item(const LayerDesc &L, int ch0, unsigned char *smem, int qmax,
                                          unsigned mode)
 {
@@ -1329,6 +1333,7 @@ __device__ __forceinline__ void run_item(const LayerDesc &L, int ch0, unsigned c
         if (m1 < L.M) channel_single(L, m1, smem + static_cast<size_t>(threadIdx.x) * L.slice_bytes, qmax, mode);
         return;
     }
+    const bool own = kScales == kOwnScales || (kScales == kEither && L.sin);
     Group G;
     G.g = L.g;
     G.sh = L.g_shift;
@@ -1341,7 +1346,10 @@ __device__ __forceinline__ void run_item(const LayerDesc &L, int ch0, unsigned c
         SQ_DBG(ch0 >= 0 && L.g >= 8 && (1 << L.g_shift) == L.g && row_bytes(L.g, L.off_vi) <= L.slice_bytes &&
                static_cast<size_t>(gi + 1) * L.slice_bytes <= dynamic_smem_bytes(), 5);
         if (L.g >= 32 && m >= L.M) return;
-        if (kClip && L.sin) row_body<true, kGroup, 0>(L, m, G, slice, qmax, mode, m < L.M);
+        if (own && kScales == kEither) row_body<true, kGroup, 0>(L, m, G, slice, qmax, mode, m < L.M);
+        else if (own && L.g == 8) row_body<true, kGroup, 8>(L, m, G, slice, qmax, mode, m < L.M);
+        else if (own && L.g == 16) row_body<true, kGroup, 16>(L, m, G, slice, qmax, mode, m < L.M);
+        else if (own) row_body<true, kGroup, 32>(L, m, G, slice, qmax, mode, true);
         else if (L.g == 8) row_body<false, kGroup, 8>(L, m, G, slice, qmax, mode, m < L.M);
         else if (L.g == 16) row_body<false, kGroup, 16>(L, m, G, slice, qmax, mode, m < L.M);
         else row_body<false, kGroup, 32>(L, m, G, slice, qmax, mode, true);
@@ -1352,9 +1360,9 @@ __device__ __forceinline__ void run_item(const LayerDesc &L, int ch0, unsigned c
         SQ_DBG(ch0 >= 0 && L.g >= 32 && (1 << L.g_shift) == L.g && conv_bytes(L.g, L.NK, L.K) <= L.slice_bytes &&
                static_cast<size_t>(gi + 1) * L.slice_bytes <= dynamic_smem_bytes(), 6);
         if (L.K == 9 && (mode & 2u)) {
-            if (kClip && L.sin) conv_body<9, true>(L, m, G, slice, qmax, mode);
+            if (own) conv_body<9, true>(L, m, G, slice, qmax, mode);
             else conv_body<9, false>(L, m, G, slice, qmax, mode);
-        } else if (kClip && L.sin) {
+        } else if (own) {
             conv_body<0, true>(L, m, G, slice, qmax, mode);
         } else if (L.K == 7 && (mode & 2u)) {
             conv_body<7, false>(L, m, G, slice, qmax, mode);
@@ -1372,7 +1380,7 @@ __device__ __forceinline__ void run_item(const LayerDesc &L, int ch0, unsigned c
     if (s == 0.0f) return;   // staging wait ran out (status word set); nothing is written
     if (L.K > 1) {   // E + C without K
         channel_body_ec(L, m, G, slice, s, mode);
-    } else if (kClip && L.sin) {   // 1x1 rows too long for the registers of one thread block
+    } else if (own) {   // 1x1 rows too long for the registers of one thread block
         float sc = L.sin[m];
         if (!(sc > 0.0f && sc < __int_as_float(0x7f800000))) sc = 1.0f;
         channel_body_clip(L, m, G, slice, sc, mode, qmax);
@@ -1383,10 +1391,9 @@ __device__ __forceinline__ void run_item(const LayerDesc &L, int ch0, unsigned c
     }
 }
 
-// kClip: layers of the launch have scales of their own.  (Without the bodies for these the others keep their values in
-// registers.  A spilled one comes back from L2, the L1 being shared memory: with 968 B of spill loads in a kernel for both four
+// (Without the bodies for scales of the layers' own the others keep their values in registers.  A spilled one comes back from L2, the L1 being shared memory: with 968 B of spill loads in a kernel for both four
 // 512x512x3x3 layers took 28.6 us on a B200, with 396 B 24.8.)
-template <bool kClip>
+template <Scales kScales>
 __global__ void __launch_bounds__(kCtaThreads, SQ_MIN_CTAS)
 squant_model_kernel(const __grid_constant__ LaunchTable tbl, int qmax, unsigned mode)
 {
@@ -1398,7 +1405,7 @@ squant_model_kernel(const __grid_constant__ LaunchTable tbl, int qmax, unsigned 
         if (layer + step < tbl.n_layers && tbl.first_item[layer + step] <= item) layer += step;
     const LayerDesc &L = tbl.layers[layer];
     const int ch0 = (item - tbl.first_item[layer]) * (kCtaThreads >> L.g_shift);
-    run_item<kClip>(L, ch0, smem, qmax, mode);
+    run_item<kScales>(L, ch0, smem, qmax, mode);
 }
 
 // The same with the descriptors in a table in global memory (used by the entry point whose
@@ -1410,7 +1417,7 @@ squant_table_kernel(const LayerDesc *__restrict__ layers, const Item *__restrict
     extern __shared__ __align__(16) unsigned char smem[];
     const Item it = items[blockIdx.x];
     const LayerDesc L = layers[it.layer];
-    run_item<true>(L, it.ch0, smem, qmax, mode);
+    run_item<kEither>(L, it.ch0, smem, qmax, mode);
 }
 
 }  // namespace sq

@@ -623,6 +623,59 @@ __device__ __forceinline__ float4 row_error_sums(const int4 p)
     return make_float4(a.x, a.y, b.x, b.y);
 }
 
+// The same where the clip of Sec. 2.2 can fire; `er`: the elements' error sums.  A flip is barred exactly where w/s lies beyond the
+// last code: at the last code itself the perturbation is 0 and the element no candidate.  What is left of its perturbation
+// only adds to the sum: whole codes and sum64.
+struct RowClip {
+    float xmin, xmax;
+    int whole;   // in codes
+    long long sum64;
+};
+template <bool kErr>
+__device__ __forceinline__ unsigned row_vector_clip(const float4 w, const E2 &c2, RowSums &R, RowClip &C, int which, int4 &p, float4 &er)
+{
+    const float2 wa = make_float2(w.x, w.y), wb = make_float2(w.z, w.w);
+    const float2 xa = __fmul2_rn(wa, c2.y), xb = __fmul2_rn(wb, c2.y);
+    float2 Xa = __ffma2_rn(__ffma2_rn(xa, c2.ns2, wa), c2.y, xa), Xb = __ffma2_rn(__ffma2_rn(xb, c2.ns2, wb), c2.y, xb);
+    float2 ra = make_float2(0.0f, 0.0f), rb = ra;
+    const bool beyond = fmaxf(fmaxf(Xa.x, Xa.y), fmaxf(Xb.x, Xb.y)) > C.xmax || fminf(fminf(Xa.x, Xa.y), fminf(Xb.x, Xb.y)) < C.xmin;
+    if (beyond) {
+        const float2 ya = make_float2(fminf(fmaxf(Xa.x, C.xmin), C.xmax), fminf(fmaxf(Xa.y, C.xmin), C.xmax));
+        const float2 yb = make_float2(fminf(fmaxf(Xb.x, C.xmin), C.xmax), fminf(fmaxf(Xb.y, C.xmin), C.xmax));
+        ra = __ffma2_rn(Xa, c2.neg1, ya);
+        rb = __ffma2_rn(Xb, c2.neg1, yb);
+        Xa = ya;
+        Xb = yb;
+        // whole codes and the rest of each
+        const float2 ma = __ffma2_rn(c2.magic, c2.neg1, __fadd2_rn(ra, c2.magic)), mb = __ffma2_rn(c2.magic, c2.neg1, __fadd2_rn(rb, c2.magic));
+        const float2 fa = __ffma2_rn(ma, c2.neg1, ra), fb = __ffma2_rn(mb, c2.neg1, rb);
+        const int i0 = __float2int_rn(fa.x), i1 = __float2int_rn(fa.y), i2 = __float2int_rn(fb.x), i3 = __float2int_rn(fb.y);
+        C.whole += __float2int_rn(__fmul_rn(__fadd_rn(__fadd_rn(ma.x, ma.y), __fadd_rn(mb.x, mb.y)), 0x1p-30f));
+        C.sum64 += static_cast<long long>(i0 + i1) + (i2 + i3);
+        if (kErr) {   // (from 2^23 units on an element is whole)
+            ra = __fadd2_rn(ma, make_float2(__int2float_rn(i0), __int2float_rn(i1)));
+            rb = __fadd2_rn(mb, make_float2(__int2float_rn(i2), __int2float_rn(i3)));
+        }
+    }
+    const float2 ta = __fadd2_rn(Xa, c2.magic), tb = __fadd2_rn(Xb, c2.magic);
+    const float2 Pa = __ffma2_rn(Xa, c2.neg1, __ffma2_rn(c2.magic, c2.neg1, ta)), Pb = __ffma2_rn(Xb, c2.neg1, __ffma2_rn(c2.magic, c2.neg1, tb));
+    p = make_int4(__float2int_rn(Pa.x), __float2int_rn(Pa.y), __float2int_rn(Pb.x), __float2int_rn(Pb.y));
+    R.fs = __fadd2_rn(R.fs, Pa);
+    R.fs = __fadd2_rn(R.fs, Pb);
+    R.sum += static_cast<unsigned>(p.x) + static_cast<unsigned>(p.y);
+    R.sum += static_cast<unsigned>(p.z) + static_cast<unsigned>(p.w);
+    R.hi[which] = __vimax3_s32(__vimax3_s32(R.hi[which], p.x, p.y), p.z, p.w);
+    R.lo[which] = __vimin3_s32(__vimin3_s32(R.lo[which], p.x, p.y), p.z, p.w);
+    if (kErr) {   // (one of the two is 0)
+        const float2 k30 = make_float2(0x1p-30f, 0x1p-30f);
+        const float2 a = __fmul2_rn(__fadd2_rn(make_float2(__int2float_rn(p.x), __int2float_rn(p.y)), ra), k30);
+        const float2 b = __fmul2_rn(__fadd2_rn(make_float2(__int2float_rn(p.z), __int2float_rn(p.w)), rb), k30);
+        er = make_float4(a.x, a.y, b.x, b.y);
+    }
+    return __byte_perm(__byte_perm(__float_as_uint(ta.x), __float_as_uint(ta.y), 0x0040),
+                       __byte_perm(__float_as_uint(tb.x), __float_as_uint(tb.y), 0x0040), 0x5410);
+}
+
 // The loops over a thread's vectors, which lie kStep vectors apart (a constant: the addresses of a step are immediates).
 template <int kStep>
 __device__ __forceinline__ float row_stage(float4 *w, const float4 *src, int vecs)
@@ -638,31 +691,39 @@ __device__ __forceinline__ float row_stage(float4 *w, const float4 *src, int vec
     }
     return amax;
 }
-template <int kStep, bool kErr>
-__device__ __forceinline__ void row_quantize(float4 *w, unsigned *codes, float4 *kerr, int vecs, const E2 &c2, RowSums &R)
+template <int kStep, bool kErr, bool kClip>
+__device__ __forceinline__ void row_quantize(float4 *w, unsigned *codes, float4 *kerr, int vecs, const E2 &c2, RowSums &R, RowClip &C)
 {
+    auto vector = [&](int at, int which) {
+        int4 p;
+        float4 er;
+        if (kClip) codes[at] = row_vector_clip<kErr>(w[at], c2, R, C, which, p, er);
+        else codes[at] = row_vector(w[at], c2, R, which, p);
+        reinterpret_cast<int4 *>(w)[at] = p;
+        if (kErr) __stcs(kerr + at, kClip ? er : row_error_sums(p));
+    };
 #pragma unroll 1
     for (; vecs > 1; vecs -= 2) {
-        const float4 w0 = w[0], w1 = w[kStep];
-        int4 p0, p1;
-        codes[0] = row_vector(w0, c2, R, 0, p0);
-        codes[kStep] = row_vector(w1, c2, R, 1, p1);
-        reinterpret_cast<int4 *>(w)[0] = p0;
-        reinterpret_cast<int4 *>(w)[kStep] = p1;
-        if (kErr) {
-            __stcs(kerr, row_error_sums(p0));
-            __stcs(kerr + kStep, row_error_sums(p1));
-            kerr += 2 * kStep;
+        if (kClip) {
+            vector(0, 0);
+            vector(kStep, 1);
+        } else {
+            const float4 w0 = w[0], w1 = w[kStep];
+            int4 p0, p1;
+            codes[0] = row_vector(w0, c2, R, 0, p0);
+            codes[kStep] = row_vector(w1, c2, R, 1, p1);
+            reinterpret_cast<int4 *>(w)[0] = p0;
+            reinterpret_cast<int4 *>(w)[kStep] = p1;
+            if (kErr) {
+                __stcs(kerr, row_error_sums(p0));
+                __stcs(kerr + kStep, row_error_sums(p1));
+            }
         }
+        if (kErr) kerr += 2 * kStep;
         w += 2 * kStep;
         codes += 2 * kStep;
     }
-    if (vecs > 0) {
-        int4 p;
-        codes[0] = row_vector(w[0], c2, R, 0, p);
-        reinterpret_cast<int4 *>(w)[0] = p;
-        if (kErr) __stcs(kerr, row_error_sums(p));
-    }
+    if (vecs > 0) vector(0, 0);
 }
 
 // kClip: the clip of Sec. 2.2 can fire (caller-supplied scales): codes are clamped, sums are 64
@@ -751,12 +812,16 @@ __device__ __forceinline__ void row_body(const LayerDesc &L, int m, const Group 
     R.sum = 0u;
     R.fs = make_float2(0.0f, 0.0f);
     R.hi[0] = R.hi[1] = R.lo[0] = R.lo[1] = 0;   // of the even and the odd ones of the thread's vectors
-    long long sum64 = 0;
+    RowClip C;
+    C.xmin = static_cast<float>(qmin) * 1073741824.0f;
+    C.xmax = static_cast<float>(qmax) * 1073741824.0f;
+    C.whole = 0;   // kClip: what is not in R.sum
+    C.sum64 = 0;
     {
         const float s2 = fast ? __fmul_rn(s, 0x1p-30f) : 0.0f;
         const E2 c2 = make_e2(fast ? __frcp_rn(s2) : 0.0f, s2);
-        const float tmin = kMagic + static_cast<float>(qmin) * 1073741824.0f, tmax = kMagic + static_cast<float>(qmax) * 1073741824.0f;
         const bool kvec = ((reinterpret_cast<uintptr_t>(kerr) - 4 * r) & 15) == 0;
+        const float tmin = kMagic + C.xmin, tmax = kMagic + C.xmax;
         auto quantize = [&](const float4 w, int4 &p, float2 &oa, float2 &ob, int which) -> unsigned {
             float2 Pa, Pb;
             unsigned c4;
@@ -795,10 +860,10 @@ __device__ __forceinline__ void row_body(const LayerDesc &L, int m, const Group 
                 oa = make_float2(__int2float_rn(p.x), __int2float_rn(p.y));
                 ob = make_float2(__int2float_rn(p.z), __int2float_rn(p.w));
             } else {
-                row_clip_one(Pa.x, p.x, c4, qmin, qmax, sum64, oa.x);
-                row_clip_one(Pa.y, p.y, c4 >> 8, qmin, qmax, sum64, oa.y);
-                row_clip_one(Pb.x, p.z, c4 >> 16, qmin, qmax, sum64, ob.x);
-                row_clip_one(Pb.y, p.w, c4 >> 24, qmin, qmax, sum64, ob.y);
+                row_clip_one(Pa.x, p.x, c4, qmin, qmax, C.sum64, oa.x);
+                row_clip_one(Pa.y, p.y, c4 >> 8, qmin, qmax, C.sum64, oa.y);
+                row_clip_one(Pb.x, p.z, c4 >> 16, qmin, qmax, C.sum64, ob.x);
+                row_clip_one(Pb.y, p.w, c4 >> 24, qmin, qmax, C.sum64, ob.y);
             }
             const int h = __vimax3_s32(__vimax3_s32(p.x, p.y, p.z), p.w, 0), l = __vimin3_s32(__vimin3_s32(p.x, p.y, p.z), p.w, 0);
             if (which == 0) { R.hi[0] = max(R.hi[0], h); R.lo[0] = min(R.lo[0], l); }
@@ -808,10 +873,10 @@ __device__ __forceinline__ void row_body(const LayerDesc &L, int m, const Group 
             ob = __fmul2_rn(ob, k30);
             return c4;
         };
-        if (!kClip && kLanes != 0 && __all_sync(kFull, fast && (!kerr || kvec))) {   // (uniform for groups of whole warps)
+        if (kLanes != 0 && __all_sync(kFull, fast && (!kerr || kvec))) {   // (uniform for groups of whole warps)
             constexpr int kStep = kLanes ? kLanes : 1;
-            if (kerr) row_quantize<kStep, true>(reinterpret_cast<float4 *>(Pbuf) + q0, cbuf + q0, reinterpret_cast<float4 *>(kerr - r) + q0, vecs, c2, R);
-            else row_quantize<kStep, false>(reinterpret_cast<float4 *>(Pbuf) + q0, cbuf + q0, nullptr, vecs, c2, R);
+            if (kerr) row_quantize<kStep, true, kClip>(reinterpret_cast<float4 *>(Pbuf) + q0, cbuf + q0, reinterpret_cast<float4 *>(kerr - r) + q0, vecs, c2, R, C);
+            else row_quantize<kStep, false, kClip>(reinterpret_cast<float4 *>(Pbuf) + q0, cbuf + q0, nullptr, vecs, c2, R, C);
         } else {
 #pragma unroll 1
             for (int i = 0; i < vecs; ++i) {
@@ -844,7 +909,9 @@ __device__ __forceinline__ void row_body(const LayerDesc &L, int m, const Group 
     long long ec = 0;
     if ((mode & 4u) || L.cerr) {
         int up = 0, down = 0;
-        ec = owner_sum<kOwn, kClip, false>(G, S, sum64, R.sum, __float2int_rn(__fmul_rn(__fadd_rn(R.fs.x, R.fs.y), 0x1p-17f)), up, down);
+        const int apx = __float2int_rn(__fmul_rn(__fadd_rn(R.fs.x, R.fs.y), 0x1p-17f));
+        if (kClip) C.sum64 += static_cast<long long>(C.whole) * kOne + static_cast<long long>(apx) * (1ll << 17) + static_cast<int>(R.sum - (static_cast<unsigned>(apx) << 17));
+        ec = owner_sum<kOwn, kClip, false>(G, S, C.sum64, R.sum, apx, up, down);
     }
 
     // ---- SQuant-C: Algorithm 2 on the channel, the perturbations are the keys
@@ -915,7 +982,8 @@ __device__ __forceinline__ void row_body(const LayerDesc &L, int m, const Group 
                 if (kerr) kerr[n] = __fmul_rn(__int2float_rn(sgn > 0 ? a - kOne : kOne - a), 0x1p-30f);
             };
             const int vtop = kHalf + (1 << 14) + 1;
-            const int k_eff = select_top<kOwn>(G, prepare, count, listing, [] {}, each, [](int) { return 0u; }, flip, kOwn == kBlock ? 2 * g : per * g, L.N >= kRowDirect,
+            const bool direct = L.N >= kRowDirect && (g > 32 || __any_sync(kFull, want && kc < S.cap));   // (of a clipped row kc can be huge)
+            const int k_eff = select_top<kOwn>(G, prepare, count, listing, [] {}, each, [](int) { return 0u; }, flip, kOwn == kBlock ? 2 * g : per * g, direct,
                                                list_start(kc, 2.0f, vtop, max(N, 1)), vtop, vtop, 2.0f, kc, N, want, S, 1);
             ec -= static_cast<long long>(sgn) * k_eff * kOne;
         }

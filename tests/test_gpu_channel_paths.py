@@ -109,6 +109,26 @@ def test_rows_whose_list_starts_at_a_guess(n):
         check(ws, bits, start=bits % 3)
 
 
+@pytest.mark.parametrize("bits,clip", [(2, 0.97), (4, 0.7), (8, 0.5), (3, 0.2), (8, 0.1), (6, 0.04)])
+def test_elements_at_and_far_beyond_the_clip_range(bits, clip):
+    """Scales of the caller's from just below absmax (elements on the last code) to far below (sums of many whole codes, kernels
+    whose every candidate is flipped), rows in groups of every kind and 3x3 kernels; with absmax layers in the same call too."""
+    ws = [w for i, s in enumerate([(37, 100, 1, 1), (20, 300, 1, 1), (9, 701, 1, 1), (5, 3000, 1, 1), (19, 33, 3, 3), (5, 513, 3, 3)]) for w in layers(s, 7 * bits + i)]
+    check(ws, bits, clip=clip)
+    check(ws, bits, flags=0, start=1, outputs=True, clip=clip)
+    bufs = []
+    for i, w in enumerate(ws):
+        b = sq.alloc_outputs(torch.from_numpy(w).cuda())
+        if i % 2:
+            a = np.abs(w).reshape(w.shape[0], -1).max(1)
+            b.scales_in = torch.from_numpy((np.where(a > 0, a, 1) * clip / (2 ** (bits - 1) - 1)).astype(np.float32)).cuda()
+        bufs.append(b)
+    sq.squant_quantize_model(bufs, bits=bits)
+    for b, w in zip(bufs, ws):
+        r = oracle.quantize_layer(w, bits=bits, scales_in=None if b.scales_in is None else b.scales_in.cpu().numpy(), details=True)
+        assert np.array_equal(b.codes.cpu().numpy(), r.codes) and np.array_equal(b.kernel_err.cpu().numpy().view(np.int32), r.kernel_err.view(np.int32))
+
+
 @pytest.mark.parametrize("shape", [(2, 1, 1, 45857), (3, 2, 1, 22928), (2, 9, 1, 5095), (2, 200, 1, 229), (5, 106, 7, 7), (9, 52, 7, 7), (9, 103, 5, 5)])
 def test_larger_kernels_at_the_sizes_that_share_a_thread_block(shape):
     """The longest channels of few large kernels that one thread block, or two and four channels that share one, hold;
