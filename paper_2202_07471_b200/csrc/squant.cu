@@ -32,7 +32,6 @@ constexpr size_t kMaxPlans = 64;
 constexpr int kLongChannel = 8192;           // weights: longer channels are launched apart from the others
 constexpr int kStreamKernels = 1184;         // 3x3 channels of at least as many kernels go to the streaming kernel (stream_eligible)
 constexpr int kGroupedSmemGoal = 55 << 10;   // shared memory of a grouped CTA with which four of them share a multiprocessor
-constexpr int kLongRow512 = 22000;           // weights: see build_param_plan
 constexpr int kSmSmem = 228 << 10;           // shared memory of a multiprocessor; every thread block takes 1 KB of it for the system
 constexpr int kBlockSmemReserved = 1 << 10;
 constexpr int kWideSmemGoal = 112 << 10;     // the same of a cluster's thread block: two of them
@@ -350,7 +349,7 @@ struct ParamPlan {
     struct Wide { LayerDesc d; int cluster, kpc, smem; };
     std::vector<Wide> wide;
     // row kernel (1x1 rows too long for a group): one item per output channel
-    enum RowForm { kRow512, kLong512, kLong256 };   // row_body with 512 threads, long_row_body with 512, with 256
+    enum RowForm { kRow512, kLong512, kRow256 };   // row_body with 512 threads, long_row_body with 512, row_body with 256
     struct Rows { sq::LaunchTable table; RowForm form; int grid, smem; };
     std::vector<Rows> rows;
     // streaming kernel (layers of long 3x3 channels): one item per output channel
@@ -463,48 +462,45 @@ int build_param_plan(const squant_layer *layers, int32_t n_layers, const squant_
     }
     // Long rows, a thread block per output channel, in one of three forms.  row_body holds 5 B of shared memory a weight,
     // long_row_body 4 (5 of packed codes).  What counts is how many threads a multiprocessor holds and over how many
-    // vectors a thread spreads the code that runs once.  us a call on a B200, row_body / long_row_body:
-    //   - Many rows of up to 16 K weights: long_row_body with 256 threads.  Where four such thread blocks fit a multiprocessor
-    //     (13 K weights) the line is at one and a half waves of them: rows of 12,000 weights 700 28.8 / 29.9, 1000 37.9 / 35.7, 1500 49.9 / 46.9,
-    //     4096 119.5 / 96.9; with packed codes (10 K weights) at two: rows of 9000 1000 30.7 / 31.6, 1500 41.3 / 41.2, 2000 52.1 / 48.6.
-    //     Where three fit, at four, and not with packed codes or supplied scales: rows of 15,001 1000 42.9 / 47.3, 1500 59.6 / 58.9,
-    //     2000 75.2 / 72.9, 4096 143.7 / 133.4; 2000 of 13,500 with packed codes 63.0 / 71.9.
-    //   - More rows of over 22 K weights than multiprocessors, neither packed codes nor supplied scales: long_row_body with 512
-    //     threads, of which two blocks fit a multiprocessor up to 26 K weights and of row_body one (2000 rows of 17,000 78.2 / 81.4, of
-    //     20,000 86.1 / 88.9, of 25,001 143.4 / 109.4, of 32,768 157.4 / 155.1; 300 of 25,001 32.3 / 30.1; 16 of 25,001 14.3 / 15.7).
-    //   - All others row_body: few rows take the time of one row's chain, which is shorter there (16 rows of 9000 8.2 / 10.3, 1000 of
-    //     16,384 42.6 / 48.4, with packed codes 39.1 / 58.4).
-    const auto small_blocks = [&](int i) {   // of 256 threads on a multiprocessor
-        const int bytes = sq::long_row_bytes(256, (descs[i].N + 6) >> 2, pack, sq::kBlock);
-        return descs[i].N > sq::kRowSmallElems ? 0 : std::min(4, kSmSmem / (bytes + kBlockSmemReserved));
+    // vectors a thread spreads the code that runs once.  us a call on a B200, row_body with 256 / with 512 threads / long_row_body with 512:
+    //   - More than two and a quarter rows a multiprocessor, so short that three thread blocks of 256 threads fit one (14.8 K weights): those
+    //     (rows of 9000 300 12.5 / 12.3 / 14.4, 400 14.4 / 15.8 / 18.7, 4096 69.9 / 94.1 / 117; of 12,000 100 12.9 / 10.3 / 12.8, 500 19.5 / 20.5 /
+    //     25.0, 4096 89.6 / 105 / 128; 4096 of 14,100 106.7 / 124.1 / 142.3, of 15,001 135.3 / 127.7 / 153.8; 2000 of 9000 with packed codes
+    //     40.2 / 51.2 / 69.2; 1500 of 9000 with scales of their own 39.4 / 47.4 / 65.7).
+    //   - More rows than multiprocessors of which two thread blocks fit one only in long_row_body (22 to 27 K weights), neither packed codes nor
+    //     scales of their own: that (2000 rows of 25,001 - / 127.2 / 110.7, 300 - / 30.7 / 30.8, 1000 of 22,100 - / 49.6 / 57.1, 300 of 30,000
+    //     - / 31.2 / 36.9).
+    //   - All others row_body with 512 threads.
+    const auto blocks = [&](int bytes) { return kSmSmem / (bytes + kBlockSmemReserved); };   // on a multiprocessor
+    const auto small_blocks = [&](int i) { return std::min(4, blocks(sq::row_bytes(256, (descs[i].N + 6) >> 2, sq::kBlock))); };
+    const auto only_long = [&](int i) {
+        const int vecs = (descs[i].N + 6) >> 2;
+        return !pack && !descs[i].sin && blocks(sq::row_bytes(512, vecs, sq::kBlock)) < 2 && blocks(sq::long_row_bytes(512, vecs, pack, sq::kBlock)) >= 2;
     };
-    const auto codes_only = [&](int i) { return !pack && !descs[i].sin; };
-    int64_t four = 0, three = 0, longer = 0;   // rows
+    int64_t small = 0, longer = 0;   // rows
     for (int i : rows) {
-        const int small = small_blocks(i);
-        if (small == 4) four += descs[i].M;
-        if (small == 3 && codes_only(i)) three += descs[i].M;
-        if (descs[i].N > kLongRow512 && codes_only(i)) longer += descs[i].M;
+        if (small_blocks(i) >= 3) small += descs[i].M;
+        if (only_long(i)) longer += descs[i].M;
     }
     const auto form_of = [&](int i) {
-        const int small = small_blocks(i);
-        if (small == 4 && four > (pack ? 8ll : 6ll) * sms) return ParamPlan::kLong256;
-        if (small == 3 && codes_only(i) && three > 12ll * sms) return ParamPlan::kLong256;
-        return descs[i].N > kLongRow512 && codes_only(i) && longer > sms ? ParamPlan::kLong512 : ParamPlan::kRow512;
+        if (small_blocks(i) >= 3 && 4 * small > 9ll * sms) return ParamPlan::kRow256;
+        return only_long(i) && longer > sms ? ParamPlan::kLong512 : ParamPlan::kRow512;
     };
+    // Rows of 256 threads of which four thread blocks fit a multiprocessor have a launch apart from those of which three do.
+    const auto launch_of = [&](int i) { return form_of(i) == ParamPlan::kRow256 ? 8 - small_blocks(i) : static_cast<int>(form_of(i)); };
     std::stable_sort(rows.begin(), rows.end(), [&](int a, int b) {   // by form, longest first
-        return form_of(a) != form_of(b) ? form_of(a) < form_of(b) : descs[a].N > descs[b].N;
+        return launch_of(a) != launch_of(b) ? launch_of(a) < launch_of(b) : descs[a].N > descs[b].N;
     });
     for (size_t base = 0; base < rows.size();) {
         const ParamPlan::RowForm form = form_of(rows[base]);
         size_t n = 0;
         int smem = 0;
-        while (base + n < rows.size() && n < sq::kMaxParamLayers && form_of(rows[base + n]) == form) {
+        while (base + n < rows.size() && n < sq::kMaxParamLayers && launch_of(rows[base + n]) == launch_of(rows[base])) {
             LayerDesc &d = descs[rows[base + n]];
             d.off_vi = (d.N + 6) >> 2;
             d.off_ev = regular_rows(d);
-            smem = std::max(smem, form == ParamPlan::kRow512 ? sq::row_bytes(512, d.off_vi, sq::kBlock)
-                                                             : sq::long_row_bytes(form == ParamPlan::kLong512 ? 512 : 256, d.off_vi, pack, sq::kBlock));
+            smem = std::max(smem, form == ParamPlan::kLong512 ? sq::long_row_bytes(512, d.off_vi, pack, sq::kBlock)
+                                                              : sq::row_bytes(form == ParamPlan::kRow512 ? 512 : 256, d.off_vi, sq::kBlock));
             ++n;
         }
         p.rows.emplace_back();
@@ -605,7 +601,7 @@ int device_smem_limit(int device, int &limit)
             SQ_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, v));
         SQ_CUDA(cudaFuncSetAttribute(sq::squant_table_kernel,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, v));
-        SQ_CUDA(cudaFuncSetAttribute((sq::squant_row_kernel<256, true>),
+        SQ_CUDA(cudaFuncSetAttribute((sq::squant_row_kernel<256, false>),
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, v));
         SQ_CUDA(cudaFuncSetAttribute((sq::squant_row_kernel<512, true>),
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, v));
@@ -729,7 +725,7 @@ int launch_plan(const ParamPlan &p, cudaStream_t stream)
     for (const ParamPlan::Rows &r : p.rows) {
         if (r.form == ParamPlan::kRow512) sq::squant_row_kernel<512, false><<<r.grid, 512, r.smem, stream>>>(r.table, p.qmax, p.mode);
         else if (r.form == ParamPlan::kLong512) sq::squant_row_kernel<512, true><<<r.grid, 512, r.smem, stream>>>(r.table, p.qmax, p.mode);
-        else sq::squant_row_kernel<256, true><<<r.grid, 256, r.smem, stream>>>(r.table, p.qmax, p.mode);
+        else sq::squant_row_kernel<256, false><<<r.grid, 256, r.smem, stream>>>(r.table, p.qmax, p.mode);
         SQ_CUDA(cudaGetLastError());
         g_launches.fetch_add(1, std::memory_order_relaxed);
     }

@@ -965,7 +965,7 @@ __device__ __forceinline__ void row_body(const LayerDesc &L, int m, const Group 
                 }
             };
             auto count = [&](int t, int) {
-                if (kOwn == kBlock) return __syncthreads_count(m0 >= t) + __syncthreads_count(m1 >= t);
+                if (kOwn == kBlock) return __syncthreads_count(max(m0, m1) >= t);
                 if (g <= 32) return __popc(__ballot_sync(kFull, m0 >= t) & gmask) + __popc(__ballot_sync(kFull, m1 >= t) & gmask);
                 int c = 0;
 #pragma unroll 1
@@ -983,7 +983,7 @@ __device__ __forceinline__ void row_body(const LayerDesc &L, int m, const Group 
             };
             const int vtop = kHalf + (1 << 14) + 1;
             const bool direct = L.N >= kRowDirect && (g > 32 || __any_sync(kFull, want && kc < S.cap));   // (of a clipped row kc can be huge)
-            const int k_eff = select_top<kOwn>(G, prepare, count, listing, [] {}, each, [](int) { return 0u; }, flip, kOwn == kBlock ? 2 * g : per * g, direct,
+            const int k_eff = select_top<kOwn>(G, prepare, count, listing, [] {}, each, [](int) { return 0u; }, flip, kOwn == kBlock ? g : per * g, direct,
                                                list_start(kc, 2.0f, vtop, max(N, 1)), vtop, vtop, 2.0f, kc, N, want, S, 1);
             ec -= static_cast<long long>(sgn) * k_eff * kOne;
         }

@@ -1,5 +1,5 @@
 // Output channels that are too long for a group of the grouped kernel: 1x1 rows of more than 8 K weights
-// get a thread block of 256 or 512 threads each (by long_row_body here or by row_body, see build_param_plan), and channels that do not fit one thread block's shared memory a
+// get a thread block of 256 or 512 threads each (by row_body, a few sizes by long_row_body here, see build_param_plan), and channels that do not fit one thread block's shared memory a
 // cluster of 2, 4 or 8 of them, each with a contiguous run of the channel's kernels.  What a channel needs
 // as a whole travels through distributed shared memory (plain loads from the other thread blocks' shared
 // memory; no multicast anywhere): absmax, error sum, the counts of SQuant-C's search and the short lists
@@ -458,7 +458,6 @@ __device__ __forceinline__ void long_row_body(const LayerDesc &L, int m, const G
 
 // Rows of more than 8 K weights, one thread block per output channel.  kLong: by long_row_body, else by row_body.
 // Which form a row takes: build_param_plan.
-constexpr int kRowSmallElems = 16384;   // longest row of 256 threads
 template <int kThreads, bool kLong>
 __global__ void __launch_bounds__(kThreads, 1024 / kThreads)
 squant_row_kernel(const __grid_constant__ LaunchTable tbl, int qmax, unsigned mode)
