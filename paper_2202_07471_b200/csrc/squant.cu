@@ -722,35 +722,56 @@ int launch_plan(const ParamPlan &p, cudaStream_t stream)
         SQ_CUDA(cudaGetLastError());
         g_launches.fetch_add(1, std::memory_order_relaxed);
     }
-    for (const ParamPlan::Rows &r : p.rows) {
-        if (r.form == ParamPlan::kRow512) sq::squant_row_kernel<512, false><<<r.grid, 512, r.smem, stream>>>(r.table, p.qmax, p.mode);
-        else if (r.form == ParamPlan::kLong512) sq::squant_row_kernel<512, true><<<r.grid, 512, r.smem, stream>>>(r.table, p.qmax, p.mode);
-        else sq::squant_row_kernel<256, false><<<r.grid, 256, r.smem, stream>>>(r.table, p.qmax, p.mode);
-        SQ_CUDA(cudaGetLastError());
-        g_launches.fetch_add(1, std::memory_order_relaxed);
+    // The row and cluster kernels may start before the launch in front of them has ended (see next_launch_may_start).  Not the streaming
+    // kernels, which may share a scratch area, nor the grouped one (the wait at its end would cost it registers), nor what a graph captures.
+    bool early = false;
+    if (p.streams.size() + p.rows.size() + p.grouped.size() + p.wide.size() > 1) {
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        SQ_CUDA(cudaStreamIsCapturing(stream, &cap));
+        early = cap == cudaStreamCaptureStatusNone;
     }
+    bool first = p.streams.empty() && p.grouped.empty();
+    const auto launch = [&](auto kernel, bool early_kernel, int grid, int threads, int smem, int cluster, const auto &...args) -> int {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(static_cast<unsigned>(grid));
+        cfg.blockDim = dim3(static_cast<unsigned>(threads));
+        cfg.dynamicSmemBytes = static_cast<size_t>(smem);
+        cfg.stream = stream;
+        cudaLaunchAttribute attr[2];
+        if (cluster > 1) {
+            attr[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
+            attr[cfg.numAttrs].val.clusterDim.x = static_cast<unsigned>(cluster);
+            attr[cfg.numAttrs].val.clusterDim.y = 1;
+            attr[cfg.numAttrs].val.clusterDim.z = 1;
+            ++cfg.numAttrs;
+        }
+        if (early && early_kernel && !first) {
+            attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+            attr[cfg.numAttrs].val.programmaticStreamSerializationAllowed = 1;
+            ++cfg.numAttrs;
+        }
+        cfg.attrs = attr;
+        first = first && !early_kernel;
+        void *const argv[] = {const_cast<void *>(static_cast<const void *>(&args))...};   // (of the kernels' own types)
+        SQ_CUDA(cudaLaunchKernelExC(&cfg, reinterpret_cast<const void *>(kernel), const_cast<void **>(argv)));
+        g_launches.fetch_add(1, std::memory_order_relaxed);
+        return SQUANT_OK;
+    };
     for (const ParamPlan::Grouped &gl : p.grouped) {
         auto kernel = gl.scales == sq::kAbsmax ? sq::squant_model_kernel<sq::kAbsmax>
                       : gl.scales == sq::kOwnScales ? sq::squant_model_kernel<sq::kOwnScales> : sq::squant_model_kernel<sq::kEither>;
-        kernel<<<gl.grid, sq::kCtaThreads, gl.smem, stream>>>(gl.table, p.qmax, p.mode);
-        SQ_CUDA(cudaGetLastError());
-        g_launches.fetch_add(1, std::memory_order_relaxed);
+        const int rc = launch(kernel, false, gl.grid, sq::kCtaThreads, gl.smem, 1, gl.table, p.qmax, p.mode);
+        if (rc) return rc;
+    }
+    for (const ParamPlan::Rows &r : p.rows) {
+        auto kernel = r.form == ParamPlan::kRow512 ? sq::squant_row_kernel<512, false>
+                      : r.form == ParamPlan::kLong512 ? sq::squant_row_kernel<512, true> : sq::squant_row_kernel<256, false>;
+        const int rc = launch(kernel, true, r.grid, r.form == ParamPlan::kRow256 ? 256 : 512, r.smem, 1, r.table, p.qmax, p.mode);
+        if (rc) return rc;
     }
     for (const ParamPlan::Wide &w : p.wide) {   // one cluster per output channel
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(static_cast<unsigned>(w.d.M) * w.cluster);
-        cfg.blockDim = dim3(sq::kBlockThreads);
-        cfg.dynamicSmemBytes = static_cast<size_t>(w.smem);
-        cfg.stream = stream;
-        cudaLaunchAttribute attr;
-        attr.id = cudaLaunchAttributeClusterDimension;
-        attr.val.clusterDim.x = static_cast<unsigned>(w.cluster);
-        attr.val.clusterDim.y = 1;
-        attr.val.clusterDim.z = 1;
-        cfg.attrs = &attr;
-        cfg.numAttrs = 1;
-        SQ_CUDA(cudaLaunchKernelEx(&cfg, sq::squant_wide_kernel, w.d, p.qmax, p.mode, w.kpc));
-        g_launches.fetch_add(1, std::memory_order_relaxed);
+        const int rc = launch(sq::squant_wide_kernel, true, w.d.M * w.cluster, sq::kBlockThreads, w.smem, w.cluster, w.d, p.qmax, p.mode, w.kpc);
+        if (rc) return rc;
     }
     return SQUANT_OK;
 }

@@ -173,6 +173,17 @@ __device__ __forceinline__ void bulk_store_wait()
     asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
 }
 
+// ---------------------------------------------------------------- overlap of a call's launches
+// The launches of a call work on different layers, so those of the row and cluster kernels may start while the one before still runs: their
+// thread blocks take the places that the last ones of that leave free.  Every kernel says at its start that the next may come, as
+// soon as all of its own thread blocks have started.  A launch that may come early ends no earlier than the one before (its last thread
+// block waits for that), so whatever follows the call's last launch follows all of them.
+__device__ __forceinline__ void next_launch_may_start() { asm volatile("griddepcontrol.launch_dependents;"); }
+__device__ __forceinline__ void end_after_launch_before()
+{
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) asm volatile("griddepcontrol.wait;");
+}
+
 // ---------------------------------------------------------------- group-wide reductions
 // `red` points at 16 eight-byte slots owned by the group.
 __device__ __forceinline__ float group_absmax(const Group &G, float v, void *red)
@@ -1398,6 +1409,7 @@ __global__ void __launch_bounds__(kCtaThreads, SQ_MIN_CTAS)
 squant_model_kernel(const __grid_constant__ LaunchTable tbl, int qmax, unsigned mode)
 {
     extern __shared__ __align__(16) unsigned char smem[];
+    next_launch_may_start();
     const int item = blockIdx.x;
     int layer = 0;   // uniform binary search for the last layer whose first item is <= item
 #pragma unroll 1

@@ -349,7 +349,7 @@ __device__ __forceinline__ int shared_count(int *w)
 // a = the value of a candidate in the direction of the flips, n its kernel index in the channel.  listing(t, push) calls
 // push(a, n, code) for those of the thread's elements that are at least t units, 1 <= t < top (`top` is one unit above
 // the largest possible); code is handed through to flip.  direct: from `start` on somewhat more than kc candidates are expected,
-// which are listed without a search.  If there is no such list or it will not do, the bound is searched: the threads know maxima of a
+// which are listed without a search (never with kSearchFirst).  If there is no such list or it will not do, the bound is searched: the threads know maxima of a
 // over parts of their elements, count(t) = how many of the group's nmax maxima are at least t (direct: prepare() once before, it may
 // write to shared memory).  For
 // the exact search: settle() once, then each(v, f) calls f(a, n) for those with a >= v (any v >= 1, vtop above all),
@@ -358,7 +358,7 @@ __device__ __forceinline__ int shared_count(int *w)
 // index first), by some thread of the group.  want: this group selects at all (kc >= 1).  Returns the number of
 // flips.  Every thread of the group calls it, groups that share a warp together; it starts with no barrier and
 // ends with none.
-template <Owner kOwn, class Prepare, class Count, class Listing, class Settle, class Each, class CodeOf, class Flip>
+template <Owner kOwn, bool kSearchFirst, class Prepare, class Count, class Listing, class Settle, class Each, class CodeOf, class Flip>
 __device__ __forceinline__ int select_top(const Group &G, Prepare prepare, Count count, Listing listing, Settle settle, Each each, CodeOf code_of, Flip flip, int nmax, bool direct, int start,
                                           int top, int vtop, float spread, int kc, int n_all, bool want, const Sel &S, int K)
 {
@@ -401,8 +401,9 @@ __device__ __forceinline__ int select_top(const Group &G, Prepare prepare, Count
         slow = todo && !sure;   // fewer than kc maxima are candidates at all
         todo = todo && sure;
     };
+    if (kSearchFirst) search();
 #pragma unroll 1
-    for (int round = 0;; ++round) {
+    for (int round = kSearchFirst ? 1 : 0;; ++round) {
         if (round > 0 || direct) {
             if (todo && (round > 0 || kc < cap))
                 listing(lo, [&](int a, int n, unsigned code) {
@@ -453,7 +454,7 @@ __device__ __forceinline__ int select_top(const Group &G, Prepare prepare, Count
             owner_sync<kOwn>(G);
             todo = again;
         }
-        if (round == 0) search();
+        if (!kSearchFirst && round == 0) search();
     }
     auto flip_entry = [&](unsigned long long e) {
         const unsigned low = static_cast<unsigned>(e);
@@ -983,7 +984,7 @@ __device__ __forceinline__ void row_body(const LayerDesc &L, int m, const Group 
             };
             const int vtop = kHalf + (1 << 14) + 1;
             const bool direct = L.N >= kRowDirect && (g > 32 || __any_sync(kFull, want && kc < S.cap));   // (of a clipped row kc can be huge)
-            const int k_eff = select_top<kOwn>(G, prepare, count, listing, [] {}, each, [](int) { return 0u; }, flip, kOwn == kBlock ? g : per * g, direct,
+            const int k_eff = select_top<kOwn, false>(G, prepare, count, listing, [] {}, each, [](int) { return 0u; }, flip, kOwn == kBlock ? g : per * g, direct,
                                                list_start(kc, 2.0f, vtop, max(N, 1)), vtop, vtop, 2.0f, kc, N, want, S, 1);
             ec -= static_cast<long long>(sgn) * k_eff * kOne;
         }

@@ -423,7 +423,7 @@ __device__ __forceinline__ void long_row_body(const LayerDesc &L, int m, const G
                 if (deq16) deq16[n] = static_cast<uint16_t>(bf16_bits(row_deq(c, s)));
             };
             const int nmax = kOwn == kCluster ? 4 * g * static_cast<int>(cg::this_cluster().num_blocks()) : g;
-            const int k_eff = select_top<kOwn>(G, [] {}, count, listing, settle, each, code_of, flip, nmax, false, 0, (kHalf >> 16) + 1, kHalf + (1 << 14) + 1, 2.0f, kc, L.N, want, S, 1);
+            const int k_eff = select_top<kOwn, true>(G, [] {}, count, listing, settle, each, code_of, flip, nmax, false, 0, (kHalf >> 16) + 1, kHalf + (1 << 14) + 1, 2.0f, kc, L.N, want, S, 1);
             ec -= static_cast<long long>(sgn) * k_eff * kOne;
         }
     }
@@ -463,6 +463,7 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads)
 squant_row_kernel(const __grid_constant__ LaunchTable tbl, int qmax, unsigned mode)
 {
     extern __shared__ __align__(16) unsigned char smem[];
+    next_launch_may_start();
     const int item = blockIdx.x;
     int layer = 0;
 #pragma unroll 1
@@ -484,6 +485,7 @@ squant_row_kernel(const __grid_constant__ LaunchTable tbl, int qmax, unsigned mo
         if (L.sin) row_body<true, kBlock, 32>(L, m, G, smem, qmax, mode, true);
         else row_body<false, kBlock, 32>(L, m, G, smem, qmax, mode, true);
     }
+    end_after_launch_before();
 }
 
 // Shared memory of one of a cluster's thread blocks that has `kpc` kernels of K weights.
@@ -499,6 +501,7 @@ __global__ void __launch_bounds__(kBlockThreads, 2)
 squant_wide_kernel(const LayerDesc L, int qmax, unsigned mode, int kpc)
 {
     extern __shared__ __align__(16) unsigned char smem[];
+    next_launch_may_start();
     cg::cluster_group cluster = cg::this_cluster();
     const int C = static_cast<int>(cluster.num_blocks()), rank = static_cast<int>(cluster.block_rank());
     const int m = static_cast<int>(blockIdx.x) / C;
@@ -521,6 +524,7 @@ squant_wide_kernel(const LayerDesc L, int qmax, unsigned mode, int kpc)
         else conv_body<0, false, kCluster>(L, m, G, smem, qmax, mode, n0, nloc);
     }
     cluster.sync();   // no thread block leaves while another may still read its shared memory
+    end_after_launch_before();
 }
 
 }  // namespace sq
