@@ -679,11 +679,17 @@ __device__ __forceinline__ unsigned row_vector_clip(const float4 w, const E2 &c2
 
 // The loops over a thread's vectors, which lie kStep vectors apart (a constant: the addresses of a step are immediates).
 template <int kStep>
-__device__ __forceinline__ float row_stage(float4 *w, const float4 *src, int vecs)
+__device__ __forceinline__ float row_stage(float4 *w, const float4 *src, int vecs, bool whole)
 {
     float amax = 0.0f;
+    if (whole) {
 #pragma unroll 4
-    for (int i = 0; i < vecs; ++i) copy_async16(w + i * kStep, src + i * kStep);
+        for (int i = 0; i < vecs; ++i) copy_async16(w + i * kStep, src + i * kStep);
+    } else {   // packed codes of a misaligned row
+#pragma unroll 1
+        for (int i = 0; i < vecs; ++i)
+            for (int c = 0; c < 4; ++c) copy_async4(reinterpret_cast<float *>(w + i * kStep) + c, reinterpret_cast<const float *>(src + i * kStep) + c);
+    }
     copy_async_wait();
 #pragma unroll 4
     for (int i = 0; i < vecs; ++i) {
@@ -775,10 +781,10 @@ __device__ __forceinline__ void row_body(const LayerDesc &L, int m, const Group 
         float4 *w = reinterpret_cast<float4 *>(Pbuf) + q0;
         const float4 *src = reinterpret_cast<const float4 *>(wrow - r) + q0;
         if (rag >= 0) copy_async4(Pel + rag, wrow + rag);
-        if (kLanes != 0 && (!pack || (reinterpret_cast<uintptr_t>(src) & 15) == 0)) {
-            amax = row_stage<kLanes ? kLanes : 1>(w, src, vecs);
+        const bool whole = (reinterpret_cast<uintptr_t>(src) & 15) == 0;
+        if (kLanes != 0) {
+            amax = row_stage<kLanes ? kLanes : 1>(w, src, vecs, whole);
         } else {
-            const bool whole = (reinterpret_cast<uintptr_t>(src) & 15) == 0;   // (packed codes of a misaligned row)
 #pragma unroll 1
             for (int i = 0; i < vecs; ++i) {
                 if (whole) copy_async16(w + i * step, src + i * step);
