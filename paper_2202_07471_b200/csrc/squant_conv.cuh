@@ -323,7 +323,7 @@ __device__ __forceinline__ void conv_body(const LayerDesc &L, int m, const Group
                     const float2 w2 = make_float2(w[2 * p], p < 4 ? w[2 * p + 1] : 0.0f);
                     float2 t;
                     if (!kClip) {
-                        squant_e_fast2(w2, c2, t, P2[p]);
+                        squant_e_fast2<true>(w2, c2, t, P2[p]);
                     } else {
                         // A flip is barred exactly where w/s lies beyond the last code: at the last code itself the perturbation
                         // is 0 and the element no candidate; the rest of its perturbation only adds to the sum.
@@ -336,7 +336,7 @@ __device__ __forceinline__ void conv_body(const LayerDesc &L, int m, const Group
                         rests = __fadd2_rn(rests, rest);
                         size = __fadd_rn(__fadd_rn(size, fabsf(rest.x)), fabsf(rest.y));
                         t = __fadd2_rn(Xc, c2.magic);
-                        P2[p] = __ffma2_rn(Xc, c2.neg1, __ffma2_rn(c2.magic, c2.neg1, t));
+                        P2[p] = __ffma2_rn(Xc, c2.neg1, less_magic<true>(t, c2));
                     }
                     ck[2 * p] = static_cast<unsigned char>(__float_as_uint(t.x));
                     if (p < 4) ck[2 * p + 1] = static_cast<unsigned char>(__float_as_uint(t.y));
@@ -438,7 +438,7 @@ __device__ __forceinline__ void conv_body(const LayerDesc &L, int m, const Group
             S.mx[G.t] = hi0;
             S.mx[G.t + g] = -lo0;
         }
-        ec = owner_sum<kOwn, kClip, true>(G, S, esum, static_cast<unsigned>(esum), static_cast<int>((esum + (1 << 16)) >> 17), up, down);
+        ec = owner_sum<kOwn, kClip, kLargest>(G, S, esum, static_cast<unsigned>(esum), static_cast<int>((esum + (1 << 16)) >> 17), up, down);
     }
 
     // ---- SQuant-C: Algorithm 2 on the channel, keys = the kernels' candidates

@@ -236,9 +236,10 @@ __device__ __forceinline__ float owner_absmax(const Group &G, float amax, const 
 }
 
 // Channel-wide error sum and extremes.  k64: the sum of e; else the sum of which lo32 is a thread's value
-// modulo 2^32 and apx its size in units of 2^17, off by less than 2^13 units over the channel.  kExt: up, down
-// (both >= 0) become the channel's (groups of whole warps).
-template <Owner kOwn, bool k64, bool kExt>
+// modulo 2^32 and apx its size in units of 2^17, off by less than 2^13 units over the channel.  kLargest: up, down
+// (both >= 0) become the channel's largest, kTotal: the sums of those of the warps (groups of whole warps).
+enum Extra { kNothing, kLargest, kTotal };
+template <Owner kOwn, bool k64, Extra kExtra>
 __device__ __forceinline__ long long owner_sum(const Group &G, const Sel &S, long long e, unsigned lo32, int apx, int &up, int &down)
 {
     const int lane = threadIdx.x & 31;
@@ -248,7 +249,7 @@ __device__ __forceinline__ long long owner_sum(const Group &G, const Sel &S, lon
         lo32 = static_cast<unsigned>(lanes_add(G.g, static_cast<int>(lo32)));
         apx = lanes_add(G.g, apx);
     }
-    if (kExt) {
+    if (kExtra == kLargest) {
         up = static_cast<int>(__reduce_max_sync(kFull, static_cast<unsigned>(up)));
         down = static_cast<int>(__reduce_max_sync(kFull, static_cast<unsigned>(down)));
     }
@@ -262,9 +263,12 @@ __device__ __forceinline__ long long owner_sum(const Group &G, const Sel &S, lon
                     atomicAdd(&S.part->lo32, static_cast<int>(lo32));
                     atomicAdd(&S.part->hi32, apx);
                 }
-                if (kExt) {
+                if (kExtra == kLargest) {
                     atomicMax(&S.part->up, up);
                     atomicMax(&S.part->down, down);
+                } else if (kExtra == kTotal) {
+                    atomicAdd(&S.part->up, up);
+                    atomicAdd(&S.part->down, down);
                 }
             }
             owner_sync<kOwn>(G);
@@ -283,9 +287,12 @@ __device__ __forceinline__ long long owner_sum(const Group &G, const Sel &S, lon
             lo32 = static_cast<unsigned>(__reduce_add_sync(kFull, q.x));
             apx = __reduce_add_sync(kFull, q.y);
         }
-        if (kExt) {
+        if (kExtra == kLargest) {
             up = static_cast<int>(__reduce_max_sync(kFull, static_cast<unsigned>(q.z)));
             down = static_cast<int>(__reduce_max_sync(kFull, static_cast<unsigned>(q.w)));
+        } else if (kExtra == kTotal) {
+            up = __reduce_add_sync(kFull, q.z);
+            down = __reduce_add_sync(kFull, q.w);
         }
     }
     if (k64) return e;
@@ -604,8 +611,8 @@ struct RowSums {
 __device__ __forceinline__ unsigned row_vector(const float4 w, const E2 &c2, RowSums &R, int which, int4 &p)
 {
     float2 ta, tb, Pa, Pb;
-    squant_e_fast2(make_float2(w.x, w.y), c2, ta, Pa);
-    squant_e_fast2(make_float2(w.z, w.w), c2, tb, Pb);
+    squant_e_fast2<true>(make_float2(w.x, w.y), c2, ta, Pa);
+    squant_e_fast2<true>(make_float2(w.z, w.w), c2, tb, Pb);
     p = make_int4(__float2int_rn(Pa.x), __float2int_rn(Pa.y), __float2int_rn(Pb.x), __float2int_rn(Pb.y));
     R.fs = __fadd2_rn(R.fs, Pa);
     R.fs = __fadd2_rn(R.fs, Pb);
@@ -648,7 +655,7 @@ __device__ __forceinline__ unsigned row_vector_clip(const float4 w, const E2 &c2
         Xa = ya;
         Xb = yb;
         // whole codes and the rest of each
-        const float2 ma = __ffma2_rn(c2.magic, c2.neg1, __fadd2_rn(ra, c2.magic)), mb = __ffma2_rn(c2.magic, c2.neg1, __fadd2_rn(rb, c2.magic));
+        const float2 ma = less_magic<true>(__fadd2_rn(ra, c2.magic), c2), mb = less_magic<true>(__fadd2_rn(rb, c2.magic), c2);
         const float2 fa = __ffma2_rn(ma, c2.neg1, ra), fb = __ffma2_rn(mb, c2.neg1, rb);
         const int i0 = __float2int_rn(fa.x), i1 = __float2int_rn(fa.y), i2 = __float2int_rn(fb.x), i3 = __float2int_rn(fb.y);
         C.whole += __float2int_rn(__fmul_rn(__fadd_rn(__fadd_rn(ma.x, ma.y), __fadd_rn(mb.x, mb.y)), 0x1p-30f));
@@ -659,7 +666,7 @@ __device__ __forceinline__ unsigned row_vector_clip(const float4 w, const E2 &c2
         }
     }
     const float2 ta = __fadd2_rn(Xa, c2.magic), tb = __fadd2_rn(Xb, c2.magic);
-    const float2 Pa = __ffma2_rn(Xa, c2.neg1, __ffma2_rn(c2.magic, c2.neg1, ta)), Pb = __ffma2_rn(Xb, c2.neg1, __ffma2_rn(c2.magic, c2.neg1, tb));
+    const float2 Pa = __ffma2_rn(Xa, c2.neg1, less_magic<true>(ta, c2)), Pb = __ffma2_rn(Xb, c2.neg1, less_magic<true>(tb, c2));
     p = make_int4(__float2int_rn(Pa.x), __float2int_rn(Pa.y), __float2int_rn(Pb.x), __float2int_rn(Pb.y));
     R.fs = __fadd2_rn(R.fs, Pa);
     R.fs = __fadd2_rn(R.fs, Pb);
@@ -836,8 +843,8 @@ __device__ __forceinline__ void row_body(const LayerDesc &L, int m, const Group 
                 const float2 wa = make_float2(w.x, w.y), wb = make_float2(w.z, w.w);
                 float2 ta, tb;
                 if (!kClip) {
-                    squant_e_fast2(wa, c2, ta, Pa);
-                    squant_e_fast2(wb, c2, tb, Pb);
+                    squant_e_fast2<true>(wa, c2, ta, Pa);
+                    squant_e_fast2<true>(wb, c2, tb, Pb);
                 } else {
                     const float2 xa = __fmul2_rn(wa, c2.y), xb = __fmul2_rn(wb, c2.y);
                     const float2 Xa = __ffma2_rn(__ffma2_rn(xa, c2.ns2, wa), c2.y, xa), Xb = __ffma2_rn(__ffma2_rn(xb, c2.ns2, wb), c2.y, xb);
@@ -847,8 +854,8 @@ __device__ __forceinline__ void row_body(const LayerDesc &L, int m, const Group 
                     ta.y = fminf(fmaxf(ta.y, tmin), tmax);
                     tb.x = fminf(fmaxf(tb.x, tmin), tmax);
                     tb.y = fminf(fmaxf(tb.y, tmin), tmax);
-                    Pa = __ffma2_rn(Xa, c2.neg1, __ffma2_rn(c2.magic, c2.neg1, ta));
-                    Pb = __ffma2_rn(Xb, c2.neg1, __ffma2_rn(c2.magic, c2.neg1, tb));
+                    Pa = __ffma2_rn(Xa, c2.neg1, less_magic<true>(ta, c2));
+                    Pb = __ffma2_rn(Xb, c2.neg1, less_magic<true>(tb, c2));
                 }
                 c4 = __byte_perm(__byte_perm(__float_as_uint(ta.x), __float_as_uint(ta.y), 0x0040),
                                  __byte_perm(__float_as_uint(tb.x), __float_as_uint(tb.y), 0x0040), 0x5410);
@@ -918,7 +925,7 @@ __device__ __forceinline__ void row_body(const LayerDesc &L, int m, const Group 
         int up = 0, down = 0;
         const int apx = __float2int_rn(__fmul_rn(__fadd_rn(R.fs.x, R.fs.y), 0x1p-17f));
         if (kClip) C.sum64 += static_cast<long long>(C.whole) * kOne + static_cast<long long>(apx) * (1ll << 17) + static_cast<int>(R.sum - (static_cast<unsigned>(apx) << 17));
-        ec = owner_sum<kOwn, kClip, false>(G, S, C.sum64, R.sum, apx, up, down);
+        ec = owner_sum<kOwn, kClip, kNothing>(G, S, C.sum64, R.sum, apx, up, down);
     }
 
     // ---- SQuant-C: Algorithm 2 on the channel, the perturbations are the keys

@@ -84,8 +84,8 @@ __device__ __forceinline__ void row_quad(const float4 w, const RowQuant &R, Quad
             tb.y = fminf(fmaxf(tb.y, tmin), tmax);
         }
     }
-    o.qa = __ffma2_rn(R.c2.magic, R.c2.neg1, ta);
-    o.qb = __ffma2_rn(R.c2.magic, R.c2.neg1, tb);
+    o.qa = less_magic(ta, R.c2);
+    o.qb = less_magic(tb, R.c2);
     o.Pa = __ffma2_rn(Xa, R.c2.neg1, o.qa);
     o.Pb = __ffma2_rn(Xb, R.c2.neg1, o.qb);
     o.c4 = __byte_perm(__byte_perm(__float_as_uint(ta.x), __float_as_uint(ta.y), 0x0040),
@@ -118,9 +118,9 @@ __device__ __forceinline__ unsigned row_extremes(const int4 p)
 //     quarter of its vectors (both signs, 16 bits each) and makes those of the few quarters that come into question
 //     anew, which yields the code of what is flipped too;
 //   - only codes that are to be packed wait in shared memory.
-// Against the body of the groups, with which these rows shared their code before: 256 rows of 100,352 weights 156 -> 83 us
-// on a B200 (the checked body of supplied scales until then), 4096 rows of 12,000 123.0 -> 96.9.  In groups of up to
-// 256 threads it is the slower one (65,536 rows of 256 weights 54 -> 63 us), and for few rows: there the code that runs once counts most.
+// Against the body of the groups, with which wide rows shared their code before: 256 rows of 100,352 weights 156 -> 83 us
+// on a B200 (the checked body of supplied scales until then).  Where row_body fits it is the slower one (4096 rows of 12,000 98.4 us, 89.6 in
+// row_body): the code that runs once counts.
 template <bool kClip, Owner kOwn>
 __device__ __forceinline__ void long_row_body(const LayerDesc &L, int m, const Group &G, unsigned char *slice, int qmax, unsigned mode,
                                               int n0 = 0, int nloc = 0)
@@ -312,11 +312,23 @@ __device__ __forceinline__ void long_row_body(const LayerDesc &L, int m, const G
     // ---- channel sum.  !kClip: its value modulo 2^32 is exact, its size is known from the float sums
     // (a thread's fewer than 2^7 elements of at most one half give partial sums below 2^36, each addition off by at most 2^11, so
     // its sum by less than 2^18; those of at most 2^12 threads by less than 2^30, and by 2^28 for the rounding to units of 2^17)
+    // The list of SQuant-C starts where the number of elements within `near` of one half leads one to expect somewhat more than k_c
+    // (near is in units of 2^16; evenly spread values have as many elements there as the channel sum's standard deviation).  The count travels with
+    // the channel sum, so that no barrier is spent on a search: 256 rows of 100,352 weights 76.9 -> 71.8 us a call on a B200, 8 of 200,000 19.2 -> 17.0,
+    // 1000 of 25,001 58.7 -> 56.4.  Too few seen (two bits and outliers) say nothing; a cluster then searches (256 rows of 100,352: 87.2 -> 88.8).
+    constexpr int top = (kHalf >> 16) + 1;
+    auto near_of = [](int n) { return min(max(__float2int_rn(0.58f * top * rsqrtf(static_cast<float>(n))), 1), top - 1); };
+    int above = 0, below = 0;
     long long ec = 0;
     if ((mode & 4u) || L.cerr) {
-        if (kOwn != kCluster) S.mx[G.t] = static_cast<int>(__vmaxu2(__vmaxu2(e0, e1), __vmaxu2(e2, e3)));   // SQuant-C looks for its bound among these
-        int up = 0, down = 0;
-        ec = owner_sum<kOwn, kClip, false>(G, S, sum64, sum, __float2int_rn(__fmul_rn(__fadd_rn(fs.x, fs.y), 0x1p-17f)), up, down);
+        if (mode & 4u) {   // quarters whose extremes lie near one half, of either sign
+            const unsigned th = static_cast<unsigned>(top - near_of(again(L.N))) << 16;
+            for (const unsigned e : {e0, e1, e2, e3}) {
+                above += __popc(__ballot_sync(kFull, (e << 16) >= th));
+                below += __popc(__ballot_sync(kFull, e >= th));
+            }
+        }
+        ec = owner_sum<kOwn, kClip, kTotal>(G, S, sum64, sum, __float2int_rn(__fmul_rn(__fadd_rn(fs.x, fs.y), 0x1p-17f)), above, below);
     }
 
     // ---- SQuant-C: Algorithm 2 on the channel, the perturbations are the keys
@@ -423,7 +435,13 @@ __device__ __forceinline__ void long_row_body(const LayerDesc &L, int m, const G
                 if (deq16) deq16[n] = static_cast<uint16_t>(bf16_bits(row_deq(c, s)));
             };
             const int nmax = kOwn == kCluster ? 4 * g * static_cast<int>(cg::this_cluster().num_blocks()) : g;
-            const int k_eff = select_top<kOwn, true>(G, [] {}, count, listing, settle, each, code_of, flip, nmax, false, 0, (kHalf >> 16) + 1, kHalf + (1 << 14) + 1, 2.0f, kc, L.N, want, S, 1);
+            auto prepare = [&] {
+                if (kOwn != kCluster) S.mx[G.t] = static_cast<int>(__vmaxu2(__vmaxu2(e0, e1), __vmaxu2(e2, e3)));
+            };
+            const int seen = sgn > 0 ? above : below;
+            const float goal = __fadd_rn(__fmul_rn(static_cast<float>(kc), 1.3f), 10.0f);
+            const int start = top - 1 - __float2int_rn(__fmul_rn(goal, __fdividef(static_cast<float>(near_of(again(L.N))), static_cast<float>(max(seen, 1)))));
+            const int k_eff = select_top<kOwn, false>(G, prepare, count, listing, settle, each, code_of, flip, nmax, kOwn != kCluster || seen >= 24, start, top, kHalf + (1 << 14) + 1, 2.0f, kc, L.N, want, S, 1);
             ec -= static_cast<long long>(sgn) * k_eff * kOne;
         }
     }

@@ -109,6 +109,19 @@ def test_rows_whose_list_starts_at_a_guess(n):
         check(ws, bits, start=bits % 3)
 
 
+@pytest.mark.parametrize("rows,n", [(1, 25001), (3, 24004), (3, 100352), (2, 65541)])
+def test_long_rows_whose_list_starts_at_a_guess(rows, n):
+    """Long and wide rows: a guess from the number of elements seen near one half, too few of them (two bits and outliers),
+    one-signed weights and ties."""
+    if rows == 1:   # enough of them for the long form
+        rows = torch.cuda.get_device_properties(0).multi_processor_count + 1
+    shape = (rows, n, 1, 1)
+    w = W.random_layer(shape, seed=n)
+    ws = [w, np.where(W.random_layer(shape, seed=n + 1) > 2.0 * w.std(), 8 * w, w)] + layers((3,) + shape[1:], n)
+    for bits in (2, 4, 8):
+        check(ws, bits, start=bits % 3)
+
+
 @pytest.mark.parametrize("bits,clip", [(2, 0.97), (4, 0.7), (8, 0.5), (3, 0.2), (8, 0.1), (6, 0.04)])
 def test_elements_at_and_far_beyond_the_clip_range(bits, clip):
     """Scales of the caller's from just below absmax (elements on the last code) to far below (sums of many whole codes, kernels
