@@ -941,11 +941,13 @@ __device__ __forceinline__ void row_body(const LayerDesc &L, int m, const Group 
             auto visit = [&](int t, unsigned halves, auto fn) {
                 const int tx = t + sx;
 #pragma unroll 1
-                for (; halves != 0u; halves &= halves - 1u) {
-                    const int odd = __ffs(halves) - 1;
+                while (halves != 0u) {
+                    const bool both = halves == 3u && vecs <= kRowVecs;   // in one pass
+                    const int at = both ? 0 : __ffs(halves) - 1, inc = both ? 1 : 2;
+                    halves = both ? 0u : halves & (halves - 1u);
                     unsigned hit = 0u, bit = 1u;   // a bit for each of these (at most 32) elements that counts
 #pragma unroll 2
-                    for (int i = odd; i < vecs; i += 2, bit <<= 4) {
+                    for (int i = at; i < vecs; i += inc, bit <<= 4) {
                         const int4 p = Pbuf[q0 + i * step];
                         if ((p.x ^ sx) >= tx) hit |= bit;
                         if ((p.y ^ sx) >= tx) hit |= 2u * bit;
@@ -954,7 +956,7 @@ __device__ __forceinline__ void row_body(const LayerDesc &L, int m, const Group 
                     }
 #pragma unroll 1
                     for (; hit != 0u; hit &= hit - 1u) {
-                        const int b = __ffs(hit) - 1, n = 4 * (q0 + (odd + 2 * (b >> 2)) * step) - r + (b & 3);
+                        const int b = __ffs(hit) - 1, n = 4 * (q0 + (at + inc * (b >> 2)) * step) - r + (b & 3);
                         SQ_DBG(n >= 0 && n < N, 15);
                         fn((Pel[n] ^ sx) - sx, n);
                     }
