@@ -121,7 +121,7 @@ int squant_quantize_layer(const squant_layer *layer, const squant_options *opt, 
  * that layers could be quantized in parallel, Sec. 4.2): one launch of the grouped kernel for
  * most models; layers of channels longer than 8192 weights take launches of their own: 3x3 channels
  * of 1184 input channels and more (a multiple of 4, at most 2048; SQuant-K on, absmax scales) one of
- * the persistent streaming kernel, 1x1 rows one to three of the row kernel, channels that do not fit one
+ * the persistent streaming kernel, 1x1 rows one to four of the row kernel, channels that do not fit one
  * thread block's shared memory one of the cluster kernel per layer.
  *
  *   layers, n_layers  host array of descriptors holding DEVICE pointers; n_layers >= 0
