@@ -480,6 +480,11 @@ __device__ __forceinline__ void conv_body(const LayerDesc &L, int m, const Group
                     if (a >= t) fn(a, n0 + n);
                 }
             };
+            auto tally = [&](int t) {
+                int c = 0;
+                each(t, [&](int, int) { ++c; });
+                return c;
+            };
             auto listing = [&](int t, auto push) { each(t, [&](int a, int n) { push(a, n, 0u); }); };   // (positions are with the kernels)
             auto flip = [&](int, int n_abs, unsigned) {
                 const int n = n_abs - n0;
@@ -493,7 +498,7 @@ __device__ __forceinline__ void conv_body(const LayerDesc &L, int m, const Group
             // Over-SQuant candidates reach one, but few come near it: the search starts at the largest
             const int top = (sgn > 0 ? up : down) + 1;
             const int nmax = g * (kOwn == kCluster ? static_cast<int>(cg::this_cluster().num_blocks()) : 1);
-            const int k_eff = select_top<kOwn, false>(G, [] {}, count, listing, [] {}, each, [](int) { return 0u; }, flip, nmax, false, 0, top, top, 3.0f, kc, L.N, true, S, K);
+            const int k_eff = select_top<kOwn, false>(G, [] {}, count, listing, [] {}, tally, each, [](int) { return 0u; }, flip, nmax, false, 0, top, top, 3.0f, kc, L.N, true, S, K);
             ec -= static_cast<long long>(sgn) * k_eff * kOne;
         }
     }

@@ -423,6 +423,11 @@ __device__ __forceinline__ void long_row_body(const LayerDesc &L, int m, const G
                 }
                 if (p_rag >= up || p_rag <= down) fn(abs(p_rag), n0 + rag);
             };
+            auto tally = [&](int v) {
+                int c = 0;
+                each(v, [&](int, int) { ++c; });
+                return c;
+            };
             auto code_of = [&](int n_abs) { return static_cast<unsigned>(pack ? cel[n_abs - n0] : crow[n_abs - n0]); };
             auto flip = [&](int a, int n_abs, unsigned code) {
                 const int n = n_abs - n0;
@@ -441,7 +446,7 @@ __device__ __forceinline__ void long_row_body(const LayerDesc &L, int m, const G
             const int seen = sgn > 0 ? above : below;
             const float goal = __fadd_rn(__fmul_rn(static_cast<float>(kc), 1.3f), 10.0f);
             const int start = top - 1 - __float2int_rn(__fmul_rn(goal, __fdividef(static_cast<float>(near_of(again(L.N))), static_cast<float>(max(seen, 1)))));
-            const int k_eff = select_top<kOwn, false>(G, prepare, count, listing, settle, each, code_of, flip, nmax, kOwn != kCluster || seen >= 24, start, top, kHalf + (1 << 14) + 1, 2.0f, kc, L.N, want, S, 1);
+            const int k_eff = select_top<kOwn, false>(G, prepare, count, listing, settle, tally, each, code_of, flip, nmax, kOwn != kCluster || seen >= 24, start, top, kHalf + (1 << 14) + 1, 2.0f, kc, L.N, want, S, 1);
             ec -= static_cast<long long>(sgn) * k_eff * kOne;
         }
     }

@@ -109,6 +109,24 @@ def test_rows_whose_list_starts_at_a_guess(n):
         check(ws, bits, start=bits % 3)
 
 
+@pytest.mark.parametrize("n", [180, 256, 512, 1024, 2048, 4096])
+def test_rows_of_every_number_of_flips(n):
+    """A row for each number of flips up to a quarter of its weights: first lists with and without room, searches among
+    too few maxima, exact searches from the bound of a list that was full; spread and coarse values, other rows between them."""
+    flips = np.arange(n // 4)
+    rng = np.random.default_rng(n)
+    x = rng.integers(-6, 7, (2 * flips.size, n)) + np.where(rng.random((2 * flips.size, n)) < 0.5, 0, rng.uniform(-0.49, 0.49, (2 * flips.size, n)))
+    x[::2] = rng.integers(-6, 7, (flips.size, n))
+    for k in flips:   # the first elements add up to about k
+        up = rng.uniform(0.3, 0.49, n)
+        x[2 * k, :] += np.where((np.cumsum(up) < k) if k % 3 else (np.arange(n) < k / 0.4), up if k % 3 else 0.4, 0.0)
+    x[:, 0] = 7
+    w = x.astype(np.float32)[..., None, None] / np.float32(7)
+    check([w, -w], 4)
+    check([w], 4, start=1, clip=0.99)
+    check([w], 4, clip=0.6)
+
+
 @pytest.mark.parametrize("rows,n", [(1, 25001), (3, 24004), (3, 100352), (2, 65541)])
 def test_long_rows_whose_list_starts_at_a_guess(rows, n):
     """Long and wide rows: a guess from the number of elements seen near one half, too few of them (two bits and outliers),
