@@ -599,8 +599,8 @@ int device_smem_limit(int device, int &limit)
         SQ_CUDA(cudaDeviceGetAttribute(&v, cudaDevAttrMaxSharedMemoryPerBlockOptin, device));
         for (auto kernel : {sq::squant_model_kernel<sq::kAbsmax>, sq::squant_model_kernel<sq::kOwnScales>, sq::squant_model_kernel<sq::kEither>})
             SQ_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, v));
-        SQ_CUDA(cudaFuncSetAttribute(sq::squant_table_kernel,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, v));
+        for (auto kernel : {sq::squant_table_kernel<sq::kAbsmax>, sq::squant_table_kernel<sq::kOwnScales>})
+            SQ_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, v));
         SQ_CUDA(cudaFuncSetAttribute((sq::squant_row_kernel<256, false>),
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, v));
         SQ_CUDA(cudaFuncSetAttribute((sq::squant_row_kernel<512, true>),
@@ -1080,8 +1080,8 @@ int squant_quantize_layer_noalloc(const squant_layer *layer, const squant_option
     SQ_CUDA(cudaMemcpyAsync(table, g_noalloc_host, 256 + ibytes, cudaMemcpyHostToDevice, stream));
     const LayerDesc *dl = static_cast<const LayerDesc *>(table);
     const Item *di = reinterpret_cast<const Item *>(static_cast<const unsigned char *>(table) + 256);
-    sq::squant_table_kernel<<<static_cast<unsigned>(hp.items.size()), sq::kCtaThreads, hp.smem_bytes, stream>>>(
-        dl, di, hp.qmax, hp.mode);
+    auto kernel = hp.layers[0].sin ? sq::squant_table_kernel<sq::kOwnScales> : sq::squant_table_kernel<sq::kAbsmax>;
+    kernel<<<static_cast<unsigned>(hp.items.size()), sq::kCtaThreads, hp.smem_bytes, stream>>>(dl, di, hp.qmax, hp.mode);
     SQ_CUDA(cudaGetLastError());
     g_launches.fetch_add(1, std::memory_order_relaxed);
     return SQUANT_OK;

@@ -64,6 +64,21 @@ def test_noalloc_matches_regular_entry_point_on_consecutive_calls():
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("shape", [(96, 128, 3, 3), (300, 1000, 1, 1), (70, 250, 1, 1), (5, 4096, 1, 1), (33, 40, 5, 5), (200, 1, 3, 3), (64, 8, 1, 7)])
+def test_noalloc_with_and_without_scales_of_the_callers(shape):
+    """Each has a kernel of its own: a layer of each in turn, the codes and sums of the CPU checker."""
+    w = W.random_layer(shape, seed=shape[1])
+    sc = (np.abs(w).reshape(shape[0], -1).max(1) * np.float32(0.7) / np.float32(7)).astype(np.float32)
+    for scales in (None, sc, None):
+        b = sq.alloc_outputs(torch.from_numpy(w).cuda(), dequant=True)
+        b.scales_in = None if scales is None else torch.from_numpy(scales).cuda()
+        sq.squant_quantize_layer_noalloc(b, bits=4)
+        ref = oracle.quantize_layer(w, bits=4, scales_in=scales, details=True)
+        for got, want in ((b.codes, ref.codes), (b.scales, ref.scales), (b.kernel_err, ref.kernel_err), (b.channel_err, ref.channel_err), (b.dequant, ref.dequant)):
+            assert np.array_equal(got.cpu().numpy().view(np.uint8), np.ascontiguousarray(want).view(np.uint8))
+
+
+@pytest.mark.gpu
 def test_noalloc_refuses_a_stream_that_is_being_captured():
     """The table upload reads a host image that the next call rewrites, so a captured copy would
     replay someone else's table: the call is refused before anything is enqueued, and the same
