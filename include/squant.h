@@ -141,7 +141,11 @@ int squant_quantize_layer(const squant_layer *layer, const squant_options *opt, 
  * a counter in device memory, which is part of the scratch area and so belongs to the cached launch
  * tables of these exact descriptors and the graphs captured with them:
  * two calls with the SAME descriptors must not overlap on the GPU (they would race on the
- * outputs anyway); calls with different descriptors may.  All arguments are validated
+ * outputs anyway); calls with different descriptors may.
+ * The launches of one call work on different layers and may overlap on the GPU (except those that a graph captures):
+ * no layer may read or write what another layer of the same call writes.  They start when all earlier
+ * work of the stream has ended, and whatever follows the call in the stream starts when all of them have ended.
+ * All arguments are validated
  * on the host first; a failed call launches nothing and writes nothing.  Returns SQUANT_OK or a
  * negative SQUANT_ERR_* code.
  */

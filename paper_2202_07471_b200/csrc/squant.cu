@@ -692,6 +692,18 @@ int launch_plan(const ParamPlan &p, cudaStream_t stream)
 {
     const int freed = free_dead_scratch(stream);   // of graphs and of plans that have left the cache
     if (freed) return freed;
+    // The row and cluster kernels may start before the launch in front of them has ended (see next_launch_may_start).  Not the streaming
+    // kernels, which may share a scratch area, nor the grouped one (the wait at its end would cost it registers), nor what a graph captures.
+    const size_t plain = std::max<size_t>(p.streams.size() + p.grouped.size(), 1), launches = p.streams.size() + p.grouped.size() + p.rows.size() + p.wide.size();
+    size_t j = 0;   // of this call's launches
+    bool overlap = false;
+    if (launches > plain) {
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        SQ_CUDA(cudaStreamIsCapturing(stream, &cap));
+        overlap = cap == cudaStreamCaptureStatusNone;
+    }
+    const auto early = [&](size_t i) { return overlap && i >= plain && i < launches; };
+    const auto mode = [&] { return p.mode | (early(j) ? sq::kModeMayStartEarly : 0u) | (early(j + 1) ? sq::kModeNextMayStart : 0u); };
     // long 3x3 channels first: one persistent CTA per multiprocessor
     for (ParamPlan::Stream &st : p.streams) {
         int device = 0;
@@ -715,23 +727,15 @@ int launch_plan(const ParamPlan &p, cudaStream_t stream)
         if (scratch) {
             const int grid = std::min(st.items, sms), smem = sq::stream_layout(st.nk_max, st.n_max).total;
             auto kernel = st.out ? sq::squant_stream_kernel<true> : sq::squant_stream_kernel<false>;
-            kernel<<<grid, sq::kStreamThreads, smem, stream>>>(st.table, p.qmax, p.mode, st.items, st.nk_max, st.n_max, scratch->mem, scratch->work());
+            kernel<<<grid, sq::kStreamThreads, smem, stream>>>(st.table, p.qmax, mode(), st.items, st.nk_max, st.n_max, scratch->mem, scratch->work());
         } else {
-            sq::squant_model_kernel<sq::kAbsmax><<<st.grouped_grid, sq::kCtaThreads, st.grouped_smem, stream>>>(st.grouped, p.qmax, p.mode);
+            sq::squant_model_kernel<sq::kAbsmax><<<st.grouped_grid, sq::kCtaThreads, st.grouped_smem, stream>>>(st.grouped, p.qmax, mode());
         }
         SQ_CUDA(cudaGetLastError());
         g_launches.fetch_add(1, std::memory_order_relaxed);
+        ++j;
     }
-    // The row and cluster kernels may start before the launch in front of them has ended (see next_launch_may_start).  Not the streaming
-    // kernels, which may share a scratch area, nor the grouped one (the wait at its end would cost it registers), nor what a graph captures.
-    bool early = false;
-    if (p.streams.size() + p.rows.size() + p.grouped.size() + p.wide.size() > 1) {
-        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-        SQ_CUDA(cudaStreamIsCapturing(stream, &cap));
-        early = cap == cudaStreamCaptureStatusNone;
-    }
-    bool first = p.streams.empty() && p.grouped.empty();
-    const auto launch = [&](auto kernel, bool early_kernel, int grid, int threads, int smem, int cluster, const auto &...args) -> int {
+    const auto launch = [&](auto kernel, int grid, int threads, int smem, int cluster, const auto &...args) -> int {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(static_cast<unsigned>(grid));
         cfg.blockDim = dim3(static_cast<unsigned>(threads));
@@ -745,32 +749,32 @@ int launch_plan(const ParamPlan &p, cudaStream_t stream)
             attr[cfg.numAttrs].val.clusterDim.z = 1;
             ++cfg.numAttrs;
         }
-        if (early && early_kernel && !first) {
+        if (early(j)) {
             attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
             attr[cfg.numAttrs].val.programmaticStreamSerializationAllowed = 1;
             ++cfg.numAttrs;
         }
         cfg.attrs = attr;
-        first = first && !early_kernel;
         void *const argv[] = {const_cast<void *>(static_cast<const void *>(&args))...};   // (of the kernels' own types)
         SQ_CUDA(cudaLaunchKernelExC(&cfg, reinterpret_cast<const void *>(kernel), const_cast<void **>(argv)));
         g_launches.fetch_add(1, std::memory_order_relaxed);
+        ++j;
         return SQUANT_OK;
     };
     for (const ParamPlan::Grouped &gl : p.grouped) {
         auto kernel = gl.scales == sq::kAbsmax ? sq::squant_model_kernel<sq::kAbsmax>
                       : gl.scales == sq::kOwnScales ? sq::squant_model_kernel<sq::kOwnScales> : sq::squant_model_kernel<sq::kEither>;
-        const int rc = launch(kernel, false, gl.grid, sq::kCtaThreads, gl.smem, 1, gl.table, p.qmax, p.mode);
+        const int rc = launch(kernel, gl.grid, sq::kCtaThreads, gl.smem, 1, gl.table, p.qmax, mode());
         if (rc) return rc;
     }
     for (const ParamPlan::Rows &r : p.rows) {
         auto kernel = r.form == ParamPlan::kRow512 ? sq::squant_row_kernel<512, false>
                       : r.form == ParamPlan::kLong512 ? sq::squant_row_kernel<512, true> : sq::squant_row_kernel<256, false>;
-        const int rc = launch(kernel, true, r.grid, r.form == ParamPlan::kRow256 ? 256 : 512, r.smem, 1, r.table, p.qmax, p.mode);
+        const int rc = launch(kernel, r.grid, r.form == ParamPlan::kRow256 ? 256 : 512, r.smem, 1, r.table, p.qmax, mode());
         if (rc) return rc;
     }
     for (const ParamPlan::Wide &w : p.wide) {   // one cluster per output channel
-        const int rc = launch(sq::squant_wide_kernel, true, w.d.M * w.cluster, sq::kBlockThreads, w.smem, w.cluster, w.d, p.qmax, p.mode, w.kpc);
+        const int rc = launch(sq::squant_wide_kernel, w.d.M * w.cluster, sq::kBlockThreads, w.smem, w.cluster, w.d, p.qmax, mode(), w.kpc);
         if (rc) return rc;
     }
     return SQUANT_OK;

@@ -174,14 +174,19 @@ __device__ __forceinline__ void bulk_store_wait()
 }
 
 // ---------------------------------------------------------------- overlap of a call's launches
-// The launches of a call work on different layers, so those of the row and cluster kernels may start while the one before still runs: their
-// thread blocks take the places that the last ones of that leave free.  Every kernel says at its start that the next may come, as
-// soon as all of its own thread blocks have started.  A launch that may come early ends no earlier than the one before (its last thread
-// block waits for that), so whatever follows the call's last launch follows all of them.
-__device__ __forceinline__ void next_launch_may_start() { asm volatile("griddepcontrol.launch_dependents;"); }
-__device__ __forceinline__ void end_after_launch_before()
+// The launches of a call work on different layers, so those of the row and cluster kernels may start while the one
+// before still runs: their thread blocks take the places that the last ones of that leave free.  A launch that another
+// of the call may follow early (kModeNextMayStart) says so at its start, as soon as all of its own thread blocks have
+// started.  One that may come early (kModeMayStartEarly) ends no earlier than the one before (its last thread block
+// waits for that), so whatever follows the call's last launch follows all of them; the last launch says nothing.
+constexpr unsigned kModeNextMayStart = 0x400u, kModeMayStartEarly = 0x800u;   // bits of `mode`
+__device__ __forceinline__ void next_launch_may_start(unsigned mode)
 {
-    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) asm volatile("griddepcontrol.wait;");
+    if (mode & kModeNextMayStart) asm volatile("griddepcontrol.launch_dependents;");
+}
+__device__ __forceinline__ void end_after_launch_before(unsigned mode)
+{
+    if ((mode & kModeMayStartEarly) && blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 // ---------------------------------------------------------------- group-wide reductions
@@ -1419,7 +1424,7 @@ __global__ void __launch_bounds__(kCtaThreads, SQ_MIN_CTAS)
 squant_model_kernel(const __grid_constant__ LaunchTable tbl, int qmax, unsigned mode)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    next_launch_may_start();
+    next_launch_may_start(mode);
     const int item = blockIdx.x;
     int layer = 0;   // uniform binary search for the last layer whose first item is <= item
 #pragma unroll 1

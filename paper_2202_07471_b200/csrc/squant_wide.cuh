@@ -486,7 +486,7 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads)
 squant_row_kernel(const __grid_constant__ LaunchTable tbl, int qmax, unsigned mode)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    next_launch_may_start();
+    next_launch_may_start(mode);
     const int item = blockIdx.x;
     int layer = 0;
 #pragma unroll 1
@@ -508,7 +508,7 @@ squant_row_kernel(const __grid_constant__ LaunchTable tbl, int qmax, unsigned mo
         if (L.sin) row_body<true, kBlock, 32>(L, m, G, smem, qmax, mode, true);
         else row_body<false, kBlock, 32>(L, m, G, smem, qmax, mode, true);
     }
-    end_after_launch_before();
+    end_after_launch_before(mode);
 }
 
 // Shared memory of one of a cluster's thread blocks that has `kpc` kernels of K weights.
@@ -524,7 +524,7 @@ __global__ void __launch_bounds__(kBlockThreads, 2)
 squant_wide_kernel(const LayerDesc L, int qmax, unsigned mode, int kpc)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    next_launch_may_start();
+    next_launch_may_start(mode);
     cg::cluster_group cluster = cg::this_cluster();
     const int C = static_cast<int>(cluster.num_blocks()), rank = static_cast<int>(cluster.block_rank());
     const int m = static_cast<int>(blockIdx.x) / C;
@@ -547,7 +547,7 @@ squant_wide_kernel(const LayerDesc L, int qmax, unsigned mode, int kpc)
         else conv_body<0, false, kCluster>(L, m, G, smem, qmax, mode, n0, nloc);
     }
     cluster.sync();   // no thread block leaves while another may still read its shared memory
-    end_after_launch_before();
+    end_after_launch_before(mode);
 }
 
 }  // namespace sq

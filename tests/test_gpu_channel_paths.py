@@ -484,3 +484,49 @@ def test_wide_rows_in_clusters_of_two_and_four(n):
         check([part], 4, sums=False, start=1)
         check([part], 4, flags=sq.FLAG_NARROW_RANGE | sq.FLAG_PACK_INT4, start=3)
     check([w[:9]], 8, flags=0, outputs=True, clip=0.9)
+
+
+@pytest.mark.parametrize("shapes,kernels", [([(100, 16384, 1, 1), (1, 50000, 1, 1)], ["row", "cluster"]), ([(100, 8000, 1, 1), (1, 50000, 1, 1)], ["grouped", "cluster"]),
+                                            ([(100, 8000, 1, 1), (5, 9000, 1, 1), (1, 50000, 1, 1)], ["grouped", "row", "cluster"])])
+def test_what_follows_a_call_follows_all_of_its_launches(shapes, kernels):
+    """The first launch (every row flips thousands of weights that tie) outlasts those that may start before it ends.  Its
+    outputs are copied, its weights overwritten and the call made again on the same stream, with no synchronization."""
+    assert sq.squant_plan_kernels(shapes) == kernels
+    ws = [((np.arange(np.prod(s)) % 7 - 3 + 0.4) / 7).astype(np.float32).reshape(s) if i == 0 else W.random_layer(s, seed=i) for i, s in enumerate(shapes)]
+    ws[0][:, 0] = 1.0   # scales of 1/7
+    refs = [oracle.quantize_layer(w, bits=4) for w in ws]
+    weights = [torch.from_numpy(w).cuda() for w in ws]
+    bufs = [sq.alloc_outputs(w.clone()) for w in weights]
+    call = sq.ModelCall(bufs)
+
+    def time_of(c):
+        start, end = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        torch.cuda.synchronize()
+        start.record()
+        for _ in range(10):
+            c.run()
+        end.record()
+        end.synchronize()
+        return start.elapsed_time(end)
+
+    call.run()
+    first, rest = sq.ModelCall(bufs[:1]), sq.ModelCall(bufs[1:])
+    time_of(first), time_of(rest)
+    assert time_of(first) > 1.5 * time_of(rest)
+    seen = []
+    for _ in range(10):
+        for b, w in zip(bufs, weights):
+            b.w.copy_(w)
+            b.codes.fill_(-128)
+        call.run()
+        got = [(b.codes.clone(), b.kernel_err.clone(), b.channel_err.clone()) for b in bufs]
+        for b in bufs:
+            b.w.fill_(0.0)
+        call.run()
+        seen.append((got, [b.codes.clone() for b in bufs]))
+    torch.cuda.synchronize()
+    for got, again in seen:
+        for g, a, r in zip(got, again, refs):
+            for x, want in zip(g, (r.codes, r.kernel_err, r.channel_err)):
+                assert np.array_equal(x.cpu().numpy().view(np.uint8), np.ascontiguousarray(want).view(np.uint8))
+            assert not a.any()
