@@ -468,7 +468,7 @@ int build_param_plan(const squant_layer *layers, int32_t n_layers, const squant_
         return (a.d.K > 1) != (b.d.K > 1) ? a.d.K > 1 : a.d.K == 1 && a.d.N > b.d.N;
     });
     // Long rows, a thread block per output channel, in one of three forms.  row_body holds 5 B of shared memory a weight,
-    // long_row_body 4 (5 of packed codes).  What counts is how many threads a multiprocessor holds and over how many
+    // long_row_body 4.  What counts is how many threads a multiprocessor holds and over how many
     // vectors a thread spreads the code that runs once.  us a call on a B200, row_body with 256 / with 512 threads / long_row_body with 512:
     //   - More than two and a quarter rows a multiprocessor, so short that three thread blocks of 256 threads fit one (14.8 K weights): those
     //     (rows of 9000 300 12.5 / 12.3 / 14.4, 400 14.4 / 15.8 / 18.7, 4096 69.9 / 94.1 / 117; of 12,000 100 12.9 / 10.3 / 12.8, 500 19.5 / 20.5 /
@@ -482,7 +482,7 @@ int build_param_plan(const squant_layer *layers, int32_t n_layers, const squant_
     const auto small_blocks = [&](int i) { return std::min(4, blocks(sq::row_bytes(256, (descs[i].N + 6) >> 2, sq::kBlock))); };
     const auto only_long = [&](int i) {
         const int vecs = (descs[i].N + 6) >> 2;
-        return !pack && !descs[i].sin && blocks(sq::row_bytes(512, vecs, sq::kBlock)) < 2 && blocks(sq::long_row_bytes(512, vecs, pack, sq::kBlock)) >= 2;
+        return !pack && !descs[i].sin && blocks(sq::row_bytes(512, vecs, sq::kBlock)) < 2 && blocks(sq::long_row_bytes(512, vecs, false, sq::kBlock)) >= 2;
     };
     int64_t small = 0, longer = 0;   // rows
     for (int i : rows) {
@@ -506,7 +506,7 @@ int build_param_plan(const squant_layer *layers, int32_t n_layers, const squant_
             LayerDesc &d = descs[rows[base + n]];
             d.off_vi = (d.N + 6) >> 2;
             d.off_ev = regular_rows(d);
-            smem = std::max(smem, form == ParamPlan::kLong512 ? sq::long_row_bytes(512, d.off_vi, pack, sq::kBlock)
+            smem = std::max(smem, form == ParamPlan::kLong512 ? sq::long_row_bytes(512, d.off_vi, false, sq::kBlock)
                                                               : sq::row_bytes(form == ParamPlan::kRow512 ? 512 : 256, d.off_vi, sq::kBlock));
             ++n;
         }

@@ -498,7 +498,7 @@ __device__ __forceinline__ void conv_body(const LayerDesc &L, int m, const Group
             // Over-SQuant candidates reach one, but few come near it: the search starts at the largest
             const int top = (sgn > 0 ? up : down) + 1;
             const int nmax = g * (kOwn == kCluster ? static_cast<int>(cg::this_cluster().num_blocks()) : 1);
-            const int k_eff = select_top<kOwn, false>(G, [] {}, count, listing, [] {}, tally, each, [](int) { return 0u; }, flip, nmax, false, 0, top, top, 3.0f, kc, L.N, true, S, K);
+            const int k_eff = select_top<kOwn>(G, [] {}, count, listing, [] {}, tally, each, [](int) { return 0u; }, flip, nmax, false, 0, top, top, 3.0f, kc, L.N, true, S, K);
             ec -= static_cast<long long>(sgn) * k_eff * kOne;
         }
     }

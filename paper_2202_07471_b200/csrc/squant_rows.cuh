@@ -1,5 +1,5 @@
 // 1x1 layers (fully connected and pointwise): a group of 8 to 256 threads takes a whole output
-// channel, up to 32 weights a thread, or a thread block of 512 threads a longer one.
+// channel, up to 32 weights a thread, or a thread block of 256 or 512 threads a longer one.
 //
 // Every element is its own kernel, so SQuant-K is a no-op (Sec. 3.4) and the work is absmax,
 // SQuant-E, the channel sum and SQuant-C's choice of the k_c largest perturbations of one sign.
@@ -95,7 +95,7 @@ __host__ __device__ constexpr int sel_bytes(int g, Owner own = kGroup, int K = 1
 }
 // Shared memory of a 1x1 channel of `vecs` vectors: selection, perturbations, codes.
 __host__ __device__ constexpr int row_bytes(int g, int vecs, Owner own = kGroup) { return (own == kBlock ? sel_list_bytes(g, own, 1) : sel_bytes(g, own)) + 20 * vecs; }
-// The same where a thread block or a cluster takes the row: weights, and codes if they are to be packed.
+// The same in long_row_body (a thread block or a cluster takes the row): weights, and codes if they are to be packed.
 __host__ __device__ constexpr int long_row_bytes(int g, int vecs, bool pack, Owner own) { return sel_bytes(g, own) + (pack ? 20 : 16) * vecs; }
 
 // The parts of a group's selection memory.
@@ -361,7 +361,7 @@ __device__ __forceinline__ bool guess_fits(int kc, int cap) { return kOwn == kCl
 // a = the value of a candidate in the direction of the flips, n its kernel index in the channel.  listing(t, push) calls
 // push(a, n, code) for those of the thread's elements that are at least t units, 1 <= t < top (`top` is one unit above
 // the largest possible); code is handed through to flip.  direct: from `start` on somewhat more than kc candidates are expected,
-// which are listed without a search (never with kSearchFirst).  If there is no such list or it will not do, the bound is searched: the threads know maxima of a
+// which are listed without a search.  If there is no such list or it will not do, the bound is searched: the threads know maxima of a
 // over parts of their elements, count(t) = how many of the group's nmax maxima are at least t (direct: prepare() once before, it may
 // write to shared memory).  For
 // the exact search: settle() once, then tally(v) = how many of the thread's elements have a >= v (any v >= 1, vtop above all),
@@ -370,7 +370,7 @@ __device__ __forceinline__ bool guess_fits(int kc, int cap) { return kOwn == kCl
 // index first), by some thread of the group.  want: this group selects at all (kc >= 1).  Returns the number of
 // flips.  Every thread of the group calls it, groups that share a warp together; it starts with no barrier and
 // ends with none.
-template <Owner kOwn, bool kSearchFirst, class Prepare, class Count, class Listing, class Settle, class Tally, class Each, class CodeOf, class Flip>
+template <Owner kOwn, class Prepare, class Count, class Listing, class Settle, class Tally, class Each, class CodeOf, class Flip>
 __device__ __forceinline__ int select_top(const Group &G, Prepare prepare, Count count, Listing listing, Settle settle, Tally tally, Each each, CodeOf code_of, Flip flip,
                                           int nmax, bool direct, int start, int top, int vtop, float spread, int kc, int n_all, bool want, const Sel &S, int K)
 {
@@ -414,9 +414,8 @@ __device__ __forceinline__ int select_top(const Group &G, Prepare prepare, Count
         slow = todo && !sure;   // too few maxima
         todo = todo && sure;
     };
-    if (kSearchFirst) search();
 #pragma unroll 1
-    for (int round = kSearchFirst ? 1 : 0;; ++round) {
+    for (int round = 0;; ++round) {
         if (round > 0 || direct) {
             if (todo && (round > 0 || guess_fits<kOwn>(kc, cap)))
                 listing(lo, [&](int a, int n, unsigned code) {
@@ -467,7 +466,7 @@ __device__ __forceinline__ int select_top(const Group &G, Prepare prepare, Count
             owner_sync<kOwn>(G);
             todo = again;
         }
-        if (!kSearchFirst && round == 0) search();
+        if (round == 0) search();
     }
     auto flip_entry = [&](unsigned long long e) {
         const unsigned low = static_cast<unsigned>(e);
@@ -1019,7 +1018,7 @@ __device__ __forceinline__ void row_body(const LayerDesc &L, int m, const Group 
             };
             const int vtop = kHalf + (1 << 14) + 1;
             const bool direct = L.N >= kRowDirect && (g > 32 || __any_sync(kFull, want && guess_fits<kOwn>(kc, S.cap)));   // (of a clipped row kc can be huge)
-            const int k_eff = select_top<kOwn, false>(G, prepare, count, listing, [] {}, tally, each, [](int) { return 0u; }, flip, kOwn == kBlock ? g : per * g, direct,
+            const int k_eff = select_top<kOwn>(G, prepare, count, listing, [] {}, tally, each, [](int) { return 0u; }, flip, kOwn == kBlock ? g : per * g, direct,
                                                list_start(kc, 2.0f, vtop, max(N, 1)), vtop, vtop, 2.0f, kc, N, want, S, 1);
             ec -= static_cast<long long>(sgn) * k_eff * kOne;
         }

@@ -108,7 +108,7 @@ __device__ __forceinline__ unsigned row_extremes(const int4 p)
 
 // ---------------------------------------------------------------- one 1x1 channel
 // Rows that a whole thread block (kBlock) or a cluster takes; kCluster: this thread block has the elements n0 ..
-// n0 + nloc - 1 (n0 a multiple of four).  kClip: the clip of Sec. 2.2 can fire (caller-supplied scales): codes are
+// n0 + nloc - 1 (n0 a multiple of four).  kBlock: neither packed codes nor supplied scales.  kClip: the clip of Sec. 2.2 can fire (caller-supplied scales): codes are
 // clamped, sums are 64 bit and an element whose flipped code would leave the range is no candidate.
 //
 // What bounds it is the number of instructions (and their supply: code outside loops is fetched anew by every warp):
@@ -125,6 +125,7 @@ template <bool kClip, Owner kOwn>
 __device__ __forceinline__ void long_row_body(const LayerDesc &L, int m, const Group &G, unsigned char *slice, int qmax, unsigned mode,
                                               int n0 = 0, int nloc = 0)
 {
+    static_assert(kOwn == kCluster || (kOwn == kBlock && !kClip), "");
     const int g = G.g, N = kOwn == kCluster ? nloc : L.N;   // elements here
     constexpr int stride = 32;   // a warp has a contiguous run of vectors
     const Sel S(slice, g, kOwn, 1);
@@ -137,7 +138,7 @@ __device__ __forceinline__ void long_row_body(const LayerDesc &L, int m, const G
     const float *wrow = L.w + first;
     // The row is cut into vectors at 16-byte boundaries of the weights (packed codes pair elements from
     // the row's start, so there the vectors start with the row).
-    const bool pack = (mode & kModePackInt4) != 0;
+    const bool pack = kOwn == kCluster && (mode & kModePackInt4) != 0;   // (packed codes of kBlock: row_body)
     int r = 0, q_lo = 0, q_hi = N >> 2, rag = -1;
     bool ragged = false;
     const bool regular = L.off_ev != 0;
@@ -446,7 +447,7 @@ __device__ __forceinline__ void long_row_body(const LayerDesc &L, int m, const G
             const int seen = sgn > 0 ? above : below;
             const float goal = __fadd_rn(__fmul_rn(static_cast<float>(kc), 1.3f), 10.0f);
             const int start = top - 1 - __float2int_rn(__fmul_rn(goal, __fdividef(static_cast<float>(near_of(again(L.N))), static_cast<float>(max(seen, 1)))));
-            const int k_eff = select_top<kOwn, false>(G, prepare, count, listing, settle, tally, each, code_of, flip, nmax, kOwn != kCluster || seen >= 24, start, top, kHalf + (1 << 14) + 1, 2.0f, kc, L.N, want, S, 1);
+            const int k_eff = select_top<kOwn>(G, prepare, count, listing, settle, tally, each, code_of, flip, nmax, kOwn != kCluster || seen >= 24, start, top, kHalf + (1 << 14) + 1, 2.0f, kc, L.N, want, S, 1);
             ec -= static_cast<long long>(sgn) * k_eff * kOne;
         }
     }
@@ -500,9 +501,8 @@ squant_row_kernel(const __grid_constant__ LaunchTable tbl, int qmax, unsigned mo
     G.bar = 0;
     const int m = item - tbl.first_item[layer];
     if (kLong) {
-        SQ_DBG(long_row_bytes(kThreads, L.off_vi, (mode & kModePackInt4) != 0, kBlock) <= static_cast<int>(dynamic_smem_bytes()), 10);
-        if (L.sin) long_row_body<true, kBlock>(L, m, G, smem, qmax, mode);
-        else long_row_body<false, kBlock>(L, m, G, smem, qmax, mode);
+        SQ_DBG(long_row_bytes(kThreads, L.off_vi, false, kBlock) <= static_cast<int>(dynamic_smem_bytes()) && !L.sin && !(mode & kModePackInt4), 10);
+        long_row_body<false, kBlock>(L, m, G, smem, qmax, mode);
     } else {
         SQ_DBG(row_bytes(kThreads, L.off_vi, kBlock) <= static_cast<int>(dynamic_smem_bytes()), 10);
         if (L.sin) row_body<true, kBlock, 32>(L, m, G, smem, qmax, mode, true);
