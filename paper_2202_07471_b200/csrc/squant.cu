@@ -479,7 +479,9 @@ int build_param_plan(const squant_layer *layers, int32_t n_layers, const squant_
     //     - / 31.2 / 36.9).
     //   - All others row_body with 512 threads.
     const auto blocks = [&](int bytes) { return kSmSmem / (bytes + kBlockSmemReserved); };   // on a multiprocessor
-    const auto small_blocks = [&](int i) { return std::min(4, blocks(sq::row_bytes(256, (descs[i].N + 6) >> 2, sq::kBlock))); };
+    const auto small_blocks = [&](int i) {   // of 256 threads, none if the row is too long for them
+        return descs[i].N > 4 * 2 * sq::kRowVecs * 256 ? 0 : std::min(4, blocks(sq::row_bytes(256, (descs[i].N + 6) >> 2, sq::kBlock)));
+    };
     const auto only_long = [&](int i) {
         const int vecs = (descs[i].N + 6) >> 2;
         return !pack && !descs[i].sin && blocks(sq::row_bytes(512, vecs, sq::kBlock)) < 2 && blocks(sq::long_row_bytes(512, vecs, false, sq::kBlock)) >= 2;

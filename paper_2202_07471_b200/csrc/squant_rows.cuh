@@ -30,7 +30,7 @@ namespace sq {
 
 namespace cg = cooperative_groups;
 
-constexpr int kRowVecs = 8;                       // vectors of four weights a thread of a group takes
+constexpr int kRowVecs = 8;                       // vectors of four weights a thread of a group takes; of a thread block that has a row for itself up to twice as many
 
 // Threads per channel for rows of `vecs` vectors (8, 16, .. 256), 0: too long for a group.
 __host__ __device__ inline int row_group(int vecs)
@@ -362,8 +362,8 @@ __device__ __forceinline__ bool guess_fits(int kc, int cap) { return kOwn == kCl
 // push(a, n, code) for those of the thread's elements that are at least t units, 1 <= t < top (`top` is one unit above
 // the largest possible); code is handed through to flip.  direct: from `start` on somewhat more than kc candidates are expected,
 // which are listed without a search.  If there is no such list or it will not do, the bound is searched: the threads know maxima of a
-// over parts of their elements, count(t) = how many of the group's nmax maxima are at least t (direct: prepare() once before, it may
-// write to shared memory).  For
+// over parts of their elements, count(t) = how many of the group's nmax maxima are at least t (prepare() once before, after a list that
+// will not do: it may write to shared memory.  Without `direct` it is not called, count must do without).  For
 // the exact search: settle() once, then tally(v) = how many of the thread's elements have a >= v (any v >= 1, vtop above all),
 // each(v, f) calls f(a, n) for those, code_of(n) is the code of one.  spread: the expected distance between the largest candidates in units
 // of top / n_all.  flip(a, n, code) is called once for each of the min(kc, candidates) largest (equal values: lower
@@ -946,7 +946,9 @@ __device__ __forceinline__ void row_body(const LayerDesc &L, int m, const Group 
         if (g <= 32 ? __any_sync(kFull, want) : want) {
             const int m0 = sgn > 0 ? R.hi[0] : -R.lo[0], m1 = sgn > 0 ? R.hi[1] : -R.lo[1];
             const int sx = sgn > 0 ? 0 : -1;   // p ^ sx = the value in the direction of the flips, less one if that is downward
-            // the elements of value t and more, in the vectors of `halves` (bit 0: the even ones, bit 1: the odd ones)
+            // the elements of value t and more, in the vectors of `halves` (bit 0: the even ones, bit 1: the odd ones), of which a word
+            // of hits holds at most eight
+            SQ_DBG(vecs <= 2 * kRowVecs, 27);
             auto visit = [&](int t, unsigned halves, auto fn) {
                 const int tx = t + sx;
 #pragma unroll 1
@@ -1017,7 +1019,7 @@ __device__ __forceinline__ void row_body(const LayerDesc &L, int m, const Group 
                 if (kerr) kerr[n] = __fmul_rn(__int2float_rn(sgn > 0 ? a - kOne : kOne - a), 0x1p-30f);
             };
             const int vtop = kHalf + (1 << 14) + 1;
-            const bool direct = L.N >= kRowDirect && (g > 32 || __any_sync(kFull, want && guess_fits<kOwn>(kc, S.cap)));   // (of a clipped row kc can be huge)
+            const bool direct = g > 32 || (L.N >= kRowDirect && __any_sync(kFull, want && guess_fits<kOwn>(kc, S.cap)));   // (of a clipped row kc can be huge)
             const int k_eff = select_top<kOwn>(G, prepare, count, listing, [] {}, tally, each, [](int) { return 0u; }, flip, kOwn == kBlock ? g : per * g, direct,
                                                list_start(kc, 2.0f, vtop, max(N, 1)), vtop, vtop, 2.0f, kc, N, want, S, 1);
             ec -= static_cast<long long>(sgn) * k_eff * kOne;

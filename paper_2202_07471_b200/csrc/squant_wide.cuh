@@ -24,6 +24,7 @@ constexpr int kWideMaxCluster = 8;
 // body of the grouped kernel.  Longer rows that fit one thread block still take that body, which is the slower one
 // there: 1024 rows of 32,772 weights 318 us against 99 in this kernel, of 40,000 480 against 116, 16 rows of 40,000 83 against 22.
 constexpr int kRowBlockElems = 32768;
+static_assert(kRowBlockElems <= 4 * 2 * kRowVecs * kBlockThreads, "");
 
 // ---------------------------------------------------------------- SQuant-E on four weights of a 1x1 row
 struct Quad {
@@ -447,7 +448,10 @@ __device__ __forceinline__ void long_row_body(const LayerDesc &L, int m, const G
             const int seen = sgn > 0 ? above : below;
             const float goal = __fadd_rn(__fmul_rn(static_cast<float>(kc), 1.3f), 10.0f);
             const int start = top - 1 - __float2int_rn(__fmul_rn(goal, __fdividef(static_cast<float>(near_of(again(L.N))), static_cast<float>(max(seen, 1)))));
-            const int k_eff = select_top<kOwn>(G, prepare, count, listing, settle, tally, each, code_of, flip, nmax, kOwn != kCluster || seen >= 24, start, top, kHalf + (1 << 14) + 1, 2.0f, kc, L.N, want, S, 1);
+            // (A thread block lists from the guess however few it has seen: a search and its list cost more.  1000 rows of 25,001
+            // weights at two bits with outliers 58.4 us on a B200, with the search first 64.6, without outliers 59.2 and 64.2.)
+            const bool direct = kOwn != kCluster || seen >= 24;
+            const int k_eff = select_top<kOwn>(G, prepare, count, listing, settle, tally, each, code_of, flip, nmax, direct, start, top, kHalf + (1 << 14) + 1, 2.0f, kc, L.N, want, S, 1);
             ec -= static_cast<long long>(sgn) * k_eff * kOne;
         }
     }
