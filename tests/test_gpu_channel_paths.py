@@ -448,29 +448,43 @@ def test_long_and_wide_rows_without_sums(n):
     check(ws, 4, clip=0.7, sums=False)
 
 
-@pytest.mark.parametrize("n,waves", [(8200, 6), (8193, 8), (10001, 8), (12290, 6), (13100, 6), (13500, 12), (16384, 12), (16387, 1), (22001, 1), (26500, 1)])
-def test_forms_of_long_rows(n, waves):
-    """Rows of the row kernel on either side of the numbers, in rows a multiprocessor, from which they take another form:
-    every output form in each, and a call of all forms."""
+@pytest.mark.parametrize("n,form", [(8193, "256"), (10985, "256"), (10986, "256"), (13500, "256"), (14877, "256"), (14878, "512"), (16387, "512"), (22313, "512"),
+                                    (22314, "long"), (25001, "long"), (26869, "long"), (26870, "512")])
+def test_forms_of_long_rows(n, form):
+    """Rows of the row kernel on either side of the lengths (four and three thread blocks of 256 threads on a multiprocessor;
+    two of 512 only in long_row_body) and of the numbers of rows (two and a quarter a multiprocessor; one) from which they take
+    another form, every output form in each.  The form shows in the number of launches of a call that has another
+    layer in row_body with 512 threads."""
     sms = torch.cuda.get_device_properties(0).multi_processor_count
-    w = adversarial_layer((waves * sms + 1, n, 1, 1), seed=n)
-    check([w], 4)
-    check([w[1:]], 4)
-    check([w], 4, sums=False, start=1)
-    check([w], 4, flags=sq.FLAG_NARROW_RANGE | sq.FLAG_PACK_INT4, start=2)
-    if n in (8193, 16384, 22001):
-        check([w], 8, flags=0, outputs=True, start=3)
-        check([w], 4, clip=0.8)
-        check([w], 3, mode=sq.MODE_E | sq.MODE_C)
+    few = 9 * sms // 4 if n < 20000 else sms
+    w, other = adversarial_layer((few + 1, n, 1, 1), seed=n), adversarial_layer((1, 14900, 1, 1), seed=1)
+
+    def launches(w, *args, **kw):
+        n0 = sq.squant_launch_count()
+        check([w, other], *args, **kw)
+        return sq.squant_launch_count() - n0
+
+    apart, small = (1 if form == "512" else 2), (2 if form == "256" else 1)   # long_row_body: neither packed codes nor supplied scales
+    assert launches(w, 4) == apart
+    assert launches(w[1:], 4) == 1
+    assert launches(w, 4, sums=False, start=1) == apart
+    assert launches(w, 4, flags=sq.FLAG_NARROW_RANGE | sq.FLAG_PACK_INT4, start=2) == small
+    if n not in (10985, 10986, 22313, 26870):
+        assert launches(w, 8, flags=0, outputs=True, start=3) == apart
+        if n < 15000:   # (longer rows with supplied scales go to the cluster kernel)
+            assert launches(w, 4, clip=0.8) == small
+        assert launches(w, 3, mode=sq.MODE_E | sq.MODE_C) == apart
+        assert launches(w, 4, mode=sq.MODE_E, outputs=True) == apart
 
 
 def test_call_with_every_form_of_long_rows():
     sms = torch.cuda.get_device_properties(0).multi_processor_count
-    shapes = [(12 * sms + 1, 13500, 1, 1), (6 * sms, 8201, 1, 1), (5, 12000, 1, 1), (sms, 22100, 1, 1), (7, 32768, 1, 1), (11, 17000, 1, 1), (3, 50000, 1, 1), (40, 64, 3, 3)]
+    shapes = [(sms, 14877, 1, 1), (9 * sms // 4, 8201, 1, 1), (5, 12000, 1, 1), (sms + 1, 25001, 1, 1), (7, 32768, 1, 1), (11, 17000, 1, 1), (3, 50000, 1, 1), (40, 64, 3, 3)]
     ws = [adversarial_layer(s, seed=s[1]) for s in shapes]
     n0 = sq.squant_launch_count()
     check(ws, 4, start=1)
-    assert sq.squant_launch_count() - n0 == 3 + 1 + 1   # the forms, the wide layer, the grouped launch
+    # 256 threads of which three and of which four thread blocks fit a multiprocessor, both forms with 512; the wide layer, the grouped launch
+    assert sq.squant_launch_count() - n0 == 4 + 1 + 1
 
 
 @pytest.mark.parametrize("n", [46501, 48000, 50999])

@@ -642,10 +642,13 @@ def test_checked_build_finds_no_violation_on_small_cases():
     if not os.path.exists(lib_build.LIB_DEBUG):
         pytest.skip("libsquant_debug.so has not been built")
     ws = [adversarial_layer(s, seed=9 + i) for i, s in enumerate(SWEEP_SHAPES)] + [redo_layer(64, 4, seed=4), redo_layer(2048, 4)]
+    # long rows in each form of the row kernel: enough of them for 256 threads (four thread blocks on a multiprocessor, and three) and for long_row_body, few
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    ws += [adversarial_layer(s, seed=s[1]) for s in ((2 * sms, 8201, 1, 1), (sms, 14877, 1, 1), (sms + 1, 22401, 1, 1), (3, 16387, 1, 1))]
     # long 3x3 channels (streaming kernel): special channels, heavy ties (digit-by-digit selection), a partial last warp
     ws += [adversarial_layer((150, 1200, 3, 3), seed=77), adversarial_layer((15, 1000, 3, 3), seed=79), coarse(W.random_layer((5, 2048, 3, 3), seed=78), steps=24, div=4)]
     ref = run_gpu(ws, 4, EKC)
-    assert_kernels(ref[-3:], ["stream", "grouped", "stream"])
+    assert_kernels(ref[-7:], 4 * ["row"] + ["stream", "grouped", "stream"])
     sq.use_library(lib_build.LIB_DEBUG)
     try:
         checked, n, site = sq.squant_debug_violations()
