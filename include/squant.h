@@ -144,7 +144,9 @@ int squant_quantize_layer(const squant_layer *layer, const squant_options *opt, 
  * outputs anyway); calls with different descriptors may.
  * The launches of one call work on different layers and may overlap on the GPU (except those that a graph captures):
  * no layer may read or write what another layer of the same call writes.  They start when all earlier
- * work of the stream has ended, and whatever follows the call in the stream starts when all of them have ended.
+ * work of the stream has ended, and whatever follows the call in the stream starts when all of them have ended - but a
+ * kernel that the caller launches behind a call with programmatic stream serialization may start as soon as the last launch has
+ * started, and must wait (cudaGridDependencySynchronize) before it touches what the call reads or writes.
  * All arguments are validated
  * on the host first; a failed call launches nothing and writes nothing.  Returns SQUANT_OK or a
  * negative SQUANT_ERR_* code.

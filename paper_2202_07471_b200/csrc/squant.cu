@@ -711,8 +711,8 @@ int launch_plan(const ParamPlan &p, cudaStream_t stream)
         SQ_CUDA(cudaStreamIsCapturing(stream, &cap));
         overlap = cap == cudaStreamCaptureStatusNone;
     }
-    const auto early = [&](size_t i) { return overlap && i >= plain && i < launches; };
-    const auto mode = [&] { return p.mode | (early(j) ? sq::kModeMayStartEarly : 0u) | (early(j + 1) ? sq::kModeNextMayStart : 0u); };
+    const auto early = [&](size_t i) { return overlap && i >= plain; };
+    const auto mode = [&] { return p.mode | (early(j) ? sq::kModeMayStartEarly : 0u); };
     // long 3x3 channels first: one persistent CTA per multiprocessor
     for (ParamPlan::Stream &st : p.streams) {
         int device = 0;
@@ -736,9 +736,9 @@ int launch_plan(const ParamPlan &p, cudaStream_t stream)
         if (scratch) {
             const int grid = std::min(st.items, sms), smem = sq::stream_layout(st.nk_max, st.n_max).total;
             auto kernel = st.out ? sq::squant_stream_kernel<true> : sq::squant_stream_kernel<false>;
-            kernel<<<grid, sq::kStreamThreads, smem, stream>>>(st.table, p.qmax, mode(), st.items, st.nk_max, st.n_max, scratch->mem, scratch->work());
+            kernel<<<grid, sq::kStreamThreads, smem, stream>>>(st.table, p.qmax, p.mode, st.items, st.nk_max, st.n_max, scratch->mem, scratch->work());
         } else {
-            sq::squant_model_kernel<sq::kAbsmax><<<st.grouped_grid, sq::kCtaThreads, st.grouped_smem, stream>>>(st.grouped, p.qmax, mode());
+            sq::squant_model_kernel<sq::kAbsmax><<<st.grouped_grid, sq::kCtaThreads, st.grouped_smem, stream>>>(st.grouped, p.qmax, p.mode);
         }
         SQ_CUDA(cudaGetLastError());
         g_launches.fetch_add(1, std::memory_order_relaxed);
@@ -773,7 +773,7 @@ int launch_plan(const ParamPlan &p, cudaStream_t stream)
     for (const ParamPlan::Grouped &gl : p.grouped) {
         auto kernel = gl.scales == sq::kAbsmax ? sq::squant_model_kernel<sq::kAbsmax>
                       : gl.scales == sq::kOwnScales ? sq::squant_model_kernel<sq::kOwnScales> : sq::squant_model_kernel<sq::kEither>;
-        const int rc = launch(kernel, gl.grid, sq::kCtaThreads, gl.smem, 1, gl.table, p.qmax, mode());
+        const int rc = launch(kernel, gl.grid, sq::kCtaThreads, gl.smem, 1, gl.table, p.qmax, p.mode);
         if (rc) return rc;
     }
     for (const ParamPlan::Rows &r : p.rows) {

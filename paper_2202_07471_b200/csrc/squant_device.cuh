@@ -175,15 +175,14 @@ __device__ __forceinline__ void bulk_store_wait()
 
 // ---------------------------------------------------------------- overlap of a call's launches
 // The launches of a call work on different layers, so those of the row and cluster kernels may start while the one
-// before still runs: their thread blocks take the places that the last ones of that leave free.  A launch that another
-// of the call may follow early (kModeNextMayStart) says so at its start, as soon as all of its own thread blocks have
-// started.  One that may come early (kModeMayStartEarly) ends no earlier than the one before (its last thread block
-// waits for that), so whatever follows the call's last launch follows all of them; the last launch says nothing.
-constexpr unsigned kModeNextMayStart = 0x400u, kModeMayStartEarly = 0x800u;   // bits of `mode`
-__device__ __forceinline__ void next_launch_may_start(unsigned mode)
-{
-    if (mode & kModeNextMayStart) asm volatile("griddepcontrol.launch_dependents;");
-}
+// before still runs: their thread blocks take the places that the last ones of that leave free.  Every kernel says at
+// its start that the next may come, as soon as all of its own thread blocks have started; whatever is launched in the
+// ordinary way waits for its end all the same, and starts the sooner after it (256x256x3x3 7.6 us a call on a B200,
+// 8.1 if only launches say so that another of their call may follow early; MobileNetV2 shapes 15.6 and 15.9).  A launch that may come early
+// (kModeMayStartEarly) ends no earlier than the one before (its last thread block waits for that), so whatever
+// follows the call's last launch follows all of them.
+constexpr unsigned kModeMayStartEarly = 0x400u;   // a bit of `mode`
+__device__ __forceinline__ void next_launch_may_start() { asm volatile("griddepcontrol.launch_dependents;"); }
 __device__ __forceinline__ void end_after_launch_before(unsigned mode)
 {
     if ((mode & kModeMayStartEarly) && blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -1424,7 +1423,7 @@ __global__ void __launch_bounds__(kCtaThreads, SQ_MIN_CTAS)
 squant_model_kernel(const __grid_constant__ LaunchTable tbl, int qmax, unsigned mode)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    next_launch_may_start(mode);
+    next_launch_may_start();
     const int item = blockIdx.x;
     int layer = 0;   // uniform binary search for the last layer whose first item is <= item
 #pragma unroll 1

@@ -416,7 +416,7 @@ squant_stream_kernel(const __grid_constant__ LaunchTable tbl, int qmax, unsigned
                      unsigned char *held_scratch, unsigned *work)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    next_launch_may_start(mode);
+    next_launch_may_start();
     const StreamLayout lay = stream_layout(nk_max, n_max);
     StreamCtrl *ctrl = reinterpret_cast<StreamCtrl *>(smem + lay.off_ctrl);
     const int tid = threadIdx.x;

@@ -491,7 +491,7 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads)
 squant_row_kernel(const __grid_constant__ LaunchTable tbl, int qmax, unsigned mode)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    next_launch_may_start(mode);
+    next_launch_may_start();
     const int item = blockIdx.x;
     int layer = 0;
 #pragma unroll 1
@@ -531,7 +531,7 @@ __global__ void __launch_bounds__(kBlockThreads, 2)
 squant_wide_kernel(const LayerDesc L, int qmax, unsigned mode, int kpc)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    next_launch_may_start(mode);
+    next_launch_may_start();
     cg::cluster_group cluster = cg::this_cluster();
     const int C = static_cast<int>(cluster.num_blocks()), rank = static_cast<int>(cluster.block_rank());
     const int m = static_cast<int>(blockIdx.x) / C;
