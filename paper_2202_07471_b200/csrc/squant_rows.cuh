@@ -595,18 +595,25 @@ __device__ __forceinline__ void row_clip_one(float Pf, int &P, unsigned c, int q
 }
 
 // ---------------------------------------------------------------- one 1x1 channel
-// Where a list for SQuant-C starts: from there on kc + kc / 4 + 6 of n_all values that are spread evenly from -top / 2 * spread
-// to top / 2 * spread are expected (2 to 3 % of such lists are too short).
-__device__ __forceinline__ int list_start(int kc, float spread, int top, int n_all)
+// Where a list for SQuant-C starts: from there on kc + kc / 4 + `more` of n_all values that are spread evenly from
+// -top / 2 * spread to top / 2 * spread are expected.
+__device__ __forceinline__ int list_start(int kc, float spread, int top, int n_all, float more)
 {
-    const float goal = static_cast<float>(kc) + static_cast<float>(kc >> 2) + 6.0f;
+    const float goal = static_cast<float>(kc) + static_cast<float>(kc >> 2) + more;
     return top - 1 - __float2int_rz(__fmul_rn(__fmul_rn(goal, spread), __fdividef(static_cast<float>(top), static_cast<float>(n_all))));
 }
 
-// Weights: SQuant-C of shorter rows (which groups of at most a warp take) searches its bound first, since the guess takes in too many of their elements (the guess /
-// the search first, us on a B200: 131,072 rows of 64 49.2 / 45.0, 65,536 of 96 31.9 / 30.0, of 128 33.0 / 32.4, of 160 37.1 / 36.9, of 192 39.1 / 41.1,
-// 32,768 of 256 29.7 / 34.4).
+// Weights: SQuant-C of shorter rows (which groups of at most a warp take) searches its bound first, since the guess takes
+// in too many of their elements (the guess / the search first, us on a B200: 131,072 rows of 64 49.2 / 45.0, 65,536 of 96
+// 31.9 / 30.0, of 128 33.0 / 32.4, of 160 37.1 / 36.9, of 192 39.1 / 41.1, 32,768 of 256 29.7 / 34.4).
 constexpr int kRowDirect = 176;
+// Where a thread has at most two vectors (launches that do not fill the GPU, whose rows have several times the threads), the
+// launch takes the time of its slowest row.  One list in 300 was too short with 6 more than kc * 5 / 4, which cost that
+// row a search and a second list; with 10 it is one in 3000.  Groups of up to a warp search first: of so few
+// elements to a maximum the search takes hardly too many.  us on a B200, before / with 10 / and that: 300 rows of 700
+// 7.5 / 6.2 / 6.2, 1000 of 512 8.2 / 6.7 / 6.7, 2000 of 256 8.2 / 8.2 / 7.2.  With more vectors a thread the longer
+// list costs more than it saves (16,384 rows of 512 23.4 / 25.6, ResNet-18 shapes 29.1 / 31.8).
+constexpr int kRowFew = 2 * 4;   // elements
 
 // What a thread knows of the perturbations it has made: their sum modulo 2^32 and as floats, the extremes over
 // every other vector.
@@ -1019,9 +1026,10 @@ __device__ __forceinline__ void row_body(const LayerDesc &L, int m, const Group 
                 if (kerr) kerr[n] = __fmul_rn(__int2float_rn(sgn > 0 ? a - kOne : kOne - a), 0x1p-30f);
             };
             const int vtop = kHalf + (1 << 14) + 1;
-            const bool direct = g > 32 || (L.N >= kRowDirect && __any_sync(kFull, want && guess_fits<kOwn>(kc, S.cap)));   // (of a clipped row kc can be huge)
+            const bool few = L.N <= kRowFew * g;
+            const bool direct = g > 32 || (!few && L.N >= kRowDirect && __any_sync(kFull, want && guess_fits<kOwn>(kc, S.cap)));   // (of a clipped row kc can be huge)
             const int k_eff = select_top<kOwn>(G, prepare, count, listing, [] {}, tally, each, [](int) { return 0u; }, flip, kOwn == kBlock ? g : per * g, direct,
-                                               list_start(kc, 2.0f, vtop, max(N, 1)), vtop, vtop, 2.0f, kc, N, want, S, 1);
+                                               list_start(kc, 2.0f, vtop, max(N, 1), few ? 10.0f : 6.0f), vtop, vtop, 2.0f, kc, N, want, S, 1);
             ec -= static_cast<long long>(sgn) * k_eff * kOne;
         }
     }
