@@ -467,17 +467,24 @@ int build_param_plan(const squant_layer *layers, int32_t n_layers, const squant_
     std::stable_sort(p.wide.begin(), p.wide.end(), [](const ParamPlan::Wide &a, const ParamPlan::Wide &b) {
         return (a.d.K > 1) != (b.d.K > 1) ? a.d.K > 1 : a.d.K == 1 && a.d.N > b.d.N;
     });
-    // Long rows, a thread block per output channel, in one of three forms.  row_body holds 5 B of shared memory a weight,
-    // long_row_body 4.  What counts is how many threads a multiprocessor holds and over how many
-    // vectors a thread spreads the code that runs once.  us a call on a B200, row_body with 256 / with 512 threads / long_row_body with 512:
-    //   - More than two and a quarter rows a multiprocessor, so short that three thread blocks of 256 threads fit one (14.8 K weights): those
-    //     (rows of 9000 300 12.5 / 12.3 / 14.4, 400 14.4 / 15.8 / 18.7, 4096 69.9 / 94.1 / 117; of 12,000 100 12.9 / 10.3 / 12.8, 500 19.5 / 20.5 /
-    //     25.0, 4096 89.6 / 105 / 128; 4096 of 14,100 106.7 / 124.1 / 142.3, of 15,001 135.3 / 127.7 / 153.8; 2000 of 9000 with packed codes
-    //     40.2 / 51.2 / 69.2; 1500 of 9000 with scales of their own 39.4 / 47.4 / 65.7).
-    //   - More rows than multiprocessors of which two thread blocks fit one only in long_row_body (22 to 27 K weights), neither packed codes nor
-    //     scales of their own: that (2000 rows of 25,001 - / 127.2 / 110.7, 300 - / 30.7 / 30.8, 1000 of 22,100 - / 49.6 / 57.1, 300 of 30,000
-    //     - / 31.2 / 36.9).
+    // Long rows, a thread block per output channel, in one of three forms.  row_body holds 5 B of shared memory a
+    // weight, long_row_body 4.  What counts is how many threads a multiprocessor holds and over how many vectors a
+    // thread spreads the code that runs once.
+    //   - More than two and a quarter rows a multiprocessor, so short that three thread blocks of 256 threads fit one
+    //     (14.8 K weights): row_body with 256 threads.
+    //   - More rows than multiprocessors of which two thread blocks fit one only in long_row_body (22 to 27 K
+    //     weights), neither packed codes nor scales of their own: long_row_body with 512 threads.
     //   - All others row_body with 512 threads.
+    // us a call on a B200, row_body with 256 threads / with 512 / long_row_body with 512:
+    //   rows of 9000       300 12.5 / 12.3 / 14.4, 400 14.4 / 15.8 / 18.7, 4096 69.9 / 94.1 / 117
+    //     packed codes     2000 40.2 / 51.2 / 69.2
+    //     their own scales 1500 39.4 / 47.4 / 65.7
+    //   of 12,000          100 12.9 / 10.3 / 12.8, 500 19.5 / 20.5 / 25.0, 4096 89.6 / 105 / 128
+    //   of 14,100          4096 106.7 / 124.1 / 142.3
+    //   of 15,001          4096 135.3 / 127.7 / 153.8
+    //   of 22,100          1000 - / 49.6 / 57.1
+    //   of 25,001          300 - / 30.7 / 30.8, 2000 - / 127.2 / 110.7
+    //   of 30,000          300 - / 31.2 / 36.9
     const auto blocks = [&](int bytes) { return kSmSmem / (bytes + kBlockSmemReserved); };   // on a multiprocessor
     const auto small_blocks = [&](int i) {   // of 256 threads, none if the row is too long for them
         return descs[i].N > 4 * 2 * sq::kRowVecs * 256 ? 0 : std::min(4, blocks(sq::row_bytes(256, (descs[i].N + 6) >> 2, sq::kBlock)));
@@ -701,8 +708,9 @@ int launch_plan(const ParamPlan &p, cudaStream_t stream)
 {
     const int freed = free_dead_scratch(stream);   // of graphs and of plans that have left the cache
     if (freed) return freed;
-    // The row and cluster kernels may start before the launch in front of them has ended (see next_launch_may_start).  Not the streaming
-    // kernels, which may share a scratch area, nor the grouped one (the wait at its end would cost it registers), nor what a graph captures.
+    // The row and cluster kernels may start before the launch in front of them has ended (see next_launch_may_start).
+    // Not the streaming kernels, which may share a scratch area, nor the grouped one (the wait at its end would cost
+    // it registers), nor what a graph captures.
     const size_t plain = std::max<size_t>(p.streams.size() + p.grouped.size(), 1), launches = p.streams.size() + p.grouped.size() + p.rows.size() + p.wide.size();
     size_t j = 0;   // of this call's launches
     bool overlap = false;

@@ -124,10 +124,11 @@ __device__ __noinline__ KernelOut64 kernel_clip_out(float *wk, int K, float s, b
     return o;
 }
 
-// A 3x3 kernel under the clip that the straight-line selection does not settle, from its weights, scale in the range of the
-// reciprocal sequence (y, s2: as in squant_e_fast).  Most have elements that lie two codes and more beyond the range, and every
-// candidate is flipped.  Out of line.  (Four 512x512x3x3 layers with scales of 0.7 absmax: 59.5 us on a B200 with every kernel that has codes on the edge of
-// the range settled by kernel_clip, 41.1 with all but these in line.)
+// A 3x3 kernel under the clip that the straight-line selection does not settle, from its weights, scale in the range
+// of the reciprocal sequence (y, s2: as in squant_e_fast).  Most have elements that lie two codes and more beyond the
+// range, and every candidate is flipped.  Out of line.  (Four 512x512x3x3 layers with scales of 0.7 absmax: 59.5 us
+// on a B200 with every kernel that has codes on the edge of the range settled by kernel_clip, 41.1 with all but these
+// in line.)
 __device__ __noinline__ KernelOut64 kernel9_beyond(float *wk, float y, float s2, int qmin, int qmax, unsigned char *ck)
 {
     const float xmin = static_cast<float>(qmin) * 1073741824.0f, xmax = static_cast<float>(qmax) * 1073741824.0f;

@@ -1416,8 +1416,9 @@ __device__ __forceinline__ void run_item(const LayerDesc &L, int ch0, unsigned c
     }
 }
 
-// (Without the bodies for scales of the layers' own the others keep their values in registers.  A spilled one comes back from L2, the L1 being shared memory: with 968 B of spill loads in a kernel for both four
-// 512x512x3x3 layers took 28.6 us on a B200, with 396 B 24.8.)
+// (Without the bodies for scales of the layers' own the others keep their values in registers.  A spilled one comes
+// back from L2, the L1 being shared memory: with 968 B of spill loads in a kernel for both four 512x512x3x3 layers
+// took 28.6 us on a B200, with 396 B 24.8.)
 template <Scales kScales>
 __global__ void __launch_bounds__(kCtaThreads, SQ_MIN_CTAS)
 squant_model_kernel(const __grid_constant__ LaunchTable tbl, int qmax, unsigned mode)

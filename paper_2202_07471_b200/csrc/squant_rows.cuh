@@ -1,25 +1,23 @@
-// 1x1 layers (fully connected and pointwise): a group of 8 to 256 threads takes a whole output
-// channel, up to 32 weights a thread, or a thread block of 256 or 512 threads a longer one.
+// 1x1 layers (fully connected and pointwise): a group of 8 to 256 threads takes a whole output channel, up to 32
+// weights a thread, or a thread block of 256 or 512 threads a longer one.
 //
-// Every element is its own kernel, so SQuant-K is a no-op (Sec. 3.4) and the work is absmax,
-// SQuant-E, the channel sum and SQuant-C's choice of the k_c largest perturbations of one sign.
-// What bounds such a channel is not bandwidth but instructions and the chain of its steps: by way
-// of staged weights, a histogram in shared atomics and a 256-bin scan per channel, a ResNet-50
-// spent 70 thread-instructions per weight, most of them fixed costs of short channels.  Here
-//   - the weights are requested all at once and put into shared memory, each thread's for itself (no
-//     barrier); the perturbations take their place, where a thread looks again only if its largest one
-//     comes into question;
+// Every element is its own kernel, so SQuant-K is a no-op (Sec. 3.4) and the work is absmax, SQuant-E, the channel
+// sum and SQuant-C's choice of the k_c largest perturbations of one sign. What bounds such a channel is not bandwidth
+// but instructions and the chain of its steps: by way of staged weights, a histogram in shared atomics and a 256-bin
+// scan per channel, a ResNet-50 spent 70 thread-instructions per weight, most of them fixed costs of short channels.
+// Here
+//   - the weights are requested all at once and put into shared memory, each thread's for itself (no barrier); the
+//     perturbations take their place, where a thread looks again only if its largest one comes into question;
 //   - short channels share a warp (8 or 16 threads each), so the fixed costs are shared too;
-//   - SQuant-C needs no histogram.  Each thread knows its largest candidates; a value T0 that at
-//     least k_c of those maxima reach is a lower bound of the k_c-th largest candidate whatever the
-//     distribution, and few other elements reach it (with k_c of m maxima about m ln(m / (m - k_c))
-//     elements).  T0 is searched among the maxima, the elements from T0 on are listed, and those of
-//     the first k_c ranks are flipped.  What that cannot settle (k_c beyond the number of maxima, a
-//     full list) goes to an exact search by counting.
-// With squant_conv.cuh: ResNet-50 shapes 84.5 -> 65.6 us device time on a B200.  With loops of constant strides over a thread's vectors (a
-// warp of a longer row has a contiguous run of them), 22 instead of 30 thread-instructions a weight for SQuant-E in rows of 4096, and a list
-// that is made at a guessed bound before any search: 2 x 4096 rows of 4096 weights at 8 bit 65.5 -> 53.0 us a call, 16,384 of 512 29.2 -> 23.8,
-// 32,768 of 256 35.9 -> 28.9.
+//   - SQuant-C needs no histogram.  Each thread knows its largest candidates; a value T0 that at least k_c of those
+//     maxima reach is a lower bound of the k_c-th largest candidate whatever the distribution, and few other elements
+//     reach it (with k_c of m maxima about m ln(m / (m - k_c)) elements).  T0 is searched among the maxima, the
+//     elements from T0 on are listed, and those of the first k_c ranks are flipped.  What that cannot settle (k_c
+//     beyond the number of maxima, a full list) goes to an exact search by counting.
+// With squant_conv.cuh: ResNet-50 shapes 84.5 -> 65.6 us device time on a B200.  With loops of constant strides over
+// a thread's vectors (a warp of a longer row has a contiguous run of them), 22 instead of 30 thread-instructions a
+// weight for SQuant-E in rows of 4096, and a list that is made at a guessed bound before any search: 2 x 4096 rows of
+// 4096 weights at 8 bit 65.4 -> 55.4 us a call, 16,384 of 512 29.2 -> 23.4, 32,768 of 256 35.9 -> 26.8.
 #pragma once
 
 #include <cooperative_groups.h>
@@ -30,7 +28,7 @@ namespace sq {
 
 namespace cg = cooperative_groups;
 
-constexpr int kRowVecs = 8;                       // vectors of four weights a thread of a group takes; of a thread block that has a row for itself up to twice as many
+constexpr int kRowVecs = 8;   // vectors of four weights a thread of a group takes; twice as many where a thread block has a row for itself
 
 // Threads per channel for rows of `vecs` vectors (8, 16, .. 256), 0: too long for a group.
 __host__ __device__ inline int row_group(int vecs)
@@ -49,7 +47,8 @@ struct SelScratch {
     int pad;
 };
 
-// What a warp (of a cluster: a thread block) contributes: absmax (bit pattern of a non-negative float) first, then error sum and extremes of the candidates.
+// What a warp (of a cluster: a thread block) contributes: absmax (bit pattern of a non-negative float) first, then
+// error sum and extremes of the candidates.
 constexpr int kMaxWarps = 16;   // of a channel in one thread block
 struct WarpPart {
     int lo32, hi32;   // the error sum: modulo 2^32 and, in units of 2^17, its size; or both halves of 64 bits
@@ -70,13 +69,14 @@ __host__ __device__ constexpr int sel_warps(int g, Owner own, int K) { return g 
 // Kernels of more than nine elements: a thread's maximum is put in when the direction of the flips is known, one word
 // instead of two and a barrier more, which the few kernels of such a channel hardly notice.
 __host__ __device__ constexpr bool late_maxima(int K) { return K > 9; }
-// Entries of a list.  Groups of eight threads: 40, with which four thread blocks with 32 rows of 256 weights each share a multiprocessor
-// (with 64 three: ResNet-50 shapes 62.3 us on a B200, 57.4 with 40; mixed kernel sizes 47.1, 41.9; 65,536 rows of 192 weights alone
-// 38.3, 41.1, a matter of their last wave).  Groups of 64, 128 and 256 threads on larger kernels: as many as make the group's selection memory
-// 1,056, 2,144 and 3,104 B, with late maxima 1,056, 1,568 and 3,120 B.  The last figure is part of the longest
-// channel of few kernels that a thread block takes; the others decide how many channels share one (512 channels of 106
-// 7x7 kernels, four layers: two channels to a thread block 49.6 us on a B200, one 70.9).  The weights follow, so a multiple of 32 B: rows of
-// whole 32-byte sectors copied to an odd multiple of 16 cost 2000 rows of 21,000 weights 98.0 us instead of 91.8.
+// Entries of a list.  Groups of eight threads: 40, with which four thread blocks with 32 rows of 256 weights each
+// share a multiprocessor (with 64 three: ResNet-50 shapes 62.3 us on a B200, 57.4 with 40; mixed kernel sizes 47.1,
+// 41.9; 65,536 rows of 192 weights alone 38.3, 41.1, a matter of their last wave).  Groups of 64, 128 and 256 threads
+// on larger kernels: as many as make the group's selection memory 1,056, 2,144 and 3,104 B, with late maxima 1,056,
+// 1,568 and 3,120 B.  The last figure is part of the longest channel of few kernels that a thread block takes; the
+// others decide how many channels share one (512 channels of 106 7x7 kernels, four layers: two channels to a thread
+// block 49.6 us on a B200, one 70.9).  The weights follow, so a multiple of 32 B: rows of whole 32-byte sectors
+// copied to an odd multiple of 16 cost 2000 rows of 21,000 weights 98.0 us instead of 91.8.
 __host__ __device__ constexpr int sel_cap(int g, int K = 1)
 {
     return K == 1 ? (g == 8 ? 40 : g <= 64 ? 64 : (g > 256 ? 472 : g))   // (472: 4,128 B with the parts)
@@ -362,9 +362,9 @@ __device__ __forceinline__ bool guess_fits(int kc, int cap) { return kOwn == kCl
 // push(a, n, code) for those of the thread's elements that are at least t units, 1 <= t < top (`top` is one unit above
 // the largest possible); code is handed through to flip.  direct: from `start` on somewhat more than kc candidates are expected,
 // which are listed without a search.  If there is no such list or it will not do, the bound is searched: the threads know maxima of a
-// over parts of their elements, count(t) = how many of the group's nmax maxima are at least t (prepare() once before, after a list that
-// will not do: it may write to shared memory.  Without `direct` it is not called, count must do without).  For
-// the exact search: settle() once, then tally(v) = how many of the thread's elements have a >= v (any v >= 1, vtop above all),
+// over parts of their elements, count(t) = how many of the group's nmax maxima are at least t (prepare() once before,
+// after a list that will not do: it may write to shared memory.  Without `direct` it is not called, count must do
+// without).  For the exact search: settle() once, then tally(v) = how many of the thread's elements have a >= v (any v >= 1, vtop above all),
 // each(v, f) calls f(a, n) for those, code_of(n) is the code of one.  spread: the expected distance between the largest candidates in units
 // of top / n_all.  flip(a, n, code) is called once for each of the min(kc, candidates) largest (equal values: lower
 // index first), by some thread of the group.  want: this group selects at all (kc >= 1).  Returns the number of
@@ -1027,7 +1027,8 @@ __device__ __forceinline__ void row_body(const LayerDesc &L, int m, const Group 
             };
             const int vtop = kHalf + (1 << 14) + 1;
             const bool few = L.N <= kRowFew * g;
-            const bool direct = g > 32 || (!few && L.N >= kRowDirect && __any_sync(kFull, want && guess_fits<kOwn>(kc, S.cap)));   // (of a clipped row kc can be huge)
+            // (of a clipped row kc can be huge)
+            const bool direct = g > 32 || (!few && L.N >= kRowDirect && __any_sync(kFull, want && guess_fits<kOwn>(kc, S.cap)));
             const int k_eff = select_top<kOwn>(G, prepare, count, listing, [] {}, tally, each, [](int) { return 0u; }, flip, kOwn == kBlock ? g : per * g, direct,
                                                list_start(kc, 2.0f, vtop, max(N, 1), few ? 10.0f : 6.0f), vtop, vtop, 2.0f, kc, N, want, S, 1);
             ec -= static_cast<long long>(sgn) * k_eff * kOne;

@@ -1,15 +1,16 @@
-// Output channels that are too long for a group of the grouped kernel: 1x1 rows of more than 8 K weights
-// get a thread block of 256 or 512 threads each (by row_body, a few sizes by long_row_body here, see build_param_plan), and channels that do not fit one thread block's shared memory a
-// cluster of 2, 4 or 8 of them, each with a contiguous run of the channel's kernels.  What a channel needs
-// as a whole travels through distributed shared memory (plain loads from the other thread blocks' shared
-// memory; no multicast anywhere): absmax, error sum, the counts of SQuant-C's search and the short lists
-// of its candidates, which every thread block collects for itself, so that all of them take the same
-// decisions without a leader.
+// Output channels that are too long for a group of the grouped kernel: 1x1 rows of more than 8 K weights get a thread
+// block of 256 or 512 threads each (by row_body, a few sizes by long_row_body here, see build_param_plan), and
+// channels that do not fit one thread block's shared memory a cluster of 2, 4 or 8 of them, each with a contiguous
+// run of the channel's kernels.  What a channel needs as a whole travels through distributed shared memory (plain
+// loads from the other thread blocks' shared memory; no multicast anywhere): absmax, error sum, the counts of
+// SQuant-C's search and the short lists of its candidates, which every thread block collects for itself, so that all
+// of them take the same decisions without a leader.
 //
-// Channels this wide can hold 2^16 and more kernels, the size from which the one element that sits on
-// the edge of the clip range (|w/s| a shade above qmax) can make it into a top-k: an element whose flipped
-// code would leave the range is no candidate.  Rows look for it where it can matter, among candidates of at most
-// 2^16 units of 2^-30, which only the exact search takes (rows of the row kernel are shorter); larger kernels run the body that checks every candidate.
+// Channels this wide can hold 2^16 and more kernels, the size from which the one element that sits on the edge of the
+// clip range (|w/s| a shade above qmax) can make it into a top-k: an element whose flipped code would leave the range
+// is no candidate.  Rows look for it where it can matter, among candidates of at most 2^16 units of 2^-30, which only
+// the exact search takes (rows of the row kernel are shorter); larger kernels run the body that checks every
+// candidate.
 //
 // Two thread blocks per multiprocessor where the channel can be cut that small.
 #pragma once
@@ -20,9 +21,10 @@ namespace sq {
 
 static_assert(kBlockThreads == 1 << 9, "");
 constexpr int kWideMaxCluster = 8;
-// Longest row of the row kernel (168 KB of shared memory with packed codes or in row_body); up to here it was laid out and compared with the staged
-// body of the grouped kernel.  Longer rows that fit one thread block still take that body, which is the slower one
-// there: 1024 rows of 32,772 weights 318 us against 99 in this kernel, of 40,000 480 against 116, 16 rows of 40,000 83 against 22.
+// Longest row of the row kernel (168 KB of shared memory with packed codes or in row_body); up to here it was laid
+// out and compared with the staged body of the grouped kernel.  Longer rows that fit one thread block still take that
+// body, which is the slower one there: 1024 rows of 32,772 weights 318 us against 99 in this kernel, of 40,000 480
+// against 116, 16 rows of 40,000 83 against 22.
 constexpr int kRowBlockElems = 32768;
 static_assert(kRowBlockElems <= 4 * 2 * kRowVecs * kBlockThreads, "");
 
@@ -108,9 +110,10 @@ __device__ __forceinline__ unsigned row_extremes(const int4 p)
 }
 
 // ---------------------------------------------------------------- one 1x1 channel
-// Rows that a whole thread block (kBlock) or a cluster takes; kCluster: this thread block has the elements n0 ..
-// n0 + nloc - 1 (n0 a multiple of four).  kBlock: neither packed codes nor supplied scales.  kClip: the clip of Sec. 2.2 can fire (caller-supplied scales): codes are
-// clamped, sums are 64 bit and an element whose flipped code would leave the range is no candidate.
+// Rows that a whole thread block (kBlock) or a cluster takes; kCluster: this thread block has the elements n0 .. n0 +
+// nloc - 1 (n0 a multiple of four).  kBlock: neither packed codes nor supplied scales.  kClip: the clip of Sec. 2.2
+// can fire (caller-supplied scales): codes are clamped, sums are 64 bit and an element whose flipped code would leave
+// the range is no candidate.
 //
 // What bounds it is the number of instructions (and their supply: code outside loops is fetched anew by every warp):
 //   - codes, error sums and dequantized weights leave as SQuant-E makes them, and SQuant-C corrects the few elements
@@ -119,9 +122,9 @@ __device__ __forceinline__ unsigned row_extremes(const int4 p)
 //     quarter of its vectors (both signs, 16 bits each) and makes those of the few quarters that come into question
 //     anew, which yields the code of what is flipped too;
 //   - only codes that are to be packed wait in shared memory.
-// Against the body of the groups, with which wide rows shared their code before: 256 rows of 100,352 weights 156 -> 83 us
-// on a B200 (the checked body of supplied scales until then).  Where row_body fits it is the slower one (4096 rows of 12,000 98.4 us, 89.6 in
-// row_body): the code that runs once counts.
+// Against the body of the groups, with which wide rows shared their code before: 256 rows of 100,352 weights 156 ->
+// 83 us on a B200 (the checked body of supplied scales until then).  Where row_body fits it is the slower one (4096
+// rows of 12,000 128 us with 512 threads, in row_body with 256 89.6): the code that runs once counts.
 template <bool kClip, Owner kOwn>
 __device__ __forceinline__ void long_row_body(const LayerDesc &L, int m, const Group &G, unsigned char *slice, int qmax, unsigned mode,
                                               int n0 = 0, int nloc = 0)
@@ -312,12 +315,15 @@ __device__ __forceinline__ void long_row_body(const LayerDesc &L, int m, const G
     }
 
     // ---- channel sum.  !kClip: its value modulo 2^32 is exact, its size is known from the float sums
-    // (a thread's fewer than 2^7 elements of at most one half give partial sums below 2^36, each addition off by at most 2^11, so
-    // its sum by less than 2^18; those of at most 2^12 threads by less than 2^30, and by 2^28 for the rounding to units of 2^17)
-    // The list of SQuant-C starts where the number of elements within `near` of one half leads one to expect somewhat more than k_c
-    // (near is in units of 2^16; evenly spread values have as many elements there as the channel sum's standard deviation).  The count travels with
-    // the channel sum, so that no barrier is spent on a search: 256 rows of 100,352 weights 76.9 -> 71.8 us a call on a B200, 8 of 200,000 19.2 -> 17.0,
-    // 1000 of 25,001 58.7 -> 56.4.  Too few seen (two bits and outliers) say nothing; a cluster then searches (256 rows of 100,352: 87.2 -> 88.8).
+    // (a thread's fewer than 2^7 elements of at most one half give partial sums below 2^36, each addition off by at
+    // most 2^11, so its sum by less than 2^18; those of at most 2^12 threads by less than 2^30, and by 2^28 for the
+    // rounding to units of 2^17)
+    // The list of SQuant-C starts where the number of elements within `near` of one half leads one to expect somewhat
+    // more than k_c (near is in units of 2^16; evenly spread values have as many elements there as the channel sum's
+    // standard deviation).  The count travels with the channel sum, so that no
+    // barrier is spent on a search: 256 rows of 100,352 weights 76.9 -> 71.8 us a call on a B200, 8 of 200,000 19.2
+    // -> 17.0, 1000 of 25,001 58.7 -> 56.4.  Too few seen (two bits and outliers) say nothing; a cluster then
+    // searches (256 rows of 100,352: 86.6 -> 88.1).
     constexpr int top = (kHalf >> 16) + 1;
     auto near_of = [](int n) { return min(max(__float2int_rn(0.58f * top * rsqrtf(static_cast<float>(n))), 1), top - 1); };
     int above = 0, below = 0;
