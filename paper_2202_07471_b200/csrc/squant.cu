@@ -460,13 +460,6 @@ int build_param_plan(const squant_layer *layers, int32_t n_layers, const squant_
         order.push_back(i);
         if (kernels) kernels[i] = SQUANT_KERNEL_GROUPED;
     }
-    // Larger kernels first, whose clusters run longer than those of rows, and long rows before shorter ones, so that short
-    // clusters end the call (us on a B200: 256 rows of 100,352 weights and then 64 channels of 8192 3x3 kernels 92.3, the other
-    // way round 87.0; 300 rows of 51,268, 150 channels of 5200 3x3 kernels, 9 rows of 200,001 and 6 channels of 19,000 as
-    // given 116.7, sorted 108.5; 40 rows of 100,352, 10 of 190,000 and 20 of 60,000, one wave, 32.5 and 33.3).
-    std::stable_sort(p.wide.begin(), p.wide.end(), [](const ParamPlan::Wide &a, const ParamPlan::Wide &b) {
-        return (a.d.K > 1) != (b.d.K > 1) ? a.d.K > 1 : a.d.K == 1 && a.d.N > b.d.N;
-    });
     // Long rows, a thread block per output channel, in one of three forms.  row_body holds 5 B of shared memory a
     // weight, long_row_body 4.  What counts is how many threads a multiprocessor holds and over how many vectors a
     // thread spreads the code that runs once.
@@ -623,8 +616,8 @@ int device_smem_limit(int device, int &limit)
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, v));
         SQ_CUDA(cudaFuncSetAttribute((sq::squant_row_kernel<512, false>),
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, v));
-        for (auto kernel : {sq::squant_wide_kernel<true>, sq::squant_wide_kernel<false>})
-            SQ_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, v));
+        SQ_CUDA(cudaFuncSetAttribute(sq::squant_wide_kernel,
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, v));
         SQ_CUDA(cudaFuncSetAttribute(sq::squant_stream_kernel<false>,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, v));
         SQ_CUDA(cudaFuncSetAttribute(sq::squant_stream_kernel<true>,
@@ -791,8 +784,7 @@ int launch_plan(const ParamPlan &p, cudaStream_t stream)
         if (rc) return rc;
     }
     for (const ParamPlan::Wide &w : p.wide) {   // one cluster per output channel
-        auto kernel = w.d.K == 1 ? sq::squant_wide_kernel<true> : sq::squant_wide_kernel<false>;
-        const int rc = launch(kernel, w.d.M * w.cluster, sq::kBlockThreads, w.smem, w.cluster, w.d, p.qmax, mode(), w.kpc);
+        const int rc = launch(sq::squant_wide_kernel, w.d.M * w.cluster, sq::kBlockThreads, w.smem, w.cluster, w.d, p.qmax, mode(), w.kpc);
         if (rc) return rc;
     }
     return SQUANT_OK;

@@ -529,10 +529,7 @@ __host__ __device__ inline long long wide_bytes(int kpc, int K, bool pack)
     return K == 1 ? long_row_bytes(kBlockThreads, (kpc + 6) >> 2, pack, kCluster) : conv_bytes(kBlockThreads, static_cast<int>(nk), K, kCluster);
 }
 
-// One output channel per cluster; grid = channels * cluster size.  kRows: 1x1 channels (L.off_vi = vectors of a run), else
-// larger kernels.  (Apart they keep all values in registers; with both in one kernel 8 B were spilled: 220 rows of 193,269
-// weights without SQuant-C 94.0 us on a B200, 93.5, 43 of 176,510 without its sums 26.5, 26.2.)
-template <bool kRows>
+// One output channel per cluster; grid = channels * cluster size.  L.off_vi = vectors of a run (1x1).
 __global__ void __launch_bounds__(kBlockThreads, 2)
 squant_wide_kernel(const LayerDesc L, int qmax, unsigned mode, int kpc)
 {
@@ -549,7 +546,7 @@ squant_wide_kernel(const LayerDesc L, int qmax, unsigned mode, int kpc)
     G.bar = 0;
     SQ_DBG(wide_bytes(kpc, L.K, (mode & kModePackInt4) != 0) <= static_cast<long long>(dynamic_smem_bytes()), 11);
     const bool range = L.sin != nullptr || L.N >= 65536;   // a flip can be barred by the clip range
-    if (kRows) {
+    if (L.K == 1) {
         if (L.sin) long_row_body<true, kCluster>(L, m, G, smem, qmax, mode, n0, nloc);
         else long_row_body<false, kCluster>(L, m, G, smem, qmax, mode, n0, nloc);
     } else if (L.K == 9 && (mode & 2u)) {
