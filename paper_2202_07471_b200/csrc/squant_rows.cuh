@@ -701,27 +701,10 @@ __device__ __forceinline__ unsigned row_vector_clip(const float4 w, const E2 &c2
 }
 
 // The loops over a thread's vectors, which lie kStep vectors apart (a constant: the addresses of a step are immediates).
-// kFew: at most two of them take a way of their own, shorter than what the unrolled loops leave for them (us a call on a
-// B200: 2000 rows of 256 weights 7.2 -> 6.8, of 200 8.1 -> 7.3, 700 of 461 8.0 -> 7.0, 256 of 1024 6.6 -> 6.4; two layers of 4096
-// of 4096 at 8 bit 55.5 -> 56.2).  Not in the bodies of supplied scales, which would spill 432 B instead of 180.
-template <int kStep, bool kFew>
+template <int kStep>
 __device__ __forceinline__ float row_stage(float4 *w, const float4 *src, int vecs, bool whole)
 {
     float amax = 0.0f;
-    if (kFew && __builtin_expect(whole && vecs <= 2, 0)) {
-        if (vecs > 0) copy_async16(w, src);
-        if (vecs > 1) copy_async16(w + kStep, src + kStep);
-        copy_async_wait();
-        if (vecs > 0) {
-            const float4 v = w[0];
-            amax = absmax3(absmax3(amax, v.x, v.y), v.z, v.w);
-        }
-        if (vecs > 1) {
-            const float4 v = w[kStep];
-            amax = absmax3(absmax3(amax, v.x, v.y), v.z, v.w);
-        }
-        return amax;
-    }
     if (whole) {
 #pragma unroll 4
         for (int i = 0; i < vecs; ++i) copy_async16(w + i * kStep, src + i * kStep);
@@ -823,7 +806,7 @@ __device__ __forceinline__ void row_body(const LayerDesc &L, int m, const Group 
         if (rag >= 0) copy_async4(Pel + rag, wrow + rag);
         const bool whole = (reinterpret_cast<uintptr_t>(src) & 15) == 0;
         if (kLanes != 0) {
-            amax = row_stage<kLanes ? kLanes : 1, kOwn == kGroup && kLanes == 32 && !kClip>(w, src, vecs, whole);
+            amax = row_stage<kLanes ? kLanes : 1>(w, src, vecs, whole);
         } else {
 #pragma unroll 1
             for (int i = 0; i < vecs; ++i) {
